@@ -23,11 +23,15 @@ constexpr int kOffW1 = 0, kOffB1 = kOffW1 + kMlpH * kMlpIn, kOffW2 = kOffB1 + kM
 constexpr int kFragL1 = 8 * 1 * 2 * 32, kFragL2 = 8 * 4 * 2 * 32, kFragL3 = 1 * 4 * 2 * 32;
 constexpr int kMlpSmemWords = kFragL1 + kFragL2 + kFragL3 + kMlpH + kMlpH + kMlpOut;
 
-// Fill the shared image from the BF16 blob (all threads of the block take part).
-__device__ __forceinline__ void mlp_stage(const __nv_bfloat16 *__restrict__ w, uint32_t *__restrict__ s) {
-  auto pk = [](const __nv_bfloat16 *p, int r, int c0, int ncol, int ld) -> uint32_t {
-    const unsigned short lo = c0 < ncol ? __bfloat16_as_ushort(p[r * ld + c0]) : 0;
-    const unsigned short hi = c0 + 1 < ncol ? __bfloat16_as_ushort(p[r * ld + c0 + 1]) : 0;
+__device__ __forceinline__ __nv_bfloat16 mlp_weight(__nv_bfloat16 w) { return w; }
+__device__ __forceinline__ __nv_bfloat16 mlp_weight(float w) { return __float2bfloat16_rn(w); }  // an FP32 master copy
+
+// Fill the shared image from the weight blob (all threads of the block take part).
+template <class T>
+__device__ __forceinline__ void mlp_stage(const T *__restrict__ w, uint32_t *__restrict__ s) {
+  auto pk = [](const T *p, int r, int c0, int ncol, int ld) -> uint32_t {
+    const unsigned short lo = c0 < ncol ? __bfloat16_as_ushort(mlp_weight(p[r * ld + c0])) : 0;
+    const unsigned short hi = c0 + 1 < ncol ? __bfloat16_as_ushort(mlp_weight(p[r * ld + c0 + 1])) : 0;
     return (uint32_t)lo | ((uint32_t)hi << 16);
   };
   for (int i = threadIdx.x; i < kFragL1 + kFragL2 + kFragL3; i += blockDim.x) {
@@ -56,7 +60,7 @@ __device__ __forceinline__ void mlp_stage(const __nv_bfloat16 *__restrict__ w, u
   float *bias = reinterpret_cast<float *>(s + kFragL1 + kFragL2 + kFragL3);
   for (int i = threadIdx.x; i < kMlpH + kMlpH + kMlpOut; i += blockDim.x) {
     const int o = i < kMlpH ? kOffB1 + i : (i < 2 * kMlpH ? kOffB2 + i - kMlpH : kOffB3 + i - 2 * kMlpH);
-    bias[i] = __bfloat162float(w[o]);
+    bias[i] = __bfloat162float(mlp_weight(w[o]));
   }
 }
 
