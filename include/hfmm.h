@@ -128,22 +128,19 @@ typedef struct {
                           does not depend on scheduling).  A leaf against itself stays one-sided.
                           Needs mac_mode 0 and size_rule 1 (the walk is then symmetric); ignores
                           use_graph.  The partials take 12 bytes per (entry, source particle). */
-  int list_init;       /* initial capacity, in entries, of every traversal list (frontier, M2L, P2P,
-                          segments, runs) of a new context: 0 = a guess scaled with n and leaf_max;
+  int list_init;       /* initial capacity, in entries, of every traversal list (open lists, M2L, P2P;
+                          k-d tree: frontier) of a new context: 0 = a guess scaled with n and leaf_max;
                           a small value makes the walk overflow and repeat with grown lists (the
                           lists come out the same either way) */
   int sink_batches;    /* hfmm_short_range_forces in batches of sinks (0 = automatic: one batch
                           while the first guess of the P2P list stays below 2^28 entries, else
                           batches of about 2^27 guessed entries; 1..4096 = that many).  The walk
-                          takes the top levels once (4, 5 or 6 of them as the batches grow),
-                          then each batch of sink cells (a contiguous Morton range, about equal
-                          particle counts) walks to the
-                          leaves, and its lists are grouped and evaluated before the next batch
-                          reuses the list memory, so memory and the 32-bit list bounds apply per
-                          batch.  The lists hold the same entries, split by sink; a leaf above
-                          the split level sums its entries in two groups (rounding differs from
-                          one batch in the last bits).  Not in graph mode; after a call in more than one
-                          batch the P2P / M2L lists cannot be exported. */
+                          visits the cells with children once, then each batch of leaves (a range
+                          of the leaves in breadth-first order, about equal numbers) is walked, and
+                          its lists are evaluated before the next batch reuses the list memory, so
+                          memory and the 32-bit list bounds apply per batch.  The lists hold the same
+                          entries, split by sink; a leaf's are all in its batch.  Not in graph mode;
+                          after a call in more than one batch the P2P / M2L lists cannot be exported. */
   int tree;            /* 0 = Morton octree (the default; every option above applies);
                           1 = the ORB / k-d tree of Sec. 2.1 (Fig. 1) and Sec. 4: a node of more than
                           leaf_max particles gives the first floor(n / 2) of them, in the order of

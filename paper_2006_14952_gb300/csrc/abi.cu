@@ -136,16 +136,14 @@ namespace {
 template <class F>
 void for_each_buffer(Ctx &c, F f) {
   DBuf *bufs[] = {&c.key, &c.key_alt, &c.idx, &c.idx_alt, &c.xs, &c.pm4, &c.perm, &c.cell, &c.range, &c.kids,
-                  &c.leaves, &c.bounds, &c.nkids, &c.koff, &c.front, &c.front_next, &c.cls, &c.counts, &c.offs,
+                  &c.leaves, &c.bounds, &c.nkids, &c.koff, &c.front, &c.front_next, &c.offs, &c.wnode, &c.wqueue, &c.wspill, &c.obeg, &c.ocnt, &c.open, &c.openc,
                   &c.m2l, &c.m2l_alt, &c.p2p, &c.p2p_alt, &c.m2l_beg, &c.m2l_end, &c.p2p_beg, &c.p2p_end, &c.M,
                   &c.L, &c.tmp, &c.tmp2, &c.d_small, &c.hpos, &c.hmass, &c.hacc, &c.m2l_mid, &c.tab,
-                  &c.mlp_w, &c.cand, &c.mlp_scratch, &c.fseg, &c.fseg_next, &c.seg_a, &c.seg_b, &c.acc_a,
-                  &c.acc_b, &c.segbase, &c.btot2, &c.rm_key, &c.rm_beg, &c.rm_cnt, &c.rp_key, &c.rp_beg,
-                  &c.rp_cnt, &c.segpre, &c.ctot, &c.tstate, &c.rm_rank, &c.rp_rank, &c.rcnt_m, &c.rcnt_p,
+                  &c.mlp_w, &c.cand, &c.mlp_scratch, &c.tstate,
                   &c.mut_cnt, &c.mut_poff, &c.mut_key, &c.mut_key_alt, &c.mut_val, &c.mut_val_alt,
                   &c.mut_bounds, &c.mut_small, &c.mut_part, &c.mut_lkey, &c.mut_lval, &c.lo_flag,
                   &c.lo_rank, &c.lo_meta, &c.lo_sink, &c.lo_tcnt, &c.lo_toff, &c.lo_scr,
-                  &c.pacc, &c.tf_pairs, &c.tf_segs, &c.tf_sst, &c.lpt_order, &c.lpt_tmp, &c.kd.xw,
+                  &c.pacc, &c.lpt_order, &c.lpt_tmp, &c.kd.xw,
                   &c.kd.ord[0], &c.kd.ord[1], &c.kd.ord[2], &c.kd.ord2[0], &c.kd.ord2[1], &c.kd.ord2[2],
                   &c.kd.side, &c.kd.flag, &c.kd.scan, &c.kd.pnode, &c.kd.nflag, &c.kd.nscan, &c.kd.first,
                   &c.kd.count, &c.kd.child, &c.kd.parent, &c.kd.axis, &c.kd.box, &c.kd.geo, &c.kd.geof, &c.kd.hs,
@@ -278,7 +276,6 @@ cudaError_t whole_call_graph(Ctx &c, float *acc, cudaStream_t st, bool prof, boo
   *ok = false;
   if (!c.gstream && (e = cudaStreamCreateWithFlags(&c.gstream, cudaStreamNonBlocking)) != cudaSuccess) return e;
   if ((e = traverse_graph_prepare(c)) != cudaSuccess) return e;
-  if ((e = sort_lists_prepare(c)) != cudaSuccess) return e;
   // during the capture the list sizes are their capacities on the host
   c.nm2l = (int64_t)c.cap_m2l;
   c.np2p = (int64_t)c.cap_p2p;
@@ -461,8 +458,8 @@ std::vector<uint64_t> step_signature(Ctx &c, const double *pos, const float *vel
   for (DBuf *b : pmb) v.push_back((uint64_t)(uintptr_t)b->p);
   uint64_t dtb;
   std::memcpy(&dtb, &dt, 8);
-  const uint64_t rest[] = {(uint64_t)c.n, c.cap_nodes, (uint64_t)c.cap_levels, c.cap_front, c.cap_m2l, c.cap_p2p,
-                           c.cap_seg, c.cap_run, (uint64_t)c.pm_plan_r2c, (uint64_t)c.pm_plan_c2r,
+  const uint64_t rest[] = {(uint64_t)c.n, c.cap_nodes, (uint64_t)c.cap_levels, c.cap_open, c.cap_m2l, c.cap_p2p,
+                           (uint64_t)c.pm_plan_r2c, (uint64_t)c.pm_plan_c2r,
                            (uint64_t)(uintptr_t)pos, (uint64_t)(uintptr_t)vel, (uint64_t)(uintptr_t)acc,
                            (uint64_t)(uintptr_t)c.mass_ref, dtb};
   v.insert(v.end(), rest, rest + sizeof(rest) / sizeof(rest[0]));
@@ -493,7 +490,6 @@ cudaError_t step_graph(Ctx &c, double *pos, float *vel, float *acc, double dt, c
   if ((e = ensure(c.M, eb)) != cudaSuccess) return e;
   if ((e = ensure(c.L, eb)) != cudaSuccess) return e;
   if ((e = traverse_graph_prepare(c)) != cudaSuccess) return e;
-  if ((e = sort_lists_prepare(c)) != cudaSuccess) return e;
   if ((e = pm_prepare(c)) != cudaSuccess) return e;
   std::vector<uint64_t> sig = step_signature(c, pos, vel, acc, dt);
   if (!c.gexec_step || sig != c.step_sig) {
@@ -736,6 +732,12 @@ int hfmm_get_stats(hfmm_ctx *h, hfmm_stats *o) {
   return HFMM_OK;
 }
 
+// The walk places each sink's entries together, the sinks in no fixed order: rows go out by
+// (order, sink), a sink's own entries in the order they are summed in.
+static void by_sink(std::vector<uint64_t> &v) {
+  std::stable_sort(v.begin(), v.end(), [](uint64_t a, uint64_t b) { return a >> kSinkShift < b >> kSinkShift; });
+}
+
 int hfmm_export(hfmm_ctx *h, int what, void *buf, size_t *bytes) {
   if (!h || !bytes) return HFMM_ERR_ARG;
   Ctx &c = h->c;
@@ -843,6 +845,7 @@ int hfmm_export(hfmm_ctx *h, int what, void *buf, size_t *bytes) {
       std::vector<uint64_t> v(c.nm2l);
       e = cudaMemcpy(v.data(), c.m2l.p, c.nm2l * 8, cudaMemcpyDeviceToHost);
       if (e != cudaSuccess) break;
+      by_sink(v);
       int64_t *o = static_cast<int64_t *>(buf);
       for (int64_t t = 0; t < c.nm2l; ++t) o[t] = pair_order(v[t]);
       break;
@@ -853,6 +856,7 @@ int hfmm_export(hfmm_ctx *h, int what, void *buf, size_t *bytes) {
       std::vector<uint64_t> v(cnt);
       e = cudaMemcpy(v.data(), (what == HFMM_EXPORT_P2P ? c.p2p : c.m2l).p, cnt * 8, cudaMemcpyDeviceToHost);
       if (e != cudaSuccess) break;
+      by_sink(v);
       int64_t *o = static_cast<int64_t *>(buf);
       for (int64_t t = 0; t < cnt; ++t) {
         o[3 * t] = pair_sink(v[t]);

@@ -323,28 +323,22 @@ struct Ctx {
   DBuf bounds, nkids, koff, tstate;  // build scratch
   uint64_t cap_nodes = 0;
 
-  // traversal
-  DBuf front, front_next, cls, counts, offs;
-  // sink-major walk: segment of each sink cell (per level), segment sinks and totals,
-  // segment bases, runs of M2L / P2P entries per (sink, level)
-  DBuf fseg, fseg_next, seg_a, seg_b, acc_a, acc_b, segbase, btot2, segpre, ctot;
-  DBuf rm_key, rm_beg, rm_cnt, rp_key, rp_beg, rp_cnt;
-  // runs per sink (counters during the walk) and each run's rank among its sink's runs
-  DBuf rm_rank, rp_rank, rcnt_m, rcnt_p;
-  uint64_t cap_seg = 0, cap_run = 0;
-  int64_t nrun_m = 0, nrun_p = 0, frontier_items = 0;
+  // traversal: node records, each node's parent's open list, open lists
+  DBuf wnode, wqueue, wspill, obeg, ocnt, open, openc;
+  DBuf front, front_next;  // k-d walk: frontier (ping-pong); its lists' sorts borrow them as scratch
+  DBuf offs;               // scan scratch
+  int64_t frontier_items = 0;
   DBuf m2l, m2l_alt, p2p, p2p_alt;  // packed u64 entries
   int64_t nm2l = 0, np2p = 0;
   int traverse_iters = 0;
   int64_t traverse_walks = 0;  // walks of the last traversal (1 + repeats after an overflow)
-  uint64_t cap_front = 0, cap_m2l = 0, cap_p2p = 0;  // traversal capacities (entries)
+  uint64_t cap_open = 0, cap_m2l = 0, cap_p2p = 0;  // traversal capacities (entries)
   int cap_levels = 0;  // graph mode: tree levels the level loops cover
   double walk_share = 1.0;  // sink batches: the share of the walk one batch takes (first list guesses)
   int last_batches = 1;     // sink batches of the last short-range call
   bool lists_split = false; // the last short-range call's lists were evaluated in parts (not kept)
   DBuf pacc;                // sink batches: P2P accelerations [3][n], added by L2P
   DBuf lpt_order, lpt_tmp;  // P2P: the sink leaves longest first, and its buckets and counters
-  DBuf tf_pairs, tf_segs, tf_sst;  // sink batches: the frontier the top levels leave
   DBuf m2l_beg, m2l_end, p2p_beg, p2p_end;  // u32 [nnodes] CSR bounds by sink
   DBuf m2l_mid;  // u32 [nnodes]: [beg, mid) table pairs, [mid, end) per-pair operator
 
@@ -442,8 +436,8 @@ cudaError_t m2l_pass_tc(Ctx &c, int q, cudaStream_t st);
 // (plus add[3][n], input order, when given).
 cudaError_t downward(Ctx &c, float *acc, cudaStream_t st, const float *add = nullptr);
 // The short-range call in sink batches (upward pass done by the caller; L must
-// be zero): the walk over the top levels, then per batch of sinks the rest of
-// the walk, list grouping, M2L and P2P (into c.pacc), then L2L and L2P + P2P.
+// be zero): the walk over the cells with children and their M2L, then per batch
+// of leaves the rest of the walk, M2L and P2P (into c.pacc), then L2L and L2P + P2P.
 cudaError_t short_range_batched(Ctx &c, float *acc, int nbatch, cudaStream_t st);
 // The batches the next short-range call takes (sink_batches, or the automatic count).
 int sink_batches_for(const Ctx &c);
@@ -458,7 +452,6 @@ void pm_release(Ctx &c);
 // walk fitted their capacities (device flags; null pointers: always).
 struct StepGuard {
   const int *tree_overflow = nullptr, *walk_overflow = nullptr;
-  const unsigned long long *walk_left = nullptr;
 };
 StepGuard step_guard(Ctx &c);
 cudaError_t kick_guarded(float *vel, const float *acc, int64_t n, double h, StepGuard g, cudaStream_t st);
@@ -468,13 +461,10 @@ cudaError_t drift(double *pos, const float *vel, int64_t n, double dt, double bo
 // Cut-off P2P, added to the accelerations written by downward().
 cudaError_t p2p_pass(Ctx &c, float *acc, cudaStream_t st);
 // Graph mode: the walk without its host read-back (sizes every buffer first; the
-// read-back after the graph reports whether the lists fit), and the device
-// address of the walk's run counts (0 M2L, 1 P2P).
+// read-back after the graph reports whether the lists fit).
 cudaError_t traverse_graph_prepare(Ctx &c);
 cudaError_t traverse_graph_launch(Ctx &c, cudaStream_t st);
 cudaError_t traverse_graph_finish(Ctx &c, cudaStream_t st, bool *ok);
-const unsigned long long *walk_run_counts(Ctx &c, int which);
-cudaError_t sort_lists_prepare(Ctx &c);
 // Graph mode for the step: the octree build without its read-back.
 cudaError_t build_tree_prepare(Ctx &c, int64_t n);
 cudaError_t build_tree_launch(Ctx &c, const double *pos, const float *mass, int64_t n, cudaStream_t st);

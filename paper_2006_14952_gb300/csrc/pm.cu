@@ -234,7 +234,7 @@ __global__ void k_interpolate(const double *__restrict__ xs, const uint32_t *__r
 
 __global__ void k_kick(float *__restrict__ vel, const float *__restrict__ acc, int64_t n3, float h, StepGuard g) {
   const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (g.tree_overflow && (*g.tree_overflow || *g.walk_overflow || *g.walk_left)) return;
+  if (g.tree_overflow && (*g.tree_overflow || *g.walk_overflow)) return;
   if (i < n3) vel[i] = fmaf(h, acc[i], vel[i]);
 }
 
