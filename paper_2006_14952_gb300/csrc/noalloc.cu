@@ -14,8 +14,8 @@ namespace {
 constexpr int64_t kNoAllocMaxN = HFMM_NOALLOC_MAX_N;
 constexpr size_t kAltKeyBytes = (size_t)kNoAllocMaxN * sizeof(uint64_t);
 constexpr size_t kAltIdxBytes = (size_t)kNoAllocMaxN * sizeof(uint32_t);
-// sort histograms / offsets / scan partials for kNoAllocMaxN keys, rounded up
-constexpr size_t kSortScratchBytes = (size_t)2 * 256 * ((kNoAllocMaxN + 2047) / 2048) * sizeof(uint32_t) + 4096;
+// the sort's digit totals and look-back tables for up to kNoAllocMaxN keys, rounded up
+constexpr size_t kSortScratchBytes = (size_t)2 * 256 * ((kNoAllocMaxN + 2047) / 2048) * sizeof(uint32_t) + 16384;
 constexpr size_t kScratchBytes = kAltKeyBytes + kAltIdxBytes + kSortScratchBytes;
 
 // Shared by every call on a device; held until the process exits.
