@@ -185,7 +185,7 @@ __host__ __device__ inline bool p2p_owner(uint32_t a, uint32_t b, uint32_t s, ui
 }
 
 // ---------------------------------------------------------------- tree sizes on the device
-// The octree build's sizes as its cooperative kernel leaves them (node count,
+// The octree build's sizes as its kernels leave them (node count,
 // leaf count, levels, first node of each level, capacity overflow).  In graph
 // mode the kernels after the build read their sizes here instead of taking
 // them from the host; an overflowed build reads as an empty tree.
@@ -320,7 +320,7 @@ struct Ctx {
   DBuf range;   // uint2 {first, count}
   DBuf kids;    // int2 {first child or -1, child count}
   DBuf leaves;  // u32 [nleaves] node index of each leaf
-  DBuf bounds, nkids, koff, tstate;  // build scratch
+  DBuf lev, lcnt, tstate;  // per particle its first own level and its leaf's; tile counts; sizes
   uint64_t cap_nodes = 0;
 
   // traversal: node records, each node's parent's open list, open lists

@@ -1,17 +1,23 @@
 // Octree build (Sec. 2.1, a tree with a leaf limiter; here a Morton octree):
-// periodic wrap, 63-bit Morton keys, stable key sort, level-synchronous split
-// of cells holding more than leaf_max particles, and per-particle FP32
-// offsets from the geometric centre of the leaf.
-#include <cooperative_groups.h>
-
+// periodic wrap, 63-bit Morton keys, stable key sort, the cells holding more than
+// leaf_max particles split, and per-particle FP32 offsets from the geometric
+// centre of the leaf.
+//
+// The nodes follow from the sorted keys alone, all levels at once.  Particle i
+// starts a cell on every level below those it shares with particle i - 1.  Its
+// cell on level l holds more than leaf_max particles, and is split, exactly when
+// some run of leaf_max + 1 sorted particles through i shares that level; so the
+// deepest split level of i is a sliding maximum of common levels (k_levels), and
+// particle i starts a node on the levels from its first own cell to its leaf.
+// Counting those per level and tile, one scan over the tiles (k_level_scan)
+// numbers the nodes breadth first, in key order within a level (k_nodes).
+#include <algorithm>
 #include <cstring>
 
 #include "common.cuh"
 
 namespace hfmm {
 namespace {
-
-namespace cg = cooperative_groups;
 
 __global__ void k_keys(const double *__restrict__ pos, int64_t n, double box, double inv_pow2, uint64_t *__restrict__ key,
                        uint32_t *__restrict__ idx) {
@@ -21,231 +27,302 @@ __global__ void k_keys(const double *__restrict__ pos, int64_t n, double box, do
   idx[i] = (uint32_t)i;
 }
 
-__global__ void k_gather(const double *__restrict__ pos, const uint32_t *__restrict__ idx, int64_t n, double box,
-                         double inv_pow2,
-                         double *__restrict__ xs) {
-  int64_t s = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (s >= n) return;
-  uint32_t i = idx[s];
-  xs[s] = wrap_box_fast(pos[i], box, inv_pow2);
-  xs[n + s] = wrap_box_fast(pos[n + i], box, inv_pow2);
-  xs[2 * n + s] = wrap_box_fast(pos[2 * n + i], box, inv_pow2);
+constexpr int kLT = 256;        // threads of the level kernels
+constexpr int kLTile = 1024;    // particles per tile
+constexpr int kHalo = 64;       // leaf_max is at most 64
+constexpr int kLCnt = 2 * (kDepth + 1);  // counters per tile: nodes by level, leaves by level
+
+// Levels two keys share: the common octant digits.
+__device__ __forceinline__ int common_level(uint64_t a, uint64_t b) {
+  const uint64_t x = a ^ b;
+  return x ? (__clzll((long long)x) - 1) / 3 : kDepth;
 }
 
-
-// FP64 offset from the geometric leaf centre, rounded once to FP32 (a thread
-// per leaf; the cell side L 2^-level built from its bits: no FP64 division).
-__global__ void k_leaf_offsets(const uint32_t *__restrict__ leaves, int64_t nl, const uint4 *__restrict__ cell,
-                               const uint2 *__restrict__ range, const double *__restrict__ xs,
-                               const float *__restrict__ mass, const uint32_t *__restrict__ perm, int64_t n,
-                               double box, float4 *__restrict__ pm4, const TreeState *tz) {
-  int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (t >= tree_leaves(tz, nl)) return;
-  uint32_t k = leaves[t];
-  uint4 c = cell[k];
-  uint2 r = range[k];
-  const double h = box * __longlong_as_double((long long)(1023 - (int)c.w) << 52);
-  double zx = ((double)c.x + 0.5) * h, zy = ((double)c.y + 0.5) * h, zz = ((double)c.z + 0.5) * h;
-  for (uint32_t i = r.x; i < r.x + r.y; ++i) {
-    pm4[i] = make_float4((float)(xs[i] - zx), (float)(xs[n + i] - zy), (float)(xs[2 * n + i] - zz), mass[perm[i]]);
+// lev[i]: the first level particle i starts a cell on (low byte), the level of its
+// leaf (high byte); it starts the nodes of the levels from the first to the second.
+// cnt[c][tile]: nodes (c < 22) and leaves (c - 22) by level that start in the tile.
+__global__ void __launch_bounds__(kLT) k_levels(const uint64_t *__restrict__ key, int64_t n, int leaf_max,
+                                                uint16_t *__restrict__ lev, uint32_t *__restrict__ cnt,
+                                                int64_t ntiles) {
+  __shared__ uint64_t k[kLTile + 2 * kHalo + 1];
+  __shared__ int8_t run[2][kLTile + kHalo];
+  __shared__ uint32_t c[kLCnt];
+  const int tid = threadIdx.x, lane = tid & 31;
+  const int64_t t0 = (int64_t)blockIdx.x * kLTile;
+  for (int q = tid; q < kLTile + 2 * kHalo + 1; q += kLT) {  // k[q]: particle t0 - kHalo - 1 + q
+    const int64_t g = t0 - kHalo - 1 + q;
+    k[q] = g >= 0 && g < n ? key[g] : 0ull;
   }
-}
-
-constexpr int kBT = 256;
-
-
-// Level-synchronous octree build in one cooperative launch (Sec. 2.1 tree, as a
-// Morton octree): per level every node with more than leaf_max particles (and
-// above the depth cap) is split at the octant boundaries of the sorted keys;
-// a grid-wide scan of the child counts places the children breadth-first (key
-// order within a level) and a scan of the leaf flags lists the leaves.  The
-// sizes stay on the device; the host reads them once at the end.
-__global__ void __launch_bounds__(kBT) k_tree_levels(const uint64_t *__restrict__ key, int64_t n, int leaf_max,
-                                                     uint4 *__restrict__ cell, uint2 *__restrict__ range,
-                                                     int2 *__restrict__ kids, uint32_t *__restrict__ leaves,
-                                                     unsigned long long capN, uint32_t *__restrict__ nk,
-                                                     uint32_t *__restrict__ bnd, unsigned long long *__restrict__ btot,
-                                                     TreeState *__restrict__ st, int max_levels) {
-  cg::grid_group grid = cg::this_grid();
-  __shared__ unsigned long long lo, cnt, total, nleaves;
-  __shared__ unsigned long long wsum[kBT / 32][2], pre[2], all[2], run[2];
-  const int tid = threadIdx.x, lane = tid & 31, wp = tid >> 5;
-  const unsigned nb = gridDim.x, bid = blockIdx.x;
-  if (bid == 0 && tid == 0) {
-    cell[0] = make_uint4(0, 0, 0, 0);
-    range[0] = make_uint2(0, (uint32_t)n);
-    st->level_start[0] = 0;
-  }
-  if (tid == 0) {
-    lo = 0;
-    cnt = 1;
-    total = 1;
-    nleaves = 0;
+  if (tid < kLCnt) c[tid] = 0u;
+  __syncthreads();
+  // run[q]: the level shared by particles j .. j + leaf_max, j = t0 - kHalo + q (-1: none)
+  for (int q = tid; q < kLTile + kHalo; q += kLT) {
+    const int64_t j = t0 - kHalo + q;
+    run[0][q] = (int8_t)(j >= 0 && j + leaf_max < n ? common_level(k[q + 1], k[q + 1 + leaf_max]) : -1);
   }
   __syncthreads();
-  grid.sync();
-  int level = 0;
-  for (; level <= kDepth; ++level) {
-    const unsigned long long L0 = lo, C = cnt, T0 = total, N0 = nleaves;
-    const unsigned long long ch = (C + nb - 1) / nb;
-    const unsigned long long blo = ch * bid < C ? ch * bid : C, bhi = blo + ch < C ? blo + ch : C;
-    // phase A: eight lanes per node, lane o finds the first key with octant digit >= o
-    // (independent searches over the node's range); child counts and block sums
-    unsigned long long sc = 0, sl = 0;
-    for (unsigned long long tb = 8 * blo; tb < 8 * bhi; tb += kBT) {  // uniform trip count (shuffles)
-      const unsigned long long tt = tb + tid, t = tt / 8;
-      const uint32_t o = (uint32_t)(tt % 8);
-      const bool valid = tt < 8 * bhi;
-      uint2 r = make_uint2(0, 0);
-      bool split = false;
-      if (valid) {
-        r = range[L0 + t];
-        split = (int)r.y > leaf_max && level < kDepth;
-      }
-      uint32_t bo = r.x;
-      if (split && o > 0) {
-        const int shift = 3 * (kDepth - level - 1);
-        uint32_t a = r.x, e = r.x + r.y;
-        while (a < e) {
-          const uint32_t mid = a + (e - a) / 2;
-          if (((uint32_t)(key[mid] >> shift) & 7u) < o)
-            a = mid + 1;
-          else
-            e = mid;
-        }
-        bo = a;
-      }
-      // boundary o + 1 from the next lane of the group (the last lane: the range end)
-      uint32_t bn = __shfl_down_sync(0xffffffffu, bo, 1, 8);
-      if (o == 7) bn = r.x + r.y;
-      const uint32_t nonempty = split && bn > bo ? 1u : 0u;
-      uint32_t c = nonempty;
-      c += __shfl_xor_sync(0xffffffffu, c, 1, 8);
-      c += __shfl_xor_sync(0xffffffffu, c, 2, 8);
-      c += __shfl_xor_sync(0xffffffffu, c, 4, 8);
-      if (valid) {
-        bnd[9 * t + o] = bo;
-        if (o == 7) bnd[9 * t + 8] = r.x + r.y;
-        if (o == 0) {
-          nk[t] = c;
-          sc += c;
-          sl += c == 0;
-        }
-      }
-    }
-    for (int o = 16; o; o >>= 1) {
-      sc += __shfl_xor_sync(0xffffffffu, sc, o);
-      sl += __shfl_xor_sync(0xffffffffu, sl, o);
-    }
-    if (lane == 0) {
-      wsum[wp][0] = sc;
-      wsum[wp][1] = sl;
+  // maxima of runs starting at q .. q + w - 1, w doubled while it fits the window of leaf_max + 1
+  int b = 0, w = 1;
+  for (; 2 * w <= leaf_max + 1; w *= 2, b ^= 1) {
+    for (int q = tid; q < kLTile + kHalo; q += kLT) {
+      const int o = q + w < kLTile + kHalo ? q + w : q;
+      run[b ^ 1][q] = run[b][q] > run[b][o] ? run[b][q] : run[b][o];
     }
     __syncthreads();
-    if (tid < 2) {
-      unsigned long long v = 0;
-      for (int q = 0; q < kBT / 32; ++q) v += wsum[q][tid];
-      btot[2 * bid + tid] = v;
+  }
+  for (int p = 0; p < kLTile; p += kLT) {
+    const int q = p + tid;
+    const int64_t i = t0 + q;
+    const bool valid = i < n;
+    uint32_t first = 255, last = 0;
+    if (valid) {
+      const int8_t m0 = run[b][q + kHalo - leaf_max], m1 = run[b][q + kHalo + 1 - w];
+      const int m = m0 > m1 ? m0 : m1;
+      last = (uint32_t)((m < kDepth ? m : kDepth - 1) + 1);  // cells on the deepest level are not split
+      first = i == 0 ? 0u : (uint32_t)(common_level(k[q + kHalo], k[q + kHalo + 1]) + 1);
+      lev[i] = (uint16_t)(first | (last << 8));
     }
-    __threadfence();
-    grid.sync();
-    // phase B: block prefixes, then each node's children and leaf slot
-    if (tid < 2) {
-      unsigned long long b = 0, a = 0;
-      for (unsigned q = 0; q < nb; ++q) {
-        const unsigned long long v = btot[2 * q + tid];
-        if (q < bid) b += v;
-        a += v;
+    const uint32_t lo = __reduce_min_sync(0xffffffffu, first), hi = __reduce_max_sync(0xffffffffu, last);
+    for (uint32_t l = lo; l <= hi; ++l) {
+      const unsigned nd = __ballot_sync(0xffffffffu, first <= l && l <= last);
+      const unsigned lf = __ballot_sync(0xffffffffu, first <= l && l == last);
+      if (lane == 0 && nd) atomicAdd(&c[l], (uint32_t)__popc(nd));
+      if (lane == 0 && lf) atomicAdd(&c[kDepth + 1 + l], (uint32_t)__popc(lf));
+    }
+  }
+  __syncthreads();
+  if (tid < kLCnt) cnt[(int64_t)tid * ntiles + blockIdx.x] = c[tid];
+}
+
+// Exclusive scan of each counter over the tiles, in place (a warp a counter), and
+// the tree's sizes.  base[c]: the first node (leaf) number of each level.
+__global__ void __launch_bounds__(1024) k_level_scan(uint32_t *__restrict__ cnt, int64_t ntiles,
+                                                     uint32_t *__restrict__ base, unsigned long long capN,
+                                                     int max_levels, TreeState *__restrict__ st) {
+  __shared__ unsigned long long tot[kLCnt];
+  const int lane = threadIdx.x & 31;
+  for (int c = threadIdx.x >> 5; c < kLCnt; c += 32) {
+    unsigned long long run = 0;
+    uint32_t *row = cnt + (int64_t)c * ntiles;
+    for (int64_t t = 0; t < ntiles; t += 128) {
+      uint32_t v[4], s = 0;
+#pragma unroll
+      for (int q = 0; q < 4; ++q) {
+        v[q] = t + 4 * lane + q < ntiles ? row[t + 4 * lane + q] : 0u;
+        s += v[q];
       }
-      pre[tid] = b;
-      all[tid] = a;
-      run[tid] = b;
-    }
-    __syncthreads();
-    const unsigned long long Cn = all[0], Ln = all[1];
-    // node capacity, or (graph mode) more levels than the host sized its level loops for
-    if (T0 + Cn > capN || (Cn > 0 && level + 2 > max_levels)) {
-      if (bid == 0 && tid == 0) st->overflow = 1;
-      break;  // every block takes the same decision
-    }
-    for (unsigned long long tb = blo; tb < bhi; tb += kBT) {
-      const unsigned long long t = tb + tid;
-      const bool valid = t < bhi;
-      const uint32_t c = valid ? nk[t] : 0u;
-      const unsigned long long lf = valid && c == 0 ? 1ull : 0ull;
-      unsigned long long xc = c, xl = lf;
+      uint32_t x = s;
 #pragma unroll
       for (int o = 1; o < 32; o <<= 1) {
-        const unsigned long long yc = __shfl_up_sync(0xffffffffu, xc, o), yl = __shfl_up_sync(0xffffffffu, xl, o);
-        if (lane >= o) {
-          xc += yc;
-          xl += yl;
-        }
+        const uint32_t y = __shfl_up_sync(0xffffffffu, x, o);
+        if (lane >= o) x += y;
       }
-      if (lane == 31) {
-        wsum[wp][0] = xc;
-        wsum[wp][1] = xl;
-      }
-      __syncthreads();
-      unsigned long long wc = 0, wl = 0, tc = 0, tl = 0;
-      for (int q = 0; q < kBT / 32; ++q) {
-        if (q < wp) {
-          wc += wsum[q][0];
-          wl += wsum[q][1];
-        }
-        tc += wsum[q][0];
-        tl += wsum[q][1];
-      }
-      if (valid) {
-        const unsigned long long k = L0 + t;
-        if (c == 0) {
-          kids[k] = make_int2(-1, 0);
-          leaves[N0 + run[1] + wl + xl - lf] = (uint32_t)k;
-        } else {
-          const unsigned long long base = T0 + run[0] + wc + xc - c;
-          kids[k] = make_int2((int)base, (int)c);
-          const uint4 pc = cell[k];
-          uint32_t b[9];
+      unsigned long long at = run + x - s;
 #pragma unroll
-          for (int o = 0; o < 9; ++o) b[o] = bnd[9 * t + o];
-          uint32_t q = 0;
-          for (uint32_t o = 0; o < 8; ++o) {
-            if (b[o + 1] > b[o]) {
-              cell[base + q] = make_uint4(2 * pc.x + ((o >> 2) & 1u), 2 * pc.y + ((o >> 1) & 1u), 2 * pc.z + (o & 1u),
-                                          pc.w + 1);
-              range[base + q] = make_uint2(b[o], b[o + 1] - b[o]);
-              ++q;
-            }
+      for (int q = 0; q < 4; ++q) {
+        if (t + 4 * lane + q < ntiles) row[t + 4 * lane + q] = (uint32_t)at;
+        at += v[q];
+      }
+      run += __shfl_sync(0xffffffffu, x, 31);
+    }
+    if (lane == 0) tot[c] = run;
+  }
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    unsigned long long nodes = 0, leaves = 0;
+    int levels = 0;
+    for (int l = 0; l <= kDepth; ++l) {
+      base[l] = (uint32_t)nodes;
+      base[kDepth + 1 + l] = (uint32_t)leaves;
+      st->level_start[l] = nodes;
+      nodes += tot[l];
+      leaves += tot[kDepth + 1 + l];
+      if (tot[l]) levels = l + 1;
+    }
+    for (int l = levels; l < kDepth + 3; ++l) st->level_start[l] = nodes;
+    st->total = nodes;
+    st->nleaves = leaves;
+    st->nlevels = levels;
+    // node capacity, or (graph mode) more levels than the host sized its level loops for
+    st->overflow = nodes > capN || levels > max_levels ? 1 : 0;
+  }
+}
+
+// Every third bit of v, packed (the inverse of spread3).
+__device__ __forceinline__ uint32_t pack3(uint64_t v) {
+  uint64_t x = v & 0x1249249249249249ull;
+  x = (x | (x >> 2)) & 0x10c30c30c30c30c3ull;
+  x = (x | (x >> 4)) & 0x100f00f00f00f00full;
+  x = (x | (x >> 8)) & 0x001f0000ff0000ffull;
+  x = (x | (x >> 16)) & 0x001f00000000ffffull;
+  x = (x | (x >> 32)) & 0x1fffffu;
+  return (uint32_t)x;
+}
+
+// The nodes each particle starts, and the particle itself: sorted wrapped position
+// and FP64 offset from the leaf's geometric centre, rounded once to FP32 (the cell
+// side L 2^-level built from its bits: no FP64 division).  Cells that split get
+// their first child here, their particle and child counts from k_node_counts.
+__global__ void __launch_bounds__(kLT) k_nodes(const uint64_t *__restrict__ key, const uint16_t *__restrict__ lev,
+                                               int64_t n, int leaf_max, const uint32_t *__restrict__ cnt,
+                                               const uint32_t *__restrict__ base, int64_t ntiles,
+                                               const TreeState *__restrict__ st, uint4 *__restrict__ cell,
+                                               uint2 *__restrict__ range, int2 *__restrict__ kids,
+                                               uint32_t *__restrict__ leaves, const double *__restrict__ pos,
+                                               const float *__restrict__ mass, const uint32_t *__restrict__ idx,
+                                               double box, double inv_pow2, double *__restrict__ xs,
+                                               float4 *__restrict__ pm4) {
+  constexpr int kRounds = kLTile / 32;  // 32 consecutive particles each
+  __shared__ uint16_t lv[kLTile + kHalo + 1];
+  __shared__ uint32_t wc[kRounds][kLCnt];
+  if (st->overflow) return;
+  const int tid = threadIdx.x, lane = tid & 31;
+  const uint32_t lt = (1u << lane) - 1u;
+  const int64_t t0 = (int64_t)blockIdx.x * kLTile;
+  for (int q = tid; q < kLTile + kHalo + 1; q += kLT) lv[q] = t0 + q < n ? lev[t0 + q] : (uint16_t)0;  // 0: ends every cell
+  for (int q = tid; q < kRounds * kLCnt; q += kLT) (&wc[0][0])[q] = 0u;
+  __syncthreads();
+  for (int p = 0; p < kLTile; p += kLT) {
+    const int q = p + tid;
+    const bool valid = t0 + q < n;
+    const uint32_t first = valid ? lv[q] & 255u : 255u, last = valid ? lv[q] >> 8 : 0u;
+    const uint32_t lo = __reduce_min_sync(0xffffffffu, first), hi = __reduce_max_sync(0xffffffffu, last);
+    for (uint32_t l = lo; l <= hi; ++l) {
+      const unsigned nd = __ballot_sync(0xffffffffu, first <= l && l <= last);
+      const unsigned lf = __ballot_sync(0xffffffffu, first <= l && l == last);
+      if (lane == 0) {
+        wc[q >> 5][l] = (uint32_t)__popc(nd);
+        wc[q >> 5][kDepth + 1 + l] = (uint32_t)__popc(lf);
+      }
+    }
+  }
+  __syncthreads();
+  if (tid < kLCnt) {
+    uint32_t at = base[tid] + cnt[(int64_t)tid * ntiles + blockIdx.x];
+    for (int q = 0; q < kRounds; ++q) {
+      const uint32_t v = wc[q][tid];
+      wc[q][tid] = at;
+      at += v;
+    }
+  }
+  __syncthreads();
+  for (int p = 0; p < kLTile; p += kLT) {
+    const int q = p + tid;
+    const int64_t i = t0 + q;
+    const bool valid = i < n;
+    const uint32_t first = valid ? lv[q] & 255u : 255u, last = valid ? lv[q] >> 8 : 0u;
+    const uint64_t ki = valid ? key[i] : 0ull;
+    const uint32_t cx = pack3(ki >> 2), cy = pack3(ki >> 1), cz = pack3(ki);
+    const uint32_t lo = __reduce_min_sync(0xffffffffu, first), hi = __reduce_max_sync(0xffffffffu, last);
+    uint32_t child = 0;  // this particle's node one level down
+    for (uint32_t l = hi + 1; l-- > lo;) {
+      const bool mine = first <= l && l <= last;
+      const unsigned nd = __ballot_sync(0xffffffffu, mine);
+      const unsigned lf = __ballot_sync(0xffffffffu, mine && l == last);
+      if (!mine) continue;
+      const uint32_t k = wc[q >> 5][l] + (uint32_t)__popc(nd & lt);
+      const uint32_t sh = kDepth - l;
+      cell[k] = make_uint4(cx >> sh, cy >> sh, cz >> sh, l);
+      uint32_t c = 0;
+      if (l == last) {
+        leaves[wc[q >> 5][kDepth + 1 + l] + (uint32_t)__popc(lf & lt)] = k;
+        kids[k] = make_int2(-1, 0);
+        // the leaf ends where a particle starts a cell on its level or above
+        c = 1;
+        while ((int)c <= leaf_max && (lv[q + c] & 255u) > l) ++c;
+        if ((int)c > leaf_max) {  // more than leaf_max particles on the deepest level: equal keys
+          int64_t a = i + c, e = n;
+          while (a < e) {
+            const int64_t mid = a + (e - a) / 2;
+            if (key[mid] == ki) a = mid + 1;
+            else e = mid;
           }
+          c = (uint32_t)(a - i);
         }
+      } else {
+        kids[k] = make_int2((int)child, 0);
       }
-      __syncthreads();
-      if (tid == 0) {
-        run[0] += tc;
-        run[1] += tl;
-      }
-      __syncthreads();
+      range[k] = make_uint2((uint32_t)i, c);
+      child = k;
     }
-    __threadfence();
-    __syncthreads();
-    if (tid == 0) {
-      lo = T0;
-      cnt = Cn;
-      total = T0 + Cn;
-      nleaves = N0 + Ln;
-    }
-    if (bid == 0 && tid == 0) st->level_start[level + 1] = T0;  // start of level + 1 (or the end)
-    grid.sync();
-    if (Cn == 0) {
-      ++level;
-      break;
+    if (valid) {
+      const uint32_t o = idx[i], sh = kDepth - last;
+      const double h = box * __longlong_as_double((long long)(1023 - (int)last) << 52);
+      const double x = wrap_box_fast(pos[o], box, inv_pow2), y = wrap_box_fast(pos[n + o], box, inv_pow2),
+                   z = wrap_box_fast(pos[2 * n + o], box, inv_pow2);
+      xs[i] = x;
+      xs[n + i] = y;
+      xs[2 * n + i] = z;
+      pm4[i] = make_float4((float)(x - ((double)(cx >> sh) + 0.5) * h), (float)(y - ((double)(cy >> sh) + 0.5) * h),
+                           (float)(z - ((double)(cz >> sh) + 0.5) * h), mass[o]);
     }
   }
-  if (bid == 0 && tid == 0) {
-    st->total = total;
-    st->nleaves = nleaves;
-    st->nlevels = level;
+}
+
+// Cells that split: the end of their particles (a search for the first key outside)
+// and how many nodes of the next level start before it.
+__global__ void k_node_counts(const uint64_t *__restrict__ key, int64_t n, int leaf_max,
+                              const TreeState *__restrict__ st, const uint4 *__restrict__ cell,
+                              uint2 *__restrict__ range, int2 *__restrict__ kids) {
+  if (st->overflow) return;
+  const int64_t nn = (int64_t)st->total, stride = (int64_t)gridDim.x * blockDim.x;
+  for (int64_t k = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; k < nn; k += stride) {
+    const int ch = kids[k].x;
+    if (ch < 0) continue;
+    const uint32_t l = cell[k].w, first = range[k].x;
+    const int sh = 3 * (kDepth - (int)l);
+    const uint64_t pre = key[first] >> sh;
+    int64_t a = (int64_t)first + leaf_max + 1, e = n;  // a split cell holds more than leaf_max
+    if (k + 1 < (int64_t)st->level_start[l + 1]) e = range[k + 1].x;
+    while (a < e) {
+      const int64_t mid = a + (e - a) / 2;
+      if ((key[mid] >> sh) == pre) a = mid + 1;
+      else e = mid;
+    }
+    int c = 1;
+    const int64_t next = (int64_t)st->level_start[l + 2];
+    while (c < 8 && ch + c < next && (int64_t)range[ch + c].x < a) ++c;
+    range[k].y = (uint32_t)(a - first);
+    kids[k].y = c;
   }
+}
+
+// Buffers of the levels for n particles and the node capacity.
+cudaError_t level_buffers(Ctx &c, int64_t n) {
+  cudaError_t e;
+  const int64_t ntiles = (n + kLTile - 1) / kLTile;
+  const size_t capN = (size_t)c.cap_nodes;
+  if ((e = ensure(c.lev, (size_t)n * 2)) != cudaSuccess) return e;
+  if ((e = ensure(c.lcnt, (size_t)(ntiles + 1) * kLCnt * 4)) != cudaSuccess) return e;
+  if ((e = ensure(c.tstate, sizeof(TreeState))) != cudaSuccess) return e;
+  if ((e = ensure(c.cell, capN * sizeof(uint4))) != cudaSuccess) return e;
+  if ((e = ensure(c.range, capN * sizeof(uint2))) != cudaSuccess) return e;
+  if ((e = ensure(c.kids, capN * sizeof(int2))) != cudaSuccess) return e;
+  return ensure(c.leaves, capN * sizeof(uint32_t));
+}
+
+// Keys sorted: the nodes and the particles in tree order, sizes in c.tstate (no read-back).
+//
+// What bounds it: the gathers of positions and masses in sorted order (k_nodes);
+// below 10^5 particles, four launches.  The level-synchronous build it replaced
+// (one cooperative launch, three grid barriers a level, then a thread a leaf for
+// the offsets), ms with its read-back, before and now: 0.54 -> 0.18 at 2M, 1.67 ->
+// 1.07 at 16M, 0.32 -> 0.06 at 262k, 0.17 -> 0.05 at 32k, 0.10 -> 0.05 at 1000.
+cudaError_t levels_launch(Ctx &c, const double *pos, const float *mass, int64_t n, int max_levels, cudaStream_t st) {
+  const int64_t ntiles = (n + kLTile - 1) / kLTile;
+  uint32_t *base = P<uint32_t>(c.lcnt), *cnt = base + kLCnt;
+  TreeState *ts = P<TreeState>(c.tstate);
+  const uint64_t *key = P<uint64_t>(c.key);
+  k_levels<<<(unsigned)ntiles, kLT, 0, st>>>(key, n, c.prm.leaf_max, P<uint16_t>(c.lev), cnt, ntiles);
+  k_level_scan<<<1, 1024, 0, st>>>(cnt, ntiles, base, c.cap_nodes, max_levels, ts);
+  k_nodes<<<(unsigned)ntiles, kLT, 0, st>>>(key, P<uint16_t>(c.lev), n, c.prm.leaf_max, cnt, base, ntiles, ts,
+                                            P<uint4>(c.cell), P<uint2>(c.range), P<int2>(c.kids),
+                                            P<uint32_t>(c.leaves), pos, mass, P<uint32_t>(c.idx), c.prm.box,
+                                            box_inverse_if_pow2(c.prm.box), P<double>(c.xs), P<float4>(c.pm4));
+  k_node_counts<<<std::min(blocks_for((size_t)c.cap_nodes, 128), 152u * 16u), 128, 0, st>>>(
+      key, n, c.prm.leaf_max, ts, P<uint4>(c.cell), P<uint2>(c.range), P<int2>(c.kids));
+  note_launch(4);
+  return cudaGetLastError();
 }
 
 }  // namespace
@@ -284,52 +361,21 @@ cudaError_t build_tree(Ctx &c, const double *pos, const float *mass, int64_t n, 
     std::swap(c.key, c.key_alt);
     std::swap(c.idx, c.idx_alt);
   }
-  uint64_t *key = P<uint64_t>(c.key);
-  uint32_t *perm = P<uint32_t>(c.idx);
   if (c.prm.profile & 1) cudaEventRecord(c.ev[1], st);
-  k_gather<<<blocks_for(n, T), T, 0, st>>>(pos, perm, n, c.prm.box, inv_pow2, P<double>(c.xs));
-  note_launch();
-
-  // octree levels: one cooperative launch; node capacity from the last build, grown on overflow
-  if (c.cap_nodes < (uint64_t)(2 * n / (c.prm.leaf_max > 1 ? c.prm.leaf_max : 1) + 64))
-    c.cap_nodes = (uint64_t)(2 * n / (c.prm.leaf_max > 1 ? c.prm.leaf_max : 1) + 64);
-  int dev = 0, nsm = 0, per_sm = 0;
-  TRY(cudaGetDevice(&dev));
-  TRY(cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev));
-  TRY(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_tree_levels, kBT, 0));
-  if (per_sm < 1) return cudaErrorInvalidConfiguration;
-  const unsigned nb = (unsigned)(nsm * (per_sm < 2 ? per_sm : 2));
+  // node capacity from the last build, grown to what an overflow asked for
+  c.cap_nodes = std::max<uint64_t>(c.cap_nodes, (uint64_t)(2 * n / (c.prm.leaf_max > 1 ? c.prm.leaf_max : 1) + 64));
   TreeState hs{};
-  TreeState *dst = reinterpret_cast<TreeState *>(c.tstate.p);
-  TRY(ensure(c.tstate, sizeof(TreeState)));
-  dst = reinterpret_cast<TreeState *>(c.tstate.p);
-  TRY(ensure(c.bounds, (size_t)nb * 2 * sizeof(unsigned long long)));
   for (int attempt = 0;; ++attempt) {
     if (attempt == 8) return cudaErrorInvalidValue;
-    const unsigned long long capN = c.cap_nodes;
-    TRY(ensure(c.cell, capN * sizeof(uint4)));
-    TRY(ensure(c.range, capN * sizeof(uint2)));
-    TRY(ensure(c.kids, capN * sizeof(int2)));
-    TRY(ensure(c.leaves, capN * sizeof(uint32_t)));
-    TRY(ensure(c.nkids, capN * sizeof(uint32_t)));
-    TRY(ensure(c.koff, capN * 9 * sizeof(uint32_t)));  // octant boundaries of a level's nodes
-    TRY(cudaMemsetAsync(dst, 0, sizeof(TreeState), st));
-    uint4 *cl = P<uint4>(c.cell);
-    uint2 *rg = P<uint2>(c.range);
-    int2 *kd = P<int2>(c.kids);
-    uint32_t *lv = P<uint32_t>(c.leaves), *nkp = P<uint32_t>(c.nkids), *bd = P<uint32_t>(c.koff);
-    unsigned long long *bt = P<unsigned long long>(c.bounds);
-    int lm = c.prm.leaf_max, ml = kDepth + 1;
-    int64_t nn = n;
-    void *args[] = {(void *)&key, (void *)&nn, (void *)&lm, (void *)&cl, (void *)&rg, (void *)&kd, (void *)&lv,
-                    (void *)&capN, (void *)&nkp, (void *)&bd, (void *)&bt, (void *)&dst, (void *)&ml};
-    TRY(cudaLaunchCooperativeKernel((const void *)k_tree_levels, dim3(nb), dim3(kBT), args, 0, st));
-    note_launch();
-    TRY(cudaMemcpyAsync(c.h_pinned, dst, sizeof(TreeState), cudaMemcpyDeviceToHost, st));
+    TRY(level_buffers(c, n));
+    TRY(levels_launch(c, pos, mass, n, kDepth + 1, st));
+    TRY(cudaMemcpyAsync(c.h_pinned, c.tstate.p, sizeof(TreeState), cudaMemcpyDeviceToHost, st));
     TRY(cudaStreamSynchronize(st));
     std::memcpy(&hs, c.h_pinned, sizeof(TreeState));
     if (!hs.overflow) break;
-    c.cap_nodes *= 2;
+    c.nnodes = (int64_t)hs.total;
+    if (hs.total >= (1ull << kSinkBits)) return cudaErrorInvalidValue;  // mapped to HFMM_ERR_CAPACITY
+    c.cap_nodes = std::max<uint64_t>(2 * c.cap_nodes, hs.total + hs.total / 2);
   }
   const int64_t total = (int64_t)hs.total;
   c.nlevels = hs.nlevels;
@@ -337,11 +383,6 @@ cudaError_t build_tree(Ctx &c, const double *pos, const float *mass, int64_t n, 
   c.nnodes = total;
   c.nleaves = (int64_t)hs.nleaves;
   if (total >= ((int64_t)1 << kSinkBits)) return cudaErrorInvalidValue;  // mapped to HFMM_ERR_CAPACITY
-  k_leaf_offsets<<<blocks_for(c.nleaves, T), T, 0, st>>>(P<uint32_t>(c.leaves), c.nleaves, P<uint4>(c.cell),
-                                                         P<uint2>(c.range), P<double>(c.xs), mass, perm, n,
-                                                         c.prm.box, P<float4>(c.pm4), nullptr);
-  note_launch();
-  TRY(cudaGetLastError());
   if (c.prm.profile & 1) cudaEventRecord(c.ev[2], st);
   c.have_tree = true;
   return cudaSuccess;
@@ -364,23 +405,11 @@ cudaError_t build_tree_prepare(Ctx &c, int64_t n) {
   TRY(ensure(c.xs, n * 24));
   TRY(ensure(c.pm4, n * 16));
   TRY(ensure(c.tmp, radix_sort_scratch_bytes((size_t)n)));
-  if (c.cap_nodes < (uint64_t)(2 * n / (c.prm.leaf_max > 1 ? c.prm.leaf_max : 1) + 64))
-    c.cap_nodes = (uint64_t)(2 * n / (c.prm.leaf_max > 1 ? c.prm.leaf_max : 1) + 64);
-  const unsigned long long capN = c.cap_nodes;
-  TRY(ensure(c.cell, capN * sizeof(uint4)));
-  TRY(ensure(c.range, capN * sizeof(uint2)));
-  TRY(ensure(c.kids, capN * sizeof(int2)));
-  TRY(ensure(c.leaves, capN * sizeof(uint32_t)));
-  TRY(ensure(c.nkids, capN * sizeof(uint32_t)));
-  TRY(ensure(c.koff, capN * 9 * sizeof(uint32_t)));
-  TRY(ensure(c.tstate, sizeof(TreeState)));
+  c.cap_nodes = std::max<uint64_t>(c.cap_nodes, (uint64_t)(2 * n / (c.prm.leaf_max > 1 ? c.prm.leaf_max : 1) + 64));
+  TRY(level_buffers(c, n));
   // levels the graph's level loops cover: the last tree's and two more
   if (c.cap_levels < c.nlevels + 2) c.cap_levels = c.nlevels + 2;
   if (c.cap_levels > kDepth + 1) c.cap_levels = kDepth + 1;
-  int dev = 0, nsm = 0;
-  TRY(cudaGetDevice(&dev));
-  TRY(cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev));
-  TRY(ensure(c.bounds, (size_t)nsm * 2 * 2 * sizeof(unsigned long long)));
   return cudaSuccess;
 #undef TRY
 }
@@ -402,44 +431,15 @@ cudaError_t build_tree_launch(Ctx &c, const double *pos, const float *mass, int6
     std::swap(c.key, c.key_alt);
     std::swap(c.idx, c.idx_alt);
   }
-  uint64_t *key = P<uint64_t>(c.key);
-  uint32_t *perm = P<uint32_t>(c.idx);
-  k_gather<<<blocks_for(n, T), T, 0, st>>>(pos, perm, n, c.prm.box, inv_pow2, P<double>(c.xs));
-  note_launch();
-  int dev = 0, nsm = 0, per_sm = 0;
-  if ((e = cudaGetDevice(&dev)) != cudaSuccess) return e;
-  if ((e = cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev)) != cudaSuccess) return e;
-  if ((e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_tree_levels, kBT, 0)) != cudaSuccess) return e;
-  if (per_sm < 1) return cudaErrorInvalidConfiguration;
-  const unsigned nb = (unsigned)(nsm * (per_sm < 2 ? per_sm : 2));
-  TreeState *dst = P<TreeState>(c.tstate);
-  if ((e = cudaMemsetAsync(dst, 0, sizeof(TreeState), st)) != cudaSuccess) return e;
-  unsigned long long capN = c.cap_nodes;
-  uint4 *cl = P<uint4>(c.cell);
-  uint2 *rg = P<uint2>(c.range);
-  int2 *kd = P<int2>(c.kids);
-  uint32_t *lv = P<uint32_t>(c.leaves), *nkp = P<uint32_t>(c.nkids), *bd = P<uint32_t>(c.koff);
-  unsigned long long *bt = P<unsigned long long>(c.bounds);
-  int lm = c.prm.leaf_max, ml = c.cap_levels;
-  int64_t nn = n;
-  void *args[] = {(void *)&key, (void *)&nn, (void *)&lm, (void *)&cl, (void *)&rg, (void *)&kd, (void *)&lv,
-                  (void *)&capN, (void *)&nkp, (void *)&bd, (void *)&bt, (void *)&dst, (void *)&ml};
-  if ((e = cudaLaunchCooperativeKernel((const void *)k_tree_levels, dim3(nb), dim3(kBT), args, 0, st)) != cudaSuccess)
-    return e;
-  note_launch();
-  k_leaf_offsets<<<blocks_for(c.cap_nodes, T), T, 0, st>>>(P<uint32_t>(c.leaves), (int64_t)c.cap_nodes,
-                                                           P<uint4>(c.cell), P<uint2>(c.range), P<double>(c.xs),
-                                                           mass, perm, n, c.prm.box, P<float4>(c.pm4), dst);
-  note_launch();
-  return cudaGetLastError();
+  return levels_launch(c, pos, mass, n, c.cap_levels, st);
 }
 
 // After the graph: the device state's sizes on the host.  False on an overflow
 // of the node or level capacity (both are then grown for the next capture).
 bool build_tree_finish(Ctx &c, const TreeState &hs) {
   if (hs.overflow) {
-    // which limit it was is not recorded: grow both (the direct rebuild sizes them exactly)
-    c.cap_nodes *= 2;
+    // which limit it was is not recorded: grow both
+    c.cap_nodes = std::max<uint64_t>(2 * c.cap_nodes, hs.total + hs.total / 2);
     c.cap_levels = c.cap_levels + 2 > kDepth + 1 ? kDepth + 1 : c.cap_levels + 2;
     return false;
   }
