@@ -63,8 +63,9 @@ __global__ void __launch_bounds__(256) k_mlp_infer(const __nv_bfloat16 *__restri
 // is split exactly into three BF16 terms (8 + 8 + 8 significant bits), three MMAs
 // whose products are again exact in FP32.  The tensor cores do not round their
 // accumulator to nearest: chained over all of a block's tiles the gradients came
-// out 2.4e-6 from the FP64 ones (3e-7 in FP32 arithmetic), so every 16 samples
-// start from zero and are added to the running sums in FP32.
+// out 2.4e-6 from the FP64 ones (3e-7 in FP32 arithmetic), and chained over a
+// layer's 64 inputs the bias of the logits alone moved them by 1e-6.  So every
+// MMA group sums 16 terms from zero, and the groups are added in FP32.
 //
 // The sample tile of 64 (16 rows a warp) keeps the staged operands within 73 KB,
 // so that three blocks share an SM: 12 warps cover the latency of the staging.
@@ -101,6 +102,14 @@ __device__ __forceinline__ void mma_bf16_1688(float (&c)[4], uint32_t a0, uint32
   asm volatile("mma.sync.aligned.m16n8k8.row.col.f32.bf16.bf16.f32 {%0,%1,%2,%3}, {%4,%5}, {%6}, {%0,%1,%2,%3};"
                : "+f"(c[0]), "+f"(c[1]), "+f"(c[2]), "+f"(c[3])
                : "r"(a0), "r"(a1), "r"(b0));
+}
+
+// c += a b with the products summed from zero and added in FP32.
+__device__ __forceinline__ void mma_add(float (&c)[4], const uint32_t (&a)[4], uint32_t b0, uint32_t b1) {
+  float p[4] = {0.f, 0.f, 0.f, 0.f};
+  mma_bf16_16816(p, a, b0, b1);
+#pragma unroll
+  for (int q = 0; q < 4; ++q) c[q] += p[q];
 }
 
 __device__ __forceinline__ void ldsm4t(uint32_t (&r)[4], const __nv_bfloat16 *p) {
@@ -183,9 +192,10 @@ __global__ void __launch_bounds__(kGradThreads, 3) k_mlp_grad(const float *__res
     uint32_t f[4][4], m1 = 0, m2 = 0;
 #pragma unroll
     for (int nt = 0; nt < 8; ++nt) {
-      const float b0 = bias[nt * 8 + 2 * t], b1 = bias[nt * 8 + 2 * t + 1];
-      float c[4] = {b0, b1, b0, b1};
+      float c[4] = {0.f, 0.f, 0.f, 0.f};
       mma_bf16_16816(c, a, sw[(nt * 2 + 0) * 32 + lane], sw[(nt * 2 + 1) * 32 + lane]);
+#pragma unroll
+      for (int q = 0; q < 4; ++q) c[q] += bias[nt * 8 + 2 * t + (q & 1)];
 #pragma unroll
       for (int q = 0; q < 4; ++q) m1 |= (c[q] > 0.f ? 1u : 0u) << (4 * nt + q);
       const uint32_t lo = pack_bf16(fmaxf(c[0], 0.f), fmaxf(c[1], 0.f));
@@ -198,11 +208,12 @@ __global__ void __launch_bounds__(kGradThreads, 3) k_mlp_grad(const float *__res
     uint32_t h2[4][4];
 #pragma unroll
     for (int nt = 0; nt < 8; ++nt) {
-      const float b0 = bias[kMlpH + nt * 8 + 2 * t], b1 = bias[kMlpH + nt * 8 + 2 * t + 1];
-      float c[4] = {b0, b1, b0, b1};
+      float c[4];
+#pragma unroll
+      for (int q = 0; q < 4; ++q) c[q] = bias[kMlpH + nt * 8 + 2 * t + (q & 1)];
 #pragma unroll
       for (int kt = 0; kt < 4; ++kt)
-        mma_bf16_16816(c, f[kt], s2[((nt * 4 + kt) * 2 + 0) * 32 + lane], s2[((nt * 4 + kt) * 2 + 1) * 32 + lane]);
+        mma_add(c, f[kt], s2[((nt * 4 + kt) * 2 + 0) * 32 + lane], s2[((nt * 4 + kt) * 2 + 1) * 32 + lane]);
 #pragma unroll
       for (int q = 0; q < 4; ++q) m2 |= (c[q] > 0.f ? 1u : 0u) << (4 * nt + q);
       const uint32_t lo = pack_bf16(fmaxf(c[0], 0.f), fmaxf(c[1], 0.f));
@@ -215,8 +226,7 @@ __global__ void __launch_bounds__(kGradThreads, 3) k_mlp_grad(const float *__res
     const float b0 = bias[2 * kMlpH + 2 * t], b1 = bias[2 * kMlpH + 2 * t + 1];
     float z[4] = {b0, b1, b0, b1};
 #pragma unroll
-    for (int kt = 0; kt < 4; ++kt)
-      mma_bf16_16816(z, h2[kt], s3[(kt * 2 + 0) * 32 + lane], s3[(kt * 2 + 1) * 32 + lane]);
+    for (int kt = 0; kt < 4; ++kt) mma_add(z, h2[kt], s3[(kt * 2 + 0) * 32 + lane], s3[(kt * 2 + 1) * 32 + lane]);
     // ---- softmax over the quad's 8 logits of each row, loss, d3 = weight (p - onehot)
     float mx0 = fmaxf(z[0], z[1]), mx8 = fmaxf(z[2], z[3]);
 #pragma unroll
@@ -324,10 +334,14 @@ __global__ void __launch_bounds__(kGradThreads, 3) k_mlp_grad(const float *__res
     for (int nt = 0; nt < 8; ++nt) {
       float c[4] = {0.f, 0.f, 0.f, 0.f};
 #pragma unroll
-      for (int q = 2; q >= 0; --q)
+      for (int kt = 0; kt < 4; ++kt) {
+        float p[4] = {0.f, 0.f, 0.f, 0.f};
 #pragma unroll
-        for (int kt = 0; kt < 4; ++kt)
-          mma_bf16_16816(c, d2[q][kt], w2t[((kt * 8 + nt) * 2 + 0) * 32 + lane], w2t[((kt * 8 + nt) * 2 + 1) * 32 + lane]);
+        for (int q = 2; q >= 0; --q)
+          mma_bf16_16816(p, d2[q][kt], w2t[((kt * 8 + nt) * 2 + 0) * 32 + lane], w2t[((kt * 8 + nt) * 2 + 1) * 32 + lane]);
+#pragma unroll
+        for (int q = 0; q < 4; ++q) c[q] += p[q];
+      }
 #pragma unroll
       for (int q = 0; q < 4; ++q) c[q] = (m1 >> (4 * nt + q)) & 1u ? c[q] : 0.f;
       uint32_t w0[3], w8[3];
