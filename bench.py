@@ -45,10 +45,11 @@ UNIT = "forces/s"
 FP32_LANES_PER_SM = 128
 N_SM = 152
 # FP32 work of one P2P pair inside the cut-off (FMA = 2 flop): separation (3),
-# r^2 (1 mul + 2 fma = 5), rsqrt (1), u = r^2 r^-1 - R_c / 2 (1 fma = 2), the
-# truncation factor S = exp2(r^2 k) Q(u) with Q of degree 9 (exponent 1 +
-# exp2 1 + 9 fma 18 + product 1 = 21), -S m / r^3 (4), accumulation (3 fma = 6).
-P2P_FLOPS_PER_PAIR = 42
+# r^2 (1 mul + 2 fma = 5), rsqrt (1), the truncation factor over r, Q / r = P(v) / r + a
+# with v = 1 / (1/r + p) and P of degree 4 (add 1 + reciprocal 1 + 4 fma 8 + 1 fma 2 =
+# 12), exp2(r^2 k) (1 + 1), r^-2 and the products with it and m (4), accumulation
+# (3 fma = 6).
+P2P_FLOPS_PER_PAIR = 33
 # The same count for the polynomial split (Sec. 5): separation 3, r^2 5,
 # rsqrt 1, r^-3 2, -(r^-3 + c0 + c1 r^2) m (1 fma + 1 add + 1 mul = 4),
 # accumulation 6.

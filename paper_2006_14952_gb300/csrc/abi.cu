@@ -5,6 +5,7 @@
 #include <cstdio>
 #include <cstring>
 #include <new>
+#include <utility>
 #include <vector>
 
 #include "common.cuh"
@@ -93,36 +94,83 @@ void mac_integer_thresholds(Ctx &c) {
   }
 }
 
+namespace {
+
+// Solve the n x n system A x = b in place (Gaussian elimination, partial pivoting); false if singular.
+bool solve_small(int n, double (*A)[6], double *b) {
+  for (int k = 0; k < n; ++k) {
+    int piv = k;
+    for (int i = k + 1; i < n; ++i)
+      if (std::fabs(A[i][k]) > std::fabs(A[piv][k])) piv = i;
+    if (!(std::fabs(A[piv][k]) > 0)) return false;
+    for (int j = 0; j < n; ++j) std::swap(A[k][j], A[piv][j]);
+    std::swap(b[k], b[piv]);
+    for (int i = k + 1; i < n; ++i) {
+      const double f = A[i][k] / A[k][k];
+      for (int j = k; j < n; ++j) A[i][j] -= f * A[k][j];
+      b[i] -= f * b[k];
+    }
+  }
+  for (int k = n - 1; k >= 0; --k) {
+    for (int j = k + 1; j < n; ++j) b[k] -= A[k][j] * b[j];
+    b[k] /= A[k][k];
+  }
+  return true;
+}
+
+}  // namespace
+
 PairFit fit_pair_factor(double rs, double rc) {
-  constexpr int N = 10;
-  const double pi = 3.14159265358979323846;
-  const double xc = rc / rs;
-  double fk[N], cj[N], T[N + 1][N], mono[N];
-  for (int k = 0; k < N; ++k) {
-    double t = 0.5 * (1.0 + std::cos(pi * (k + 0.5) / N));
-    double x = xc * t;
-    fk[k] = std::exp(0.25 * x * x) * std::erfc(0.5 * x) + x / std::sqrt(pi);
+  const double pi = 3.14159265358979323846, xc = rc / rs;
+  auto q_of = [&](double x) { return std::exp(0.25 * x * x) * std::erfc(0.5 * x) + x / std::sqrt(pi); };
+  // basis at x: (v / v_c)^k, k = 0..4, then x / x_c; v = x / (1 + p x)
+  auto basis = [&](double x, double p, double (&f)[6]) {
+    const double v = x / (1.0 + p * x) * (1.0 + p * xc) / xc;
+    f[0] = 1.0;
+    for (int k = 1; k < 5; ++k) f[k] = f[k - 1] * v;
+    f[5] = x / xc;
+  };
+  constexpr int kTest = 49;
+  double xt[kTest], qt[kTest];
+  for (int i = 0; i < kTest; ++i) {
+    xt[i] = xc * i / (kTest - 1);
+    qt[i] = q_of(xt[i]);
   }
-  for (int j = 0; j < N; ++j) {
-    double s = 0.0;
-    for (int k = 0; k < N; ++k) s += fk[k] * std::cos(pi * j * (k + 0.5) / N);
-    cj[j] = (j == 0 ? 1.0 : 2.0) * s / N;
+  double best = 1e300, bc[6] = {1, 0, 0, 0, 0, 0}, bp = 0.2;
+  for (int ip = 0; ip < 13; ++ip) {
+    const double p = 0.1 + 0.025 * ip, vc = xc / (1.0 + p * xc);
+    for (int n = 5; n <= 6; ++n) {  // without and with the linear term
+      double A[6][6], c[6] = {0, 0, 0, 0, 0, 0};
+      for (int i = 0; i < n; ++i) {
+        const double v = vc * 0.5 * (1.0 - std::cos(pi * (i + 0.5) / n)), x = v / (1.0 - p * v);
+        basis(x, p, A[i]);
+        c[i] = q_of(x);
+      }
+      if (!solve_small(n, A, c)) continue;
+      // the largest relative error, with half an FP32 unit of every term's size
+      double cost = 0.0;
+      for (int i = 0; i < kTest; ++i) {
+        double f[6], s = 0.0, t = 0.0;
+        basis(xt[i], p, f);
+        for (int k = 0; k < n; ++k) {
+          s += c[k] * f[k];
+          t += std::fabs(c[k] * f[k]);
+        }
+        cost = std::max(cost, std::fabs(s / qt[i] - 1.0) + std::ldexp(t / qt[i], -24));
+      }
+      if (cost < best) {
+        best = cost;
+        bp = p;
+        for (int k = 0; k < 6; ++k) bc[k] = c[k];
+      }
+    }
   }
-  // T_j(s) as monomial coefficients in s = 2r / R_c - 1 (the interval's midpoint at 0)
-  std::memset(T, 0, sizeof(T));
-  T[0][0] = 1.0;
-  T[1][1] = 1.0;
-  for (int j = 1; j + 1 < N; ++j)
-    for (int i = 0; i < N; ++i) T[j + 1][i] = (i ? 2.0 * T[j][i - 1] : 0.0) - T[j - 1][i];
-  for (int i = 0; i < N; ++i) {
-    mono[i] = 0.0;
-    for (int j = 0; j < N; ++j) mono[i] += cj[j] * T[j][i];
-  }
-  // in powers of u = r - R_c / 2 (s = u * 2 / R_c): small coefficients, a well-conditioned Horner sum
   PairFit f;
+  const double vc = rs * xc / (1.0 + bp * xc);
   double sc = 1.0;
-  for (int i = 0; i < N; ++i, sc *= 2.0 / rc) f.c[i] = (float)(mono[i] * sc);
-  f.rmid = (float)(0.5 * rc);
+  for (int k = 0; k < 5; ++k, sc /= vc) f.c[k] = (float)(bc[k] * sc);
+  f.a = (float)(bc[5] / rc);
+  f.p = (float)(bp / rs);
   f.rc2 = (float)(rc * rc);
   f.kexp = (float)(-1.4426950408889634 / (4.0 * rs * rs));
   return f;

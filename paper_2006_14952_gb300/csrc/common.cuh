@@ -250,20 +250,23 @@ cudaError_t radix_sort_u64_into(uint64_t *keys, uint32_t *vals, uint64_t *keys_a
                                 cudaStream_t st);
 
 // ---------------------------------------------------------------- pair force
-// S(x) = erfc(x/2) + x e^(-x^2/4) / sqrt(pi) = exp2(r^2 kexp) Q(r / R_c),
-// Q(t) = sum_j c[j] t^j (degree 9), kexp = -log2(e) / (4 r_s^2).
 // 1/L when the box side L is a power of two (then exact), else 0
 inline double box_inverse_if_pow2(double box) {
   int e = 0;
   return std::frexp(box, &e) == 0.5 ? 1.0 / box : 0.0;
 }
 
+// S(x) = erfc(x/2) + x e^(-x^2/4) / sqrt(pi) = exp2(r^2 kexp) Q(x), x = r / r_s,
+// Q(x) = e^(x^2/4) erfc(x/2) + x / sqrt(pi), kexp = -log2(e) / (4 r_s^2).  Q is
+// evaluated as sum_k c[k] v^k + a r, v = r / (1 + p r): the first part decays like
+// 1/x, which a degree-4 polynomial in v follows to 5.5e-7 at R_c = 4.5 r_s (a
+// polynomial in r needs degree 9 for 1.2e-6), and v = 1 / (1/r + p) is one
+// reciprocal.
 struct PairFit {
-  float c[10];  // Q = sum_i c[i] u^i, u = r - rmid
-  float rmid, rc2, kexp;
+  float c[5], a, p, rc2, kexp;
 };
-// Chebyshev interpolation (10 nodes on [0, R_c]) of e^(x^2/4) erfc(x/2) + x/sqrt(pi),
-// x = r / r_s, in FP64, expanded in powers of u = r - R_c / 2 and rounded to FP32.
+// Interpolation of Q on [0, R_c] at Chebyshev nodes in v, in FP64; p (in units of
+// 1 / r_s, 0.1 .. 0.4) and whether a is used are chosen for the smallest error.
 PairFit fit_pair_factor(double rs, double rc);
 struct Ctx;
 void mac_integer_thresholds(Ctx &c);

@@ -531,7 +531,7 @@ constexpr int kKdStage = 64;
 // kCount (statistics runs): also count the pairs inside (0, R_c) into *useful.
 // kSplit: 0 the Gaussian pair force of Sec. 2.2, 1 the polynomial one of Sec. 5.
 template <bool kCount, int kSplit>
-__global__ void __launch_bounds__(kT) k_kd_p2p(const uint32_t *__restrict__ leaves, int64_t nl,
+__global__ void __launch_bounds__(kT, 2) k_kd_p2p(const uint32_t *__restrict__ leaves, int64_t nl,
                                                const uint32_t *__restrict__ first, const uint32_t *__restrict__ count,
                                                KdGeo Gm, const uint32_t *__restrict__ beg,
                                                const uint32_t *__restrict__ end, const uint64_t *__restrict__ lst,
@@ -655,20 +655,7 @@ __global__ void __launch_bounds__(kT) k_kd_p2p(const uint32_t *__restrict__ leav
         const bool in0 = r2.x < fit.rc2 && r2.x > 0.f, in1 = r2.y < fit.rc2 && r2.y > 0.f;
         if (kCount && real) n_in += (uint32_t)in0 + (uint32_t)in1;
         // outside (0, R_c) the values below may be inf / NaN; the selects discard them
-        const float2 ri = make_float2(rsqrt_mufu(r2.x), rsqrt_mufu(r2.y));
-        const float2 r3 = __fmul2_rn(__fmul2_rn(ri, ri), ri);
-        float2 fs;
-        if constexpr (kSplit == 1) {
-          // m (1/r^3 - 5 / (2 R_c^3) + 3 r^2 / (2 R_c^5))
-          fs = __fmul2_rn(__fadd2_rn(r3, __ffma2_rn(r2, fit.pc1, fit.pc0)), w);
-        } else {
-          const float2 u = __ffma2_rn(r2, ri, fit.nrmid);  // r - R_c / 2
-          float2 qv = fit.c[9];
-#pragma unroll
-          for (int i = 8; i >= 0; --i) qv = __ffma2_rn(qv, u, fit.c[i]);
-          const float2 ea = __fmul2_rn(r2, fit.kexp);
-          fs = __fmul2_rn(__fmul2_rn(__fmul2_rn(make_float2(exp2_mufu(ea.x), exp2_mufu(ea.y)), qv), r3), w);
-        }
+        float2 fs = __fmul2_rn(pair_factor2<kSplit>(r2, fit), w);
         fs.x = in0 ? fs.x : 0.f;
         fs.y = in1 ? fs.y : 0.f;
         ax = __ffma2_rn(fs, dx, ax);
@@ -684,7 +671,7 @@ __global__ void __launch_bounds__(kT) k_kd_p2p(const uint32_t *__restrict__ leav
           pair2(px, py, pz, w, n1x, n1y, n1z, a1x, a1y, a1z, has1);
         }
       } else {
-#pragma unroll 4
+#pragma unroll 8
         for (uint32_t j = 0; j < kept; j += 2) {
           const float2 px = *reinterpret_cast<const float2 *>(X + j), py = *reinterpret_cast<const float2 *>(Y + j);
           const float2 pz = *reinterpret_cast<const float2 *>(Z + j), w = *reinterpret_cast<const float2 *>(Wm + j);

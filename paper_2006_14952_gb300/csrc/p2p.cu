@@ -32,10 +32,7 @@
 // massless source far outside the cut-off.
 //
 // Pair force (Gaussian split): a = -m S(x) r / r^3, S(x) = erfc(x/2) + x e^(-x^2/4) / sqrt(pi),
-// x = r / r_s, evaluated as S = exp2(-x^2 log2(e) / 4) * Q(r) with Q a degree-9
-// polynomial interpolating e^(x^2/4) erfc(x/2) + x / sqrt(pi) at Chebyshev
-// nodes on [0, R_c], expanded in powers of u = r - R_c / 2 (coefficients from
-// the host, fit_pair_factor()).
+// x = r / r_s, evaluated as in PairFit (common.cuh) and pair_factor2 (p2p_common.cuh).
 #include "p2p_common.cuh"
 
 namespace hfmm {
@@ -317,21 +314,7 @@ __global__ void __launch_bounds__(256, 2) k_p2p(const uint32_t *__restrict__ ite
           const bool in1 = (r2.y < fit.rc2) && (r2.y > 0.f);
           if (kCount) n_in += (uint32_t)in0 + (uint32_t)in1;
           // outside (0, R_c) the values below may be inf/NaN; the selects discard them
-          const float2 rinv = make_float2(rsqrt_mufu(r2.x), rsqrt_mufu(r2.y));
-          const float2 r3 = __fmul2_rn(__fmul2_rn(rinv, rinv), rinv);
-          float2 f;
-          if constexpr (kSplit == 1) {
-            // -m (1/r^3 - 5 / (2 R_c^3) + 3 r^2 / (2 R_c^5))
-            f = __fmul2_rn(__fadd2_rn(r3, __ffma2_rn(r2, fit.pc1, fit.pc0)), make_float2(B.z, B.w));
-          } else {
-            const float2 tt = __ffma2_rn(r2, rinv, fit.nrmid);  // u = r - R_c / 2
-            float2 qv = fit.c[9];
-#pragma unroll
-            for (int j = 8; j >= 0; --j) qv = __ffma2_rn(qv, tt, fit.c[j]);
-            const float2 ea = __fmul2_rn(r2, fit.kexp);
-            const float2 sfac = __fmul2_rn(make_float2(exp2_mufu(ea.x), exp2_mufu(ea.y)), qv);
-            f = __fmul2_rn(__fmul2_rn(sfac, r3), make_float2(B.z, B.w));  // -S m / r^3
-          }
+          float2 f = __fmul2_rn(pair_factor2<kSplit>(r2, fit), make_float2(B.z, B.w));  // w = -m
           f.x = in0 ? f.x : 0.f;
           f.y = in1 ? f.y : 0.f;
           sx = __ffma2_rn(f, dx, sx);

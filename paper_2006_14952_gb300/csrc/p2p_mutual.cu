@@ -308,19 +308,7 @@ __global__ void __launch_bounds__(256, 2)
                 const bool in1 = (r2.y < fit.rc2) && (r2.y > 0.f);
                 if (kCount)
                   n_in += (uint32_t)in0 * (s0[u] != kNoSlot ? 2u : 1u) + (uint32_t)in1 * (s1[u] != kNoSlot ? 2u : 1u);
-                const float2 rinv = make_float2(rsqrt_mufu(r2.x), rsqrt_mufu(r2.y));
-                const float2 r3 = __fmul2_rn(__fmul2_rn(rinv, rinv), rinv);
-                float2 g;  // -f_(1)(r): S / r^3 (Gaussian) or 1/r^3 - 5 / (2 R_c^3) + 3 r^2 / (2 R_c^5)
-                if constexpr (kSplit == 1) {
-                  g = __fadd2_rn(r3, __ffma2_rn(r2, fit.pc1, fit.pc0));
-                } else {
-                  const float2 tt = __ffma2_rn(r2, rinv, fit.nrmid);
-                  float2 qv = fit.c[9];
-#pragma unroll
-                  for (int j = 8; j >= 0; --j) qv = __ffma2_rn(qv, tt, fit.c[j]);
-                  const float2 ea = __fmul2_rn(r2, fit.kexp);
-                  g = __fmul2_rn(__fmul2_rn(make_float2(exp2_mufu(ea.x), exp2_mufu(ea.y)), qv), r3);
-                }
+                float2 g = pair_factor2<kSplit>(r2, fit);
                 g.x = in0 ? g.x : 0.f;
                 g.y = in1 ? g.y : 0.f;
                 // on the sink: m_j f_(1) d = (-m_j) g d; on the sources: m_i g d
