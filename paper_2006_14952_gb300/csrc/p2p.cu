@@ -38,6 +38,14 @@
 namespace hfmm {
 namespace {
 
+// Order of the work items (k_lpt_hist, k_lpt_place): items and work by bucket, placing cursors.
+constexpr int kLptBuckets = 64;
+constexpr unsigned kLptWarps = 152 * 16;  // warps the GPU holds of k_p2p
+struct LptState {
+  unsigned long long work;
+  unsigned n_items, pad;
+  unsigned hist[kLptBuckets], cursor[kLptBuckets];
+};
 
 // kCap: source particles per fill (even); dynamic shared memory: 2 x 8 x kCap float4.
 // kSplit 0: the Gaussian truncation S(x) above; 1: the polynomial truncation of
@@ -50,9 +58,26 @@ __global__ void __launch_bounds__(256, 2) k_p2p(const uint32_t *__restrict__ ite
                                                 const uint64_t *__restrict__ lst, const float4 *__restrict__ pm4,
                                                 const uint32_t *__restrict__ perm, int64_t n, float box, PairFit2 fit,
                                                 float G, float *__restrict__ acc_out,
-                                                unsigned long long *__restrict__ ctr, const unsigned *__restrict__ n_items) {
+                                                unsigned long long *__restrict__ ctr,
+                                                const LptState *__restrict__ lpt) {
   extern __shared__ float4 p2p_smem[];
-  const int64_t nl = *n_items;  // work items: a leaf's chunk of up to 32 sinks (leaf index, chunk in bit 31)
+  __shared__ float4 part[8][32];  // a shared item's sums, by warp and sink
+  __shared__ unsigned next_shared, n_shared;
+  const unsigned nl = lpt->n_items;  // work items: a leaf's chunk of up to 32 sinks (leaf index, chunk in bit 31)
+  unsigned *taken = reinterpret_cast<unsigned *>(ctr);  // items handed out: to warps, to blocks
+  if (threadIdx.x < 32) {
+    // the items heavy enough to be shared: the first buckets, of work (entries x sinks) above half
+    // a warp's share of it all, and of at least 2^14 (512 entries of 32 sinks: 64 for each of the
+    // eight warps, or the prefetch chain they start with is most of what they do)
+    const unsigned long long half = max(lpt->work / (2ull * kLptWarps), (1ull << 14) - 1ull);
+    unsigned c = 0;
+    for (int b = threadIdx.x; b < kLptBuckets; b += 32)
+      if (lpt->hist[b] && (1ull << (63 - b)) > half) c += lpt->hist[b];
+    c = __reduce_add_sync(0xffffffffu, c);
+    if (threadIdx.x == 0) n_shared = c;
+  }
+  __syncthreads();
+  bool shared_phase = true;
   // per warp: the 32 list entries of the pending fill (first particle, exclusive
   // candidate offset, leaf-centre offset in the sink's frame), each candidate's
   // entry, and the chunk's sink bounding box (lo xyz, hi xyz)
@@ -70,15 +95,30 @@ __global__ void __launch_bounds__(256, 2) k_p2p(const uint32_t *__restrict__ ite
   const float half_unit = box / (float)kHalfBox;
   uint32_t n_in = 0;  // pairs inside the cut-off (profile mode only)
   for (;;) {
-    unsigned long long t = 0;
-    if (lane == 0) t = atomicAdd(ctr, 1ull);
-    t = __shfl_sync(0xffffffffu, t, 0);
-    if ((int64_t)t >= nl) break;
+    unsigned t = 0;
+    if (shared_phase) {  // a block's eight warps take an eighth of the item's list each
+      if (threadIdx.x == 0) next_shared = atomicAdd(taken + 1, 1u);
+      __syncthreads();
+      t = next_shared;
+      __syncthreads();
+      if (t >= n_shared) {
+        shared_phase = false;
+        continue;
+      }
+    } else {
+      if (lane == 0) t = n_shared + atomicAdd(taken, 1u);
+      t = __shfl_sync(0xffffffffu, t, 0);
+      if (t >= nl) break;
+    }
     const uint32_t item = items[t], k = item & 0x7fffffffu;
     const uint4 ca = cell[k];
     const uint2 r = range[k];
-    const uint32_t tb = beg[k], te = end[k];
-    if (tb == te) continue;  // no sources (in sink batches: a leaf of another batch)
+    uint32_t tb = beg[k], te = end[k];
+    if (shared_phase) {
+      const uint32_t share = (te - tb + 7u) / 8u;
+      tb = min(tb + share * wid, te);
+      te = min(tb + share, te);
+    }
 
     // the entry window at q + lane, prefetched in two steps: the list word
     // (fetch_lst, while the previous fill is evaluated), then the source leaf's
@@ -353,12 +393,33 @@ __global__ void __launch_bounds__(256, 2) k_p2p(const uint32_t *__restrict__ ite
           sy += v.y;
           sz += v.z;
         }
-        const uint32_t o = perm[cbase + lane];
-        acc_out[o] += G * sx;
-        acc_out[n + o] += G * sy;
-        acc_out[2 * n + o] += G * sz;
+        if (shared_phase) {
+          part[wid][lane] = make_float4(sx, sy, sz, 0.f);
+        } else {
+          const uint32_t o = perm[cbase + lane];
+          acc_out[o] += G * sx;
+          acc_out[n + o] += G * sy;
+          acc_out[2 * n + o] += G * sz;
+        }
       }
       __syncwarp();
+      if (shared_phase) {
+        __syncthreads();
+        if (wid == 0 && lane < cs) {  // the warps' sums in order
+          float sx = 0.f, sy = 0.f, sz = 0.f;
+#pragma unroll
+          for (int w = 0; w < 8; ++w) {
+            const float4 v = part[w][lane];
+            sx += v.x;
+            sy += v.y;
+            sz += v.z;
+          }
+          const uint32_t o = perm[cbase + lane];
+          acc_out[o] += G * sx;
+          acc_out[n + o] += G * sy;
+          acc_out[2 * n + o] += G * sz;
+        }
+      }
     }
   }
   if (kCount) {
@@ -369,7 +430,13 @@ __global__ void __launch_bounds__(256, 2) k_p2p(const uint32_t *__restrict__ ite
 }
 
 // Longest-first order of the work (list scheduling: the persistent grid takes
-// items in this order).  An item is one chunk of up to 32 sinks of a leaf
+// items in this order).  Where the heaviest items outweigh a warp's share of the
+// whole they set the time however they are ordered: those (k_p2p) are each shared by
+// a block's eight warps, an eighth of the list a warp, before the others start:
+// 1.40 -> 1.02 ms at 262k clustered particles, 0.91 -> 0.59 at 300k (polynomial
+// split), nothing at 2M, where no item is that heavy.  Shared from 2^13: 0.48
+// instead of 0.41 ms at 100k uniform; every item above half a share, whatever its
+// size: 0.15 instead of 0.115 at 32k.  An item is one chunk of up to 32 sinks of a leaf
 // (leaves of 33..64 particles give two, so the heaviest leaves' work is split
 // between two warps; the chunks' sums are independent, so the forces do not
 // change).  An item's work is about the leaf's list entries times its sinks;
@@ -378,13 +445,11 @@ __global__ void __launch_bounds__(256, 2) k_p2p(const uint32_t *__restrict__ ite
 // and placed bucket by bucket, heaviest first.  Leaves with empty lists (other
 // sink batches) give no item.  The order within a bucket does not matter: each
 // item's sums are its own warp's.
-constexpr int kLptBuckets = 64;
-
 __global__ void k_lpt_hist(const uint32_t *__restrict__ leaves, int64_t nl, const uint2 *__restrict__ range,
                            const uint32_t *__restrict__ beg, const uint32_t *__restrict__ end,
-                           uint8_t *__restrict__ bucket, unsigned *__restrict__ hist, unsigned *__restrict__ n_items,
-                           const TreeState *tz) {
+                           uint8_t *__restrict__ bucket, LptState *__restrict__ lpt, const TreeState *tz) {
   __shared__ unsigned h[kLptBuckets];
+  unsigned long long work = 0;
   for (int i = threadIdx.x; i < kLptBuckets; i += blockDim.x) h[i] = 0u;
   __syncthreads();
   nl = tree_leaves(tz, nl);
@@ -399,30 +464,33 @@ __global__ void k_lpt_hist(const uint32_t *__restrict__ leaves, int64_t nl, cons
         const uint32_t cs = min(32u, cnt - 32u * c);
         b = (uint8_t)__clzll((unsigned long long)ent * cs);  // heavier: smaller bucket index
         atomicAdd(&h[b], 1u);
+        work += (unsigned long long)ent * cs;
       }
       bucket[2 * t + c] = b;
     }
   }
+#pragma unroll
+  for (int o = 16; o; o >>= 1) work += __shfl_xor_sync(0xffffffffu, work, o);
+  if ((threadIdx.x & 31) == 0 && work) atomicAdd(&lpt->work, work);
   __syncthreads();
   for (int i = threadIdx.x; i < kLptBuckets; i += blockDim.x)
     if (h[i]) {
-      atomicAdd(&hist[i], h[i]);
-      atomicAdd(n_items, h[i]);
+      atomicAdd(&lpt->hist[i], h[i]);
+      atomicAdd(&lpt->n_items, h[i]);
     }
 }
 
 // Ranks within a block from shared-memory counters, one global reservation per
 // (block, bucket): the few heavy buckets take few global atomics.
 __global__ void k_lpt_place(const uint32_t *__restrict__ leaves, int64_t nl, const uint8_t *__restrict__ bucket,
-                            const unsigned *__restrict__ hist, unsigned *__restrict__ cursor,
-                            uint32_t *__restrict__ order, const TreeState *tz) {
+                            LptState *__restrict__ lpt, uint32_t *__restrict__ order, const TreeState *tz) {
   __shared__ unsigned base[kLptBuckets], cnt[kLptBuckets];
   for (int i = threadIdx.x; i < kLptBuckets; i += blockDim.x) cnt[i] = 0u;
   if (threadIdx.x == 0) {
     unsigned run = 0;
     for (int i = 0; i < kLptBuckets; ++i) {
       base[i] = run;
-      run += hist[i];
+      run += lpt->hist[i];
     }
   }
   __syncthreads();
@@ -440,7 +508,7 @@ __global__ void k_lpt_place(const uint32_t *__restrict__ leaves, int64_t nl, con
   }
   __syncthreads();
   for (int i = threadIdx.x; i < kLptBuckets; i += blockDim.x)
-    if (cnt[i]) base[i] += atomicAdd(&cursor[i], cnt[i]);
+    if (cnt[i]) base[i] += atomicAdd(&lpt->cursor[i], cnt[i]);
   __syncthreads();
   if (valid) {
     const uint32_t a = leaves[t];
@@ -479,21 +547,19 @@ cudaError_t p2p_pass(Ctx &c, float *acc, cudaStream_t st) {
   // the leaves longest first
   const TreeState *tz = c.graph_tree ? P<TreeState>(c.tstate) : nullptr;
   if ((e = ensure(c.lpt_order, (size_t)c.nleaves * 8)) != cudaSuccess) return e;
-  if ((e = ensure(c.lpt_tmp, (size_t)c.nleaves * 2 + (2 * kLptBuckets + 4) * sizeof(unsigned) + 64)) != cudaSuccess)
-    return e;
-  unsigned *hist = P<unsigned>(c.lpt_tmp), *cursor = hist + kLptBuckets, *n_items = cursor + kLptBuckets;
-  uint8_t *bucket = reinterpret_cast<uint8_t *>(n_items + 4);
-  if ((e = cudaMemsetAsync(hist, 0, (2 * kLptBuckets + 4) * sizeof(unsigned), st)) != cudaSuccess) return e;
+  if ((e = ensure(c.lpt_tmp, (size_t)c.nleaves * 2 + sizeof(LptState))) != cudaSuccess) return e;
+  LptState *lpt = P<LptState>(c.lpt_tmp);
+  uint8_t *bucket = reinterpret_cast<uint8_t *>(lpt + 1);
+  if ((e = cudaMemsetAsync(lpt, 0, sizeof(LptState), st)) != cudaSuccess) return e;
   if (c.prm.leaf_max > 64) return cudaErrorInvalidValue;  // two chunks per leaf at most
   k_lpt_hist<<<blocks_for(c.nleaves, T), T, 0, st>>>(P<uint32_t>(c.leaves), c.nleaves, P<uint2>(c.range),
-                                                      P<uint32_t>(c.p2p_beg), P<uint32_t>(c.p2p_end), bucket, hist,
-                                                      n_items, tz);
-  k_lpt_place<<<blocks_for(c.nleaves, T), T, 0, st>>>(P<uint32_t>(c.leaves), c.nleaves, bucket, hist, cursor,
+                                                      P<uint32_t>(c.p2p_beg), P<uint32_t>(c.p2p_end), bucket, lpt, tz);
+  k_lpt_place<<<blocks_for(c.nleaves, T), T, 0, st>>>(P<uint32_t>(c.leaves), c.nleaves, bucket, lpt,
                                                        P<uint32_t>(c.lpt_order), tz);
   note_launch(2);
   kern<<<g, T, dyn, st>>>(P<uint32_t>(c.lpt_order), P<uint4>(c.cell), P<uint2>(c.range), P<uint32_t>(c.p2p_beg),
                         P<uint32_t>(c.p2p_end), P<uint64_t>(c.p2p), P<float4>(c.pm4), P<uint32_t>(c.idx), c.n,
-                        (float)c.prm.box, fit2, (float)c.prm.G, acc, ctr, n_items);
+                        (float)c.prm.box, fit2, (float)c.prm.G, acc, ctr, lpt);
   note_launch();
   return cudaGetLastError();
 }
