@@ -502,7 +502,7 @@ std::vector<uint64_t> step_signature(Ctx &c, const double *pos, const float *vel
     v.push_back((uint64_t)(uintptr_t)b.p);
     v.push_back((uint64_t)b.cap);
   });
-  DBuf *pmb[] = {&c.pm_q, &c.pm_rho, &c.pm_mk, &c.pm_ak, &c.pm_a, &c.pm_gtab};
+  DBuf *pmb[] = {&c.pm_q, &c.pm_rho, &c.pm_mk, &c.pm_ak, &c.pm_a, &c.pm_gtab, &c.pm_win};
   for (DBuf *b : pmb) v.push_back((uint64_t)(uintptr_t)b->p);
   uint64_t dtb;
   std::memcpy(&dtb, &dt, 8);

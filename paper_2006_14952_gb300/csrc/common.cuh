@@ -386,6 +386,7 @@ struct Ctx {
   // tile pair counts and offsets, grouped pairs
   DBuf lo_flag, lo_rank, lo_meta, lo_sink, lo_tcnt, lo_toff, lo_scr;
   KdTree kd;  // tree = 1
+  DBuf pm_win;           // sinc window of one axis by index (PM Green function)
   DBuf pm_gtab;          // polynomial split: long-range Green function per integer |k|^2
   size_t pm_gtab_n = 0;  // its length (0: not built)
   int pm_plan_r2c = -1, pm_plan_c2r = -1;

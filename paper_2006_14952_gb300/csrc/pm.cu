@@ -27,12 +27,22 @@
 namespace hfmm {
 namespace {
 
-__global__ void k_mass_absmax(const float4 *__restrict__ pm4, int64_t n, unsigned *__restrict__ out) {
+// Four loads in flight a thread: one at a time the pass took 23 us at 2M, four times its bytes' worth.
+__global__ void __launch_bounds__(256) k_mass_absmax(const float4 *__restrict__ pm4, int64_t n,
+                                                     unsigned *__restrict__ out) {
+  __shared__ unsigned sv[8];
   unsigned v = 0;
-  for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x)
-    v = max(v, __float_as_uint(fabsf(pm4[i].w)));  // non-negative floats order like their bit patterns
-  for (int o = 16; o; o >>= 1) v = max(v, __shfl_xor_sync(0xffffffffu, v, o));
-  if ((threadIdx.x & 31) == 0 && v) atomicMax(out, v);
+  const int64_t i0 = (int64_t)blockIdx.x * 1024 + threadIdx.x;
+#pragma unroll
+  for (int q = 0; q < 4; ++q)  // non-negative floats order like their bit patterns
+    if (i0 + 256 * q < n) v = max(v, __float_as_uint(fabsf(pm4[i0 + 256 * q].w)));
+  v = __reduce_max_sync(0xffffffffu, v);
+  if ((threadIdx.x & 31) == 0) sv[threadIdx.x >> 5] = v;
+  __syncthreads();
+  if (threadIdx.x < 8) {
+    v = __reduce_max_sync(0xffu, sv[threadIdx.x]);
+    if (threadIdx.x == 0 && v) atomicMax(out, v);
+  }
 }
 
 // Fixed-point scale 2^s with N * max|m| * 2^s <= 2^61 (its exponent s).
@@ -97,80 +107,78 @@ __device__ __forceinline__ void cic_setup(const double *__restrict__ xs, int64_t
 
 // CIC mass assignment in 64-bit fixed point: corner value round(m 2^s w_x w_y w_z)
 // (FP32 product, one rounding to an integer).  Consecutive particles (Morton
-// order) mostly share their base mesh point: the lanes of a warp with the same
-// base point form groups (match on the point's index); when every group is a run
-// of adjacent lanes, each run adds its eight corner values with a segmented
-// shuffle sum (integers: exact, so the mesh is the same as with one atomic per
-// particle) and the run's first lane issues the eight atomics; otherwise every
-// lane issues its own.
-__global__ void k_deposit(const double *__restrict__ xs, const float4 *__restrict__ pm4, int64_t n, double to_mesh,
-                          int tm_exp, double box, int ng, const unsigned *__restrict__ mmax, unsigned long long *__restrict__ q) {
+// order) mostly share their base mesh point: each run of adjacent lanes with the
+// same base point adds its eight corner values with a segmented shuffle sum
+// (integers: exact, so the mesh is the same as with one atomic per particle), in
+// as many steps as the warp's longest run needs, and the run's first lane issues
+// the eight atomics.  Bound by the 64-bit atomics (76 us at 2M clustered, as with
+// match_any groups and all five steps before).
+__global__ void __launch_bounds__(256) k_deposit(const double *__restrict__ xs, const float4 *__restrict__ pm4,
+                                                 int64_t n, double to_mesh, int tm_exp, double box, int ng,
+                                                 const unsigned *__restrict__ mmax, unsigned long long *__restrict__ q) {
   const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   const int lane = threadIdx.x & 31;
   const bool valid = i < n;  // whole warps stay for the warp-wide steps
   int i0[3] = {0, 0, 0};
   float d[3] = {0.f, 0.f, 0.f};
   float ms = 0.f;
-  uint32_t key = 0xffffffffu - (uint32_t)lane;  // distinct keys (above any mesh index) for lanes past n
+  uint32_t key = 0xffffffffu;  // lanes past n: a run of their own (mesh indices are below 2^30)
   if (valid) {
     cic_setup(xs, n, i, to_mesh, tm_exp, box, ng, i0, d);
     ms = ldexpf(pm4[i].w, fixed_exponent(mmax, n));
     key = ((uint32_t)i0[0] * (uint32_t)ng + (uint32_t)i0[1]) * (uint32_t)ng + (uint32_t)i0[2];
   }
-  const unsigned grp = __match_any_sync(0xffffffffu, key);
-  const int first = __ffs(grp) - 1, last = 31 - __clz(grp);
-  const unsigned run = (unsigned)((1ull << (last - first + 1)) - 1ull);
-  const bool agg = __all_sync(0xffffffffu, (grp >> first) == run);
+  const uint32_t left = __shfl_up_sync(0xffffffffu, key, 1);
+  const unsigned heads = __ballot_sync(0xffffffffu, lane == 0 || left != key);
+  const unsigned after = lane == 31 ? 0u : heads >> (lane + 1);  // heads beyond this lane
+  const int last = after ? lane + __ffs(after) - 1 : 31;         // last lane of this lane's run
+  const bool head = (heads >> lane) & 1u;
+  const int longest = (int)__reduce_max_sync(0xffffffffu, head && valid ? (unsigned)(last - lane + 1) : 1u);
 #pragma unroll
-  for (int ox = 0; ox < 2; ++ox) {
-    const float wx = ox ? d[0] : 1.f - d[0];
-    const int gx = i0[0] + ox == ng ? 0 : i0[0] + ox;
-#pragma unroll
-    for (int oy = 0; oy < 2; ++oy) {
-      const float wy = oy ? d[1] : 1.f - d[1];
-      const int gy = i0[1] + oy == ng ? 0 : i0[1] + oy;
-#pragma unroll
-      for (int oz = 0; oz < 2; ++oz) {
-        const float wz = oz ? d[2] : 1.f - d[2];
-        const int gz = i0[2] + oz == ng ? 0 : i0[2] + oz;
-        long long v = valid ? __float2ll_rn(ms * (wx * wy * wz)) : 0ll;
-        unsigned long long *dst = q + ((int64_t)gx * ng + gy) * ng + gz;
-        if (agg) {
-#pragma unroll
-          for (int o = 1; o < 32; o <<= 1) {
-            const long long t = __shfl_down_sync(0xffffffffu, v, o);
-            if (lane + o <= last) v += t;
-          }
-          if (valid && lane == first) atomicAdd(dst, (unsigned long long)v);
-        } else if (valid) {
-          atomicAdd(dst, (unsigned long long)v);
-        }
-      }
+  for (int c = 0; c < 8; ++c) {
+    const int ox = c >> 2, oy = (c >> 1) & 1, oz = c & 1;
+    const float wx = ox ? d[0] : 1.f - d[0], wy = oy ? d[1] : 1.f - d[1], wz = oz ? d[2] : 1.f - d[2];
+    long long v = valid ? __float2ll_rn(ms * (wx * wy * wz)) : 0ll;
+    for (int o = 1; o < longest; o <<= 1) {
+      const long long t = __shfl_down_sync(0xffffffffu, v, o);
+      if (lane + o <= last) v += t;
+    }
+    if (valid && head) {
+      const int gx = i0[0] + ox == ng ? 0 : i0[0] + ox, gy = i0[1] + oy == ng ? 0 : i0[1] + oy,
+                gz = i0[2] + oz == ng ? 0 : i0[2] + oz;
+      atomicAdd(q + ((int64_t)gx * ng + gy) * ng + gz, (unsigned long long)v);
     }
   }
 }
 
-// Mesh density: the fixed-point sums times 2^-s (exact scaling), rounded to FP32.
-__global__ void k_fixed_to_real(const unsigned long long *__restrict__ q, int64_t cells, const unsigned *mmax,
-                                int64_t n, float *__restrict__ rho) {
-  const double inv = ldexp(1.0, -fixed_exponent(mmax, n));
-  const int64_t stride = (int64_t)gridDim.x * blockDim.x;
-  for (int64_t g = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; g < cells; g += stride)
-    rho[g] = (float)((double)(long long)q[g] * inv);
+// Mesh density: the fixed-point sums rounded to FP32, times 2^-s (exact, in two
+// factors: s can exceed the FP32 exponent range).  No FP64 arithmetic (26 us at
+// 128^3 with it).
+__global__ void __launch_bounds__(256) k_fixed_to_real(const unsigned long long *__restrict__ q, int64_t cells,
+                                                       const unsigned *mmax, int64_t n, float *__restrict__ rho) {
+  const int s = fixed_exponent(mmax, n);
+  const float f0 = ldexpf(1.f, -(s / 2)), f1 = ldexpf(1.f, -(s - s / 2));
+  const int64_t g0 = (int64_t)blockIdx.x * 1024 + threadIdx.x;
+#pragma unroll
+  for (int k = 0; k < 4; ++k) {
+    const int64_t g = g0 + 256 * k;
+    if (g < cells) rho[g] = __ll2float_rn((long long)q[g]) * f0 * f1;
+  }
 }
 
-__device__ __forceinline__ float sincf_(float x) { return fabsf(x) < 1e-4f ? 1.f - x * x / 6.f : sinf(x) / x; }
-
 // m(k) -> the three gradient components i k_d G(k) m(k) / L^3 (R2C layout [ng][ng][ng/2+1]).
+// win[i] = sinc(k_i h / 2) by axis index (the window of one axis; made with the plans);
 // gtab == nullptr: the Gaussian Green function; otherwise gtab[i^2 + j^2 + l^2]
 // holds the long-range Green function at that integer |k|^2 (units (2 pi / L)^2).
-__global__ void k_green(const cufftComplex *__restrict__ mk, int ng, float box, float rs, float G,
-                        const float *__restrict__ gtab, cufftComplex *__restrict__ ak) {
-  const int nz = ng / 2 + 1;
-  const int64_t total = (int64_t)ng * ng * nz;
-  const int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+__global__ void __launch_bounds__(256) k_green(const cufftComplex *__restrict__ mk, int ng, float box, float rs, float G,
+                                               const float *__restrict__ win, const float *__restrict__ gtab,
+                                               cufftComplex *__restrict__ ak) {
+  const uint32_t nz = (uint32_t)ng / 2 + 1;
+  const uint32_t total = (uint32_t)ng * (uint32_t)ng * nz;  // pm_grid <= 1024: below 2^30
+  const uint32_t t = blockIdx.x * blockDim.x + threadIdx.x;
   if (t >= total) return;
-  const int iz = (int)(t % nz), iy = (int)((t / nz) % ng), ix = (int)(t / ((int64_t)nz * ng));
+  const uint32_t row = t / nz;
+  const int iz = (int)(t - row * nz), ix = (int)(row / (uint32_t)ng), iy = (int)row - ix * ng;
   const float kf = 2.f * 3.14159265358979f / box;
   const int jx = ix <= ng / 2 ? ix : ix - ng, jy = iy <= ng / 2 ? iy : iy - ng;
   const float kx = kf * (float)jx;
@@ -179,8 +187,7 @@ __global__ void k_green(const cufftComplex *__restrict__ mk, int ng, float box, 
   const float k2 = kx * kx + ky * ky + kz * kz;
   float g = 0.f;
   if (k2 > 0.f) {
-    const float hh = 0.5f * box / (float)ng;
-    const float w = sincf_(kx * hh) * sincf_(ky * hh) * sincf_(kz * hh);
+    const float w = win[ix] * win[iy] * win[iz];
     const float w2 = w * w;  // W(k) = (product of sincs)^2, divided out twice
     if (gtab)
       g = G * gtab[jx * jx + jy * jy + iz * iz] / (w2 * w2) / (box * box * box);
@@ -194,7 +201,7 @@ __global__ void k_green(const cufftComplex *__restrict__ mk, int ng, float box, 
 #pragma unroll
   for (int d = 0; d < 3; ++d) {
     const float s = kd[d] * g;  // i s (re + i im) = -s im + i s re
-    ak[d * total + t] = make_float2(-s * m.y, s * m.x);
+    ak[(size_t)d * total + t] = make_float2(-s * m.y, s * m.x);
   }
 }
 
@@ -203,6 +210,7 @@ __global__ void k_interpolate(const double *__restrict__ xs, const uint32_t *__r
                               float *__restrict__ acc) {
   const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= n) return;
+  const uint32_t o = perm[i];
   int i0[3];
   float d[3];
   cic_setup(xs, n, i, to_mesh, tm_exp, box, ng, i0, d);
@@ -227,9 +235,10 @@ __global__ void k_interpolate(const double *__restrict__ xs, const uint32_t *__r
       }
     }
   }
-  const uint32_t o = perm[i];
+  // one addition per address, sent to L2 without reading it here: the scattered sectors cross
+  // once, and the index is fetched ahead of the mesh (120 -> 54 us at 2M)
 #pragma unroll
-  for (int k = 0; k < 3; ++k) acc[k * n + o] += s[k];
+  for (int k = 0; k < 3; ++k) atomicAdd(acc + k * n + o, s[k]);
 }
 
 __global__ void k_kick(float *__restrict__ vel, const float *__restrict__ acc, int64_t n3, float h, StepGuard g) {
@@ -267,6 +276,7 @@ void pm_release(Ctx &c) {
   release(c.pm_ak);
   release(c.pm_a);
   release(c.pm_gtab);
+  release(c.pm_win);
   c.pm_gtab_n = 0;
 }
 
@@ -347,6 +357,15 @@ cudaError_t pm_prepare(Ctx &c) {
       return e;
     c.pm_plan_c2r = p;
   }
+  if (!c.pm_win.p) {  // sinc(k_i h / 2) = sinc(pi i / N_g) by axis index (i and N_g - i alike)
+    std::vector<float> win(ng);
+    for (int i = 0; i < ng; ++i) {
+      const double x = M_PI * (i <= ng / 2 ? i : ng - i) / ng;
+      win[i] = (float)(x > 0 ? std::sin(x) / x : 1.0);
+    }
+    if ((e = ensure(c.pm_win, ng * 4)) != cudaSuccess) return e;
+    if ((e = cudaMemcpy(c.pm_win.p, win.data(), ng * 4, cudaMemcpyHostToDevice)) != cudaSuccess) return e;
+  }
   if (c.prm.split == 1 && (e = green_table_poly(c)) != cudaSuccess) return e;
   return cudaSuccess;
 }
@@ -368,22 +387,19 @@ cudaError_t pm_long_range(Ctx &c, float *acc, cudaStream_t st) {
   int tm_exp = 0;  // N_g / L = 2^tm_exp exactly (both powers of two), else the FP64 route
   const bool pow2 = std::frexp(to_mesh, &tm_exp) == 0.5 && box_inverse_if_pow2(c.prm.box) != 0.0;
   tm_exp = pow2 ? tm_exp - 1 : kNoExp;
-  unsigned gm = blocks_for(c.n, T);
-  if (gm > 152 * 16) gm = 152 * 16;
-  k_mass_absmax<<<gm, T, 0, st>>>(P<float4>(c.pm4), c.n, mmax);
+  k_mass_absmax<<<blocks_for(c.n, 1024), T, 0, st>>>(P<float4>(c.pm4), c.n, mmax);
   k_deposit<<<blocks_for(c.n, T), T, 0, st>>>(P<double>(c.xs), P<float4>(c.pm4), c.n, to_mesh, tm_exp, c.prm.box,
                                               ng, mmax,
                                               P<unsigned long long>(c.pm_q));
-  unsigned gc = blocks_for(cells, T);
-  if (gc > 152 * 16) gc = 152 * 16;
-  k_fixed_to_real<<<gc, T, 0, st>>>(P<unsigned long long>(c.pm_q), cells, mmax, c.n,
-                                                      P<float>(c.pm_rho));
+  k_fixed_to_real<<<blocks_for(cells, 1024), T, 0, st>>>(P<unsigned long long>(c.pm_q), cells, mmax, c.n,
+                                                         P<float>(c.pm_rho));
   note_launch(3);
   if ((e = cudaGetLastError()) != cudaSuccess) return e;
   if ((e = fft_error(cufftExecR2C(c.pm_plan_r2c, P<cufftReal>(c.pm_rho), P<cufftComplex>(c.pm_mk)))) != cudaSuccess)
     return e;
   k_green<<<blocks_for(kcells, T), T, 0, st>>>(P<cufftComplex>(c.pm_mk), ng, (float)c.prm.box, (float)c.rs,
-                                               (float)c.prm.G, c.prm.split == 1 ? P<float>(c.pm_gtab) : nullptr,
+                                               (float)c.prm.G, P<float>(c.pm_win),
+                                               c.prm.split == 1 ? P<float>(c.pm_gtab) : nullptr,
                                                P<cufftComplex>(c.pm_ak));
   note_launch();
   if ((e = cudaGetLastError()) != cudaSuccess) return e;
