@@ -341,6 +341,7 @@ def gen_tc(P, bf=False):
         return f"const float h = tf32_round({v}); hi[{dst}] = h; lo[{dst}] = {v} - h;"
 
     L = [f"template <> struct {'TCStoreBF' if bf else 'TCStore'}<{P}> {{",
+         f"  template <int G, int g>  // the coefficients c = g mod G\n"
          f"  static __device__ __forceinline__ void store_d(float rx, float ry, float rz, const float (&f)[{P + 1}],"
          f" const float (&U)[{P + 1}], {T} *__restrict__ hi, {T} *__restrict__ lo, const int (&xo)[8]) {{"]
     nm = {}
@@ -370,7 +371,8 @@ def gen_tc(P, bf=False):
                     t = f"f[{o}]" if a == (0, 0, 0) else f"{nm[a]} * f[{o}]"
                     parts.append(t if co == 1 else f"{float(co)}f * {t}")
         off = (ci >> 3) * 8 * row + (ci & 7) * row
-        L.append(f"    {{ const float d = U[{cn}] * ({' + '.join(parts)}); {split('d', f'{off} + xo[{ci & 7}]')} }}")
+        L.append(f"    if constexpr ({ci} % G == g) {{ const float d = U[{cn}] * ({' + '.join(parts)});"
+                 f" {split('d', f'{off} + xo[{ci & 7}]')} }}")
     L.append("  }")
     L.append(f"  static __device__ __forceinline__ void store_m(const float *__restrict__ Mb, float vr, float s,"
              f" {T} *__restrict__ hi, {T} *__restrict__ lo, const int (&xo)[8]) {{")

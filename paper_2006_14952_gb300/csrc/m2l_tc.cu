@@ -16,17 +16,28 @@
 // |n|+|m| <= p of P are used, so at most C(p+6,6) / NC^2 of the tensor work is
 // algorithmic (462 / 3136 at p = 5).
 //
-// CTA = 128 threads, one sink at a time (work counter).  A chunk of 128 pairs:
-// thread t computes pair t's D' and M' (generated TCStore / TCStoreBF bodies)
-// and writes them to the K-major, 128-byte-swizzled tiles (one 128-byte row per
-// matrix row holds 32 TF32 or 64 BF16 pairs: 4 or 2 tiles per chunk); one
-// thread then issues tiles x 4 K-steps x 3 split products of tcgen05.mma
-// (M = 128 rows c, N = NCP columns m) into the sink's TMEM accumulator and
-// commits to an mbarrier.  After
-// the last chunk the four warps read their 32 TMEM lanes (rows c), stage P in
-// shared memory and thread n forms L~_n = sum_m P[n+m][m].  Waits are bounded;
-// on a timeout the kernel records an error, waits (with the full limit) for the
-// MMAs it already issued, and returns after freeing TMEM.
+// A worker is 4 warps with one sink at a time; a CTA has four (a kernel that
+// allocates tensor memory gets one CTA an SM).  A chunk is 32 pairs: three warps
+// compute and store a third of the pairs' D' each (generated TCStore / TCStoreBF
+// bodies), one their M', to K-major, 128-byte-swizzled tiles (one 128-byte row per
+// matrix row); one thread issues the K-steps the chunk's pairs need x 3 split
+// products of tcgen05.mma (M = 128 rows c, N = NCP columns m) into the worker's
+// TMEM accumulator and commits to an mbarrier, and the next chunk's entries and
+// cells are fetched meanwhile.  After the last chunk the warps read their 32 TMEM
+// lanes (rows c), stage P in shared memory, and four lanes form each L~_n = sum_m
+// P[n+m][m] from a table of the places.  Waits are bounded; on a timeout the worker
+// records an error and leaves its loop, the MMAs it already issued are waited for
+// (with the full limit), and the CTA returns after freeing TMEM.
+//
+// What bounds it: the latency of a worker's chain (entries, cells, multipoles ->
+// operands -> MMA -> accumulator -> L), hidden by the other workers only.  Hence the
+// small chunk, with tiles cut to the rows that are written (the MMA's 128-row reads
+// run on into the next tile, whose values only reach rows of P that are never
+// read): 47 KB a worker at p = 6.  Four warps an SM with 128-pair chunks, every
+// thread computing both operands and all four K-tiles issued whatever the list's
+// length, took 20.8 ms for the 33M pairs of the 2M learned step instead of 8.4 (issue
+// 36%, tensor pipe 22% with four workers; 8.6 without the row prefetch).
+#include <algorithm>
 #include <type_traits>
 
 #include "common.cuh"
@@ -36,19 +47,47 @@
 namespace hfmm {
 namespace {
 
-constexpr int kThreads = 128;
-constexpr int kChunk = 128;  // pairs per chunk (4 tiles of 32)
+constexpr int kWorkers = 4;     // sinks at a time per CTA, four warps each
+constexpr int kThreads = 128 * kWorkers;
+constexpr int kChunk = 32;      // pairs per chunk: one lane each
+constexpr int kSinkBatch = 16;  // nodes taken from the work counter at a time
 constexpr uint32_t kWaitLimit = 1u << 22;
 
 __host__ __device__ constexpr int ncp_of(int p) { return (ncoef(p) + 15) / 16 * 16; }
 __host__ __device__ constexpr int tmem_cols_of(int p) {
   return ncp_of(p) <= 32 ? 32 : (ncp_of(p) <= 64 ? 64 : (ncp_of(p) <= 128 ? 128 : 256));
 }
-// 128-byte tiles per 128-pair chunk: 32 TF32 or 64 BF16 pairs per row
-__host__ __device__ constexpr int tiles_of(bool bf) { return bf ? 2 : 4; }
-// dynamic shared memory: 1 KB alignment slack + A (hi, lo) tiles x 16 KB each + B (hi, lo) tiles x NCP x 128 B each
-__host__ __device__ constexpr size_t smem_of(int p, bool bf) {
-  return 1024 + 2 * (size_t)tiles_of(bf) * 16384 + 2 * (size_t)tiles_of(bf) * ncp_of(p) * 128;
+// bytes of one A tile (rows c < NC, whole 8-row groups) and of one B tile (NCP rows)
+__host__ __device__ constexpr int a_bytes_of(int p) { return (ncoef(p) + 7) / 8 * 1024; }
+__host__ __device__ constexpr int b_bytes_of(int p) { return ncp_of(p) * 128; }
+// a worker's shared memory: A hi, lo + B hi, lo; at least the P staging and what the MMA's
+// 128-row reads of A lo span
+__host__ __device__ constexpr size_t worker_bytes(int p) {
+  const size_t tiles = 2 * (size_t)a_bytes_of(p) + 2 * (size_t)b_bytes_of(p);
+  const size_t reach = (size_t)a_bytes_of(p) + 16384, stage = (size_t)ncoef(p) * (ncoef(p) | 1) * 4;
+  const size_t most = tiles > reach ? (tiles > stage ? tiles : stage) : (reach > stage ? reach : stage);
+  return (most + 1023) / 1024 * 1024;
+}
+// dynamic shared memory: 1 KB alignment slack and the workers'
+__host__ __device__ constexpr size_t smem_of(int p) { return 1024 + kWorkers * worker_bytes(p); }
+// terms of L~: sum over n of the m with |n| + |m| <= p
+__host__ __device__ constexpr int terms_of(int p) {
+  int t = 0;
+  for (int k = 0; k <= p; ++k) t += (k + 1) * (k + 2) / 2 * ncoef(p - k);
+  return t;
+}
+
+// 16 accumulator columns of this warp's 32 lanes.
+__device__ __forceinline__ void tmem_ld16(uint32_t taddr, float (&v)[16]) {
+  uint32_t r[16];
+  asm volatile(
+      "tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15}, [%16];"
+      : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]), "=r"(r[8]),
+        "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15])
+      : "r"(taddr));
+  asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
+#pragma unroll
+  for (int i = 0; i < 16; ++i) v[i] = __uint_as_float(r[i]);
 }
 
 template <int P, bool kBF>
@@ -57,44 +96,56 @@ __global__ void __launch_bounds__(kThreads, 1)
              const uint32_t *__restrict__ end, const uint64_t *__restrict__ lst, const float *__restrict__ M,
              float *__restrict__ L, int ldm, float inv_rs, unsigned long long *__restrict__ ctr,
              int *__restrict__ status, uint32_t chunk_wait) {
-  constexpr int NC = ncoef(P);
-  constexpr int NCP = ncp_of(P);
-  constexpr uint32_t TCOLS = tmem_cols_of(P);
+  constexpr int NC = ncoef(P), NCP = ncp_of(P);
+  constexpr int kLd = NC | 1;  // row stride of the P staging (odd: no bank conflicts)
+  constexpr uint32_t WCOLS = tmem_cols_of(P);  // accumulator columns of a worker
+  constexpr uint32_t TCOLS = kWorkers * WCOLS;
+  static_assert(TCOLS <= 512, "tensor memory");
   constexpr uint32_t IDESC = kBF ? idesc_bf16(128, NCP) : idesc_tf32(128, NCP);
-  constexpr int kTiles = tiles_of(kBF), kPerRow = kChunk / kTiles;  // tiles per chunk, pairs per 128-byte row
+  constexpr int kStep = kBF ? 16 : 8;  // pairs per K-step (32 bytes)
   using T = typename std::conditional<kBF, __nv_bfloat16, float>::type;
   extern __shared__ unsigned char smem_raw[];
-  __shared__ uint64_t mbar;
+  __shared__ uint64_t mbars[kWorkers];
   __shared__ uint32_t tmem_slot;
-  __shared__ uchar4 mi[kNCMax];
-  __shared__ uint32_t next_sink;
-  __shared__ int abort_flag;
+  __shared__ uint16_t place[terms_of(P)];  // of each term P[n+m][m], by n then m
+  __shared__ uint16_t tbeg[NC + 1];
+  __shared__ uint32_t sink_list[kWorkers][kSinkBatch];
+  __shared__ int sink_count[kWorkers], aborts[kWorkers];
 
-  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-  unsigned char *base = (unsigned char *)(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);
-  T *a_hi = reinterpret_cast<T *>(base);  // kTiles tiles x 128 rows x kPerRow elements (16 KB each)
-  T *a_lo = a_hi + kTiles * 128 * kPerRow;
-  T *b_hi = a_lo + kTiles * 128 * kPerRow;  // kTiles tiles x NCP rows x kPerRow elements
-  T *b_lo = b_hi + kTiles * NCP * kPerRow;
-  float *pbuf = reinterpret_cast<float *>(base);  // P staging after a sink's last chunk (NC^2 floats)
+  // a worker's four warps (its warp w reads TMEM lanes 32 w ..) meet at a barrier of their own
+  const int worker = threadIdx.x >> 7, tid = threadIdx.x & 127, lane = tid & 31, warp = tid >> 5;
+  uint32_t *sinks = sink_list[worker];
+  volatile int &n_sinks = sink_count[worker], &abort_flag = aborts[worker];
+  auto sync = [&]() { asm volatile("bar.sync %0, 128;" ::"r"(worker + 1) : "memory"); };
+  unsigned char *base =
+      (unsigned char *)(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023) + worker * worker_bytes(P);
+  unsigned char *a_hi = base, *a_lo = a_hi + a_bytes_of(P), *b_hi = a_lo + a_bytes_of(P), *b_lo = b_hi + b_bytes_of(P);
+  float *pbuf = reinterpret_cast<float *>(base);  // P staging after a sink's last chunk
 
-  for (int c = tid; c < NC; c += kThreads) {
+  __shared__ uchar4 mi[NC];
+  if (threadIdx.x < NC) {
     int x, y, z;
-    mdecode(c, x, y, z);
-    mi[c] = make_uchar4((unsigned char)x, (unsigned char)y, (unsigned char)z, (unsigned char)(x + y + z));
+    mdecode(tid, x, y, z);
+    mi[tid] = make_uchar4((unsigned char)x, (unsigned char)y, (unsigned char)z, (unsigned char)(x + y + z));
   }
-  // operand tiles start at zero.  Rows >= NC of B stay zero; rows >= NC of A may
-  // later hold the P staging of a finished sink, which only feeds rows of P
-  // that are never read.
-  {
-    uint32_t *w = reinterpret_cast<uint32_t *>(base);
-    for (int i = tid; i < (2 * kTiles * 16384 + 2 * kTiles * NCP * 128) / 4; i += kThreads) w[i] = 0u;
+  __syncthreads();
+  if (threadIdx.x < NC) {
+    const uchar4 n = mi[tid];
+    int at = 0;
+    for (int q = 0; q < tid; ++q) at += ncoef(P - mi[q].w);
+    tbeg[tid] = (uint16_t)at;
+    const int rem = ncoef(P - n.w);
+    if (tid == NC - 1) tbeg[NC] = (uint16_t)(at + rem);
+    for (int e = 0; e < rem; ++e) {
+      const uchar4 m = mi[e];
+      place[at + e] = (uint16_t)(midx(n.x + m.x, n.y + m.y, n.z + m.z) * kLd + e);
+    }
   }
   if (tid == 0) {
-    asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(smem_u32(&mbar)));
+    asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(smem_u32(&mbars[worker])));
     abort_flag = 0;
   }
-  if (warp == 0) {
+  if (threadIdx.x < 32) {
     asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(&tmem_slot)),
                  "r"(TCOLS));
     asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;");
@@ -103,158 +154,182 @@ __global__ void __launch_bounds__(kThreads, 1)
   asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
   __syncthreads();
   asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-  const uint32_t tmem = tmem_slot;
-  const uint32_t mb = smem_u32(&mbar);
+  const uint32_t tmem0 = tmem_slot, tmem = tmem0 + worker * WCOLS;
+  const uint32_t mb = smem_u32(&mbars[worker]);
   uint32_t phase = 0;
   const float kInvSqrtPi = 0.56418958354775628f;
 
-  // this thread's column k within its tile and the swizzled element offsets of
-  // that column (16-byte chunks XOR the row mod 8 within each 8-row atom)
-  const int kq = tid / kPerRow, kk = tid % kPerRow;
+  // the swizzled element offsets of this lane's column (16-byte chunks XOR the row mod 8
+  // within each 8-row group); BF16 rows hold the 32 pairs in their first half
   constexpr int kEl = 16 / (int)sizeof(T);  // elements per 16-byte chunk
   int xo[8];
 #pragma unroll
-  for (int j = 0; j < 8; ++j) xo[j] = (((kk / kEl) ^ j) * kEl) + (kk % kEl);
-  T *my_ahi = a_hi + kq * 128 * kPerRow, *my_alo = a_lo + kq * 128 * kPerRow;
-  T *my_bhi = b_hi + kq * NCP * kPerRow, *my_blo = b_lo + kq * NCP * kPerRow;
+  for (int j = 0; j < 8; ++j) xo[j] = (((lane / kEl) ^ j) * kEl) + (lane % kEl);
 
   for (;;) {
-    if (tid == 0) {
-      uint32_t s = 0xffffffffu;
-      for (;;) {  // next sink with M2L pairs
-        unsigned long long t = atomicAdd(ctr, 1ull);
+    // ---- the next nodes with M2L pairs
+    if (warp == 0) {
+      int got = 0;
+      for (;;) {
+        unsigned long long t = 0;
+        if (lane == 0) t = atomicAdd(ctr, (unsigned long long)kSinkBatch);
+        t = __shfl_sync(0xffffffffu, t, 0);
         if ((int64_t)t >= nn) break;
-        if (end[t] > beg[t]) {
-          s = (uint32_t)t;
-          break;
-        }
+        const int64_t k = (int64_t)t + lane;
+        const bool has = lane < kSinkBatch && k < nn && end[k] > beg[k];
+        const unsigned m = __ballot_sync(0xffffffffu, has);
+        if (has) sinks[__popc(m & ((1u << lane) - 1u))] = (uint32_t)k;
+        got = __popc(m);
+        if (got) break;
       }
-      next_sink = s;
+      if (lane == 0) n_sinks = got;
     }
-    __syncthreads();
-    const uint32_t k = next_sink;
-    if (k == 0xffffffffu || abort_flag) break;
-    const uint4 ca = cell[k];
-    const uint32_t tb = beg[k], te = end[k];
-    const uint32_t nch = (te - tb + kChunk - 1) / kChunk;
-    for (uint32_t ch = 0; ch < nch; ++ch) {
-      const uint32_t t = tb + ch * kChunk + tid;
-      const bool valid = t < te;
-      float rx = 1.f, ry = 0.f, rz = 0.f, x = 1.f, u = 0.f, vr = 0.f, s = 0.f;
-      const float *Mb = M;
-      if (valid) {
-        const uint64_t e = lst[t];
-        const uint32_t b = pair_src(e);
-        const uint4 cb = cell[b];
-        int64_t dd[3];
-        half_delta(ca, cb, pair_shift(e), dd);
-        const float Rx = -(float)dd[0], Ry = -(float)dd[1], Rz = -(float)dd[2];
-        const float r2 = Rx * Rx + Ry * Ry + Rz * Rz;
-        const float rinv = rsqrtf(r2);
-        rx = Rx * rinv;
-        ry = Ry * rinv;
-        rz = Rz * rinv;
-        x = r2 * rinv * inv_rs;
-        u = (float)(2 * half_width(ca.w)) * rinv;
-        vr = (float)half_width(cb.w) / (float)half_width(ca.w);  // v / u = h_B / h_A
-        s = 1.f;
-        Mb = M + (size_t)b * ldm;
+    sync();
+    const int ns = n_sinks;
+    if (ns == 0 || abort_flag) break;
+    // this lane's pair of the next chunk, fetched while the chunk before it is in the MMA
+    uint32_t k = sinks[0], tb = beg[k], te = end[k], t0 = tb;
+    uint4 ca = cell[k], cb = ca;
+    uint64_t e = 0;
+    auto fetch = [&]() {
+      e = t0 + lane < te ? lst[t0 + lane] : 0ull;
+      cb = t0 + lane < te ? cell[pair_src(e)] : ca;
+      if (warp == 1) {  // the multipole rows into L1
+        const char *row = reinterpret_cast<const char *>(M + (size_t)pair_src(e) * ldm);
+#pragma unroll
+        for (int o = 0; o < NC * 4; o += 128) asm volatile("prefetch.global.L1 [%0];" ::"l"(row + o));
       }
-      float f[P + 1];
-      f[0] = erfcf(0.5f * x);
-      float tk = -x * kInvSqrtPi * __expf(-0.25f * x * x);
-      const float hx2 = 0.5f * x * x;
+    };
+    fetch();
+    for (int si = 0; si < ns; ++si) {
+      const uint32_t sink = k, sink_end = te;
+      for (bool first = true, more = true; more; first = false) {
+        const uint32_t cnt = sink_end - t0 < (uint32_t)kChunk ? sink_end - t0 : (uint32_t)kChunk;
+        const bool valid = (uint32_t)lane < cnt;
+        if (warp != 1) {  // D': a third of the coefficients each
+          float rx = 1.f, ry = 0.f, rz = 0.f, x = 1.f, u = 0.f;
+          if (valid) {
+            int dd[3];
+            half_delta32(ca, cb, pair_shift(e), dd);
+            const float Rx = -(float)dd[0], Ry = -(float)dd[1], Rz = -(float)dd[2];
+            const float r2 = Rx * Rx + Ry * Ry + Rz * Rz;
+            const float rinv = rsqrtf(r2);
+            rx = Rx * rinv;
+            ry = Ry * rinv;
+            rz = Rz * rinv;
+            x = r2 * rinv * inv_rs;
+            u = (float)(2 * half_width(ca.w)) * rinv;
+          }
+          float f[P + 1];
+          f[0] = erfcf(0.5f * x);
+          float tk = -x * kInvSqrtPi * __expf(-0.25f * x * x);
+          const float hx2 = 0.5f * x * x;
 #pragma unroll
-      for (int q = 0; q < P; ++q) {
-        f[q + 1] = -(float)(2 * q + 1) * f[q] + tk;
-        tk = -tk * hx2;
-      }
-      float U[P + 1];
-      U[0] = u;
+          for (int q = 0; q < P; ++q) {
+            f[q + 1] = -(float)(2 * q + 1) * f[q] + tk;
+            tk = -tk * hx2;
+          }
+          float U[P + 1];
+          U[0] = u;
 #pragma unroll
-      for (int q = 1; q <= P; ++q) U[q] = U[q - 1] * u;
-      if constexpr (kBF) {
-        TCStoreBF<P>::store_d(rx, ry, rz, f, U, my_ahi, my_alo, xo);
-        TCStoreBF<P>::store_m(Mb, vr, s, my_bhi, my_blo, xo);
-      } else {
-        TCStore<P>::store_d(rx, ry, rz, f, U, my_ahi, my_alo, xo);
-        TCStore<P>::store_m(Mb, vr, s, my_bhi, my_blo, xo);
-      }
-      asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
-      __syncthreads();
-      if (tid == 0) {
-        asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-#pragma unroll
-        for (int q = 0; q < kTiles; ++q) {
-#pragma unroll
-          for (int j = 0; j < 4; ++j) {  // K-steps of 32 bytes: 8 TF32 or 16 BF16 pairs
-            const uint32_t aoff = (uint32_t)(q * 16384 + j * 32), boff = (uint32_t)(q * NCP * 128 + j * 32);
-            const uint64_t ah = desc_sw128(smem_u32(a_hi) + aoff), al = desc_sw128(smem_u32(a_lo) + aoff);
-            const uint64_t bh = desc_sw128(smem_u32(b_hi) + boff), bl = desc_sw128(smem_u32(b_lo) + boff);
+          for (int q = 1; q <= P; ++q) U[q] = U[q - 1] * u;
+          T *hi = reinterpret_cast<T *>(a_hi), *lo = reinterpret_cast<T *>(a_lo);
+          using Store = typename std::conditional<kBF, TCStoreBF<P>, TCStore<P>>::type;
+          if (warp == 0) Store::template store_d<3, 0>(rx, ry, rz, f, U, hi, lo, xo);
+          else if (warp == 2) Store::template store_d<3, 1>(rx, ry, rz, f, U, hi, lo, xo);
+          else Store::template store_d<3, 2>(rx, ry, rz, f, U, hi, lo, xo);
+        } else {
+          const float vr = (float)half_width(cb.w) / (float)half_width(ca.w);  // v / u = h_B / h_A
+          const float *Mb = M + (size_t)pair_src(e) * ldm;
+          T *hi = reinterpret_cast<T *>(b_hi), *lo = reinterpret_cast<T *>(b_lo);
+          if constexpr (kBF) TCStoreBF<P>::store_m(Mb, vr, valid ? 1.f : 0.f, hi, lo, xo);
+          else TCStore<P>::store_m(Mb, vr, valid ? 1.f : 0.f, hi, lo, xo);
+        }
+        asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+        sync();
+        if (tid == 0) {
+          asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+          const uint32_t steps = (cnt + kStep - 1) / kStep;
+          for (uint32_t j = 0; j < steps; ++j) {
+            const uint32_t off = j * 32;
+            const uint64_t ah = desc_sw128(smem_u32(a_hi) + off), al = desc_sw128(smem_u32(a_lo) + off);
+            const uint64_t bh = desc_sw128(smem_u32(b_hi) + off), bl = desc_sw128(smem_u32(b_lo) + off);
+            const uint32_t acc = (!first || j != 0) ? 1u : 0u;
             if constexpr (kBF) {
-              mma_bf16(tmem, ah, bh, IDESC, (ch | q | j) ? 1u : 0u);
+              mma_bf16(tmem, ah, bh, IDESC, acc);
               mma_bf16(tmem, ah, bl, IDESC, 1u);
               mma_bf16(tmem, al, bh, IDESC, 1u);
             } else {
-              mma_tf32(tmem, ah, bh, IDESC, (ch | q | j) ? 1u : 0u);
+              mma_tf32(tmem, ah, bh, IDESC, acc);
               mma_tf32(tmem, ah, bl, IDESC, 1u);
               mma_tf32(tmem, al, bh, IDESC, 1u);
             }
           }
+          mma_commit(mb);
         }
-        mma_commit(mb);
-      }
-      const bool ok = mbar_wait(mb, phase, chunk_wait);
-      phase ^= 1u;
-      if (!ok) {
-        if (lane == 0) {
+        t0 += kChunk;
+        more = t0 < sink_end;
+        if (!more && si + 1 < ns) {
+          k = sinks[si + 1];
+          t0 = tb = beg[k];
+          te = end[k];
+          ca = cell[k];
+        }
+        fetch();
+        const bool ok = mbar_wait(mb, phase, chunk_wait);
+        phase ^= 1u;
+        if (!ok && lane == 0) {
           atomicExch(status, 1);
           abort_flag = 1;
         }
+        sync();
+        if (abort_flag) break;
+        asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
       }
-      __syncthreads();
       if (abort_flag) break;
+      // ---- TMEM rows 32 warp + lane hold P[c][0..NCP); stage rows c < NC
+      const int c = warp * 32 + lane;
+      if (warp * 32 < NC) {
+#pragma unroll
+        for (int col = 0; col < NCP; col += 16) {
+          float v[16];
+          tmem_ld16(tmem + ((uint32_t)(warp * 32) << 16) + (uint32_t)col, v);
+          if (c < NC) {
+#pragma unroll
+            for (int i = 0; i < 16; ++i)
+              if (col + i < NC) pbuf[c * kLd + col + i] = v[i];
+          }
+        }
+      }
+      asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+      sync();
+      // ---- four lanes an output, every fourth term each
+      for (int o = tid; o < 4 * NC; o += 128) {
+        const int n = o >> 2;
+        float acc = 0.f;
+        for (int e = tbeg[n] + (o & 3); e < tbeg[n + 1]; e += 4) acc += pbuf[place[e]];
+        const unsigned quad = 0xfu << (lane & 28);
+        acc += __shfl_xor_sync(quad, acc, 1);
+        acc += __shfl_xor_sync(quad, acc, 2);
+        if ((o & 3) == 0) L[(size_t)sink * ldm + n] += acc;
+      }
+      sync();  // the operand tiles are rewritten
       asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
     }
     if (abort_flag) break;
-    // TMEM rows 32*warp + lane hold P[c][0..NCP); stage rows c < NC
-    const int c = warp * 32 + lane;
-#pragma unroll
-    for (int col = 0; col < NCP; col += 8) {
-      float v[8];
-      tmem_ld8(tmem + ((uint32_t)(warp * 32) << 16) + (uint32_t)col, v);
-      if (c < NC) {
-#pragma unroll
-        for (int i = 0; i < 8; ++i)
-          if (col + i < NC) pbuf[c * NC + col + i] = v[i];
-      }
-    }
-    asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
-    __syncthreads();
-    if (tid < NC) {
-      const uchar4 n = mi[tid];
-      float acc = 0.f;
-      const int rem = ncoef(P - n.w);
-      for (int e = 0; e < rem; ++e) {
-        const uchar4 m = mi[e];
-        acc += pbuf[midx(n.x + m.x, n.y + m.y, n.z + m.z) * NC + e];
-      }
-      L[(size_t)k * ldm + tid] += acc;
-    }
-    __syncthreads();
-    asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
   }
   // the MMAs of an abandoned chunk may still be running: wait for them with the
   // full limit before the tensor memory they write is freed
   if (abort_flag && tid == 0) mbar_wait(mb, phase ^ 1u, kWaitLimit);
   asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
   __syncthreads();
-  if (warp == 0) asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(TCOLS));
+  if (threadIdx.x < 32)
+    asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem0), "r"(TCOLS));
 }
 
 template <int P, bool kBF>
 cudaError_t launch_tc(Ctx &c, cudaStream_t st) {
-  const size_t smem = smem_of(P, kBF);
+  const size_t smem = smem_of(P);
   cudaError_t e = cudaFuncSetAttribute(k_m2l_tc<P, kBF>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   if (e != cudaSuccess) return e;
   // d_small[5] = work counter, d_small[6] = status word
@@ -262,10 +337,11 @@ cudaError_t launch_tc(Ctx &c, cudaStream_t st) {
   int *status = reinterpret_cast<int *>(hfmm::P<uint64_t>(c.d_small) + 6);
   if ((e = cudaMemsetAsync(ctr, 0, 8, st)) != cudaSuccess) return e;  // the status word is zeroed once per call
   int nsm = 0, dev = 0;
-  cudaGetDevice(&dev);
-  cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);
+  if ((e = cudaGetDevice(&dev)) != cudaSuccess) return e;
+  if ((e = cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev)) != cudaSuccess) return e;
+  const unsigned grid = std::min((unsigned)nsm, blocks_for((size_t)c.nnodes, kSinkBatch));  // persistent
   const float inv_rs = (float)(c.prm.box / (double)kHalfBox / c.rs);
-  k_m2l_tc<P, kBF><<<nsm > 0 ? nsm : 152, kThreads, smem, st>>>(
+  k_m2l_tc<P, kBF><<<grid, kThreads, smem, st>>>(
       c.nnodes, hfmm::P<uint4>(c.cell), hfmm::P<uint32_t>(c.m2l_beg), hfmm::P<uint32_t>(c.m2l_end),
       hfmm::P<uint64_t>(c.m2l), hfmm::P<float>(c.M), hfmm::P<float>(c.L), c.ldm, inv_rs, ctr, status,
       c.prm.tc_wait_polls > 0 ? (uint32_t)c.prm.tc_wait_polls : c.prm.tc_wait_polls < 0 ? 0u : kWaitLimit);
