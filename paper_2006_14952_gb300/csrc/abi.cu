@@ -193,9 +193,9 @@ void for_each_buffer(Ctx &c, F f) {
                   &c.lo_rank, &c.lo_meta, &c.lo_sink, &c.lo_tcnt, &c.lo_toff, &c.lo_scr,
                   &c.pacc, &c.lpt_order, &c.lpt_tmp, &c.kd.xw,
                   &c.kd.ord[0], &c.kd.ord[1], &c.kd.ord[2], &c.kd.ord2[0], &c.kd.ord2[1], &c.kd.ord2[2],
-                  &c.kd.side, &c.kd.flag, &c.kd.scan, &c.kd.pnode, &c.kd.nflag, &c.kd.nscan, &c.kd.first,
+                  &c.kd.side, &c.kd.place, &c.kd.first,
                   &c.kd.count, &c.kd.child, &c.kd.parent, &c.kd.axis, &c.kd.box, &c.kd.geo, &c.kd.geof, &c.kd.hs,
-                  &c.kd.ctr, &c.kd.lv};
+                  &c.kd.ctr};
   for (DBuf *b : bufs) f(*b);
 }
 

@@ -7,19 +7,21 @@
 //   - positions wrapped (x - L floor(x / L), as for the octree); for each axis d
 //     the particle indices sorted once by (coordinate d, input index) with the
 //     stable radix sort of order-preserving 64-bit keys;
-//   - a level's node reads its particles' bounding box from the first and last
-//     entries of its range in the three orders; above leaf_max it splits on the
-//     axis of largest extent (the lowest on a tie): the first floor(n / 2)
-//     particles of that axis' order form the first child.  The other orders are
-//     partitioned stably by the particles' side: an exclusive scan of the side
-//     flags over all positions, less its value at the node's first position,
-//     ranks a particle among the second child's particles.  So every order stays
-//     sorted inside every node, and inside a leaf the x order is the particle
-//     order (that of (x, input index)); the three orders are flagged, scanned
-//     (one scan over the concatenated flags) and scattered together;
-//   - the counts of a level differ by at most one, so the depth follows from N
-//     and leaf_max on the host; each level's extent stays on the device (the
-//     kernels read it) and is read back once, after the last level.
+//   - the shape of the tree follows from n and leaf_max alone (the counts of a level
+//     are floor and ceil of n / 2^level; KdShape below): no scan, no read-back;
+//   - a node reads its particles' bounding box from the first and last entries of
+//     its range in the three orders; above leaf_max it splits on the axis of
+//     largest extent (the lowest on a tie): the first floor(n / 2) particles of that
+//     axis' order form the first child.  The orders are partitioned stably by the
+//     particles' side, so every order stays sorted inside every node, and inside a
+//     leaf the x order is the particle order (that of (x, input index)).  Nodes above
+//     2048 particles: three kernels a level over all particles (k_kd_axis, k_kd_side,
+//     k_kd_part); below, one block takes a node to its leaves (k_kd_subtree).
+// A level over all particles is bound by its passes (a random byte a particle and order,
+// two 4-byte streams an order, about 80 us at 2M); with nine launches a level to the
+// leaves, its scans of 3 n flags and a node number a particle, the build of 2M particles
+// (17 levels) took 2.45 ms; ten levels so and the rest in shared memory: 1.12 ms.  2048 is
+// what a block's 48 KB hold (24 bytes a particle), four blocks an SM.
 // Node geometry: the box centre c, half extents e, side (largest extent) in FP64,
 // and the expansion scale h = L 2^-j >= side (j <= 21, the octree's deepest
 // cell side): P2M offsets over h stay within [-1/2, 1/2] and the scale ratios of
@@ -54,7 +56,6 @@ namespace hfmm {
 namespace {
 
 constexpr int kT = 256;
-constexpr int kKdMaxLevels = 64;
 
 __global__ void k_kd_wrap(const double *__restrict__ pos, int64_t n, double box, double inv_pow2,
                           double *__restrict__ xw) {
@@ -73,164 +74,369 @@ __global__ void k_kd_keys(const double *__restrict__ x, int64_t n, uint64_t *__r
   val[i] = (uint32_t)i;
 }
 
-__global__ void k_kd_root(int64_t n, uint32_t *first, uint32_t *count, int *parent, unsigned long long *lv) {
-  first[0] = 0;
-  count[0] = (uint32_t)n;
-  parent[0] = -1;
-  lv[0] = 0;
-  lv[1] = 1;
+// The shape of the tree: levels 0 .. depth are complete; on level `depth` the counts are
+// q = floor(n / 2^depth) <= leaf_max and q + 1, and the `nsplit` nodes above leaf_max (q =
+// leaf_max only) have the last level's nodes as children.  Node (l, j) of a complete level
+// is number 2^l - 1 + j; with first(l, j) - j q of the nodes before it one larger than
+// the others, the children of (depth, j) are numbers 2^(depth + 1) - 1 + 2 (first - j q) and + 1.
+struct KdShape {
+  int64_t n;
+  int leaf_max, depth;
+  int64_t q, nsplit;
+  __host__ __device__ int64_t last_start() const { return ((int64_t)2 << depth) - 1; }
+  __host__ __device__ int64_t nodes() const { return last_start() + 2 * nsplit; }
+  __host__ __device__ int64_t leaves() const { return ((int64_t)1 << depth) + nsplit; }
+};
+KdShape kd_shape(int64_t n, int leaf_max) {
+  KdShape s{n, leaf_max, 0, n, 0};
+  while (s.q > leaf_max) {
+    ++s.depth;
+    s.q = n >> s.depth;
+  }
+  if (s.q == leaf_max) s.nsplit = n - (s.q << s.depth);
+  return s;
 }
 
-// The extent [lo, hi) of tree level l on the device: lv[2 l], lv[2 l + 1].
-__device__ __forceinline__ void level_extent(const unsigned long long *lv, int l, int64_t &lo, int64_t &hi) {
-  lo = (int64_t)lv[2 * l];
-  hi = (int64_t)lv[2 * l + 1];
+// Particle range of node (l, j), j's bits from the top (0: first child).
+__device__ __forceinline__ void kd_range(int64_t n, int l, uint32_t j, uint32_t &f, uint32_t &m) {
+  f = 0;
+  m = (uint32_t)n;
+  for (int b = l - 1; b >= 0; --b) {
+    const uint32_t h = m / 2;
+    if ((j >> b) & 1u) {
+      f += h;
+      m -= h;
+    } else {
+      m = h;
+    }
+  }
+}
+// The node of level l that holds position i of the range [f, f + m): its number among
+// them, and its range.
+__device__ __forceinline__ uint32_t kd_find(uint32_t i, int l, uint32_t &f, uint32_t &m) {
+  uint32_t j = 0;
+  for (int b = 0; b < l; ++b) {
+    const uint32_t h = m / 2;
+    const uint32_t up = i - f >= h ? 1u : 0u;
+    f += up ? h : 0u;
+    m = up ? m - h : h;
+    j = 2 * j + up;
+  }
+  return j;
 }
 
-// One level's nodes: bounding box and split decision (split flags zero up to `bound`
-// nodes, the grid's size, so the scan of a level of unknown size on the host works).
-__global__ void k_kd_level(const unsigned long long *__restrict__ lv, int level, int64_t bound, int leaf_max,
-                           const double *__restrict__ xw, int64_t n,
-                           const uint32_t *__restrict__ o0, const uint32_t *__restrict__ o1,
-                           const uint32_t *__restrict__ o2, const uint32_t *__restrict__ first,
-                           const uint32_t *__restrict__ count, double *__restrict__ box, int64_t cap,
-                           int *__restrict__ axis, uint32_t *__restrict__ nflag) {
-  const int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (t >= bound) return;
-  int64_t lo, hi;
-  level_extent(lv, level, lo, hi);
-  if (t >= hi - lo) {
-    nflag[t] = 0u;
+// Ranges, children, parents and the leaf list.
+__global__ void k_kd_topology(KdShape S, uint32_t *__restrict__ first, uint32_t *__restrict__ count,
+                              int *__restrict__ child, int *__restrict__ parent, uint32_t *__restrict__ leaves) {
+  const int64_t k = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+  if (k >= S.last_start()) return;
+  const int l = 63 - __clzll((unsigned long long)k + 1);
+  const uint32_t j = (uint32_t)(k + 1 - ((int64_t)1 << l));
+  uint32_t f, m;
+  kd_range(S.n, l, j, f, m);
+  first[k] = f;
+  count[k] = m;
+  parent[k] = k == 0 ? -1 : (int)((k - 1) / 2);
+  if (l < S.depth) {
+    child[k] = (int)(2 * k + 1);
     return;
   }
-  const int64_t k = lo + t;
-  const uint32_t f = first[k], m = count[k];
-  const uint32_t *ord[3] = {o0, o1, o2};
+  const int64_t larger = S.nsplit ? (int64_t)f - (int64_t)j * S.q : 0;  // nodes before this one that split
+  if ((int64_t)m <= S.leaf_max) {
+    child[k] = -1;
+    leaves[j - larger] = (uint32_t)k;
+    return;
+  }
+  const int64_t c = S.last_start() + 2 * larger;
+  child[k] = (int)c;
+  first[c] = f;
+  count[c] = m / 2;
+  first[c + 1] = f + m / 2;
+  count[c + 1] = m - m / 2;
+  const int64_t at = ((int64_t)1 << S.depth) - S.nsplit + 2 * larger;
+  for (int e = 0; e < 2; ++e) {
+    child[c + e] = -1;
+    parent[c + e] = (int)k;
+    leaves[at + e] = (uint32_t)(c + e);
+  }
+}
+
+// Bounding box of the node over positions [f, f + m) of the three orders, and the axis of
+// its largest extent (the lowest on a tie).
+template <class Order>
+__device__ __forceinline__ int kd_box(const double *__restrict__ xw, int64_t n, uint32_t f, uint32_t m, Order ord,
+                                      double *__restrict__ box, int64_t cap, int64_t k) {
   double best = 0.0;
   int ax = 0;
 #pragma unroll
   for (int d = 0; d < 3; ++d) {
-    const double a = xw[d * n + ord[d][f]], b = xw[d * n + ord[d][f + m - 1]];
+    const double a = xw[d * n + ord(d, f)], b = xw[d * n + ord(d, f + m - 1)];
     box[d * cap + k] = a;
     box[(3 + d) * cap + k] = b;
     const double ext = __dsub_rn(b, a);
-    if (d == 0 || ext > best) {  // the lowest axis of the largest extent
+    if (d == 0 || ext > best) {
       best = ext;
       ax = d;
     }
   }
-  const bool split = (int64_t)m > leaf_max;
-  axis[k] = split ? ax : -1;
-  nflag[t] = split ? 1u : 0u;
+  return ax;
 }
 
-__global__ void k_kd_children(const unsigned long long *__restrict__ lv, int level, const int *__restrict__ axis,
-                              const uint32_t *__restrict__ nscan, uint32_t *__restrict__ first,
-                              uint32_t *__restrict__ count, int *__restrict__ child, int *__restrict__ parent) {
-  const int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  int64_t lo, hi;
-  level_extent(lv, level, lo, hi);
-  if (t >= hi - lo) return;
-  const int64_t k = lo + t;
-  if (axis[k] < 0) {
-    child[k] = -1;
-    return;
-  }
-  const int64_t ch = hi + 2 * (int64_t)nscan[t];
-  const uint32_t f = first[k], m = count[k];
-  child[k] = (int)ch;
-  first[ch] = f;
-  count[ch] = m / 2;
-  first[ch + 1] = f + m / 2;
-  count[ch + 1] = m - m / 2;
-  parent[ch] = parent[ch + 1] = (int)k;
+struct KdOrders {
+  const uint32_t *o[3];
+};
+
+// One complete level's nodes: box and split axis (every node of the level splits).
+__global__ void k_kd_axis(int64_t n, int level, const double *__restrict__ xw, KdOrders O, double *__restrict__ box,
+                          int64_t cap, int *__restrict__ axis) {
+  const int64_t j = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+  if (j >= ((int64_t)1 << level)) return;
+  uint32_t f, m;
+  kd_range(n, level, (uint32_t)j, f, m);
+  const int64_t k = ((int64_t)1 << level) - 1 + j;
+  axis[k] = kd_box(xw, n, f, m, [&](int d, uint32_t i) { return O.o[d][i]; }, box, cap, k);
 }
 
-// The next level's extent: [hi, hi + 2 splits).
-__global__ void k_kd_next(unsigned long long *__restrict__ lv, int level, const uint64_t *__restrict__ nsplit) {
-  lv[2 * level + 2] = lv[2 * level + 1];
-  lv[2 * level + 3] = lv[2 * level + 1] + 2ull * nsplit[0];
-}
-
-// The side of every particle of a node split on this level (positions of earlier leaves: node < lo).
-__global__ void k_kd_side(int64_t n, const unsigned long long *__restrict__ lv, int level,
-                          const uint32_t *__restrict__ pnode, const uint32_t *__restrict__ first,
-                          const uint32_t *__restrict__ count, const int *__restrict__ axis,
-                          const uint32_t *__restrict__ o0, const uint32_t *__restrict__ o1,
-                          const uint32_t *__restrict__ o2, uint8_t *__restrict__ side) {
+// The side of every particle: in the second half of its node's range in the split axis' order.
+__global__ void k_kd_side(int64_t n, int level, const int *__restrict__ axis, KdOrders O, uint8_t *__restrict__ side) {
   const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= n) return;
-  const int64_t lo = (int64_t)lv[2 * level];
-  const uint32_t k = pnode[i];
-  if ((int64_t)k < lo) return;
-  const int a = axis[k];
-  if (a < 0) return;
-  const uint32_t p = a == 0 ? o0[i] : a == 1 ? o1[i] : o2[i];
-  side[p] = (uint32_t)i - first[k] >= count[k] / 2 ? 1 : 0;
+  uint32_t f = 0, m = (uint32_t)n;
+  const uint32_t j = kd_find((uint32_t)i, level, f, m);
+  const int a = axis[((int64_t)1 << level) - 1 + j];
+  side[a == 0 ? O.o[0][i] : a == 1 ? O.o[1][i] : O.o[2][i]] = (uint32_t)i - f >= m / 2 ? 1 : 0;
 }
 
-// The side flags of the three orders, concatenated ([3][n]; zero outside the nodes
-// split on this level), for one scan over all of them.
-__global__ void k_kd_flag(int64_t n, const unsigned long long *__restrict__ lv, int level,
-                          const uint32_t *__restrict__ pnode, const int *__restrict__ axis,
-                          const uint32_t *__restrict__ o0, const uint32_t *__restrict__ o1,
-                          const uint32_t *__restrict__ o2, const uint8_t *__restrict__ side,
-                          uint32_t *__restrict__ flag) {
-  const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (i >= n) return;
-  const int64_t lo = (int64_t)lv[2 * level];
-  const uint32_t k = pnode[i];
-  const bool split = (int64_t)k >= lo && axis[k] >= 0;
-  flag[i] = split ? side[o0[i]] : 0u;
-  flag[n + i] = split ? side[o1[i]] : 0u;
-  flag[2 * n + i] = split ? side[o2[i]] : 0u;
-}
-
-// Stable partition of the three orders inside every node split on this level:
-// in order d a particle of the second child is preceded in it by scan[d n + i] -
-// scan[d n + first] such particles (the scan runs over the concatenated flags).
-__global__ void k_kd_scatter(int64_t n, const unsigned long long *__restrict__ lv, int level,
-                             const uint32_t *__restrict__ pnode, const uint32_t *__restrict__ first,
-                             const uint32_t *__restrict__ count, const int *__restrict__ axis,
-                             const uint32_t *__restrict__ o0, const uint32_t *__restrict__ o1,
-                             const uint32_t *__restrict__ o2, const uint8_t *__restrict__ side,
-                             const uint32_t *__restrict__ scan, uint32_t *__restrict__ r0,
-                             uint32_t *__restrict__ r1, uint32_t *__restrict__ r2) {
-  const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (i >= n) return;
-  const int64_t lo = (int64_t)lv[2 * level];
-  const uint32_t k = pnode[i];
-  const uint32_t *ord[3] = {o0, o1, o2};
-  uint32_t *out[3] = {r0, r1, r2};
-  if ((int64_t)k < lo || axis[k] < 0) {
+// Stable partition of the three orders inside every node of a level.  A particle of the
+// second child is preceded in its node by r others of it: the tile's exclusive scan of the
+// side flags, the flags of all tiles before (published counts, looked back over), less
+// those of the nodes before, whose second children are known from the counts alone.
+constexpr int kPartItems = 8, kPartTile = kT * kPartItems;
+constexpr unsigned kPartPolls = 1u << 20;
+__global__ void __launch_bounds__(kT) k_kd_part(int64_t n, int level, KdOrders O, uint32_t *__restrict__ r0,
+                                                uint32_t *__restrict__ r1, uint32_t *__restrict__ r2,
+                                                const uint8_t *__restrict__ side, unsigned *__restrict__ ticket,
+                                                volatile unsigned long long *look, unsigned ntiles) {
+  __shared__ uint32_t wsum[kT / 32];
+  __shared__ unsigned tile_s;
+  __shared__ unsigned long long before_s;
+  const int tid = threadIdx.x, lane = tid & 31, w = tid >> 5;
+  if (tid == 0) tile_s = atomicAdd(ticket, 1u);
+  __syncthreads();
+  // tiles of the three orders in turn; the scan starts anew with each order
+  const unsigned tile = tile_s, d = tile / ntiles, t = tile - d * ntiles;
+  const uint32_t *ord = O.o[d];
+  uint32_t *out = d == 0 ? r0 : d == 1 ? r1 : r2;
+  const int64_t i0 = (int64_t)t * kPartTile + (int64_t)w * 32 * kPartItems + lane;
+  uint32_t v[kPartItems], fl[kPartItems], ex[kPartItems], c = 0;
 #pragma unroll
-    for (int d = 0; d < 3; ++d) out[d][i] = ord[d][i];
-    return;
-  }
-  const uint32_t f = first[k], nl = count[k] / 2;
+  for (int q = 0; q < kPartItems; ++q) v[q] = i0 + 32 * q < n ? ord[i0 + 32 * q] : 0u;
 #pragma unroll
-  for (int d = 0; d < 3; ++d) {
-    const uint32_t v = ord[d][i];
-    const uint32_t r = scan[d * n + i] - scan[d * n + f];  // particles of the second child before position i
-    out[d][side[v] ? f + nl + r : (uint32_t)i - r] = v;
+  for (int q = 0; q < kPartItems; ++q) fl[q] = i0 + 32 * q < n ? side[v[q]] : 0u;
+#pragma unroll
+  for (int q = 0; q < kPartItems; ++q) {
+    const unsigned b = __ballot_sync(0xffffffffu, fl[q] != 0);
+    ex[q] = c + (uint32_t)__popc(b & ((1u << lane) - 1u));
+    c += (uint32_t)__popc(b);
+  }
+  if (lane == 0) wsum[w] = c;
+  __syncthreads();
+  uint32_t wb = 0, all = 0;
+#pragma unroll
+  for (int q = 0; q < kT / 32; ++q) {
+    if (q < w) wb += wsum[q];
+    all += wsum[q];
+  }
+  if (w == 0) {
+    constexpr unsigned long long kAgg = 1ull << 62, kInc = 2ull << 62, kVal = kAgg - 1ull;
+    if (lane == 0) look[tile] = (t == 0 ? kInc : kAgg) | all;
+    // look back, 32 tiles at a time: up to the nearest published inclusive count
+    unsigned long long before = 0;
+    bool lost = false;
+    for (long long at = (long long)t - 1; at >= 0;) {
+      unsigned long long x = kInc;  // before the order's first tile: nothing
+      for (unsigned poll = 0;; ++poll) {
+        if (at - lane >= 0) x = look[d * ntiles + (unsigned)(at - lane)];
+        if (__all_sync(0xffffffffu, (x >> 62) != 0)) break;
+        if (poll == kPartPolls) {
+          lost = true;
+          break;
+        }
+      }
+      if (lost) break;
+      const unsigned inc = __ballot_sync(0xffffffffu, (x >> 62) == 2);
+      const int stop = inc ? __ffs(inc) - 1 : 31;
+      unsigned long long s = lane <= stop ? (at - lane >= 0 ? x & kVal : 0ull) : 0ull;
+#pragma unroll
+      for (int o = 16; o; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+      before += s;
+      if (inc) break;
+      at -= 32;
+    }
+    if (lost) {  // waited long enough: count the flags before this tile
+      before = 0;
+      for (int64_t p = lane; p < (int64_t)t * kPartTile; p += 32) before += side[ord[p]];
+#pragma unroll
+      for (int o = 16; o; o >>= 1) before += __shfl_xor_sync(0xffffffffu, before, o);
+    }
+    if (lane == 0) {
+      if (t > 0) look[tile] = kInc | (before + all);
+      before_s = before;
+    }
+  }
+  __syncthreads();
+  const int64_t base = (int64_t)before_s + wb, q0 = n >> level;
+#pragma unroll
+  for (int q = 0; q < kPartItems; ++q) {
+    const int64_t i = i0 + 32 * q;
+    if (i >= n) continue;
+    uint32_t f = 0, m = (uint32_t)n;
+    const int64_t j = kd_find((uint32_t)i, level, f, m);
+    // second children of the j nodes before: q0 and q0 + 1 particles, larger = f - j q0 of the latter
+    const int64_t larger = (int64_t)f - j * q0;
+    const int64_t nodes_before = (j - larger) * (q0 - q0 / 2) + larger * (q0 + 1 - (q0 + 1) / 2);
+    const uint32_t r = (uint32_t)(base + ex[q] - nodes_before);
+    out[fl[q] ? f + m / 2 + r : (uint32_t)i - r] = v[q];
   }
 }
 
-__global__ void k_kd_pnode(int64_t n, const unsigned long long *__restrict__ lv, int level,
-                           uint32_t *__restrict__ pnode, const uint32_t *__restrict__ first,
-                           const uint32_t *__restrict__ count, const int *__restrict__ child) {
-  const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (i >= n) return;
-  const int64_t lo = (int64_t)lv[2 * level];
-  const uint32_t k = pnode[i];
-  if ((int64_t)k < lo || child[k] < 0) return;
-  pnode[i] = (uint32_t)child[k] + ((uint32_t)i - first[k] >= count[k] / 2 ? 1u : 0u);
+// A node of at most 2048 particles to its leaves, one block: the orders as 16-bit places
+// in the node's x order, partitioned level by level in shared memory.
+constexpr int kSub = 2048;
+__global__ void __launch_bounds__(kT) k_kd_subtree(KdShape S, int top, const double *__restrict__ xw, KdOrders O,
+                                                   uint32_t *__restrict__ place, uint32_t *__restrict__ out,
+                                                   double *__restrict__ box, int64_t cap, int *__restrict__ axis) {
+  constexpr int kPer = kSub / kT;
+  __shared__ uint32_t id[kSub];           // the node's particles in x order
+  __shared__ __align__(16) uint16_t ord[2][3][kSub];  // the three orders, before and after a level
+  __shared__ uint16_t scan[3][kSub];         // second-child particles before each position
+  __shared__ uint8_t side[kSub], sax[kSub];  // per particle; split axis per node of the level (3: a leaf)
+  const int tid = threadIdx.x, lane = tid & 31, w = tid >> 5;
+  const int64_t n = S.n;
+  uint32_t f0, m0;
+  kd_range(n, top, blockIdx.x, f0, m0);
+  for (uint32_t i = tid; i < m0; i += kT) {
+    const uint32_t p = O.o[0][f0 + i];
+    id[i] = p;
+    place[p] = i;
+    ord[0][0][i] = (uint16_t)i;
+  }
+  __syncthreads();
+  for (uint32_t i = tid; i < m0; i += kT) {
+    ord[0][1][i] = (uint16_t)place[O.o[1][f0 + i]];
+    ord[0][2][i] = (uint16_t)place[O.o[2][f0 + i]];
+  }
+  __syncthreads();
+  int b = 0;
+  for (int l = top; l <= S.depth; ++l) {
+    const int r = l - top;
+    // ---- the level's nodes: boxes, axes
+    for (uint32_t jj = tid; jj < (1u << r); jj += kT) {
+      uint32_t f = 0, m = m0;
+      for (int q = r - 1; q >= 0; --q) {
+        const uint32_t h = m / 2;
+        if ((jj >> q) & 1u) {
+          f += h;
+          m -= h;
+        } else {
+          m = h;
+        }
+      }
+      const int64_t j = ((int64_t)blockIdx.x << r) + jj, k = ((int64_t)1 << l) - 1 + j;
+      const int a = kd_box(xw, n, f, m, [&](int d, uint32_t i) { return id[ord[b][d][i]]; }, box, cap, k);
+      const bool split = (int64_t)m > S.leaf_max;
+      axis[k] = split ? a : -1;
+      sax[jj] = split ? (uint8_t)a : (uint8_t)3;
+    }
+    __syncthreads();
+    if (l == S.depth && S.nsplit == 0) break;
+    // ---- sides
+    for (uint32_t i = tid; i < m0; i += kT) {
+      uint32_t f = 0, m = m0;
+      const int a = sax[kd_find(i, r, f, m)];
+      if (a < 3) side[ord[b][a][i]] = i - f >= m / 2 ? 1 : 0;
+      else side[ord[b][0][i]] = 0;
+    }
+    __syncthreads();
+    // ---- scans of the three orders at once (counts below 2^20 each)
+    {
+      uint32_t bits = 0;
+      unsigned long long s = 0;
+#pragma unroll
+      for (int q = 0; q < kPer; ++q) {
+        const uint32_t i = (uint32_t)tid * kPer + q;
+#pragma unroll
+        for (int d = 0; d < 3; ++d)
+          if (i < m0 && side[ord[b][d][i]]) {
+            bits |= 1u << (3 * q + d);
+            s += 1ull << (20 * d);
+          }
+      }
+      unsigned long long x = s;
+#pragma unroll
+      for (int o = 1; o < 32; o <<= 1) {
+        const unsigned long long y = __shfl_up_sync(0xffffffffu, x, o);
+        if (lane >= o) x += y;
+      }
+      // the warps' totals in the orders' other half, which the partition writes after the next barrier
+      unsigned long long *wsum = reinterpret_cast<unsigned long long *>(&ord[b ^ 1][0][0]);
+      if (lane == 31) wsum[w] = x;
+      __syncthreads();
+      unsigned long long at = x - s;
+      for (int q = 0; q < w; ++q) at += wsum[q];
+#pragma unroll
+      for (int q = 0; q < kPer; ++q) {
+        const uint32_t i = (uint32_t)tid * kPer + q;
+#pragma unroll
+        for (int d = 0; d < 3; ++d) {
+          scan[d][i] = (uint16_t)((at >> (20 * d)) & 0xfffffu);
+          if ((bits >> (3 * q + d)) & 1u) at += 1ull << (20 * d);
+        }
+      }
+    }
+    __syncthreads();
+    // ---- stable partition inside every node that splits
+    for (uint32_t i = tid; i < m0; i += kT) {
+      uint32_t f = 0, m = m0;
+      const bool split = sax[kd_find(i, r, f, m)] < 3;
+#pragma unroll
+      for (int d = 0; d < 3; ++d) {
+        const uint16_t v = ord[b][d][i];
+        const uint32_t before = (uint32_t)scan[d][i] - scan[d][f];
+        ord[b ^ 1][d][split ? (side[v] ? f + m / 2 + before : i - before) : i] = v;
+      }
+    }
+    __syncthreads();
+    b ^= 1;
+    // ---- the children of a level that splits in part: the last level's boxes
+    if (l == S.depth) {
+      for (uint32_t jj = tid; jj < (1u << r); jj += kT) {
+        if (sax[jj] == 3) continue;
+        uint32_t f = 0, m = m0;
+        for (int q = r - 1; q >= 0; --q) {
+          const uint32_t h = m / 2;
+          if ((jj >> q) & 1u) {
+            f += h;
+            m -= h;
+          } else {
+            m = h;
+          }
+        }
+        const int64_t j = ((int64_t)blockIdx.x << r) + jj;
+        const int64_t c = S.last_start() + 2 * ((int64_t)f0 + f - j * S.q);
+        auto at = [&](int d, uint32_t i) { return id[ord[b][d][i]]; };
+        kd_box(xw, n, f, m / 2, at, box, cap, c);
+        kd_box(xw, n, f + m / 2, m - m / 2, at, box, cap, c + 1);
+        axis[c] = axis[c + 1] = -1;
+      }
+    }
+  }
+  for (uint32_t i = tid; i < m0; i += kT) out[f0 + i] = id[ord[b][0][i]];
 }
 
 // Centre, half extents, side and expansion scale of every node.
 __global__ void k_kd_geo(int64_t nn, int64_t cap, const double *__restrict__ box, double L, double *__restrict__ geo,
-                         float *__restrict__ geof, float *__restrict__ hs, const int *__restrict__ child,
-                         uint32_t *__restrict__ lflag) {
+                         float *__restrict__ geof, float *__restrict__ hs, const int *__restrict__ child) {
   const int64_t k = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (k >= nn) return;
   double side = 0.0;
@@ -251,24 +457,21 @@ __global__ void k_kd_geo(int64_t nn, int64_t cap, const double *__restrict__ box
   double h = L;
   for (int j = 0; j < kDepth && side <= 0.5 * h; ++j) h *= 0.5;
   hs[k] = (float)h;
-  lflag[k] = child[k] < 0 ? 1u : 0u;
-}
-
-__global__ void k_kd_leaves(int64_t nn, const uint32_t *__restrict__ lflag, const uint32_t *__restrict__ lscan,
-                            uint32_t *__restrict__ leaves) {
-  const int64_t k = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (k >= nn || !lflag[k]) return;
-  leaves[lscan[k]] = (uint32_t)k;
 }
 
 // Particles in tree order: positions, input index, offset from the leaf's box centre and mass.
 __global__ void k_kd_particles(int64_t n, const uint32_t *__restrict__ o0, const double *__restrict__ xw,
-                               const float *__restrict__ mass, const uint32_t *__restrict__ pnode,
+                               const float *__restrict__ mass, KdShape S,
                                const double *__restrict__ geo, int64_t cap, double *__restrict__ xs,
                                uint32_t *__restrict__ perm, float4 *__restrict__ pm4) {
   const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= n) return;
-  const uint32_t p = o0[i], k = pnode[i];
+  // the leaf of position i
+  uint32_t f = 0, m = (uint32_t)n;
+  const int64_t j = kd_find((uint32_t)i, S.depth, f, m);
+  int64_t k = ((int64_t)1 << S.depth) - 1 + j;
+  if ((int64_t)m > S.leaf_max) k = S.last_start() + 2 * ((int64_t)f - j * S.q) + ((uint32_t)i - f >= m / 2 ? 1 : 0);
+  const uint32_t p = o0[i];
   float off[3];
 #pragma unroll
   for (int d = 0; d < 3; ++d) {
@@ -891,10 +1094,12 @@ cudaError_t kd_build_tree(Ctx &c, const double *pos, const float *mass, int64_t 
     c.have_tree = true;
     return cudaSuccess;
   }
-  // a leaf of a split node holds at least floor((leaf_max + 1) / 2) particles
+  const KdShape S = kd_shape(n, c.prm.leaf_max);
+  const int64_t nn = S.nodes(), cap = nn + 2;
+  // the nodes that n particles can take in the worst case must fit the lists' node bits
   const int64_t lmin = std::max(1, (c.prm.leaf_max + 1) / 2);
-  const int64_t cap = 2 * ((n + lmin - 1) / lmin) + 2;
-  if (cap > ((int64_t)1 << kSinkBits)) return cudaErrorInvalidValue;  // mapped to HFMM_ERR_CAPACITY
+  if (2 * ((n + lmin - 1) / lmin) + 2 > ((int64_t)1 << kSinkBits))
+    return cudaErrorInvalidValue;  // mapped to HFMM_ERR_CAPACITY
   kd.cap = cap;
   if (c.prm.profile & 1) cudaEventRecord(c.ev[0], st);
   TRY(ensure(kd.xw, (size_t)n * 24));
@@ -903,11 +1108,7 @@ cudaError_t kd_build_tree(Ctx &c, const double *pos, const float *mass, int64_t 
     TRY(ensure(kd.ord2[d], (size_t)n * 4));
   }
   TRY(ensure(kd.side, (size_t)n));
-  TRY(ensure(kd.flag, (size_t)n * 12));
-  TRY(ensure(kd.scan, (size_t)n * 12));
-  TRY(ensure(kd.pnode, (size_t)n * 4));
-  TRY(ensure(kd.nflag, (size_t)cap * 4));
-  TRY(ensure(kd.nscan, (size_t)cap * 4));
+  TRY(ensure(kd.place, (size_t)n * 4));
   TRY(ensure(kd.first, (size_t)cap * 4));
   TRY(ensure(kd.count, (size_t)cap * 4));
   TRY(ensure(kd.child, (size_t)cap * 4));
@@ -936,79 +1137,46 @@ cudaError_t kd_build_tree(Ctx &c, const double *pos, const float *mass, int64_t 
     if (alt) std::swap(kd.ord[d], kd.ord2[d]);
   }
   if (c.prm.profile & 1) cudaEventRecord(c.ev[1], st);
-  uint32_t *first = P<uint32_t>(kd.first), *count = P<uint32_t>(kd.count);
-  int *child = P<int>(kd.child), *parent = P<int>(kd.parent), *axis = P<int>(kd.axis);
-  TRY(ensure(kd.ctr, 128));
-  uint64_t *total = P<uint64_t>(kd.ctr) + kWalkCtr;  // after the walk's counters
-  // The depth from the counts alone: the counts of a level differ by at most one (a
-  // split gives floor and ceil halves), so [qmin, qmax] bounds them level by level.
-  int levels = 1;
-  for (int64_t qmin = n, qmax = n; qmax > c.prm.leaf_max; ++levels) {
-    qmin = std::max<int64_t>(qmin, c.prm.leaf_max + 1) / 2;
-    qmax = (qmax + 1) / 2;
+  int *child = P<int>(kd.child), *axis = P<int>(kd.axis);
+  const unsigned gn = blocks_for((size_t)n, kT), gk = blocks_for((size_t)nn, kT);
+  k_kd_topology<<<blocks_for((size_t)S.last_start(), kT), kT, 0, st>>>(
+      S, P<uint32_t>(kd.first), P<uint32_t>(kd.count), child, P<int>(kd.parent), P<uint32_t>(c.leaves));
+  note_launch();
+  auto orders = [&]() { return KdOrders{{P<uint32_t>(kd.ord[0]), P<uint32_t>(kd.ord[1]), P<uint32_t>(kd.ord[2])}}; };
+  // levels of nodes above kSub particles
+  int top = 0;
+  while (top < S.depth && ((n + ((int64_t)1 << top) - 1) >> top) > kSub) ++top;
+  const unsigned ntiles = blocks_for((size_t)n, kPartTile);
+  if (top > 0) {
+    const size_t words = 3 * (size_t)ntiles + 1;  // a level's ticket and counts
+    TRY(ensure(c.tmp2, (size_t)top * words * 8));
+    TRY(cudaMemsetAsync(c.tmp2.p, 0, (size_t)top * words * 8, st));
+    for (int l = 0; l < top; ++l) {
+      k_kd_axis<<<blocks_for((size_t)1 << l, 128), 128, 0, st>>>(n, l, xw, orders(), P<double>(kd.box), cap, axis);
+      k_kd_side<<<gn, kT, 0, st>>>(n, l, axis, orders(), P<uint8_t>(kd.side));
+      unsigned long long *lw = P<unsigned long long>(c.tmp2) + (size_t)l * words;
+      k_kd_part<<<3 * ntiles, kT, 0, st>>>(n, l, orders(), P<uint32_t>(kd.ord2[0]), P<uint32_t>(kd.ord2[1]),
+                                           P<uint32_t>(kd.ord2[2]), P<uint8_t>(kd.side),
+                                           reinterpret_cast<unsigned *>(lw), lw + 1, ntiles);
+      note_launch(3);
+      for (int d = 0; d < 3; ++d) std::swap(kd.ord[d], kd.ord2[d]);
+    }
   }
-  if (levels > kKdMaxLevels) return cudaErrorInvalidValue;
-  TRY(ensure(kd.lv, sizeof(unsigned long long) * 2 * (kKdMaxLevels + 1)));
-  unsigned long long *lv = P<unsigned long long>(kd.lv);
-  k_kd_root<<<1, 1, 0, st>>>(n, first, count, parent, lv);
+  k_kd_subtree<<<1u << top, kT, 0, st>>>(S, top, xw, orders(), P<uint32_t>(kd.place), P<uint32_t>(kd.ord2[0]),
+                                         P<double>(kd.box), cap, axis);
   note_launch();
-  TRY(cudaMemsetAsync(kd.pnode.p, 0, (size_t)n * 4, st));
-  const unsigned gn = blocks_for((size_t)n, kT);
-  // every level on the device, its extent read by the kernels (no read-back per level)
-  for (int level = 0; level < levels; ++level) {
-    const int64_t bound = std::min<int64_t>(level < 62 ? (int64_t)1 << level : cap, cap);
-    const unsigned gl = blocks_for((size_t)bound, kT);
-    k_kd_level<<<gl, kT, 0, st>>>(lv, level, bound, c.prm.leaf_max, xw, n, P<uint32_t>(kd.ord[0]),
-                                  P<uint32_t>(kd.ord[1]), P<uint32_t>(kd.ord[2]), first, count, P<double>(kd.box),
-                                  cap, axis, P<uint32_t>(kd.nflag));
-    note_launch();
-    const bool last = level + 1 == levels;  // no node of the last level splits
-    if (!last) TRY(scan_u32(P<uint32_t>(kd.nflag), P<uint32_t>(kd.nscan), total, (size_t)bound, c.tmp2, st));
-    k_kd_children<<<gl, kT, 0, st>>>(lv, level, axis, P<uint32_t>(kd.nscan), first, count, child, parent);
-    note_launch();
-    if (last) break;
-    k_kd_next<<<1, 1, 0, st>>>(lv, level, total);
-    note_launch();
-    k_kd_side<<<gn, kT, 0, st>>>(n, lv, level, P<uint32_t>(kd.pnode), first, count, axis, P<uint32_t>(kd.ord[0]),
-                                 P<uint32_t>(kd.ord[1]), P<uint32_t>(kd.ord[2]), P<uint8_t>(kd.side));
-    note_launch();
-    k_kd_flag<<<gn, kT, 0, st>>>(n, lv, level, P<uint32_t>(kd.pnode), axis, P<uint32_t>(kd.ord[0]),
-                                 P<uint32_t>(kd.ord[1]), P<uint32_t>(kd.ord[2]), P<uint8_t>(kd.side),
-                                 P<uint32_t>(kd.flag));
-    note_launch();
-    TRY(scan_u32(P<uint32_t>(kd.flag), P<uint32_t>(kd.scan), total, (size_t)(3 * n), c.tmp2, st));
-    k_kd_scatter<<<gn, kT, 0, st>>>(n, lv, level, P<uint32_t>(kd.pnode), first, count, axis, P<uint32_t>(kd.ord[0]),
-                                    P<uint32_t>(kd.ord[1]), P<uint32_t>(kd.ord[2]), P<uint8_t>(kd.side),
-                                    P<uint32_t>(kd.scan), P<uint32_t>(kd.ord2[0]), P<uint32_t>(kd.ord2[1]),
-                                    P<uint32_t>(kd.ord2[2]));
-    note_launch();
-    for (int d = 0; d < 3; ++d) std::swap(kd.ord[d], kd.ord2[d]);
-    k_kd_pnode<<<gn, kT, 0, st>>>(n, lv, level, P<uint32_t>(kd.pnode), first, count, child);
-    note_launch();
-  }
-  // the level extents back (one read-back): nodes, levels, and a full binary tree's leaves
-  uint64_t ext[2 * (kKdMaxLevels + 1)];
-  TRY(read_u64(c, lv, ext, 2 * levels, st));
-  int64_t hi = 0;
-  for (int level = 0; level < levels; ++level) {
-    if (ext[2 * level + 1] == ext[2 * level]) break;  // an empty level: the tree ended above
-    kd.level_start.push_back((int64_t)ext[2 * level + 1]);
-    hi = (int64_t)ext[2 * level + 1];
-    c.nlevels = level + 1;
-  }
-  if (hi > cap) return cudaErrorInvalidValue;
-  c.nnodes = hi;
-  const unsigned gk = blocks_for((size_t)hi, kT);
-  k_kd_geo<<<gk, kT, 0, st>>>(hi, cap, P<double>(kd.box), c.prm.box, P<double>(kd.geo), P<float>(kd.geof),
-                              P<float>(kd.hs), child, P<uint32_t>(kd.nflag));
+  std::swap(kd.ord[0], kd.ord2[0]);
+  c.nnodes = nn;
+  c.nleaves = S.leaves();
+  c.nlevels = S.depth + 1 + (S.nsplit ? 1 : 0);
+  for (int l = 0; l <= S.depth; ++l) kd.level_start.push_back(((int64_t)2 << l) - 1);
+  if (S.nsplit) kd.level_start.push_back(nn);
+  k_kd_geo<<<gk, kT, 0, st>>>(nn, cap, P<double>(kd.box), c.prm.box, P<double>(kd.geo), P<float>(kd.geof),
+                              P<float>(kd.hs), child);
   note_launch();
-  TRY(scan_u32(P<uint32_t>(kd.nflag), P<uint32_t>(kd.nscan), total, (size_t)hi, c.tmp2, st));
-  k_kd_leaves<<<gk, kT, 0, st>>>(hi, P<uint32_t>(kd.nflag), P<uint32_t>(kd.nscan), P<uint32_t>(c.leaves));
+  k_kd_particles<<<gn, kT, 0, st>>>(n, P<uint32_t>(kd.ord[0]), xw, mass, S, P<double>(kd.geo), cap, P<double>(c.xs),
+                                    P<uint32_t>(c.idx), P<float4>(c.pm4));
   note_launch();
-  k_kd_particles<<<gn, kT, 0, st>>>(n, P<uint32_t>(kd.ord[0]), xw, mass, P<uint32_t>(kd.pnode), P<double>(kd.geo),
-                                    cap, P<double>(c.xs), P<uint32_t>(c.idx), P<float4>(c.pm4));
-  note_launch();
-  c.nleaves = (hi + 1) / 2;  // every split node has two children
   if (c.prm.profile & 1) cudaEventRecord(c.ev[2], st);
   c.have_tree = true;
   return cudaGetLastError();
