@@ -35,8 +35,8 @@
 // run on into the next tile, whose values only reach rows of P that are never
 // read): 47 KB a worker at p = 6.  Four warps an SM with 128-pair chunks, every
 // thread computing both operands and all four K-tiles issued whatever the list's
-// length, took 20.8 ms for the 33M pairs of the 2M learned step instead of 8.4 (issue
-// 36%, tensor pipe 22% with four workers; 8.6 without the row prefetch).
+// length, took 20.8 ms for the 33M pairs of the 2M learned step instead of 8.6 (issue
+// 36%, tensor pipe 22%; the next rows prefetched into L1: the same).
 #include <algorithm>
 #include <type_traits>
 
@@ -194,11 +194,6 @@ __global__ void __launch_bounds__(kThreads, 1)
     auto fetch = [&]() {
       e = t0 + lane < te ? lst[t0 + lane] : 0ull;
       cb = t0 + lane < te ? cell[pair_src(e)] : ca;
-      if (warp == 1) {  // the multipole rows into L1
-        const char *row = reinterpret_cast<const char *>(M + (size_t)pair_src(e) * ldm);
-#pragma unroll
-        for (int o = 0; o < NC * 4; o += 128) asm volatile("prefetch.global.L1 [%0];" ::"l"(row + o));
-      }
     };
     fetch();
     for (int si = 0; si < ns; ++si) {
