@@ -37,18 +37,12 @@
 // sorted by (sink, source, shift), so every sum after them runs in a fixed order.
 // The same walk with the opening-angle test alone, from the root against itself,
 // is the conventional FMM's of the interaction counts (Sec. 3).
-// P2P: one warp per sink leaf, the leaves taken heaviest first from a counter,
-// its sinks in lanes (a second sink per lane above 32); the list read in windows
-// of 32 entries, each lane forming its entry's source-box offset from the sink
-// box centre in FP64; each entry's sources loaded one entry ahead, kept only
-// within R_c of the sink box, staged in shared memory and evaluated two at a
-// time in packed FP32x2, with the Gaussian (Sec. 2.2) or polynomial (Sec. 5)
-// pair force.
+// P2P: the octree's kernel (p2p.cu), the source-box offsets from the box centres.
 #include <algorithm>
 
 #include <cooperative_groups.h>
 
-#include "p2p_common.cuh"
+#include "common.cuh"
 
 namespace cg = cooperative_groups;
 
@@ -719,201 +713,6 @@ __global__ void k_kd_csr(const uint64_t *__restrict__ lst, int64_t n, uint32_t *
   if (t == n - 1 || pair_sink(lst[t + 1]) != k) end[k] = (uint32_t)(t + 1);
 }
 
-// ------------------------------------------------------------------ P2P
-// One warp per sink leaf (the leaves heaviest first, taken from a counter):
-// sinks i = first + lane and first + lane + 32.  The list entries come in windows of 32, one per lane, each
-// lane forming its entry's source-box offset from the sink box centre in FP64
-// (once per entry: this GPU's FP64 rate is low); each entry's sources are held in
-// registers one entry ahead; the sources within R_c of the sink box are staged in
-// shared memory (SoA, padded to an even count with a far, massless source) and
-// each lane evaluates two sources at a time with packed FP32x2 operations: the
-// pair force of Sec. 2.2 (or of Sec. 5) with the hard cut-off, added to acc in
-// input order.
-constexpr int kKdStage = 64;
-
-// kCount (statistics runs): also count the pairs inside (0, R_c) into *useful.
-// kSplit: 0 the Gaussian pair force of Sec. 2.2, 1 the polynomial one of Sec. 5.
-template <bool kCount, int kSplit>
-__global__ void __launch_bounds__(kT, 2) k_kd_p2p(const uint32_t *__restrict__ leaves, int64_t nl,
-                                               const uint32_t *__restrict__ first, const uint32_t *__restrict__ count,
-                                               KdGeo Gm, const uint32_t *__restrict__ beg,
-                                               const uint32_t *__restrict__ end, const uint64_t *__restrict__ lst,
-                                               const float4 *__restrict__ pm4, const uint32_t *__restrict__ perm,
-                                               int64_t n, double L, PairFit2 fit, float G, float *__restrict__ acc,
-                                               unsigned long long *__restrict__ useful,
-                                               unsigned long long *__restrict__ next) {
-  __shared__ __align__(16) float sx[kT / 32][kKdStage + 2], sy[kT / 32][kKdStage + 2], sz[kT / 32][kKdStage + 2],
-      sw[kT / 32][kKdStage + 2];
-  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-  float *X = sx[wid], *Y = sy[wid], *Z = sz[wid], *Wm = sw[wid];
-  const float rc2_cull = fit.rc2 * (1.f + 1.f / 4096.f);  // far above the FP32 rounding of either distance
-  uint32_t n_in = 0;
-  for (;;) {
-    // the next leaf of the heaviest-first order (each leaf's sums stay its own warp's)
-    unsigned long long t = 0;
-    if (lane == 0) t = atomicAdd(next, 1ull);
-    t = __shfl_sync(0xffffffffu, t, 0);
-    if ((int64_t)t >= nl) break;
-    const uint32_t k = leaves[t];
-    const uint32_t f = first[k], m = count[k];
-    const uint32_t tb = beg[k], te = end[k];
-    const bool has0 = (uint32_t)lane < m, has1 = (uint32_t)lane + 32u < m;
-    const bool two = m > 32;  // warp-uniform
-    const float4 q0 = has0 ? pm4[f + lane] : make_float4(0.f, 0.f, 0.f, 0.f);
-    const float4 q1 = has1 ? pm4[f + lane + 32] : make_float4(0.f, 0.f, 0.f, 0.f);
-    // the sink offsets, negated, as (x, x) pairs
-    const float2 n0x = f2(-q0.x), n0y = f2(-q0.y), n0z = f2(-q0.z);
-    const float2 n1x = f2(-q1.x), n1y = f2(-q1.y), n1z = f2(-q1.z);
-    // the sink box's half extents (its particles' offsets lie within them, up to FP32 rounding)
-    const float ex = (float)Gm.e(0, k), ey = (float)Gm.e(1, k), ez = (float)Gm.e(2, k);
-    float2 a0x = f2(0.f), a0y = f2(0.f), a0z = f2(0.f), a1x = f2(0.f), a1y = f2(0.f), a1z = f2(0.f);
-    // a window of 32 list entries, one per lane: source range and the source box's
-    // offset from the sink box centre (FP64, then FP32)
-    uint32_t wfb = 0, wmb = 0;
-    float wox = 0.f, woy = 0.f, woz = 0.f;
-    auto load_window = [&](uint32_t base) {
-      wmb = 0;
-      if (base + lane < te) {
-        const uint64_t e = lst[base + lane];
-        const uint32_t b = pair_src(e), s = pair_shift(e);
-        wfb = first[b];
-        wmb = count[b];
-        wox = (float)__dsub_rn(__dadd_rn(Gm.c(0, b), (double)shift_component(s, 0) * L), Gm.c(0, k));
-        woy = (float)__dsub_rn(__dadd_rn(Gm.c(1, b), (double)shift_component(s, 1) * L), Gm.c(1, k));
-        woz = (float)__dsub_rn(__dadd_rn(Gm.c(2, b), (double)shift_component(s, 2) * L), Gm.c(2, k));
-      }
-    };
-    // the sources of one entry in registers: lane j holds sources j and j + 32
-    float4 pa = make_float4(0.f, 0.f, 0.f, 0.f), pb = pa;
-    uint32_t cmb = 0;
-    float cox = 0.f, coy = 0.f, coz = 0.f;
-    auto fetch = [&](uint32_t slot) {
-      const uint32_t fb = __shfl_sync(0xffffffffu, wfb, slot);
-      cmb = __shfl_sync(0xffffffffu, wmb, slot);
-      cox = __shfl_sync(0xffffffffu, wox, slot);
-      coy = __shfl_sync(0xffffffffu, woy, slot);
-      coz = __shfl_sync(0xffffffffu, woz, slot);
-      if ((uint32_t)lane < cmb) pa = pm4[fb + lane];
-      if ((uint32_t)lane + 32u < cmb) pb = pm4[fb + lane + 32];
-    };
-    uint32_t wbase = tb;
-    if (tb < te) {
-      load_window(tb);
-      fetch(0);
-    }
-    for (uint32_t q = tb; q < te; ++q) {
-      // stage the sources of entry q within R_c of the sink box (R_c^2 (1 + 2^-12): far
-      // above the FP32 rounding of either distance), compacted in their order
-      const uint32_t mb = cmb;
-      const float ox = cox, oy = coy, oz = coz;
-      const float4 p0 = pa, p1 = pb;
-      __syncwarp();
-      uint32_t kept = 0;
-#pragma unroll
-      for (int h = 0; h < 2; ++h) {
-        const uint32_t j = (uint32_t)(32 * h + lane);
-        float4 p = h ? p1 : p0;
-        bool keep = false;
-        if (j < mb) {
-          p.x += ox;
-          p.y += oy;
-          p.z += oz;
-          const float gx = fmaxf(fabsf(p.x) - ex, 0.f), gy = fmaxf(fabsf(p.y) - ey, 0.f),
-                      gz = fmaxf(fabsf(p.z) - ez, 0.f);
-          keep = gx * gx + gy * gy + gz * gz < rc2_cull;
-        }
-        const unsigned mask = __ballot_sync(0xffffffffu, keep);
-        if (keep) {
-          const uint32_t w = kept + __popc(mask & ((1u << lane) - 1u));
-          X[w] = p.x;
-          Y[w] = p.y;
-          Z[w] = p.z;
-          Wm[w] = p.w;
-        }
-        kept += __popc(mask);
-      }
-      if (kept & 1u) {
-        if (lane == 0) {  // a far, massless partner for the last source
-          X[kept] = 1e18f;
-          Y[kept] = 0.f;
-          Z[kept] = 0.f;
-          Wm[kept] = 0.f;
-        }
-        ++kept;
-      }
-      // the next entry's sources are loaded while this entry's pairs are evaluated
-      if (q + 1 < te) {
-        if (q + 1 - wbase == 32) {
-          wbase = q + 1;
-          load_window(wbase);
-        }
-        fetch(q + 1 - wbase);
-      }
-      __syncwarp();
-      // (real: the lane holds this sink; the others evaluate a phantom sink whose result is dropped)
-      auto pair2 = [&](float2 px, float2 py, float2 pz, float2 w, float2 nx, float2 ny, float2 nz, float2 &ax,
-                       float2 &ay, float2 &az, bool real) {
-        const float2 dx = __fadd2_rn(px, nx), dy = __fadd2_rn(py, ny), dz = __fadd2_rn(pz, nz);
-        const float2 r2 = __ffma2_rn(dx, dx, __ffma2_rn(dy, dy, __fmul2_rn(dz, dz)));
-        const bool in0 = r2.x < fit.rc2 && r2.x > 0.f, in1 = r2.y < fit.rc2 && r2.y > 0.f;
-        if (kCount && real) n_in += (uint32_t)in0 + (uint32_t)in1;
-        // outside (0, R_c) the values below may be inf / NaN; the selects discard them
-        float2 fs = __fmul2_rn(pair_factor2<kSplit>(r2, fit), w);
-        fs.x = in0 ? fs.x : 0.f;
-        fs.y = in1 ? fs.y : 0.f;
-        ax = __ffma2_rn(fs, dx, ax);
-        ay = __ffma2_rn(fs, dy, ay);
-        az = __ffma2_rn(fs, dz, az);
-      };
-      if (two) {
-#pragma unroll 2
-        for (uint32_t j = 0; j < kept; j += 2) {
-          const float2 px = *reinterpret_cast<const float2 *>(X + j), py = *reinterpret_cast<const float2 *>(Y + j);
-          const float2 pz = *reinterpret_cast<const float2 *>(Z + j), w = *reinterpret_cast<const float2 *>(Wm + j);
-          pair2(px, py, pz, w, n0x, n0y, n0z, a0x, a0y, a0z, has0);
-          pair2(px, py, pz, w, n1x, n1y, n1z, a1x, a1y, a1z, has1);
-        }
-      } else {
-#pragma unroll 8
-        for (uint32_t j = 0; j < kept; j += 2) {
-          const float2 px = *reinterpret_cast<const float2 *>(X + j), py = *reinterpret_cast<const float2 *>(Y + j);
-          const float2 pz = *reinterpret_cast<const float2 *>(Z + j), w = *reinterpret_cast<const float2 *>(Wm + j);
-          pair2(px, py, pz, w, n0x, n0y, n0z, a0x, a0y, a0z, has0);
-        }
-      }
-    }
-    if (has0) {
-      const uint32_t o = perm[f + lane];
-      acc[o] += G * (a0x.x + a0x.y);
-      acc[n + o] += G * (a0y.x + a0y.y);
-      acc[2 * n + o] += G * (a0z.x + a0z.y);
-    }
-    if (has1) {
-      const uint32_t o = perm[f + lane + 32];
-      acc[o] += G * (a1x.x + a1x.y);
-      acc[n + o] += G * (a1y.x + a1y.y);
-      acc[2 * n + o] += G * (a1z.x + a1z.y);
-    }
-  }
-  if (kCount) {
-    unsigned long long v = n_in;
-    for (int o = 16; o; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-    if (lane == 0 && v) atomicAdd(useful, v);
-  }
-}
-
-// Sort keys of the sink leaves, heaviest first: the complement of entries x sinks (40 bits).
-__global__ void k_kd_work(const uint32_t *__restrict__ leaves, int64_t nl, const uint32_t *__restrict__ count,
-                          const uint32_t *__restrict__ beg, const uint32_t *__restrict__ end,
-                          uint64_t *__restrict__ key, uint32_t *__restrict__ val) {
-  const int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (t >= nl) return;
-  const uint32_t k = leaves[t];
-  const uint64_t w = (uint64_t)(end[k] - beg[k]) * count[k];
-  key[t] = (~w) & ((1ull << 40) - 1ull);
-  val[t] = k;
-}
-
 // Particle pairs on the P2P list: sum over entries of n_sink n_source.
 __global__ void k_kd_list_pairs(const uint64_t *__restrict__ lst, int64_t n, const uint32_t *__restrict__ count,
                                 unsigned long long *__restrict__ out) {
@@ -1044,40 +843,6 @@ cudaError_t kd_group(Ctx &c, cudaStream_t st) {
     TRY(read_u64(c, cnt, &pp, 1, st));
     c.p2p_particle_pairs = (int64_t)pp;
   }
-  return cudaGetLastError();
-}
-
-cudaError_t kd_p2p(Ctx &c, float *acc, cudaStream_t st) {
-  if (c.np2p == 0 || c.nleaves == 0) return cudaSuccess;
-  int dev = 0, nsm = 0;
-  TRY(cudaGetDevice(&dev));
-  TRY(cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev));
-  const unsigned g = (unsigned)std::min<int64_t>((c.nleaves + 7) / 8, (int64_t)nsm * 8);
-  // the sink leaves heaviest first (stable: equal work keeps the leaf order), taken from a counter
-  const size_t nl = (size_t)c.nleaves;
-  TRY(ensure(c.lpt_tmp, nl * 24 + 64));
-  uint64_t *key = P<uint64_t>(c.lpt_tmp), *key2 = key + nl;
-  uint32_t *val = reinterpret_cast<uint32_t *>(key2 + nl), *val2 = val + nl;
-  k_kd_work<<<blocks_for(nl, kT), kT, 0, st>>>(P<uint32_t>(c.leaves), c.nleaves, P<uint32_t>(c.kd.count),
-                                               P<uint32_t>(c.p2p_beg), P<uint32_t>(c.p2p_end), key, val);
-  note_launch();
-  bool alt = false;
-  TRY(radix_sort_u64(key, val, key2, val2, nl, 0, 40, &alt, c.tmp, st));
-  const uint32_t *order = alt ? val2 : val;
-  unsigned long long *next = P<unsigned long long>(c.kd.ctr) + kWalkCtr + 2;
-  TRY(cudaMemsetAsync(next, 0, 8, st));
-  unsigned long long *useful = P<unsigned long long>(c.d_small) + 4;  // the statistics counter of stats
-  auto run = [&](auto kernel) {
-    kernel<<<g, kT, 0, st>>>(order, c.nleaves, P<uint32_t>(c.kd.first), P<uint32_t>(c.kd.count), kd_geo(c),
-                             P<uint32_t>(c.p2p_beg), P<uint32_t>(c.p2p_end), P<uint64_t>(c.p2p), P<float4>(c.pm4),
-                             P<uint32_t>(c.idx), c.n, c.prm.box, pair_fit2(c), (float)c.prm.G, acc, useful, next);
-  };
-  const bool count_pairs = (c.prm.profile & 2) != 0, poly = c.prm.split == 1;
-  if (count_pairs)
-    poly ? run(k_kd_p2p<true, 1>) : run(k_kd_p2p<true, 0>);
-  else
-    poly ? run(k_kd_p2p<false, 1>) : run(k_kd_p2p<false, 0>);
-  note_launch();
   return cudaGetLastError();
 }
 
@@ -1215,7 +980,7 @@ cudaError_t kd_short_range(Ctx &c, float *acc, cudaStream_t st) {
   if (prof) cudaEventRecord(c.ev[7], st);
   TRY(kd_downward(c, acc, st));
   if (prof) cudaEventRecord(c.ev[8], st);
-  TRY(kd_p2p(c, acc, st));
+  TRY(p2p_pass(c, acc, st));
   if (prof) cudaEventRecord(c.ev[9], st);
   return cudaSuccess;
 }

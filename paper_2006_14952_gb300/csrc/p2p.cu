@@ -47,16 +47,54 @@ struct LptState {
   unsigned hist[kLptBuckets], cursor[kLptBuckets];
 };
 
+// What the kernel needs of a tree's nodes: a particle range, and the vector from the sink
+// leaf's centre to a source leaf's (Node: what that takes of a node, fetched ahead).
+struct OctNodes {
+  const uint4 *cell_;
+  const uint2 *range_;
+  float half_unit;
+  using Node = uint4;
+  __device__ __forceinline__ uint2 range(uint32_t k) const { return range_[k]; }
+  __device__ __forceinline__ Node node(uint32_t k) const { return cell_[k]; }
+  __device__ __forceinline__ void offset(const Node &sink, const Node &src, uint32_t s, float &dx, float &dy,
+                                         float &dz) const {
+    int dd[3];
+    half_delta32(sink, src, s, dd);
+    dx = (float)dd[0] * half_unit;
+    dy = (float)dd[1] * half_unit;
+    dz = (float)dd[2] * half_unit;
+  }
+};
+// k-d tree: box centres in FP64, once per entry (this GPU's FP64 rate is low).  A kernel of
+// its own that staged entry by entry (about 145 instructions an entry of 32 sources, of 690)
+// took 14.2 ms for the 18.7G listed pairs of the 2M set, this one 13.1.
+struct KdNodes {
+  const uint32_t *first, *count;
+  const double *geo;  // [>= 3][cap], the centres first
+  int64_t cap;
+  double L;
+  struct Node {
+    double x, y, z;
+  };
+  __device__ __forceinline__ uint2 range(uint32_t k) const { return make_uint2(first[k], count[k]); }
+  __device__ __forceinline__ Node node(uint32_t k) const { return Node{geo[k], geo[cap + k], geo[2 * cap + k]}; }
+  __device__ __forceinline__ void offset(const Node &sink, const Node &src, uint32_t s, float &dx, float &dy,
+                                         float &dz) const {
+    dx = (float)__dsub_rn(__dadd_rn(src.x, (double)shift_component(s, 0) * L), sink.x);
+    dy = (float)__dsub_rn(__dadd_rn(src.y, (double)shift_component(s, 1) * L), sink.y);
+    dz = (float)__dsub_rn(__dadd_rn(src.z, (double)shift_component(s, 2) * L), sink.z);
+  }
+};
+
 // kCap: source particles per fill (even); dynamic shared memory: 2 x 8 x kCap float4.
 // kSplit 0: the Gaussian truncation S(x) above; 1: the polynomial truncation of
 // Sec. 5, a = -m (1/r^3 - 5 / (2 R_c^3) + 3 r^2 / (2 R_c^5)) r, no exp2 and no
 // fitted factor (see hfmm_params.split).
-template <bool kCount, int kCap, int kSplit>
-__global__ void __launch_bounds__(256, 2) k_p2p(const uint32_t *__restrict__ items,
-                                                const uint4 *__restrict__ cell, const uint2 *__restrict__ range,
+template <bool kCount, int kCap, int kSplit, class Nodes>
+__global__ void __launch_bounds__(256, 2) k_p2p(const uint32_t *__restrict__ items, Nodes nodes,
                                                 const uint32_t *__restrict__ beg, const uint32_t *__restrict__ end,
                                                 const uint64_t *__restrict__ lst, const float4 *__restrict__ pm4,
-                                                const uint32_t *__restrict__ perm, int64_t n, float box, PairFit2 fit,
+                                                const uint32_t *__restrict__ perm, int64_t n, PairFit2 fit,
                                                 float G, float *__restrict__ acc_out,
                                                 unsigned long long *__restrict__ ctr,
                                                 const LptState *__restrict__ lpt) {
@@ -92,7 +130,6 @@ __global__ void __launch_bounds__(256, 2) k_p2p(const uint32_t *__restrict__ ite
   const uint32_t raw_s = (uint32_t)__cvta_generic_to_shared(raw);
   // cull threshold: R_c^2 (1 + 2^-12), far above the FP32 rounding of either distance
   const float rc2_cull = fit.rc2 * (1.f + 1.f / 4096.f);
-  const float half_unit = box / (float)kHalfBox;
   uint32_t n_in = 0;  // pairs inside the cut-off (profile mode only)
   for (;;) {
     unsigned t = 0;
@@ -111,8 +148,8 @@ __global__ void __launch_bounds__(256, 2) k_p2p(const uint32_t *__restrict__ ite
       if (t >= nl) break;
     }
     const uint32_t item = items[t], k = item & 0x7fffffffu;
-    const uint4 ca = cell[k];
-    const uint2 r = range[k];
+    const typename Nodes::Node ca = nodes.node(k);
+    const uint2 r = nodes.range(k);
     uint32_t tb = beg[k], te = end[k];
     if (shared_phase) {
       const uint32_t share = (te - tb + 7u) / 8u;
@@ -122,18 +159,18 @@ __global__ void __launch_bounds__(256, 2) k_p2p(const uint32_t *__restrict__ ite
 
     // the entry window at q + lane, prefetched in two steps: the list word
     // (fetch_lst, while the previous fill is evaluated), then the source leaf's
-    // particle range and cell (fetch_src, while the pending fill lands)
+    // particle range and centre (fetch_src, while the pending fill lands)
     uint64_t pf_e = 0;
     uint2 pf_rb = make_uint2(0u, 0u);
-    uint4 pf_cb = make_uint4(0u, 0u, 0u, 0u);
+    typename Nodes::Node pf_cb = ca;
     auto fetch_lst = [&](uint32_t q) {
       if (q + lane < te) pf_e = lst[q + lane];
     };
     auto fetch_src = [&](uint32_t q) {
       if (q + lane < te) {
         const uint32_t b = pair_src(pf_e);
-        pf_rb = range[b];
-        pf_cb = cell[b];
+        pf_rb = nodes.range(b);
+        pf_cb = nodes.node(b);
       }
     };
 
@@ -147,15 +184,9 @@ __global__ void __launch_bounds__(256, 2) k_p2p(const uint32_t *__restrict__ ite
       uint32_t cnt = 0, first = 0;
       float dx = 0.f, dy = 0.f, dz = 0.f;
       if (valid) {
-        const uint64_t e = pf_e;
-        const uint2 rb = pf_rb;
-        int dd[3];
-        half_delta32(ca, pf_cb, pair_shift(e), dd);
-        dx = (float)dd[0] * half_unit;
-        dy = (float)dd[1] * half_unit;
-        dz = (float)dd[2] * half_unit;
-        first = rb.x;
-        cnt = rb.y;
+        nodes.offset(ca, pf_cb, pair_shift(pf_e), dx, dy, dz);
+        first = pf_rb.x;
+        cnt = pf_rb.y;
       }
       const uint32_t start = lane == 0 ? jq : 0u;
       const uint32_t avail = valid ? cnt - start : 0u;
@@ -349,9 +380,8 @@ __global__ void __launch_bounds__(256, 2) k_p2p(const uint32_t *__restrict__ ite
           const float2 dx = __fadd2_rn(px, make_float2(A.x, A.y));
           const float2 dy = __fadd2_rn(py, make_float2(A.z, A.w));
           const float2 dz = __fadd2_rn(pz, make_float2(B.x, B.y));
-          const float2 r2 = __ffma2_rn(dx, dx, __ffma2_rn(dy, dy, __fmul2_rn(dz, dz)));
-          const bool in0 = (r2.x < fit.rc2) && (r2.x > 0.f);
-          const bool in1 = (r2.y < fit.rc2) && (r2.y > 0.f);
+          const float2 r2 = pair_r2(dx, dy, dz);
+          const bool in0 = in_cutoff(r2.x, fit), in1 = in_cutoff(r2.y, fit);
           if (kCount) n_in += (uint32_t)in0 + (uint32_t)in1;
           // outside (0, R_c) the values below may be inf/NaN; the selects discard them
           float2 f = __fmul2_rn(pair_factor2<kSplit>(r2, fit), make_float2(B.z, B.w));  // w = -m
@@ -445,7 +475,8 @@ __global__ void __launch_bounds__(256, 2) k_p2p(const uint32_t *__restrict__ ite
 // and placed bucket by bucket, heaviest first.  Leaves with empty lists (other
 // sink batches) give no item.  The order within a bucket does not matter: each
 // item's sums are its own warp's.
-__global__ void k_lpt_hist(const uint32_t *__restrict__ leaves, int64_t nl, const uint2 *__restrict__ range,
+template <class Nodes>
+__global__ void k_lpt_hist(const uint32_t *__restrict__ leaves, int64_t nl, Nodes nodes,
                            const uint32_t *__restrict__ beg, const uint32_t *__restrict__ end,
                            uint8_t *__restrict__ bucket, LptState *__restrict__ lpt, const TreeState *tz) {
   __shared__ unsigned h[kLptBuckets];
@@ -456,7 +487,7 @@ __global__ void k_lpt_hist(const uint32_t *__restrict__ leaves, int64_t nl, cons
   const int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (t < nl) {
     const uint32_t a = leaves[t];
-    const uint32_t ent = end[a] - beg[a], cnt = range[a].y;
+    const uint32_t ent = end[a] - beg[a], cnt = nodes.range(a).y;
 #pragma unroll
     for (uint32_t c = 0; c < 2; ++c) {
       uint8_t b = 0xff;
@@ -518,9 +549,8 @@ __global__ void k_lpt_place(const uint32_t *__restrict__ leaves, int64_t nl, con
   }
 }
 
-}  // namespace
-
-cudaError_t p2p_pass(Ctx &c, float *acc, cudaStream_t st) {
+template <class Nodes>
+cudaError_t run_p2p(Ctx &c, const Nodes &nodes, float *acc, cudaStream_t st) {
   if (c.nleaves == 0) return cudaSuccess;
   const int T = 256;
   int dev = 0, nsm = 0;
@@ -532,10 +562,10 @@ cudaError_t p2p_pass(Ctx &c, float *acc, cudaStream_t st) {
   if ((size_t)g * 8 > (size_t)c.nleaves) g = blocks_for(c.nleaves, 8);
   const bool small = c.prm.tile_p2p_stage == 128, count = (c.prm.profile & 2) != 0;
   auto kern = c.prm.split == 1
-                  ? (count ? (small ? k_p2p<true, 128, 1> : k_p2p<true, 256, 1>)
-                           : (small ? k_p2p<false, 128, 1> : k_p2p<false, 256, 1>))
-                  : (count ? (small ? k_p2p<true, 128, 0> : k_p2p<true, 256, 0>)
-                           : (small ? k_p2p<false, 128, 0> : k_p2p<false, 256, 0>));
+                  ? (count ? (small ? k_p2p<true, 128, 1, Nodes> : k_p2p<true, 256, 1, Nodes>)
+                           : (small ? k_p2p<false, 128, 1, Nodes> : k_p2p<false, 256, 1, Nodes>))
+                  : (count ? (small ? k_p2p<true, 128, 0, Nodes> : k_p2p<true, 256, 0, Nodes>)
+                           : (small ? k_p2p<false, 128, 0, Nodes> : k_p2p<false, 256, 0, Nodes>));
   // d_small[3] = work counter, d_small[4] = in-cut-off pair count (zeroed earlier when profiling)
   unsigned long long *ctr = reinterpret_cast<unsigned long long *>(P<uint64_t>(c.d_small) + 3);
   const PairFit2 fit2 = pair_fit2(c);  // the context's fit as packed operand pairs
@@ -552,16 +582,24 @@ cudaError_t p2p_pass(Ctx &c, float *acc, cudaStream_t st) {
   uint8_t *bucket = reinterpret_cast<uint8_t *>(lpt + 1);
   if ((e = cudaMemsetAsync(lpt, 0, sizeof(LptState), st)) != cudaSuccess) return e;
   if (c.prm.leaf_max > 64) return cudaErrorInvalidValue;  // two chunks per leaf at most
-  k_lpt_hist<<<blocks_for(c.nleaves, T), T, 0, st>>>(P<uint32_t>(c.leaves), c.nleaves, P<uint2>(c.range),
+  k_lpt_hist<<<blocks_for(c.nleaves, T), T, 0, st>>>(P<uint32_t>(c.leaves), c.nleaves, nodes,
                                                       P<uint32_t>(c.p2p_beg), P<uint32_t>(c.p2p_end), bucket, lpt, tz);
   k_lpt_place<<<blocks_for(c.nleaves, T), T, 0, st>>>(P<uint32_t>(c.leaves), c.nleaves, bucket, lpt,
                                                        P<uint32_t>(c.lpt_order), tz);
   note_launch(2);
-  kern<<<g, T, dyn, st>>>(P<uint32_t>(c.lpt_order), P<uint4>(c.cell), P<uint2>(c.range), P<uint32_t>(c.p2p_beg),
-                        P<uint32_t>(c.p2p_end), P<uint64_t>(c.p2p), P<float4>(c.pm4), P<uint32_t>(c.idx), c.n,
-                        (float)c.prm.box, fit2, (float)c.prm.G, acc, ctr, lpt);
+  kern<<<g, T, dyn, st>>>(P<uint32_t>(c.lpt_order), nodes, P<uint32_t>(c.p2p_beg), P<uint32_t>(c.p2p_end),
+                        P<uint64_t>(c.p2p), P<float4>(c.pm4), P<uint32_t>(c.idx), c.n, fit2, (float)c.prm.G, acc, ctr, lpt);
   note_launch();
   return cudaGetLastError();
+}
+
+}  // namespace
+
+cudaError_t p2p_pass(Ctx &c, float *acc, cudaStream_t st) {
+  if (c.prm.tree == 1)
+    return run_p2p(c, KdNodes{P<uint32_t>(c.kd.first), P<uint32_t>(c.kd.count), P<double>(c.kd.geo), c.kd.cap, c.prm.box},
+                   acc, st);
+  return run_p2p(c, OctNodes{P<uint4>(c.cell), P<uint2>(c.range), (float)c.prm.box / (float)kHalfBox}, acc, st);
 }
 
 }  // namespace hfmm

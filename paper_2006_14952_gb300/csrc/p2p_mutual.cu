@@ -303,9 +303,8 @@ __global__ void __launch_bounds__(256, 2)
                 const float2 dx = __fadd2_rn(sx, jx[u]);
                 const float2 dy = __fadd2_rn(sy, jy[u]);
                 const float2 dz = __fadd2_rn(sz, jz[u]);
-                const float2 r2 = __ffma2_rn(dx, dx, __ffma2_rn(dy, dy, __fmul2_rn(dz, dz)));
-                const bool in0 = (r2.x < fit.rc2) && (r2.x > 0.f);
-                const bool in1 = (r2.y < fit.rc2) && (r2.y > 0.f);
+                const float2 r2 = pair_r2(dx, dy, dz);
+                const bool in0 = in_cutoff(r2.x, fit), in1 = in_cutoff(r2.y, fit);
                 if (kCount)
                   n_in += (uint32_t)in0 * (s0[u] != kNoSlot ? 2u : 1u) + (uint32_t)in1 * (s1[u] != kNoSlot ? 2u : 1u);
                 float2 g = pair_factor2<kSplit>(r2, fit);
