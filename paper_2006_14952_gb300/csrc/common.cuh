@@ -486,7 +486,6 @@ cudaError_t kd_short_range(Ctx &c, float *acc, cudaStream_t st);
 cudaError_t kd_interaction_counts(Ctx &c, bool conventional, int64_t *out, cudaStream_t st);
 cudaError_t kd_upward(Ctx &c, cudaStream_t st);                // expansions.cu
 cudaError_t kd_downward(Ctx &c, float *acc, cudaStream_t st);  // expansions.cu: L2L, then L2P writing acc
-cudaError_t kd_m2l(Ctx &c, cudaStream_t st);                   // m2l.cu
 
 // Training pairs for the learned acceptance: features [n][12] and M2L errors
 // at orders 2..8 [n][7] (device buffers of the caller); *count receives n.

@@ -9,7 +9,7 @@ radial prefactors f[0..P] at r^ = 1, the sink factors U[k] = u^(k+1) and the
 source multipoles already scaled by v^|m| (Mp), and adds
     acc[n / G] += U[|n|] * sum_m Mp[m] * D^_{n+m}(R^)     (n = g mod G)
 with D^_c = sum_{k_d <= c_d/2} prod_d [c_d!/(2^k_d k_d! (c_d-2k_d)!)] R^^(c-2k) f[|c|-|k|]
-(the Cartesian derivatives of a radial function, Sec. 2.2 prefactors).  Every
+(the Cartesian derivatives of a radial function, Sec. 2.2 prefactors), formed by recurrence().  Every
 index is a literal, so the arrays live in registers.  Multi-index order: graded,
 nx descending, ny descending.
 
@@ -70,8 +70,50 @@ def hco(n, k):
     return factorial(n) // (2 ** k * factorial(k) * factorial(n - 2 * k))
 
 
-def mono_name(a):
-    return "m_%d_%d_%d" % a
+def recurrence(P, need_c, L):
+    """Emit what the D^_c of need_c are formed from; returns c -> the expression of D^_c.
+
+    D^_c = T^0_c of T^k_0 = f_k, T^k_(b+e_d) = R^_d T^(k+1)_b + b_d T^(k+1)_(b-e_d)
+    (McMurchie and Davidson 1978, for any radial function), along the axis d with the
+    smallest b_d: one instruction a term but where every b_d is 2 or more, some 230 at
+    p = 6, where the explicit sum takes 680 and rounds a little worse (rms error of a
+    D^_c against 64 bits 2.9e-7, by the recurrence 2.6e-7).
+    """
+    def step(c):
+        d = min((d for d in range(3) if c[d]), key=lambda d: c[d])
+        return d, tuple(c[e] - (e == d) for e in range(3))
+
+    def less(b, d):
+        return tuple(b[e] - (e == d) for e in range(3))
+
+    need = [set() for _ in range(P + 2)]
+    need[0] = set(need_c)
+    for k in range(P + 1):
+        for c in need[k]:
+            if sum(c):
+                d, b = step(c)
+                need[k + 1].add(b)
+                if b[d]:
+                    need[k + 1].add(less(b, d))
+
+    def term(k, c):
+        return f"f[{k}]" if sum(c) == 0 else "t%d_%d%d%d" % (k, *c)
+
+    def value(k, c):
+        if sum(c) == 0:
+            return f"f[{k}]"
+        d, b = step(c)
+        r, t1 = "r" + "xyz"[d], term(k + 1, b)
+        if b[d] == 0:
+            return f"{r} * {t1}"
+        t2 = term(k + 1, less(b, d))
+        return f"fmaf({r}, {t1}, {t2 if b[d] == 1 else '%d.f * %s' % (b[d], t2)})"
+
+    for k in range(P, 0, -1):
+        for c in sorted(need[k], key=idx):
+            if sum(c):
+                L.append(f"    const float {term(k, c)} = {value(k, c)};")
+    return lambda c: value(0, c)
 
 
 def gen_body(P, G, g):
@@ -85,57 +127,11 @@ def gen_body(P, G, g):
     ms = multi(P)
     outs = [n for n in ms if idx(n) % G == g]
     need_c = [c for c in ms if any(all(n[d] <= c[d] for d in range(3)) for n in outs)]
-    # monomials R^^a needed by the D terms
-    need_m = set()
-    for c in need_c:
-        for kx in range(c[0] // 2 + 1):
-            for ky in range(c[1] // 2 + 1):
-                for kz in range(c[2] // 2 + 1):
-                    need_m.add((c[0] - 2 * kx, c[1] - 2 * ky, c[2] - 2 * kz))
-    # close under the "parent" relation used to build them incrementally
-    def parent(a):
-        if a[2] > 0:
-            return (a[0], a[1], a[2] - 1), "rz"
-        if a[1] > 0:
-            return (a[0], a[1] - 1, a[2]), "ry"
-        return (a[0] - 1, a[1], a[2]), "rx"
-    todo = sorted(need_m, key=lambda a: sum(a))
-    have = {(0, 0, 0)}
-    full = set()
-    for a in todo:
-        chain = []
-        b = a
-        while b not in have and b != (0, 0, 0):
-            chain.append(b)
-            b = parent(b)[0]
-        for b in reversed(chain):
-            full.add(b)
-            have.add(b)
-    for a in sorted(full, key=lambda a: (sum(a), -a[0], -a[1])):
-        p, v = parent(a)
-        src = "1.f" if p == (0, 0, 0) else mono_name(p)
-        L.append(f"    const float {mono_name(a)} = {src} * {v};" if p != (0, 0, 0) else
-                 f"    const float {mono_name(a)} = {v};")
-
-    def mono(a):
-        return "1.f" if a == (0, 0, 0) else mono_name(a)
-
+    value = recurrence(P, need_c, L)
     for c in need_c:
         ci = idx(c)
         cn = sum(c)
-        terms = []
-        for kx in range(c[0] // 2 + 1):
-            for ky in range(c[1] // 2 + 1):
-                for kz in range(c[2] // 2 + 1):
-                    co = hco(c[0], kx) * hco(c[1], ky) * hco(c[2], kz)
-                    a = (c[0] - 2 * kx, c[1] - 2 * ky, c[2] - 2 * kz)
-                    o = cn - kx - ky - kz
-                    terms.append((co, a, o))
-        parts = []
-        for co, a, o in terms:
-            t = f"f[{o}]" if a == (0, 0, 0) else f"{mono(a)} * f[{o}]"
-            parts.append(t if co == 1 else f"{float(co)}f * {t}")
-        expr = " + ".join(parts)
+        expr = value(c)
         # D'_c = u^(|c|+1) D^_c; with the sources scaled by (v/u)^|m| every term
         # D'_{n+m} M''_m carries u^(|n|+1) v^|m|: one FMA per term
         L.append(f"    const float D{ci} = U[{cn}] * ({expr});")

@@ -976,7 +976,7 @@ cudaError_t kd_short_range(Ctx &c, float *acc, cudaStream_t st) {
   if (prof) cudaEventRecord(c.ev[5], st);
   TRY(kd_group(c, st));
   if (prof) cudaEventRecord(c.ev[6], st);
-  TRY(kd_m2l(c, st));
+  TRY(m2l_pass(c, c.p, st));
   if (prof) cudaEventRecord(c.ev[7], st);
   TRY(kd_downward(c, acc, st));
   if (prof) cudaEventRecord(c.ev[8], st);

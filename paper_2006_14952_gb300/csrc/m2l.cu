@@ -13,11 +13,14 @@
 // One lane per (sink, source) pair; a warp walks the pairs of one sink (lists
 // are grouped by sink), keeps its partial local expansion in registers and
 // reduces it across the warp at the end (through shared memory, in a fixed
-// order), so no atomics are used and the result is deterministic.  Each launch adds into L (one launch per order).  The expansion order is a template parameter: all
-// index arithmetic is literal in the generated straight-line bodies
-// (gen_bodies.py -> gen_bodies.cuh).  For p >= 6 the output coefficients are split
-// over G warps (slice g owns the outputs with index = g mod G); for p >= 7 the
+// order, one addition per coefficient: the result is deterministic).  Each launch
+// adds into L (one launch per order).  The expansion order is a template parameter:
+// all index arithmetic is literal in the generated straight-line bodies
+// (gen_bodies.py -> gen_bodies.cuh).  For p >= 7 the output coefficients are split
+// over G warps (slice g owns the outputs with index = g mod G) and the
 // scaled source multipoles of each lane's pair are staged in shared memory.
+#include <algorithm>
+
 #include "common.cuh"
 #include "gen_bodies.cuh"
 
@@ -62,7 +65,6 @@ __device__ __forceinline__ void m2l_sink(uint32_t k, uint32_t tb, uint32_t te, c
                                          float *__restrict__ L, int ldm, float inv_rs, float *__restrict__ wsm) {
   constexpr int NC = ncoef(P);
   constexpr int NS = (NC + G - 1) / G;
-  constexpr bool kSmem = M2LSlices<P>::kSmem;
   const int lane = threadIdx.x & 31;
   const uint4 ca = cell[k];
   float acc[NS];
@@ -88,40 +90,17 @@ __device__ __forceinline__ void m2l_sink(uint32_t k, uint32_t tb, uint32_t te, c
 #pragma unroll
     for (int q = 1; q <= P; ++q) U[q] = U[q - 1] * u;
     const float *Mb = M + (size_t)b * ldm;
-    if constexpr (kSmem) {
-      float *col = wsm + lane;
-      M2LLoad<P>::template run<32>(Mb, v, col);
-      M2LBody<P, G, g>::run(Rx * rinv, Ry * rinv, Rz * rinv, f, U, col, acc);
-    } else {
-      float Mp[NC];
-      M2LLoad<P>::template run<1>(Mb, v, Mp);
-      M2LBody<P, G, g>::run(Rx * rinv, Ry * rinv, Rz * rinv, f, U, Mp, acc);
-    }
+    float *col = wsm + lane;
+    M2LLoad<P>::template run<32>(Mb, v, col);
+    M2LBody<P, G, g>::run(Rx * rinv, Ry * rinv, Rz * rinv, f, U, col, acc);
   }
-  if constexpr (!kSmem) {
-    // sum over the lanes by a transpose in shared memory: each lane writes its
-    // partial row (stride NC + 1: no bank conflicts), then lane c adds column c
-    // over the 32 rows in lane order (deterministic) and stores it
-    static_assert(G == 1, "the transpose path sums whole rows");
 #pragma unroll
-    for (int s = 0; s < NC; ++s) wsm[lane * (NC + 1) + s] = acc[s];
-    __syncwarp();
-    for (int cix = lane; cix < NC; cix += 32) {
-      float a = 0.f;
-#pragma unroll 8
-      for (int m = 0; m < 32; ++m) a += wsm[m * (NC + 1) + cix];
-      L[(size_t)k * ldm + cix] += a;
-    }
-    __syncwarp();
-  } else {
+  for (int s = 0; s < NS; ++s) {
+    float a = acc[s];
 #pragma unroll
-    for (int s = 0; s < NS; ++s) {
-      float a = acc[s];
-#pragma unroll
-      for (int o = 16; o; o >>= 1) a += __shfl_xor_sync(0xffffffffu, a, o);
-      const int n = s * G + g;
-      if (lane == 0 && n < NC) L[(size_t)k * ldm + n] += a;
-    }
+    for (int o = 16; o; o >>= 1) a += __shfl_xor_sync(0xffffffffu, a, o);
+    const int n = s * G + g;
+    if (lane == 0 && n < NC) L[(size_t)k * ldm + n] += a;
   }
 }
 
@@ -131,31 +110,24 @@ template <int P>
 constexpr int m2l_min_blocks() { return P <= 4 ? 4 : P == 5 ? 3 : 2; }
 
 template <int P, int G, int S>
-__global__ void __launch_bounds__(128, m2l_min_blocks<P>()) k_m2l(int64_t nn, const uint4 *__restrict__ cell,
+__global__ void __launch_bounds__(128, m2l_min_blocks<P>()) k_m2l_sliced(int64_t nn, const uint4 *__restrict__ cell,
                                              const uint32_t *__restrict__ beg, const uint32_t *__restrict__ end,
                                              const uint64_t *__restrict__ lst, const float *__restrict__ M,
                                              float *__restrict__ L, int ldm, float inv_rs,
                                              const TreeState *tz) {
   extern __shared__ float sm[];
   nn = tree_nodes(tz, nn);  // graph mode: the node count from the device tree state
-  // per warp: p >= 7 the staged multipoles (32 x NC), else the reduction transpose (32 x (NC + 1))
-  float *wsm = sm + (threadIdx.x >> 5) * (M2LSlices<P>::kSmem ? ncoef(P) * 32 : 32 * (ncoef(P) + 1));
+  static_assert(M2LSlices<P>::kSmem, "orders 7 and 8");
+  float *wsm = sm + (threadIdx.x >> 5) * ncoef(P) * 32;  // per warp: the staged multipoles
   const int64_t nw = (int64_t)gridDim.x * (blockDim.x >> 5);
   for (int64_t w = (int64_t)blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5); w < nn * G; w += nw) {
     const uint32_t k = (uint32_t)(w / G);
     const int g = (int)(w % G);
     const uint32_t tb = beg[k], te = end[k];
     if (tb == te) continue;
-    if constexpr (G == 1) {
-      m2l_sink<P, 1, 0, S>(k, tb, te, cell, lst, M, L, ldm, inv_rs, wsm);
-    } else if constexpr (G == 2) {
+    if constexpr (G == 2) {
       if (g == 0) m2l_sink<P, 2, 0, S>(k, tb, te, cell, lst, M, L, ldm, inv_rs, wsm);
       else m2l_sink<P, 2, 1, S>(k, tb, te, cell, lst, M, L, ldm, inv_rs, wsm);
-    } else if constexpr (G == 4) {
-      if (g == 0) m2l_sink<P, 4, 0, S>(k, tb, te, cell, lst, M, L, ldm, inv_rs, wsm);
-      else if (g == 1) m2l_sink<P, 4, 1, S>(k, tb, te, cell, lst, M, L, ldm, inv_rs, wsm);
-      else if (g == 2) m2l_sink<P, 4, 2, S>(k, tb, te, cell, lst, M, L, ldm, inv_rs, wsm);
-      else m2l_sink<P, 4, 3, S>(k, tb, te, cell, lst, M, L, ldm, inv_rs, wsm);
     } else {
       static_assert(G == 8, "slices");
       switch (g) {
@@ -172,22 +144,219 @@ __global__ void __launch_bounds__(128, m2l_min_blocks<P>()) k_m2l(int64_t nn, co
   }
 }
 
+// Orders 1..6, either tree: one warp per sink, 32 pairs a batch.  At 254 registers eight
+// warps an SM are all there is to hide a load behind, and with the chain bounds -> entry ->
+// node in the loop a third of the warps' time went on it: while one batch is computed the
+// next one's nodes and the list entries of the one after are copied to shared memory
+// (cp.async), across sinks too.  20.4M pairs, p = 6 (2M clustered particles): 1.86 -> 1.74 ms,
+// 1.58 with the derivative tensors by recurrence (gen_bodies.py); bound by issue (65% with
+// under two warps a scheduler), half of it the contraction's 924 FMA.  The multipole rows
+// stay loads from the lanes: copied ahead as well, 1.92 (cp.async.ca), 2.2 (.cg, twice the
+// L2 sectors) or 3.2 ms (row by row: 38% more instructions).
+//
+// What the kernel needs of a tree's nodes: the staged record of a source or a sink, R = z_A
+// - z_B' in units of half_width or of length, and the scales h.
+struct OctM2L {
+  const uint4 *cell;
+  float inv_rs;  // r / r_s (Gaussian) or r / R_c (polynomial) for r in half units
+  using Staged = uint4;
+  __device__ __forceinline__ void stage(uint32_t dst, uint32_t k) const { cp16(dst, cell + k); }
+  static __device__ __forceinline__ void cp16(uint32_t dst, const void *src) {
+    asm volatile("cp.async.ca.shared.global [%0], [%1], 16;" ::"r"(dst), "l"(src) : "memory");
+  }
+  // R, h_A (in R's unit) and h_B / h_A (exact)
+  __device__ __forceinline__ void pair(const Staged &a, const Staged &b, uint32_t s, float (&R)[3], float &hA,
+                                       float &rho) const {
+    int dd[3];
+    half_delta32(a, b, s, dd);  // exact integers below 2^24
+#pragma unroll
+    for (int d = 0; d < 3; ++d) R[d] = -(float)dd[d];
+    hA = (float)(2 * half_width(a.w));
+    rho = (float)half_width(b.w) / (float)half_width(a.w);
+  }
+};
+// k-d tree: R formed in FP64 from the box centres, the scales h powers of two.
+struct KdM2L {
+  const double *geo;  // [>= 3][cap], the centres first
+  const float *hs;
+  int64_t cap;
+  double box;
+  float inv_rs;
+  struct Staged {
+    double c[3];
+    float h, pad;
+  };
+  __device__ __forceinline__ void stage(uint32_t dst, uint32_t k) const {
+#pragma unroll
+    for (int d = 0; d < 3; ++d)
+      asm volatile("cp.async.ca.shared.global [%0], [%1], 8;" ::"r"(dst + 8 * d), "l"(geo + d * cap + k) : "memory");
+    asm volatile("cp.async.ca.shared.global [%0], [%1], 4;" ::"r"(dst + 24), "l"(hs + k) : "memory");
+  }
+  __device__ __forceinline__ void pair(const Staged &a, const Staged &b, uint32_t s, float (&R)[3], float &hA,
+                                       float &rho) const {
+#pragma unroll
+    for (int d = 0; d < 3; ++d)
+      R[d] = (float)__dsub_rn(a.c[d], __dadd_rn(b.c[d], (double)shift_component(s, d) * box));
+    hA = a.h;
+    rho = b.h / a.h;
+  }
+};
+
+// A warp's shared memory.
+template <int P, class Nodes>
+struct alignas(16) M2LStage {
+  typename Nodes::Staged src[32], sink;
+  uint64_t e[2][32];              // list entries, batch by batch in turn
+  float red[32 * (ncoef(P) + 1)];  // the reduction's transpose
+};
+
+template <int P, int S, class Nodes>
+__global__ void __launch_bounds__(128, m2l_min_blocks<P>())
+    k_m2l(int64_t nn, Nodes nodes, const uint32_t *__restrict__ beg, const uint32_t *__restrict__ end,
+          const uint64_t *__restrict__ lst, const float *__restrict__ M, float *__restrict__ L, int ldm,
+          const TreeState *tz) {
+  constexpr int NC = ncoef(P);
+  static_assert(M2LSlices<P>::G == 1 && !M2LSlices<P>::kSmem, "orders 1..6");
+  using Stage = M2LStage<P, Nodes>;
+  extern __shared__ __align__(16) unsigned char m2l_smem[];
+  nn = tree_nodes(tz, nn);  // graph mode: the node count from the device tree state
+  Stage &W = reinterpret_cast<Stage *>(m2l_smem)[threadIdx.x >> 5];
+  const int lane = threadIdx.x & 31;
+  const uint32_t nw = gridDim.x * (blockDim.x >> 5);
+  // batches in order: the one computed (a), the one whose rows are in flight (b), the one
+  // whose entries are (c); k >= nn: none.  next: the sink after c's, its bounds already read
+  struct Batch {
+    uint32_t k, t, te;
+  } a, b, c, next;
+  auto bounds = [&](uint32_t k) {
+    next.k = k;
+    next.t = next.te = 0;
+    if (k < nn) {
+      next.t = beg[k];
+      next.te = end[k];
+    }
+  };
+  auto advance = [&]() {  // c to the batch after it
+    if (c.te - c.t > 32) {
+      c.t += 32;
+      return;
+    }
+    while (next.t == next.te && next.k < nn) bounds(next.k + nw);
+    c = next;
+    if (next.k < nn) bounds(next.k + nw);
+  };
+  auto shared32 = [](const void *p) { return (uint32_t)__cvta_generic_to_shared(p); };
+  int slot = 0;  // of b's entries
+  auto stage_entries = [&](int sl) {  // c's entries
+    if (c.k < nn && c.t + lane < c.te)
+      asm volatile("cp.async.ca.shared.global [%0], [%1], 8;" ::"r"(shared32(&W.e[sl][lane])), "l"(lst + c.t + lane)
+                   : "memory");
+  };
+  auto stage_rows = [&]() {  // b's rows and nodes, by its entries
+    if (b.k >= nn) return;
+    if (b.t + lane < b.te) nodes.stage(shared32(&W.src[lane]), pair_src(W.e[slot][lane]));
+    if (lane == 0) nodes.stage(shared32(&W.sink), b.k);
+  };
+  bounds(blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5));
+  c.t = c.te = 0;
+  advance();  // the first batch
+  stage_entries(0);
+  asm volatile("cp.async.commit_group;\ncp.async.wait_group 0;" ::: "memory");
+  __syncwarp();
+  b = c;
+  stage_rows();
+  advance();
+  stage_entries(1);
+  asm volatile("cp.async.commit_group;" ::: "memory");
+  float acc[NC];
+#pragma unroll
+  for (int s = 0; s < NC; ++s) acc[s] = 0.f;
+  while (b.k < nn) {
+    a = b;
+    b = c;
+    asm volatile("cp.async.wait_group 0;" ::: "memory");
+    __syncwarp();
+    const bool valid = a.t + lane < a.te;
+    float R[3] = {1.f, 0.f, 0.f}, hA = 1.f, rho = 1.f;
+    uint32_t src = 0;
+    if (valid) {
+      const uint64_t e = W.e[slot][lane];
+      src = pair_src(e);
+      nodes.pair(W.sink, W.src[lane], pair_shift(e), R, hA, rho);
+    }
+    __syncwarp();
+    slot ^= 1;
+    stage_rows();
+    advance();
+    stage_entries(slot ^ 1);
+    asm volatile("cp.async.commit_group;" ::: "memory");
+    if (valid) {
+      const float r2 = R[0] * R[0] + R[1] * R[1] + R[2] * R[2];
+      const float rinv = rsqrtf(r2);
+      float f[P + 1];
+      radial_prefactors<P, S>(r2 * rinv * nodes.inv_rs, f);
+      float U[P + 1];
+      U[0] = hA * rinv;
+#pragma unroll
+      for (int q = 1; q <= P; ++q) U[q] = U[q - 1] * U[0];
+      float Mp[NC];
+      M2LLoad<P>::template run<1>(M + (size_t)src * ldm, rho, Mp);
+      M2LBody<P, 1, 0>::run(R[0] * rinv, R[1] * rinv, R[2] * rinv, f, U, Mp, acc);
+    }
+    if (b.k == a.k) continue;  // more of this sink
+    // sum over the lanes by a transpose in shared memory: each lane writes its
+    // partial row (stride NC + 1: no bank conflicts), then lane c adds column c
+    // over the 32 rows in lane order (deterministic) and adds it to the sink's local
+    // (no other warp does: the reduction needs no answer)
+#pragma unroll
+    for (int s = 0; s < NC; ++s) {
+      W.red[lane * (NC + 1) + s] = acc[s];
+      acc[s] = 0.f;
+    }
+    __syncwarp();
+    for (int cix = lane; cix < NC; cix += 32) {
+      float sum = 0.f;
+#pragma unroll 8
+      for (int m = 0; m < 32; ++m) sum += W.red[m * (NC + 1) + cix];
+      atomicAdd(L + (size_t)a.k * ldm + cix, sum);
+    }
+    __syncwarp();
+  }
+  asm volatile("cp.async.wait_group 0;" ::: "memory");
+}
+
+template <int P, int S, class Nodes>
+cudaError_t launch(Ctx &c, const Nodes &nodes, DBuf &from, cudaStream_t st) {
+  // four sinks a warp, so that its copies overlap its arithmetic (262k clustered particles:
+  // 0.156 ms instead of 0.163 with one), one while that leaves the GPU's blocks unfilled
+  const unsigned all = blocks_for((size_t)c.nnodes, 4);
+  const unsigned cap = 152u * (unsigned)(c.prm.tile_m2l_blocks > 0 ? c.prm.tile_m2l_blocks : 64);
+  const unsigned g = std::min(cap, std::max(std::min(all, 304u), (all + 3u) / 4u));
+  const size_t smem = 4 * sizeof(M2LStage<P, Nodes>);
+  cudaError_t e = cudaFuncSetAttribute(k_m2l<P, S, Nodes>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  if (e != cudaSuccess) return e;
+  k_m2l<P, S, Nodes><<<g, 128, smem, st>>>(c.nnodes, nodes, hfmm::P<uint32_t>(from), hfmm::P<uint32_t>(c.m2l_end),
+                                           hfmm::P<uint64_t>(c.m2l), hfmm::P<float>(c.M), hfmm::P<float>(c.L), c.ldm,
+                                           c.graph_tree ? hfmm::P<TreeState>(c.tstate) : nullptr);
+  note_launch();
+  return cudaGetLastError();
+}
+
 template <int P, int S>
-cudaError_t launch(Ctx &c, cudaStream_t st) {
+cudaError_t launch_sliced(Ctx &c, cudaStream_t st) {
   constexpr int G = M2LSlices<P>::G;
   unsigned g = blocks_for((size_t)c.nnodes * G, 4);
   const unsigned cap = 152u * (unsigned)(c.prm.tile_m2l_blocks > 0 ? c.prm.tile_m2l_blocks : 64);
   if (g > cap) g = cap;
   // r / r_s (Gaussian) or r / R_c (polynomial) with r in half units: x = r_half * (L / 2^22) / scale
   const float inv_rs = (float)(c.prm.box / (double)kHalfBox / (S == 1 ? c.rc : c.rs));
-  size_t smem = M2LSlices<P>::kSmem ? (size_t)4 * ncoef(P) * 32 * sizeof(float)
-                                    : (size_t)4 * 32 * (ncoef(P) + 1) * sizeof(float);
+  const size_t smem = (size_t)4 * ncoef(P) * 32 * sizeof(float);
   if (smem > 48 * 1024) {
-    cudaError_t e = cudaFuncSetAttribute(k_m2l<P, G, S>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    cudaError_t e = cudaFuncSetAttribute(k_m2l_sliced<P, G, S>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
   }
   // the entries [mid, end) of each sink: pairs outside the operator table
-  k_m2l<P, G, S><<<g, 128, smem, st>>>(c.nnodes, hfmm::P<uint4>(c.cell), hfmm::P<uint32_t>(c.m2l_mid),
+  k_m2l_sliced<P, G, S><<<g, 128, smem, st>>>(c.nnodes, hfmm::P<uint4>(c.cell), hfmm::P<uint32_t>(c.m2l_mid),
                                     hfmm::P<uint32_t>(c.m2l_end), hfmm::P<uint64_t>(c.m2l), hfmm::P<float>(c.M),
                                     hfmm::P<float>(c.L), c.ldm, inv_rs,
                                     c.graph_tree ? hfmm::P<TreeState>(c.tstate) : nullptr);
@@ -195,113 +364,42 @@ cudaError_t launch(Ctx &c, cudaStream_t st) {
   return cudaGetLastError();
 }
 
-// M2L on the k-d tree (tree = 1; orders 1..6; split S as in k_m2l): one warp per sink node as in
-// k_m2l, with R = c_A - (c_B + s L) formed in FP64 from the box centres and the
-// scales h_A, h_B of the two nodes (powers of two: v / u = h_B / h_A is exact).
-template <int P, int S>
-__global__ void __launch_bounds__(128, m2l_min_blocks<P>()) k_kd_m2l(int64_t nn, const double *__restrict__ geo,
-                                                                 int64_t cap, const float *__restrict__ hs,
-                                                                 const uint32_t *__restrict__ beg,
-                                                                 const uint32_t *__restrict__ end,
-                                                                 const uint64_t *__restrict__ lst,
-                                                                 const float *__restrict__ M, float *__restrict__ L,
-                                                                 int ldm, double box, float inv_rs) {
-  constexpr int NC = ncoef(P);
-  static_assert(M2LSlices<P>::G == 1 && !M2LSlices<P>::kSmem, "orders 1..6");
-  extern __shared__ float sm[];
-  float *wsm = sm + (threadIdx.x >> 5) * 32 * (NC + 1);
-  const int lane = threadIdx.x & 31;
-  const int64_t nw = (int64_t)gridDim.x * (blockDim.x >> 5);
-  for (int64_t k = (int64_t)blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5); k < nn; k += nw) {
-    const uint32_t tb = beg[k], te = end[k];
-    if (tb == te) continue;
-    const double ca[3] = {geo[k], geo[cap + k], geo[2 * cap + k]};
-    const float hA = hs[k];
-    float acc[NC];
-#pragma unroll
-    for (int q = 0; q < NC; ++q) acc[q] = 0.f;
-    for (uint32_t t = tb + lane; t < te; t += 32) {
-      const uint64_t e = lst[t];
-      const uint32_t b = pair_src(e), sh = pair_shift(e);
-      float R[3];
-#pragma unroll
-      for (int d = 0; d < 3; ++d)
-        R[d] = (float)__dsub_rn(ca[d], __dadd_rn(geo[d * cap + b], (double)shift_component(sh, d) * box));
-      const float r2 = R[0] * R[0] + R[1] * R[1] + R[2] * R[2];
-      const float rinv = rsqrtf(r2);
-      float f[P + 1];
-      radial_prefactors<P, S>(r2 * rinv * inv_rs, f);
-      const float u = hA * rinv;
-      float U[P + 1];
-      U[0] = u;
-#pragma unroll
-      for (int q = 1; q <= P; ++q) U[q] = U[q - 1] * u;
-      float Mp[NC];
-      M2LLoad<P>::template run<1>(M + (size_t)b * ldm, hs[b] / hA, Mp);
-      M2LBody<P, 1, 0>::run(R[0] * rinv, R[1] * rinv, R[2] * rinv, f, U, Mp, acc);
+template <int S>
+cudaError_t run(Ctx &c, int q, cudaStream_t st) {
+  if (c.prm.tree == 1) {
+    const KdM2L nodes{P<double>(c.kd.geo), P<float>(c.kd.hs), c.kd.cap, c.prm.box,
+                      (float)(1.0 / (S == 1 ? c.rc : c.rs))};
+    switch (q) {
+      case 1: return launch<1, S>(c, nodes, c.m2l_beg, st);
+      case 2: return launch<2, S>(c, nodes, c.m2l_beg, st);
+      case 3: return launch<3, S>(c, nodes, c.m2l_beg, st);
+      case 4: return launch<4, S>(c, nodes, c.m2l_beg, st);
+      case 5: return launch<5, S>(c, nodes, c.m2l_beg, st);
+      case 6: return launch<6, S>(c, nodes, c.m2l_beg, st);
     }
-    // sum over the lanes in a fixed order (shared-memory transpose, as in k_m2l)
-#pragma unroll
-    for (int q = 0; q < NC; ++q) wsm[lane * (NC + 1) + q] = acc[q];
-    __syncwarp();
-    for (int cix = lane; cix < NC; cix += 32) {
-      float a = 0.f;
-#pragma unroll 8
-      for (int m = 0; m < 32; ++m) a += wsm[m * (NC + 1) + cix];
-      L[(size_t)k * ldm + cix] += a;
-    }
-    __syncwarp();
+    return cudaErrorInvalidValue;
   }
-}
-
-template <int P, int S>
-cudaError_t launch_kd(Ctx &c, cudaStream_t st) {
-  unsigned g = blocks_for((size_t)c.nnodes, 4);
-  const unsigned cap = 152u * (unsigned)(c.prm.tile_m2l_blocks > 0 ? c.prm.tile_m2l_blocks : 64);
-  if (g > cap) g = cap;
-  const size_t smem = (size_t)4 * 32 * (ncoef(P) + 1) * sizeof(float);
-  if (smem > 48 * 1024) {
-    cudaError_t e = cudaFuncSetAttribute(k_kd_m2l<P, S>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    if (e != cudaSuccess) return e;
+  // the entries [mid, end) of each sink: pairs outside the operator table
+  const OctM2L nodes{P<uint4>(c.cell), (float)(c.prm.box / (double)kHalfBox / (S == 1 ? c.rc : c.rs))};
+  switch (q) {
+    case 1: return launch<1, S>(c, nodes, c.m2l_mid, st);
+    case 2: return launch<2, S>(c, nodes, c.m2l_mid, st);
+    case 3: return launch<3, S>(c, nodes, c.m2l_mid, st);
+    case 4: return launch<4, S>(c, nodes, c.m2l_mid, st);
+    case 5: return launch<5, S>(c, nodes, c.m2l_mid, st);
+    case 6: return launch<6, S>(c, nodes, c.m2l_mid, st);
+    case 7: return launch_sliced<7, S>(c, st);
+    case 8: return launch_sliced<8, S>(c, st);
   }
-  k_kd_m2l<P, S><<<g, 128, smem, st>>>(c.nnodes, hfmm::P<double>(c.kd.geo), c.kd.cap, hfmm::P<float>(c.kd.hs),
-                                   hfmm::P<uint32_t>(c.m2l_beg), hfmm::P<uint32_t>(c.m2l_end),
-                                   hfmm::P<uint64_t>(c.m2l), hfmm::P<float>(c.M), hfmm::P<float>(c.L), c.ldm,
-                                   c.prm.box, (float)(1.0 / (S == 1 ? c.rc : c.rs)));
-  note_launch();
-  return cudaGetLastError();
+  return cudaErrorInvalidValue;
 }
 
 }  // namespace
 
-cudaError_t kd_m2l(Ctx &c, cudaStream_t st) {
-  if (c.nm2l == 0 || c.nnodes == 0) return cudaSuccess;
-  const bool poly = c.prm.split == 1;
-  switch (c.p) {
-    case 1: return poly ? launch_kd<1, 1>(c, st) : launch_kd<1, 0>(c, st);
-    case 2: return poly ? launch_kd<2, 1>(c, st) : launch_kd<2, 0>(c, st);
-    case 3: return poly ? launch_kd<3, 1>(c, st) : launch_kd<3, 0>(c, st);
-    case 4: return poly ? launch_kd<4, 1>(c, st) : launch_kd<4, 0>(c, st);
-    case 5: return poly ? launch_kd<5, 1>(c, st) : launch_kd<5, 0>(c, st);
-    case 6: return poly ? launch_kd<6, 1>(c, st) : launch_kd<6, 0>(c, st);
-  }
-  return cudaErrorInvalidValue;
-}
-
+// Either tree's M2L pairs at order q.
 cudaError_t m2l_pass(Ctx &c, int q, cudaStream_t st) {
   if (c.nm2l == 0 || c.nnodes == 0) return cudaSuccess;
-  const bool poly = c.prm.split == 1;
-  switch (q) {
-    case 1: return poly ? launch<1, 1>(c, st) : launch<1, 0>(c, st);
-    case 2: return poly ? launch<2, 1>(c, st) : launch<2, 0>(c, st);
-    case 3: return poly ? launch<3, 1>(c, st) : launch<3, 0>(c, st);
-    case 4: return poly ? launch<4, 1>(c, st) : launch<4, 0>(c, st);
-    case 5: return poly ? launch<5, 1>(c, st) : launch<5, 0>(c, st);
-    case 6: return poly ? launch<6, 1>(c, st) : launch<6, 0>(c, st);
-    case 7: return poly ? launch<7, 1>(c, st) : launch<7, 0>(c, st);
-    case 8: return poly ? launch<8, 1>(c, st) : launch<8, 0>(c, st);
-  }
-  return cudaErrorInvalidValue;
+  return c.prm.split == 1 ? run<1>(c, q, st) : run<0>(c, q, st);
 }
 
 }  // namespace hfmm
