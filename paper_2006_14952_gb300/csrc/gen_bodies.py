@@ -66,10 +66,6 @@ def idx(n):
     return (k * (k + 1) * (k + 2)) // 6 + j * (j + 1) // 2 + z
 
 
-def hco(n, k):
-    return factorial(n) // (2 ** k * factorial(k) * factorial(n - 2 * k))
-
-
 def recurrence(P, need_c, L):
     """Emit what the D^_c of need_c are formed from; returns c -> the expression of D^_c.
 
@@ -340,34 +336,12 @@ def gen_tc(P, bf=False):
          f"  template <int G, int g>  // the coefficients c = g mod G\n"
          f"  static __device__ __forceinline__ void store_d(float rx, float ry, float rz, const float (&f)[{P + 1}],"
          f" const float (&U)[{P + 1}], {T} *__restrict__ hi, {T} *__restrict__ lo, const int (&xo)[8]) {{"]
-    nm = {}
-    for a in ms:
-        if a == (0, 0, 0):
-            nm[a] = "1.f"
-            continue
-        if a[2] > 0:
-            p, v = (a[0], a[1], a[2] - 1), "rz"
-        elif a[1] > 0:
-            p, v = (a[0], a[1] - 1, a[2]), "ry"
-        else:
-            p, v = (a[0] - 1, a[1], a[2]), "rx"
-        name = "m_%d_%d_%d" % a
-        L.append(f"    const float {name} = {nm[p]} * {v};" if nm[p] != "1.f" else f"    const float {name} = {v};")
-        nm[a] = name
+    value = recurrence(P, ms, L)
     for c in ms:
         ci = idx(c)
         cn = sum(c)
-        parts = []
-        for kx in range(c[0] // 2 + 1):
-            for ky in range(c[1] // 2 + 1):
-                for kz in range(c[2] // 2 + 1):
-                    co = hco(c[0], kx) * hco(c[1], ky) * hco(c[2], kz)
-                    a = (c[0] - 2 * kx, c[1] - 2 * ky, c[2] - 2 * kz)
-                    o = cn - kx - ky - kz
-                    t = f"f[{o}]" if a == (0, 0, 0) else f"{nm[a]} * f[{o}]"
-                    parts.append(t if co == 1 else f"{float(co)}f * {t}")
         off = (ci >> 3) * 8 * row + (ci & 7) * row
-        L.append(f"    if constexpr ({ci} % G == g) {{ const float d = U[{cn}] * ({' + '.join(parts)});"
+        L.append(f"    if constexpr ({ci} % G == g) {{ const float d = U[{cn}] * ({value(c)});"
                  f" {split('d', f'{off} + xo[{ci & 7}]')} }}")
     L.append("  }")
     L.append(f"  static __device__ __forceinline__ void store_m(const float *__restrict__ Mb, float vr, float s,"
