@@ -346,16 +346,17 @@ def gen_tc(P, bf=False):
     L.append("  }")
     L.append(f"  static __device__ __forceinline__ void store_m(const float *__restrict__ Mb, float vr, float s,"
              f" {T} *__restrict__ hi, {T} *__restrict__ lo, const int (&xo)[8]) {{")
+    # rows are 16-byte aligned and padded: float4 loads (a lane's row is its own cache lines)
+    L.append("    const float4 *M4 = reinterpret_cast<const float4 *>(Mb);")
+    for j in range((NC + 3) // 4):
+        L.append(f"    const float4 q{j} = __ldg(M4 + {j});")
     L.append("    float q = s;")
-    for k in range(P + 1):
-        if k:
+    for ci, a in enumerate(ms):
+        if ci and sum(a) != sum(ms[ci - 1]):
             L.append("    q *= vr;")
-        for a in ms:
-            if sum(a) != k:
-                continue
-            ci = idx(a)
-            off = (ci >> 3) * 8 * row + (ci & 7) * row
-            L.append(f"    {{ const float x = __ldg(Mb + {ci}) * q; {split('x', f'{off} + xo[{ci & 7}]')} }}")
+        off = (ci >> 3) * 8 * row + (ci & 7) * row
+        comp = "q%d.%s" % (ci // 4, "xyzw"[ci % 4])
+        L.append(f"    {{ const float x = {comp} * q; {split('x', f'{off} + xo[{ci & 7}]')} }}")
     L.append("  }")
     L.append("};")
     return "\n".join(L)
