@@ -149,7 +149,7 @@ PairFit fit_pair_factor(double rs, double rc) {
       if (!solve_small(n, A, c)) continue;
       // the largest relative error, with half an FP32 unit of every term's size
       double cost = 0.0;
-      for (int i = 0; i < kTest; ++i) {
+      for (int i = kTest - 1; i >= 0 && cost < best; --i) {  // (largest near R_c)
         double f[6], s = 0.0, t = 0.0;
         basis(xt[i], p, f);
         for (int k = 0; k < n; ++k) {
@@ -184,7 +184,7 @@ namespace {
 template <class F>
 void for_each_buffer(Ctx &c, F f) {
   DBuf *bufs[] = {&c.key, &c.key_alt, &c.idx, &c.idx_alt, &c.xs, &c.pm4, &c.perm, &c.cell, &c.range, &c.kids,
-                  &c.leaves, &c.lev, &c.lcnt, &c.front, &c.front_next, &c.offs, &c.wnode, &c.wqueue, &c.wspill, &c.obeg, &c.ocnt, &c.open, &c.openc,
+                  &c.leaves, &c.lev, &c.lcnt, &c.offs, &c.wnode, &c.wqueue, &c.wspill, &c.obeg, &c.ocnt, &c.open, &c.openc,
                   &c.m2l, &c.m2l_alt, &c.p2p, &c.p2p_alt, &c.m2l_beg, &c.m2l_end, &c.p2p_beg, &c.p2p_end, &c.M,
                   &c.L, &c.tmp, &c.tmp2, &c.d_small, &c.hpos, &c.hmass, &c.hacc, &c.m2l_mid, &c.tab,
                   &c.mlp_w, &c.cand, &c.mlp_scratch, &c.tstate,
@@ -195,7 +195,7 @@ void for_each_buffer(Ctx &c, F f) {
                   &c.kd.ord[0], &c.kd.ord[1], &c.kd.ord[2], &c.kd.ord2[0], &c.kd.ord2[1], &c.kd.ord2[2],
                   &c.kd.side, &c.kd.place, &c.kd.first,
                   &c.kd.count, &c.kd.child, &c.kd.parent, &c.kd.axis, &c.kd.box, &c.kd.geo, &c.kd.geof, &c.kd.hs,
-                  &c.kd.ctr};
+                  &c.kd.open[0], &c.kd.open[1], &c.kd.obeg, &c.kd.ocnt, &c.kd.ctr};
   for (DBuf *b : bufs) f(*b);
 }
 
@@ -781,8 +781,13 @@ int hfmm_get_stats(hfmm_ctx *h, hfmm_stats *o) {
 }
 
 // The walk places each sink's entries together, the sinks in no fixed order: rows go out by
-// (order, sink), a sink's own entries in the order they are summed in.
-static void by_sink(std::vector<uint64_t> &v) {
+// (order, sink), a sink's own entries in the order they are summed in (k-d tree: by source and
+// shift).
+static void by_sink(std::vector<uint64_t> &v, bool kd) {
+  if (kd) {
+    std::sort(v.begin(), v.end());
+    return;
+  }
   std::stable_sort(v.begin(), v.end(), [](uint64_t a, uint64_t b) { return a >> kSinkShift < b >> kSinkShift; });
 }
 
@@ -893,7 +898,7 @@ int hfmm_export(hfmm_ctx *h, int what, void *buf, size_t *bytes) {
       std::vector<uint64_t> v(c.nm2l);
       e = cudaMemcpy(v.data(), c.m2l.p, c.nm2l * 8, cudaMemcpyDeviceToHost);
       if (e != cudaSuccess) break;
-      by_sink(v);
+      by_sink(v, c.prm.tree == 1);
       int64_t *o = static_cast<int64_t *>(buf);
       for (int64_t t = 0; t < c.nm2l; ++t) o[t] = pair_order(v[t]);
       break;
@@ -904,7 +909,7 @@ int hfmm_export(hfmm_ctx *h, int what, void *buf, size_t *bytes) {
       std::vector<uint64_t> v(cnt);
       e = cudaMemcpy(v.data(), (what == HFMM_EXPORT_P2P ? c.p2p : c.m2l).p, cnt * 8, cudaMemcpyDeviceToHost);
       if (e != cudaSuccess) break;
-      by_sink(v);
+      by_sink(v, c.prm.tree == 1);
       int64_t *o = static_cast<int64_t *>(buf);
       for (int64_t t = 0; t < cnt; ++t) {
         o[3 * t] = pair_sink(v[t]);

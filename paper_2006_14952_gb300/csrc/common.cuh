@@ -284,6 +284,8 @@ struct KdTree {
   DBuf geo;                      // f64 [7][cap] centre xyz, half extents xyz, side (largest extent)
   DBuf geof;                     // f32 [7][cap] the same rounded (the walk's FP32 filter)
   DBuf hs;                       // f32 [cap] expansion scale h: L 2^-j >= side, j <= 21
+  DBuf open[2];                  // walk: open lists of two levels in turn, u32
+  DBuf obeg, ocnt;               // u64, u32 [nodes]: each node's own among them
   DBuf ctr;                      // u64 [16]: the walk's counters
   std::vector<int64_t> level_start;
   int64_t cap = 0;
@@ -325,7 +327,6 @@ struct Ctx {
 
   // traversal: node records, each node's parent's open list, open lists
   DBuf wnode, wqueue, wspill, obeg, ocnt, open, openc;
-  DBuf front, front_next;  // k-d walk: frontier (ping-pong); its lists' sorts borrow them as scratch
   DBuf offs;               // scan scratch
   int64_t frontier_items = 0;
   DBuf m2l, m2l_alt, p2p, p2p_alt;  // packed u64 entries

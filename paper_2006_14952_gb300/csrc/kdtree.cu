@@ -26,17 +26,13 @@
 // and the expansion scale h = L 2^-j >= side (j <= 21, the octree's deepest
 // cell side): P2M offsets over h stay within [-1/2, 1/2] and the scale ratios of
 // the translations are powers of two.
-// Walk: one cooperative launch, level synchronous over the frontier of (sink,
-// source, shift) pairs with grid-wide barriers between the levels, one thread per
-// pair, the three rules of Sec. 2.3 on the boxes in FP64 with every operation
-// rounded on its own (no contraction, so the decisions are those of any IEEE FP64
-// evaluation in the same order), taken in FP32 wherever an error bound shows the
-// FP32 comparison cannot differ; M2L and P2P entries and the next frontier are
-// appended with warp-aggregated atomics, and when a list or the frontier outgrows
-// its buffer the buffers are grown and the walk repeated.  The lists are then
-// sorted by (sink, source, shift), so every sum after them runs in a fixed order.
-// The same walk with the opening-angle test alone, from the root against itself,
-// is the conventional FMM's of the interaction counts (Sec. 3).
+// Walk: one cooperative launch, sink-driven (k_kd_walk below): a warp takes one sink node
+// and the sources its parent left open, the three rules of Sec. 2.3 on the boxes in FP64
+// with every operation rounded on its own (no contraction, so the decisions are those of any
+// IEEE FP64 evaluation in the same order), taken in FP32 wherever an error bound shows the
+// FP32 comparison cannot differ; each sink's entries lie together in a fixed order, so every
+// sum after them runs in a fixed order.  The same walk with the opening-angle test alone,
+// from the root against itself, is the conventional FMM's of the interaction counts (Sec. 3).
 // P2P: the octree's kernel (p2p.cu), the source-box offsets from the box centres.
 #include <algorithm>
 
@@ -581,136 +577,223 @@ __device__ __forceinline__ int kd_classify(const KdGeo &G, uint32_t a, uint32_t 
   return kd_classify64_call(G, a, b, s, R);
 }
 
-// Append the entries of the lanes with `take` at consecutive slots of a list
-// (one atomic per warp); slots at or above cap are counted, not written.
-__device__ __forceinline__ void warp_append(bool take, uint64_t e, unsigned long long *ctr, uint64_t *out,
-                                            unsigned long long cap) {
-  const unsigned mask = __ballot_sync(0xffffffffu, take);
-  if (!mask) return;
-  const int lane = threadIdx.x & 31, leader = __ffs(mask) - 1;
-  unsigned long long base = 0;
-  if (lane == leader) base = atomicAdd(ctr, (unsigned long long)__popc(mask));
-  base = __shfl_sync(0xffffffffu, base, leader);
-  const unsigned long long slot = base + __popc(mask & ((1u << lane) - 1u));
-  if (take && slot < cap) out[slot] = e;
-}
+// Walk counters (u64): [0] M2L entries, [1] P2P entries, [2] status (1: the open lists
+// outgrown), [3] levels walked, [4] pairs classified, [5..7] open entries and [8..10] nodes
+// handed out of three consecutive levels (level l uses [.. + l % 3]; the one of level l + 1
+// is cleared during level l, after every block has read it at level l - 2).
+constexpr int kWalkCtr = 11;
 
-// Walk counters (u64): [0] M2L entries, [1] P2P entries, [2] status (1: the frontier
-// buffer outgrown), [3] levels walked, [4] pairs classified, [5..7] next-frontier counts
-// of three consecutive levels (level l appends to [5 + l % 3]; the one of level
-// l + 1 is cleared during level l, after every block has read it at level l - 2).
-constexpr int kWalkCtr = 8;
+struct KdWalk {
+  KdShape S;
+  KdGeo G;
+  WalkRule R;
+  const int *parent;
+  uint32_t *open[2];    // open lists of the even and the odd levels' nodes: (node, shift)
+  unsigned long long *obeg;  // per node with children: its open list
+  uint32_t *ocnt;
+  uint64_t *m2l, *p2p;
+  uint32_t *mb, *me, *pb, *pe;  // CSR bounds by sink
+  unsigned long long cap_open, cap_m2l, cap_p2p;
+  unsigned long long *ctr;
+};
 
-// The whole walk in one cooperative launch: the 27 root pairs (root, root, s) as
-// the first frontier (the conventional walk: the root against itself alone),
-// then level after level with grid-wide barriers between
-// them, until the frontier is empty or outgrows its buffer (the caller grows the
-// buffers that were outgrown, the frontier's or a list's, and walks again).
-__global__ void __launch_bounds__(kT, 4) k_kd_walk(uint64_t *__restrict__ fa, uint64_t *__restrict__ fb,
-                                                unsigned long long cap_f, uint64_t *__restrict__ m2l,
-                                                unsigned long long cap_m, uint64_t *__restrict__ p2p,
-                                                unsigned long long cap_p, unsigned long long *__restrict__ ctr,
-                                                KdGeo G, WalkRule R) {
-  cg::grid_group grid = cg::this_grid();
+constexpr int kStack = 512, kSoft = 448;  // sources a sink has still to visit
+constexpr int kStage = 1024;              // entries staged in shared memory
+constexpr int kWalkWarpWords = kStack + kStage;
+
+// One sink's session, a warp: every pair (sink, b, s) the walk meets is classified.  The
+// pairs start from those its parent left open (the root: its 27 images, or itself alone in
+// the conventional walk).  The larger of the two opens, at equal sizes both, and only a node
+// with children: a source that opens alone stays with this sink (its children go on a
+// stack), and where the sink opens, alone or with the source, the source or its children go
+// to the open list both its children start from.  The M2L entries and the P2P or open
+// entries are staged, their ranges taken with one atomic per list at the end; a session with
+// more entries than the stage holds counts them and walks again, writing in place.
+// Above kSoft waiting the stack is taken one source at a time: each adds one at most per
+// level of the tree (27 levels: node numbers are below 2^27), so it holds.
+__device__ __forceinline__ void kd_session(const KdWalk &W, uint32_t k, int level, uint32_t *stack, uint32_t *stage,
+                                           unsigned long long *nopen, unsigned long long &items) {
   const int lane = threadIdx.x & 31;
-  const unsigned long long stride = (unsigned long long)gridDim.x * blockDim.x;
-  const unsigned long long gt = (unsigned long long)blockIdx.x * blockDim.x + threadIdx.x;
-  // the root against its 27 nearest images (a conventional walk: against itself only)
-  if (R.conventional ? gt == 0 : gt < 27) fa[gt] = pack_pair(0u, 0u, R.conventional ? 13u : (uint32_t)gt);
-  unsigned long long nf = R.conventional ? 1 : 27, pairs = 0;
-  grid.sync();
-  for (int level = 0;; ++level) {
-    uint64_t *cur = (level & 1) ? fb : fa, *next = (level & 1) ? fa : fb;
-    unsigned long long *ncount = ctr + 5 + level % 3;
-    if (gt == 0) ctr[5 + (level + 1) % 3] = 0;
-    for (unsigned long long base = (unsigned long long)blockIdx.x * blockDim.x; base < nf; base += stride) {
-      const unsigned long long t = base + threadIdx.x;
-      uint32_t a = 0, b = 0, s = 0;
-      int cls = 0;
-      uint64_t e = 0;
-      float4 A0, A1, B0, B1;
-      if (t < nf) {
-        e = cur[t];
-        a = pair_sink(e);
-        b = pair_src(e);
-        s = pair_shift(e);
-        G.rec(a, A0, A1);
-        G.rec(b, B0, B1);
-        cls = kd_classify(G, a, b, s, R, A0, A1, B0, B1);
-      }
-      int ca = -1, cb = -1;
-      bool opena = false, openb = false;
-      if (cls == 2) {
-        ca = __float_as_int(A1.w);
-        cb = __float_as_int(B1.w);
-        if (ca < 0 && cb < 0) {
-          cls = 3;  // two leaves: P2P
-        } else if (ca < 0) {
-          openb = true;
-        } else if (cb < 0) {
-          opena = true;
-        } else if (A0.w != B0.w) {  // rounding to FP32 keeps the order of unequal sides
-          opena = A0.w > B0.w;
-          openb = !opena;
-        } else {
-          const double sa = G.side(a), sb = G.side(b);
-          opena = sa >= sb;
-          openb = sb >= sa;
-        }
-      }
-      warp_append(cls == 1, e, ctr + 0, m2l, cap_m);
-      warp_append(cls == 3, e, ctr + 1, p2p, cap_p);
-      // the children pairs: (opena ? 2 : 1) x (openb ? 2 : 1) of them
-      const uint32_t nkid = cls == 2 ? (opena ? 2u : 1u) * (openb ? 2u : 1u) : 0u;
-      uint32_t incl = nkid;
-#pragma unroll
-      for (int o = 1; o < 32; o <<= 1) {
-        const uint32_t y = __shfl_up_sync(0xffffffffu, incl, o);
-        if (lane >= o) incl += y;
-      }
-      const uint32_t tot = __shfl_sync(0xffffffffu, incl, 31);
-      if (tot == 0) continue;
-      unsigned long long wb = 0;
-      if (lane == 31) wb = atomicAdd(ncount, (unsigned long long)tot);
-      wb = __shfl_sync(0xffffffffu, wb, 31);
-      unsigned long long slot = wb + incl - nkid;
-      if (nkid) {
-        const uint32_t a0 = opena ? (uint32_t)ca : a, a1 = opena ? a0 + 2 : a + 1;
-        const uint32_t b0 = openb ? (uint32_t)cb : b, b1 = openb ? b0 + 2 : b + 1;
-        for (uint32_t x = a0; x < a1; ++x)
-          for (uint32_t y = b0; y < b1; ++y, ++slot)
-            if (slot < cap_f) next[slot] = pack_pair(x, y, s);
-      }
-    }
-    pairs += nf;
-    grid.sync();
-    // Every block reads the same count (this level's counter takes no appends until
-    // it is cleared two levels on), so every block takes the same decision.  The
-    // M2L and P2P counters are not read here: blocks already in the next level
-    // append to them.  An outgrown list only stops being written (the counts go on);
-    // the caller compares the final counts with the capacities.
-    const unsigned long long nn = *(volatile unsigned long long *)ncount;
-    const bool over = nn > cap_f;
-    if (over || nn == 0) {
-      if (gt == 0) {
-        ctr[2] = over ? 1ull : 0ull;
-        ctr[3] = (unsigned long long)level + 1;
-        ctr[4] = pairs;
-      }
-      return;
-    }
-    nf = nn;
+  const unsigned lt = (1u << lane) - 1u;
+  float4 A0, A1;
+  W.G.rec(k, A0, A1);
+  const int ca = __float_as_int(A1.w);
+  const bool leaf = ca < 0;
+  const uint32_t *in = W.open[(level & 1) ^ 1];
+  unsigned long long ibeg = 0;
+  uint32_t icnt = W.R.conventional ? 1u : 27u;
+  if (k != 0) {
+    const int p = W.parent[k];
+    ibeg = W.obeg[p];
+    icnt = W.ocnt[p];
   }
+  uint64_t *const m2l = W.m2l, *const p2p = W.p2p;
+  uint32_t *const out = W.open[level & 1];
+  unsigned long long bm = 0, bp = 0;
+  bool fit_m = false, fit_p = false;
+  uint32_t nm = 0, np = 0;  // M2L entries; P2P (a leaf's) or open entries
+  for (int pass = 0; pass < 2; ++pass) {
+    uint32_t pi = 0;
+    int sp = 0;
+    bool over = false;
+    nm = np = 0;
+    for (;;) {
+      // ---- the next sources: from the stack, then from the parent's open list
+      int ks = sp < 32 ? sp : 32;
+      uint32_t kl = icnt - pi < (uint32_t)(32 - ks) ? icnt - pi : (uint32_t)(32 - ks);
+      if (sp > kSoft) {
+        ks = 1;
+        kl = 0;
+      }
+      if (ks + (int)kl == 0) break;
+      const bool has = lane < ks + (int)kl;
+      uint32_t e = 0;
+      if (lane < ks) e = stack[sp - ks + lane];
+      else if (has) e = k != 0 ? in[ibeg + pi + lane - ks] : W.R.conventional ? 13u : pi + lane - ks;
+      sp -= ks;
+      pi += kl;
+      __syncwarp();
+      // ---- what becomes of each
+      const uint32_t b = e >> 5, s = e & 31u;
+      int cls = 0, cb = -1;
+      bool opena = false, openb = false;
+      if (has) {
+        float4 B0, B1;
+        W.G.rec(b, B0, B1);
+        cls = kd_classify(W.G, k, b, s, W.R, A0, A1, B0, B1);
+        cb = __float_as_int(B1.w);
+        if (cls == 2) {
+          if (leaf && cb < 0) {
+            cls = 3;  // two leaves: P2P
+          } else if (leaf) {
+            openb = true;
+          } else if (cb < 0) {
+            opena = true;
+          } else if (A0.w != B0.w) {  // rounding to FP32 keeps the order of unequal sides
+            opena = A0.w > B0.w;
+            openb = !opena;
+          } else {
+            const double sa = W.G.side(k), sb = W.G.side(b);
+            opena = sa >= sb;
+            openb = sb >= sa;
+          }
+        }
+        if (pass == 0) ++items;
+      }
+      const uint32_t kid = (uint32_t)cb << 5 | s;
+      // the source's children, to be visited by this sink
+      const unsigned mo = __ballot_sync(0xffffffffu, openb && !opena);
+      if (openb && !opena) {
+        const int at = sp + 2 * __popc(mo & lt);
+        stack[at] = kid;
+        stack[at + 1] = kid + 32u;
+      }
+      sp += 2 * __popc(mo);
+      // M2L; P2P or open (one entry, or the source's two children)
+      const bool far = cls == 1, near = cls == 3 || opena, two = opena && openb;
+      const unsigned mm = __ballot_sync(0xffffffffu, far), m1 = __ballot_sync(0xffffffffu, near),
+                     m2 = __ballot_sync(0xffffffffu, two);
+      const uint32_t im = nm + __popc(mm & lt), ip = np + __popc(m1 & lt) + __popc(m2 & lt);
+      nm += __popc(mm);
+      np += __popc(m1) + __popc(m2);
+      const uint32_t v = two ? kid : e;
+      if (pass == 0) {
+        over = over || nm + np > (uint32_t)kStage;
+        if (!over) {  // P2P or open entries from the front, M2L from the back
+          if (far) stage[kStage - 1 - im] = e;
+          if (near) stage[ip] = v;
+          if (two) stage[ip + 1] = v + 32u;
+        }
+      } else {
+        if (far && fit_m) m2l[bm + im] = pack_pair(k, 0, 0) | e;
+        if (near && fit_p) {
+          if (leaf) p2p[bp + ip] = pack_pair(k, 0, 0) | v;
+          else out[bp + ip] = v;
+        }
+        if (two && fit_p) out[bp + ip + 1] = v + 32u;
+      }
+      __syncwarp();
+    }
+    if (pass == 1) break;
+    // ---- the entries' ranges
+    if (lane == 0) {
+      if (nm) bm = atomicAdd(W.ctr + 0, (unsigned long long)nm);
+      if (np) bp = atomicAdd(leaf ? W.ctr + 1 : nopen, (unsigned long long)np);
+    }
+    bm = __shfl_sync(0xffffffffu, bm, 0);
+    bp = __shfl_sync(0xffffffffu, bp, 0);
+    fit_m = nm > 0 && bm + nm <= W.cap_m2l;
+    fit_p = np > 0 && bp + np <= (leaf ? W.cap_p2p : W.cap_open);
+    if (lane == 0) {
+      W.mb[k] = (uint32_t)bm;
+      W.me[k] = (uint32_t)bm + (fit_m ? nm : 0u);
+      W.pb[k] = leaf ? (uint32_t)bp : 0u;
+      W.pe[k] = leaf ? (uint32_t)bp + (fit_p ? np : 0u) : 0u;
+      if (!leaf) {
+        W.obeg[k] = bp;
+        W.ocnt[k] = fit_p ? np : 0u;
+      }
+    }
+    if (!over) {
+      if (fit_m)
+        for (uint32_t i = lane; i < nm; i += 32) m2l[bm + i] = pack_pair(k, 0, 0) | stage[kStage - 1 - i];
+      if (fit_p)
+        for (uint32_t i = lane; i < np; i += 32) {
+          if (leaf) p2p[bp + i] = pack_pair(k, 0, 0) | stage[i];
+          else out[bp + i] = stage[i];
+        }
+      break;
+    }
+    if (!fit_m && !fit_p) break;
+  }
+  __syncwarp();
 }
 
-// CSR bounds of a list sorted by sink.
-__global__ void k_kd_csr(const uint64_t *__restrict__ lst, int64_t n, uint32_t *__restrict__ beg,
-                         uint32_t *__restrict__ end) {
-  const int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (t >= n) return;
-  const uint32_t k = pair_sink(lst[t]);
-  if (t == 0 || pair_sink(lst[t - 1]) != k) beg[k] = (uint32_t)t;
-  if (t == n - 1 || pair_sink(lst[t + 1]) != k) end[k] = (uint32_t)(t + 1);
+// The whole walk in one cooperative launch, the tree's levels in turn with a grid-wide
+// barrier between them (an open list is complete before the children start from it), a
+// level's nodes to warps from a counter, until the last level or open lists that outgrow
+// their buffer (the caller grows the buffers that were outgrown and walks again).  Each
+// sink's entries lie together, in an order that does not depend on the schedule.
+//
+// What bounds it: instructions, in the last two levels (two thirds of the pairs); the levels
+// above by latency, one session and one barrier each.  A walk over a frontier of (sink,
+// source) pairs, two entries of 8 bytes written and read a pair, left lists to be sorted
+// by (sink, source, shift): 2.0 + 1.5 ms for 46M pairs and 21M entries (2M clustered
+// particles) instead of 1.46.
+__global__ void __launch_bounds__(kT, 4) k_kd_walk(const __grid_constant__ KdWalk W) {
+  cg::grid_group grid = cg::this_grid();
+  extern __shared__ uint32_t walk_smem[];
+  const int lane = threadIdx.x & 31;
+  uint32_t *stack = walk_smem + (threadIdx.x >> 5) * kWalkWarpWords, *stage = stack + kStack;
+  const bool first = blockIdx.x == 0 && threadIdx.x == 0;
+  const int levels = W.S.depth + 1 + (W.S.nsplit ? 1 : 0);
+  unsigned long long items = 0, most = 0;
+  int level = 0;
+  for (; level < levels; ++level) {
+    const uint32_t lo = (uint32_t)(((int64_t)1 << level) - 1);
+    const uint32_t hi = level <= W.S.depth ? (uint32_t)(((int64_t)2 << level) - 1) : (uint32_t)W.S.nodes();
+    unsigned long long *nopen = W.ctr + 5 + level % 3, *ticket = W.ctr + 8 + level % 3;
+    if (first) W.ctr[5 + (level + 1) % 3] = W.ctr[8 + (level + 1) % 3] = 0;
+    for (;;) {
+      unsigned long long t = 0;
+      if (lane == 0) t = atomicAdd(ticket, 1ull);
+      t = __shfl_sync(0xffffffffu, t, 0);
+      if (t >= hi - lo) break;
+      kd_session(W, lo + (uint32_t)t, level, stack, stage, nopen, items);
+    }
+    grid.sync();
+    // every block reads the same count, and so takes the same decision; the M2L and P2P
+    // counts are the caller's to compare with the capacities
+    most = *(volatile unsigned long long *)nopen;
+    if (most > W.cap_open) break;
+  }
+  if (first) {
+    W.ctr[2] = most > W.cap_open ? 1ull : 0ull;
+    W.ctr[3] = (unsigned long long)min(level + 1, levels);
+  }
+#pragma unroll
+  for (int o = 16; o; o >>= 1) items += __shfl_xor_sync(0xffffffffu, items, o);
+  if (lane == 0 && items) atomicAdd(W.ctr + 4, items);
 }
 
 // Particle pairs on the P2P list: sum over entries of n_sink n_source.
@@ -747,48 +830,67 @@ cudaError_t kd_walk(Ctx &c, cudaStream_t st, bool conventional = false) {
   uint64_t cap_m = std::max<uint64_t>(kd.caps[1], std::max<uint64_t>(1u << 16, 32 * nl));
   uint64_t cap_p = std::max<uint64_t>(kd.caps[2], std::max<uint64_t>(1u << 16, 256 * nl));
   if (c.prm.list_init > 0 && kd.caps[0] == 0) cap_f = cap_m = cap_p = (uint64_t)c.prm.list_init;
-  cap_f = std::max<uint64_t>(cap_f, 32);  // the 27 root pairs
+  const size_t nn = (size_t)c.nnodes;
   TRY(ensure(kd.ctr, 128));
+  TRY(ensure(kd.obeg, nn * 8));
+  TRY(ensure(kd.ocnt, nn * 4));
+  TRY(ensure(c.m2l_beg, nn * 4));
+  TRY(ensure(c.m2l_end, nn * 4));
+  TRY(ensure(c.p2p_beg, nn * 4));
+  TRY(ensure(c.p2p_end, nn * 4));
   unsigned long long *ctr = P<unsigned long long>(kd.ctr);
+  const size_t smem = (size_t)(kT / 32) * kWalkWarpWords * 4;
   int dev = 0, nsm = 0, per_sm = 0;
   TRY(cudaGetDevice(&dev));
   TRY(cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev));
-  TRY(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_kd_walk, kT, 0));
+  TRY(cudaFuncSetAttribute(k_kd_walk, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+  TRY(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_kd_walk, kT, smem));
   if (per_sm < 1) return cudaErrorInvalidConfiguration;
   const unsigned nb = (unsigned)(nsm * std::min(per_sm, 4));
-  WalkRule R;
-  R.L = c.prm.box;
-  R.rc2 = c.rc * c.rc;
-  R.theta2 = c.prm.theta * c.prm.theta;
-  R.Lf = (float)R.L;
-  R.rc2f = (float)R.rc2;
-  R.theta2f = (float)R.theta2;
-  R.dl = (float)std::ldexp(16.0 * R.L, -24);
-  R.rule = c.prm.transition_rule;
-  R.size_rule = c.prm.size_rule;
-  R.conventional = conventional ? 1 : 0;
-  KdGeo G = kd_geo(c);
+  KdWalk W;
+  W.S = kd_shape(c.n, c.prm.leaf_max);
+  W.G = KdGeo{P<double>(kd.geo), P<float>(kd.geof), kd.cap};
+  W.R.L = c.prm.box;
+  W.R.rc2 = c.rc * c.rc;
+  W.R.theta2 = c.prm.theta * c.prm.theta;
+  W.R.Lf = (float)W.R.L;
+  W.R.rc2f = (float)W.R.rc2;
+  W.R.theta2f = (float)W.R.theta2;
+  W.R.dl = (float)std::ldexp(16.0 * W.R.L, -24);
+  W.R.rule = c.prm.transition_rule;
+  W.R.size_rule = c.prm.size_rule;
+  W.R.conventional = conventional ? 1 : 0;
+  W.parent = P<int>(kd.parent);
+  W.obeg = P<unsigned long long>(kd.obeg);
+  W.ocnt = P<uint32_t>(kd.ocnt);
+  W.mb = P<uint32_t>(c.m2l_beg);
+  W.me = P<uint32_t>(c.m2l_end);
+  W.pb = P<uint32_t>(c.p2p_beg);
+  W.pe = P<uint32_t>(c.p2p_end);
+  W.ctr = ctr;
   int64_t walks = 0;
   uint64_t h[kWalkCtr];
   for (;;) {
-    if (++walks > 16) return cudaErrorInvalidValue;
-    TRY(ensure(c.front, cap_f * 8));
-    TRY(ensure(c.front_next, cap_f * 8));
+    if (++walks > 32) return cudaErrorInvalidValue;
+    for (DBuf &b : kd.open) TRY(ensure(b, cap_f * 4));
     TRY(ensure(c.m2l, cap_m * 8));
     TRY(ensure(c.p2p, cap_p * 8));
     TRY(cudaMemsetAsync(ctr, 0, kWalkCtr * 8, st));
-    uint64_t *fa = P<uint64_t>(c.front), *fb = P<uint64_t>(c.front_next), *m2l = P<uint64_t>(c.m2l),
-             *p2p = P<uint64_t>(c.p2p);
-    unsigned long long cf = cap_f, cm = cap_m, cp = cap_p;
-    void *args[] = {(void *)&fa, (void *)&fb, (void *)&cf, (void *)&m2l, (void *)&cm, (void *)&p2p, (void *)&cp,
-                    (void *)&ctr, (void *)&G, (void *)&R};
-    TRY(cudaLaunchCooperativeKernel((const void *)k_kd_walk, dim3(nb), dim3(kT), args, 0, st));
+    W.open[0] = P<uint32_t>(kd.open[0]);
+    W.open[1] = P<uint32_t>(kd.open[1]);
+    W.m2l = P<uint64_t>(c.m2l);
+    W.p2p = P<uint64_t>(c.p2p);
+    W.cap_open = cap_f;
+    W.cap_m2l = cap_m;
+    W.cap_p2p = cap_p;
+    void *args[] = {(void *)&W};
+    TRY(cudaLaunchCooperativeKernel((const void *)k_kd_walk, dim3(nb), dim3(kT), args, smem, st));
     note_launch();
     TRY(read_u64(c, ctr, h, kWalkCtr, st));
     if (!h[2] && h[0] <= cap_m && h[1] <= cap_p) break;
     // an outgrown buffer: grow what the counts ask for (the counts went on past the capacities)
-    const uint64_t nn = std::max(std::max(h[5], h[6]), h[7]);
-    if (nn > cap_f) cap_f = nn + nn / 2 + 4096;
+    const uint64_t most = std::max(std::max(h[5], h[6]), h[7]);
+    if (most > cap_f) cap_f = most + most / 2 + 4096;
     if (h[0] > cap_m) cap_m = h[0] + h[0] / 2 + 4096;
     if (h[1] > cap_p) cap_p = h[1] + h[1] / 2 + 4096;
   }
@@ -803,47 +905,19 @@ cudaError_t kd_walk(Ctx &c, cudaStream_t st, bool conventional = false) {
   return cudaSuccess;
 }
 
-cudaError_t kd_group(Ctx &c, cudaStream_t st) {
-  const size_t nn = (size_t)c.nnodes;
-  TRY(ensure(c.m2l_beg, nn * 4));
-  TRY(ensure(c.m2l_end, nn * 4));
-  TRY(ensure(c.p2p_beg, nn * 4));
-  TRY(ensure(c.p2p_end, nn * 4));
-  // the sorts' scratch: the walk's frontier buffers, free once the walk is done, when
-  // they are large enough (at 134M particles they hold tens of GB), else a buffer of its own
-  DBuf *lst[2] = {&c.m2l, &c.p2p}, *alt[2] = {&c.front_next, &c.front};
-  if (c.front_next.cap < (size_t)c.nm2l * 8) alt[0] = &c.m2l_alt;
-  if (c.front.cap < (size_t)c.np2p * 8) alt[1] = &c.p2p_alt;
-  DBuf *beg[2] = {&c.m2l_beg, &c.p2p_beg}, *end[2] = {&c.m2l_end, &c.p2p_end};
-  const int64_t len[2] = {c.nm2l, c.np2p};
-  for (int w = 0; w < 2; ++w) {
-    TRY(cudaMemsetAsync(beg[w]->p, 0, nn * 4, st));
-    TRY(cudaMemsetAsync(end[w]->p, 0, nn * 4, st));
-    if (len[w] == 0) continue;
-    TRY(ensure(*alt[w], (size_t)len[w] * 8));
-    bool in_alt = false;
-    TRY(radix_sort_u64(P<uint64_t>(*lst[w]), nullptr, P<uint64_t>(*alt[w]), nullptr, (size_t)len[w], 0,
-                       kSinkShift + kSinkBits, &in_alt, c.tmp, st));
-    if (in_alt) std::swap(*lst[w], *alt[w]);
-    k_kd_csr<<<blocks_for((size_t)len[w], kT), kT, 0, st>>>(P<uint64_t>(*lst[w]), len[w], P<uint32_t>(*beg[w]),
-                                                             P<uint32_t>(*end[w]));
+// The particle pairs on the P2P list (synchronises st).
+cudaError_t kd_particle_pairs(Ctx &c, int64_t *out, cudaStream_t st) {
+  unsigned long long *cnt = P<unsigned long long>(c.kd.ctr) + kWalkCtr + 1;
+  TRY(cudaMemsetAsync(cnt, 0, 8, st));
+  if (c.np2p > 0) {
+    k_kd_list_pairs<<<blocks_for((size_t)c.np2p, kT), kT, 0, st>>>(P<uint64_t>(c.p2p), c.np2p,
+                                                                    P<uint32_t>(c.kd.count), cnt);
     note_launch();
   }
-  // statistics runs: the particle pairs on the P2P list
-  c.p2p_particle_pairs = -1;
-  if (c.prm.profile & 2) {
-    unsigned long long *cnt = P<unsigned long long>(c.kd.ctr) + kWalkCtr + 1;
-    TRY(cudaMemsetAsync(cnt, 0, 8, st));
-    if (c.np2p > 0) {
-      k_kd_list_pairs<<<blocks_for((size_t)c.np2p, kT), kT, 0, st>>>(P<uint64_t>(c.p2p), c.np2p,
-                                                                      P<uint32_t>(c.kd.count), cnt);
-      note_launch();
-    }
-    uint64_t pp = 0;
-    TRY(read_u64(c, cnt, &pp, 1, st));
-    c.p2p_particle_pairs = (int64_t)pp;
-  }
-  return cudaGetLastError();
+  uint64_t pp = 0;
+  TRY(read_u64(c, cnt, &pp, 1, st));
+  *out = (int64_t)pp;
+  return cudaSuccess;
 }
 
 }  // namespace
@@ -953,16 +1027,7 @@ cudaError_t kd_interaction_counts(Ctx &c, bool conventional, int64_t *out, cudaS
   out[1] = c.np2p;
   out[2] = 0;
   out[3] = c.frontier_items;
-  if (c.np2p > 0) {
-    unsigned long long *cnt = P<unsigned long long>(c.kd.ctr) + kWalkCtr + 1;
-    TRY(cudaMemsetAsync(cnt, 0, 8, st));
-    k_kd_list_pairs<<<blocks_for((size_t)c.np2p, kT), kT, 0, st>>>(P<uint64_t>(c.p2p), c.np2p,
-                                                                    P<uint32_t>(c.kd.count), cnt);
-    note_launch();
-    uint64_t pp = 0;
-    TRY(read_u64(c, cnt, &pp, 1, st));
-    out[2] = (int64_t)pp;
-  }
+  if (c.np2p > 0) TRY(kd_particle_pairs(c, &out[2], st));
   return cudaSuccess;
 }
 
@@ -974,7 +1039,9 @@ cudaError_t kd_short_range(Ctx &c, float *acc, cudaStream_t st) {
   TRY(kd_walk(c, st));
   if (c.nm2l > (int64_t)UINT32_MAX || c.np2p > (int64_t)UINT32_MAX) return cudaErrorInvalidValue;
   if (prof) cudaEventRecord(c.ev[5], st);
-  TRY(kd_group(c, st));
+  // statistics runs: the particle pairs on the P2P list
+  c.p2p_particle_pairs = -1;
+  if (c.prm.profile & 2) TRY(kd_particle_pairs(c, &c.p2p_particle_pairs, st));
   if (prof) cudaEventRecord(c.ev[6], st);
   TRY(m2l_pass(c, c.p, st));
   if (prof) cudaEventRecord(c.ev[7], st);
