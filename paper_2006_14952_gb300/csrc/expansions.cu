@@ -10,12 +10,13 @@ namespace hfmm {
 namespace {
 
 // Row of NC floats at a 16-byte aligned address (rows are padded to a multiple of 4).
-template <int NC>
-__device__ __forceinline__ void load_row(const float *__restrict__ src, float (&r)[NC]) {
+// kFixed: not written by this kernel.
+template <int NC, bool kFixed = true>
+__device__ __forceinline__ void load_row(const float *src, float (&r)[NC]) {
   const float4 *s4 = reinterpret_cast<const float4 *>(src);
 #pragma unroll
   for (int q = 0; q < (NC + 3) / 4; ++q) {
-    const float4 v = __ldg(s4 + q);
+    const float4 v = kFixed ? __ldg(s4 + q) : s4[q];
     if (4 * q + 0 < NC) r[4 * q + 0] = v.x;
     if (4 * q + 1 < NC) r[4 * q + 1] = v.y;
     if (4 * q + 2 < NC) r[4 * q + 2] = v.z;
@@ -24,7 +25,7 @@ __device__ __forceinline__ void load_row(const float *__restrict__ src, float (&
 }
 
 template <int NC>
-__device__ __forceinline__ void store_row(float *__restrict__ dst, const float (&r)[NC]) {
+__device__ __forceinline__ void store_row(float *dst, const float (&r)[NC]) {
   float4 *d4 = reinterpret_cast<float4 *>(dst);
 #pragma unroll
   for (int q = 0; q < NC / 4; ++q) d4[q] = make_float4(r[4 * q], r[4 * q + 1], r[4 * q + 2], r[4 * q + 3]);
@@ -32,102 +33,170 @@ __device__ __forceinline__ void store_row(float *__restrict__ dst, const float (
   for (int c = NC / 4 * 4; c < NC; ++c) dst[c] = r[c];
 }
 
-// P2M, one thread per leaf: M~_m = sum_a mu_a (-1)^|m| / m! (u_a)^m, u = (x - z) / h.
+// P2M and L2P: kPerM and kPerL adjacent lanes a leaf, each every so many-th of its
+// particles.  A thread a leaf is bound by the chain over the particles, more lanes by P2M's
+// reduction and the loads of L2P's rows; us with 1, 2, 4, 8 lanes: 1000 uniform particles,
+// p = 4, P2M 10.6, 7.6, 6.5, -, L2P 11.5, 7.5, 5.5, 4.8; 2M clustered, p = 6, P2M 74, 70, 74, -,
+// L2P 110, 102, 97, 102; the same on the k-d tree P2M 27, 32, 36, -, L2P 64, 57, 57, 59.
+constexpr int kPerM = 2, kPerL = 4;
+
+// A leaf's row from the sums of its lanes, added in a fixed order; each stores a part.
+template <int NC>
+__device__ __forceinline__ void reduce_store(float *dst, float (&r)[NC], int part) {
+#pragma unroll
+  for (int c = 0; c < NC; ++c) {
+#pragma unroll
+    for (int o = 1; o < kPerM; o <<= 1) r[c] += __shfl_xor_sync(0xffffffffu, r[c], o);
+  }
+  float4 *d4 = reinterpret_cast<float4 *>(dst);
+#pragma unroll
+  for (int q = 0; q < NC / 4; ++q)
+    if (q % kPerM == part) d4[q] = make_float4(r[4 * q], r[4 * q + 1], r[4 * q + 2], r[4 * q + 3]);
+#pragma unroll
+  for (int c = NC / 4 * 4; c < NC; ++c)
+    if (part == 0) dst[c] = r[c];
+}
+
+// P2M: M~_m = sum_a mu_a (-1)^|m| / m! (u_a)^m, u = (x - z) / h.
 // tz (a step captured as one graph): the leaf count from the device tree state.
 template <int P>
 __global__ void k_p2m(const uint32_t *__restrict__ leaves, int64_t nl, const uint4 *__restrict__ cell,
                       const uint2 *__restrict__ range, const float4 *__restrict__ pm4, float box, int ldm,
                       float *__restrict__ M, const TreeState *tz) {
   constexpr int NC = ncoef(P);
-  int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (t >= tree_leaves(tz, nl)) return;
-  const uint32_t k = leaves[t];
-  const uint2 r = range[k];
-  const float inv_h = (float)(1u << cell[k].w) / box;
+  const int64_t t = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) / kPerM;
+  const int part = threadIdx.x % kPerM;
+  const bool valid = t < tree_leaves(tz, nl);
+  const uint32_t k = valid ? leaves[t] : 0u;
+  const uint2 r = valid ? range[k] : make_uint2(0u, 0u);
+  const float inv_h = valid ? (float)(1u << cell[k].w) / box : 0.f;
   float acc[NC];
 #pragma unroll
   for (int c = 0; c < NC; ++c) acc[c] = 0.f;
-  for (uint32_t i = r.x; i < r.x + r.y; ++i) {
+  for (uint32_t i = r.x + part; i < r.x + r.y; i += kPerM) {
     const float4 q = pm4[i];
     P2MBody<P>::run(q.x * inv_h, q.y * inv_h, q.z * inv_h, q.w, acc);
   }
   P2MBody<P>::finish(acc);
-  store_row<NC>(M + (size_t)k * ldm, acc);
+  reduce_store<NC>(M + (size_t)k * ldm, acc, valid ? part : -1);
 }
 
 // M2M, one thread per (cell of one level, child slot): each thread translates
 // one child's multipoles to the parent centre; the eight sibling threads are
 // adjacent lanes and add their results with a fixed xor-shuffle tree (the same
-// order on every run), and slot 0 stores the parent's row.  The loop is
-// block-uniform (whole warps take each trip: the shuffles see all lanes); with
-// tz (graph mode) the level's extent comes from the device tree state.
+// order on every run), and slot 0 stores the parent's row.  Every lane of a warp
+// calls it (the shuffles see all lanes).
+template <int P, bool kFixed>
+__device__ __forceinline__ void m2m_child(int64_t lo, int64_t cnt, int64_t t, const uint4 *__restrict__ cell,
+                                          const int2 *__restrict__ kids, int ldm, float *M) {
+  constexpr int NC = ncoef(P);
+  const bool in_level = t < 8 * cnt;  // whole groups of 8: cnt * 8 threads, blocks of a multiple of 8
+  const int64_t k = lo + t / 8;
+  const int slot = (int)(t % 8);
+  const int2 kd = in_level ? kids[k] : make_int2(0, 0);
+  float o[NC];
+#pragma unroll
+  for (int c = 0; c < NC; ++c) o[c] = 0.f;
+  if (slot < kd.y) {
+    const int ch = kd.x + slot;
+    const uint4 cc = cell[ch];
+    // (z_P - z_C) / H = +1/4 for the lower half of an axis, -1/4 for the upper
+    float ci[NC];
+    load_row<NC, kFixed>(M + (size_t)ch * ldm, ci);
+    M2MBody<P>::run((cc.x & 1u) ? -1.f : 1.f, (cc.y & 1u) ? -1.f : 1.f, (cc.z & 1u) ? -1.f : 1.f, ci, o);
+  }
+#pragma unroll
+  for (int c = 0; c < NC; ++c) {
+    o[c] += __shfl_xor_sync(0xffffffffu, o[c], 4);
+    o[c] += __shfl_xor_sync(0xffffffffu, o[c], 2);
+    o[c] += __shfl_xor_sync(0xffffffffu, o[c], 1);
+  }
+  if (in_level && slot == 0 && kd.y > 0) store_row<NC>(M + (size_t)k * ldm, o);
+}
+
+// One level (graph mode, tz: its extent from the device tree state).
 template <int P>
 __global__ void k_m2m(int64_t lo, int64_t cnt, const uint4 *__restrict__ cell, const int2 *__restrict__ kids, int ldm,
                       float *__restrict__ M, const TreeState *tz, int level) {
-  constexpr int NC = ncoef(P);
   tree_level(tz, level, lo, cnt);
   const int64_t stride = (int64_t)gridDim.x * blockDim.x;
-  for (int64_t b = (int64_t)blockIdx.x * blockDim.x; b < 8 * cnt; b += stride) {
-    const int64_t t = b + threadIdx.x;
-    const bool in_level = t < 8 * cnt;  // whole groups of 8: cnt * 8 threads, blocks of a multiple of 8
-    const int64_t k = lo + t / 8;
-    const int slot = (int)(t % 8);
-    const int2 kd = in_level ? kids[k] : make_int2(0, 0);
-    float o[NC];
-#pragma unroll
-    for (int c = 0; c < NC; ++c) o[c] = 0.f;
-    if (slot < kd.y) {
-      const int ch = kd.x + slot;
-      const uint4 cc = cell[ch];
-      // (z_P - z_C) / H = +1/4 for the lower half of an axis, -1/4 for the upper
-      float ci[NC];
-      load_row<NC>(M + (size_t)ch * ldm, ci);
-      M2MBody<P>::run((cc.x & 1u) ? -1.f : 1.f, (cc.y & 1u) ? -1.f : 1.f, (cc.z & 1u) ? -1.f : 1.f, ci, o);
-    }
-#pragma unroll
-    for (int c = 0; c < NC; ++c) {
-      o[c] += __shfl_xor_sync(0xffffffffu, o[c], 4);
-      o[c] += __shfl_xor_sync(0xffffffffu, o[c], 2);
-      o[c] += __shfl_xor_sync(0xffffffffu, o[c], 1);
-    }
-    if (in_level && slot == 0 && kd.y > 0) store_row<NC>(M + (size_t)k * ldm, o);
+  for (int64_t b = (int64_t)blockIdx.x * blockDim.x; b < 8 * cnt; b += stride)
+    m2m_child<P, true>(lo, cnt, b + threadIdx.x, cell, kids, ldm, M);
+}
+
+// Levels 2, 1 and 0 (at most 64 parents) in one block: a launch for each costs more than
+// their translations (upward pass and L2L of 1000 particles, p = 4, three levels: 188 -> 180 us
+// a call with the lanes above).
+constexpr int kTop = 3;
+struct TopLevels {
+  int64_t start[kTop + 1];
+  int levels;  // levels that have children, of the first kTop
+};
+
+template <int P>
+__global__ void __launch_bounds__(256) k_m2m_top(const __grid_constant__ TopLevels top, const uint4 *__restrict__ cell,
+                                                 const int2 *__restrict__ kids, int ldm, float *M,
+                                                 const TreeState *tz) {
+  for (int l = top.levels - 1; l >= 0; --l) {
+    int64_t lo = top.start[l], cnt = top.start[l + 1] - lo;
+    tree_level(tz, l, lo, cnt);
+    for (int64_t b = 0; b < 8 * cnt; b += blockDim.x)
+      m2m_child<P, false>(lo, cnt, b + threadIdx.x, cell, kids, ldm, M);
+    __syncthreads();
   }
 }
 
 // L2L, one thread per (cell of one level, child slot): the child's local
 // expansion plus the parent's translated to the child's centre.  The eight
 // siblings of a parent are neighbouring threads (one parent row load, shared).
+template <int P, bool kFixed>
+__device__ __forceinline__ void l2l_child(int64_t lo, int64_t t, const uint4 *__restrict__ cell,
+                                          const int2 *__restrict__ kids, int ldm, float *L) {
+  constexpr int NC = ncoef(P);
+  const int64_t k = lo + t / 8;
+  const int2 kd = kids[k];
+  const int slot = (int)(t % 8);
+  if (slot >= kd.y) return;
+  const int ch = kd.x + slot;
+  float pl[NC], cl[NC];
+  load_row<NC, kFixed>(L + (size_t)k * ldm, pl);
+  float *dst = L + (size_t)ch * ldm;
+  load_row<NC, kFixed>(dst, cl);
+  const uint4 cc = cell[ch];
+  // (z_C - z_P) / H = -1/4 for the lower half of an axis, +1/4 for the upper
+  L2LBody<P>::run((cc.x & 1u) ? 1.f : -1.f, (cc.y & 1u) ? 1.f : -1.f, (cc.z & 1u) ? 1.f : -1.f, pl, cl);
+  store_row<NC>(dst, cl);
+}
+
 template <int P>
 __global__ void k_l2l(int64_t lo, int64_t cnt, const uint4 *__restrict__ cell, const int2 *__restrict__ kids, int ldm,
                       float *__restrict__ L, const TreeState *tz, int level) {
-  constexpr int NC = ncoef(P);
   tree_level(tz, level, lo, cnt);
   const int64_t stride = (int64_t)gridDim.x * blockDim.x;
-  for (int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; t < 8 * cnt; t += stride) {
-    const int64_t k = lo + t / 8;
-    const int2 kd = kids[k];
-    const int slot = (int)(t % 8);
-    if (slot >= kd.y) continue;
-    const int ch = kd.x + slot;
-    float pl[NC], cl[NC];
-    load_row<NC>(L + (size_t)k * ldm, pl);
-    float *dst = L + (size_t)ch * ldm;
-    load_row<NC>(dst, cl);
-    const uint4 cc = cell[ch];
-    // (z_C - z_P) / H = -1/4 for the lower half of an axis, +1/4 for the upper
-    L2LBody<P>::run((cc.x & 1u) ? 1.f : -1.f, (cc.y & 1u) ? 1.f : -1.f, (cc.z & 1u) ? 1.f : -1.f, pl, cl);
-    store_row<NC>(dst, cl);
+  for (int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; t < 8 * cnt; t += stride)
+    l2l_child<P, true>(lo, t, cell, kids, ldm, L);
+}
+
+template <int P>
+__global__ void __launch_bounds__(256) k_l2l_top(const __grid_constant__ TopLevels top, const uint4 *__restrict__ cell,
+                                                 const int2 *__restrict__ kids, int ldm, float *L,
+                                                 const TreeState *tz) {
+  for (int l = 0; l < top.levels; ++l) {
+    int64_t lo = top.start[l], cnt = top.start[l + 1] - lo;
+    tree_level(tz, l, lo, cnt);
+    for (int64_t t = threadIdx.x; t < 8 * cnt; t += blockDim.x) l2l_child<P, false>(lo, t, cell, kids, ldm, L);
+    __syncthreads();
   }
 }
 
-// L2P, one thread per leaf: a = G h^-2 sum L~_{n+e_d} u^n / n!, written in input order.
+// L2P: a = G h^-2 sum L~_{n+e_d} u^n / n!, written in input order.
 template <int P>
 __global__ void k_l2p(const uint32_t *__restrict__ leaves, int64_t nl, const uint4 *__restrict__ cell,
                       const uint2 *__restrict__ range, const float4 *__restrict__ pm4, const uint32_t *__restrict__ perm,
                       int64_t n, float box, float G, int ldm, const float *__restrict__ L, float *__restrict__ acc,
                       const TreeState *tz, const float *__restrict__ add) {
   constexpr int NC = ncoef(P);
-  int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+  const int64_t t = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) / kPerL;
   if (t >= tree_leaves(tz, nl)) return;
   const uint32_t k = leaves[t];
   const uint2 r = range[k];
@@ -135,7 +204,7 @@ __global__ void k_l2p(const uint32_t *__restrict__ leaves, int64_t nl, const uin
   const float s = G * inv_h * inv_h;
   float l[NC];
   load_row<NC>(L + (size_t)k * ldm, l);
-  for (uint32_t i = r.x; i < r.x + r.y; ++i) {
+  for (uint32_t i = r.x + threadIdx.x % kPerL; i < r.x + r.y; i += kPerL) {
     const float4 q = pm4[i];
     float ax = 0.f, ay = 0.f, az = 0.f;
     L2PBody<P>::run(q.x * inv_h, q.y * inv_h, q.z * inv_h, l, ax, ay, az);
@@ -170,6 +239,13 @@ struct LevelLoop {
       cnt = c.level_start[l + 1] - lo;
     }
   }
+  // the first kTop levels with children
+  TopLevels top(const Ctx &c) const {
+    TopLevels t{};
+    t.levels = levels - 1 < kTop ? levels - 1 : kTop;
+    for (int l = 0; l <= t.levels && !tz; ++l) t.start[l] = c.level_start[l];
+    return t;
+  }
   unsigned grid(int64_t cnt, int T) const {
     const unsigned g = blocks_for(8 * cnt, T);
     return tz && g > 152u * 16u ? 152u * 16u : g;
@@ -181,14 +257,19 @@ cudaError_t upward_p(Ctx &c, cudaStream_t st) {
   const int T = 128;
   const float box = (float)c.prm.box;
   const LevelLoop lv(c);
-  k_p2m<P><<<blocks_for(c.nleaves, T), T, 0, st>>>(hfmm::P<uint32_t>(c.leaves), c.nleaves, hfmm::P<uint4>(c.cell), hfmm::P<uint2>(c.range),
+  k_p2m<P><<<blocks_for(c.nleaves * kPerM, T), T, 0, st>>>(hfmm::P<uint32_t>(c.leaves), c.nleaves, hfmm::P<uint4>(c.cell), hfmm::P<uint2>(c.range),
                                                    hfmm::P<float4>(c.pm4), box, c.ldm, hfmm::P<float>(c.M), lv.tz);
   note_launch();
-  for (int l = lv.levels - 2; l >= 0; --l) {
+  for (int l = lv.levels - 2; l >= kTop; --l) {
     int64_t lo, cnt;
     lv.extent(c, l, lo, cnt);
     k_m2m<P><<<lv.grid(cnt, T), T, 0, st>>>(lo, cnt, hfmm::P<uint4>(c.cell), hfmm::P<int2>(c.kids), c.ldm,
                                             hfmm::P<float>(c.M), lv.tz, l);
+    note_launch();
+  }
+  if (lv.levels > 1) {
+    k_m2m_top<P><<<1, 256, 0, st>>>(lv.top(c), hfmm::P<uint4>(c.cell), hfmm::P<int2>(c.kids), c.ldm,
+                                    hfmm::P<float>(c.M), lv.tz);
     note_launch();
   }
   return cudaGetLastError();
@@ -198,14 +279,19 @@ template <int P>
 cudaError_t downward_p(Ctx &c, float *acc, cudaStream_t st, const float *add) {
   const int T = 128;
   const LevelLoop lv(c);
-  for (int l = 0; l + 1 < lv.levels; ++l) {
+  if (lv.levels > 1) {
+    k_l2l_top<P><<<1, 256, 0, st>>>(lv.top(c), hfmm::P<uint4>(c.cell), hfmm::P<int2>(c.kids), c.ldm,
+                                    hfmm::P<float>(c.L), lv.tz);
+    note_launch();
+  }
+  for (int l = kTop; l + 1 < lv.levels; ++l) {
     int64_t lo, cnt;
     lv.extent(c, l, lo, cnt);
     k_l2l<P><<<lv.grid(cnt, T), T, 0, st>>>(lo, cnt, hfmm::P<uint4>(c.cell), hfmm::P<int2>(c.kids), c.ldm,
                                             hfmm::P<float>(c.L), lv.tz, l);
     note_launch();
   }
-  k_l2p<P><<<blocks_for(c.nleaves, T), T, 0, st>>>(hfmm::P<uint32_t>(c.leaves), c.nleaves, hfmm::P<uint4>(c.cell),
+  k_l2p<P><<<blocks_for(c.nleaves * kPerL, T), T, 0, st>>>(hfmm::P<uint32_t>(c.leaves), c.nleaves, hfmm::P<uint4>(c.cell),
                                                    hfmm::P<uint2>(c.range), hfmm::P<float4>(c.pm4), hfmm::P<uint32_t>(c.idx), c.n,
                                                    (float)c.prm.box, (float)c.prm.G, c.ldm, hfmm::P<float>(c.L), acc,
                                                    lv.tz, add);
@@ -225,19 +311,20 @@ __global__ void k_kd_p2m(const uint32_t *__restrict__ leaves, int64_t nl, const 
                          const uint32_t *__restrict__ count, const float *__restrict__ hs,
                          const float4 *__restrict__ pm4, int ldm, float *__restrict__ M) {
   constexpr int NC = ncoef(P);
-  const int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (t >= nl) return;
-  const uint32_t k = leaves[t];
-  const float inv_h = 1.f / hs[k];
+  const int64_t t = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) / kPerM;
+  const int part = threadIdx.x % kPerM;
+  const bool valid = t < nl;
+  const uint32_t k = valid ? leaves[t] : 0u, f = valid ? first[k] : 0u, m = valid ? count[k] : 0u;
+  const float inv_h = valid ? 1.f / hs[k] : 0.f;
   float acc[NC];
 #pragma unroll
   for (int q = 0; q < NC; ++q) acc[q] = 0.f;
-  for (uint32_t i = first[k]; i < first[k] + count[k]; ++i) {
+  for (uint32_t i = f + part; i < f + m; i += kPerM) {
     const float4 q = pm4[i];
     P2MBody<P>::run(q.x * inv_h, q.y * inv_h, q.z * inv_h, q.w, acc);
   }
   P2MBody<P>::finish(acc);
-  store_row<NC>(M + (size_t)k * ldm, acc);
+  reduce_store<NC>(M + (size_t)k * ldm, acc, valid ? part : -1);
 }
 
 template <int P>
@@ -290,14 +377,14 @@ __global__ void k_kd_l2p(const uint32_t *__restrict__ leaves, int64_t nl, const 
                          const float4 *__restrict__ pm4, const uint32_t *__restrict__ perm, int64_t n, float G,
                          int ldm, const float *__restrict__ L, float *__restrict__ acc) {
   constexpr int NC = ncoef(P);
-  const int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+  const int64_t t = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) / kPerL;
   if (t >= nl) return;
   const uint32_t k = leaves[t];
   const float inv_h = 1.f / hs[k];
   const float s = G * inv_h * inv_h;
   float l[NC];
   load_row<NC>(L + (size_t)k * ldm, l);
-  for (uint32_t i = first[k]; i < first[k] + count[k]; ++i) {
+  for (uint32_t i = first[k] + threadIdx.x % kPerL; i < first[k] + count[k]; i += kPerL) {
     const float4 q = pm4[i];
     float ax = 0.f, ay = 0.f, az = 0.f;
     L2PBody<P>::run(q.x * inv_h, q.y * inv_h, q.z * inv_h, l, ax, ay, az);
@@ -312,7 +399,7 @@ template <int P>
 cudaError_t kd_upward_p(Ctx &c, cudaStream_t st) {
   const int T = 128;
   KdTree &kd = c.kd;
-  k_kd_p2m<P><<<blocks_for(c.nleaves, T), T, 0, st>>>(hfmm::P<uint32_t>(c.leaves), c.nleaves,
+  k_kd_p2m<P><<<blocks_for(c.nleaves * kPerM, T), T, 0, st>>>(hfmm::P<uint32_t>(c.leaves), c.nleaves,
                                                       hfmm::P<uint32_t>(kd.first), hfmm::P<uint32_t>(kd.count),
                                                       hfmm::P<float>(kd.hs), hfmm::P<float4>(c.pm4), c.ldm,
                                                       hfmm::P<float>(c.M));
@@ -336,7 +423,7 @@ cudaError_t kd_downward_p(Ctx &c, float *acc, cudaStream_t st) {
                                                  hfmm::P<float>(kd.hs), c.ldm, hfmm::P<float>(c.L));
     note_launch();
   }
-  k_kd_l2p<P><<<blocks_for(c.nleaves, T), T, 0, st>>>(hfmm::P<uint32_t>(c.leaves), c.nleaves,
+  k_kd_l2p<P><<<blocks_for(c.nleaves * kPerL, T), T, 0, st>>>(hfmm::P<uint32_t>(c.leaves), c.nleaves,
                                                       hfmm::P<uint32_t>(kd.first), hfmm::P<uint32_t>(kd.count),
                                                       hfmm::P<float>(kd.hs), hfmm::P<float4>(c.pm4),
                                                       hfmm::P<uint32_t>(c.idx), c.n, (float)c.prm.G, c.ldm,
