@@ -16,7 +16,7 @@
 // |n|+|m| <= p of P are used, so at most C(p+6,6) / NC^2 of the tensor work is
 // algorithmic (462 / 3136 at p = 5).
 //
-// A worker is 4 warps with one sink at a time; a CTA has four (a kernel that
+// A worker is 4 warps with one sink at a time; a CTA has four or five (a kernel that
 // allocates tensor memory gets one CTA an SM).  A chunk is 32 pairs: three warps
 // compute and store a third of the pairs' D' each (generated TCStore / TCStoreBF
 // bodies), one their M', to K-major, 128-byte-swizzled tiles (one 128-byte row per
@@ -35,8 +35,11 @@
 // run on into the next tile, whose values only reach rows of P that are never
 // read): 47 KB a worker at p = 6.  Four warps an SM with 128-pair chunks, every
 // thread computing both operands and all four K-tiles issued whatever the list's
-// length, took 20.8 ms for the 33M pairs of the 2M learned step instead of 8.6 (issue
-// 36%, tensor pipe 22%; the next rows prefetched into L1: the same).
+// length, took 20.8 ms for the 33M pairs of the 2M learned step instead of 8.6; with D' by
+// recurrence 8.4, multipole rows by 16-byte loads 7.4, entries fetched two chunks ahead
+// 7.3, a fifth worker at p = 5 7.1 (issue 39%; the next rows prefetched into L1: the same;
+// the next operands formed in registers under the MMA: p = 5 3% faster, p = 6 5.2 instead
+// of 3.2 ms, its code no longer in the instruction cache).
 #include <algorithm>
 #include <type_traits>
 
@@ -47,8 +50,10 @@
 namespace hfmm {
 namespace {
 
-constexpr int kWorkers = 4;     // sinks at a time per CTA, four warps each
-constexpr int kThreads = 128 * kWorkers;
+// Sinks at a time per CTA, four warps each: at p = 6 four fill the shared memory, at p = 5
+// five do with what registers five leave a thread (96, no spills; 3.57 -> 3.37 ms of the
+// learned 2M step's p = 5 pairs, with six at 80 registers the same).
+__host__ __device__ constexpr int workers_of(int p) { return p == 5 ? 5 : 4; }
 constexpr int kChunk = 32;      // pairs per chunk: one lane each
 constexpr int kSinkBatch = 16;  // nodes taken from the work counter at a time
 constexpr uint32_t kWaitLimit = 1u << 22;
@@ -69,7 +74,7 @@ __host__ __device__ constexpr size_t worker_bytes(int p) {
   return (most + 1023) / 1024 * 1024;
 }
 // dynamic shared memory: 1 KB alignment slack and the workers'
-__host__ __device__ constexpr size_t smem_of(int p) { return 1024 + kWorkers * worker_bytes(p); }
+__host__ __device__ constexpr size_t smem_of(int p) { return 1024 + workers_of(p) * worker_bytes(p); }
 // terms of L~: sum over n of the m with |n| + |m| <= p
 __host__ __device__ constexpr int terms_of(int p) {
   int t = 0;
@@ -91,7 +96,7 @@ __device__ __forceinline__ void tmem_ld16(uint32_t taddr, float (&v)[16]) {
 }
 
 template <int P, bool kBF>
-__global__ void __launch_bounds__(kThreads, 1)
+__global__ void __launch_bounds__(128 * workers_of(P), 1)
     k_m2l_tc(int64_t nn, const uint4 *__restrict__ cell, const uint32_t *__restrict__ beg,
              const uint32_t *__restrict__ end, const uint64_t *__restrict__ lst, const float *__restrict__ M,
              float *__restrict__ L, int ldm, float inv_rs, unsigned long long *__restrict__ ctr,
@@ -99,8 +104,9 @@ __global__ void __launch_bounds__(kThreads, 1)
   constexpr int NC = ncoef(P), NCP = ncp_of(P);
   constexpr int kLd = NC | 1;  // row stride of the P staging (odd: no bank conflicts)
   constexpr uint32_t WCOLS = tmem_cols_of(P);  // accumulator columns of a worker
-  constexpr uint32_t TCOLS = kWorkers * WCOLS;
-  static_assert(TCOLS <= 512, "tensor memory");
+  constexpr int kWorkers = workers_of(P);
+  constexpr uint32_t TCOLS = kWorkers * WCOLS <= 128 ? 128 : kWorkers * WCOLS <= 256 ? 256 : 512;  // a power of two
+  static_assert(kWorkers * WCOLS <= 512, "tensor memory");
   constexpr uint32_t IDESC = kBF ? idesc_bf16(128, NCP) : idesc_tf32(128, NCP);
   constexpr int kStep = kBF ? 16 : 8;  // pairs per K-step (32 bytes)
   using T = typename std::conditional<kBF, __nv_bfloat16, float>::type;
@@ -110,11 +116,13 @@ __global__ void __launch_bounds__(kThreads, 1)
   __shared__ uint16_t place[terms_of(P)];  // of each term P[n+m][m], by n then m
   __shared__ uint16_t tbeg[NC + 1];
   __shared__ uint32_t sink_list[kWorkers][kSinkBatch];
+  __shared__ uint2 bound_list[kWorkers][kSinkBatch];  // the sinks' list bounds
   __shared__ int sink_count[kWorkers], aborts[kWorkers];
 
   // a worker's four warps (its warp w reads TMEM lanes 32 w ..) meet at a barrier of their own
   const int worker = threadIdx.x >> 7, tid = threadIdx.x & 127, lane = tid & 31, warp = tid >> 5;
   uint32_t *sinks = sink_list[worker];
+  uint2 *bounds = bound_list[worker];
   volatile int &n_sinks = sink_count[worker], &abort_flag = aborts[worker];
   auto sync = [&]() { asm volatile("bar.sync %0, 128;" ::"r"(worker + 1) : "memory"); };
   unsigned char *base =
@@ -176,9 +184,14 @@ __global__ void __launch_bounds__(kThreads, 1)
         t = __shfl_sync(0xffffffffu, t, 0);
         if ((int64_t)t >= nn) break;
         const int64_t k = (int64_t)t + lane;
-        const bool has = lane < kSinkBatch && k < nn && end[k] > beg[k];
-        const unsigned m = __ballot_sync(0xffffffffu, has);
-        if (has) sinks[__popc(m & ((1u << lane) - 1u))] = (uint32_t)k;
+        uint2 r = make_uint2(0u, 0u);
+        if (lane < kSinkBatch && k < nn) r = make_uint2(beg[k], end[k]);
+        const unsigned m = __ballot_sync(0xffffffffu, r.y > r.x);
+        if (r.y > r.x) {
+          const int at = __popc(m & ((1u << lane) - 1u));
+          sinks[at] = (uint32_t)k;
+          bounds[at] = r;
+        }
         got = __popc(m);
         if (got) break;
       }
@@ -187,101 +200,108 @@ __global__ void __launch_bounds__(kThreads, 1)
     sync();
     const int ns = n_sinks;
     if (ns == 0 || abort_flag) break;
-    // this lane's pair of the next chunk, fetched while the chunk before it is in the MMA
-    uint32_t k = sinks[0], tb = beg[k], te = end[k], t0 = tb;
-    uint4 ca = cell[k], cb = ca;
-    uint64_t e = 0;
-    auto fetch = [&]() {
-      e = t0 + lane < te ? lst[t0 + lane] : 0ull;
-      cb = t0 + lane < te ? cell[pair_src(e)] : ca;
+    // Chunks in order: the one at hand (its pair e, cb of sink ca), and the one after it,
+    // whose entry e1 is there when its cell is asked for: both fetches run under the MMA.
+    struct Chunk {
+      int si;  // ns: none
+      uint32_t t0, te;
     };
-    fetch();
-    for (int si = 0; si < ns; ++si) {
-      const uint32_t sink = k, sink_end = te;
-      for (bool first = true, more = true; more; first = false) {
-        const uint32_t cnt = sink_end - t0 < (uint32_t)kChunk ? sink_end - t0 : (uint32_t)kChunk;
-        const bool valid = (uint32_t)lane < cnt;
-        if (warp != 1) {  // D': a third of the coefficients each
-          float rx = 1.f, ry = 0.f, rz = 0.f, x = 1.f, u = 0.f;
-          if (valid) {
-            int dd[3];
-            half_delta32(ca, cb, pair_shift(e), dd);
-            const float Rx = -(float)dd[0], Ry = -(float)dd[1], Rz = -(float)dd[2];
-            const float r2 = Rx * Rx + Ry * Ry + Rz * Rz;
-            const float rinv = rsqrtf(r2);
-            rx = Rx * rinv;
-            ry = Ry * rinv;
-            rz = Rz * rinv;
-            x = r2 * rinv * inv_rs;
-            u = (float)(2 * half_width(ca.w)) * rinv;
-          }
-          float f[P + 1];
-          f[0] = erfcf(0.5f * x);
-          float tk = -x * kInvSqrtPi * __expf(-0.25f * x * x);
-          const float hx2 = 0.5f * x * x;
-#pragma unroll
-          for (int q = 0; q < P; ++q) {
-            f[q + 1] = -(float)(2 * q + 1) * f[q] + tk;
-            tk = -tk * hx2;
-          }
-          float U[P + 1];
-          U[0] = u;
-#pragma unroll
-          for (int q = 1; q <= P; ++q) U[q] = U[q - 1] * u;
-          T *hi = reinterpret_cast<T *>(a_hi), *lo = reinterpret_cast<T *>(a_lo);
-          using Store = typename std::conditional<kBF, TCStoreBF<P>, TCStore<P>>::type;
-          if (warp == 0) Store::template store_d<3, 0>(rx, ry, rz, f, U, hi, lo, xo);
-          else if (warp == 2) Store::template store_d<3, 1>(rx, ry, rz, f, U, hi, lo, xo);
-          else Store::template store_d<3, 2>(rx, ry, rz, f, U, hi, lo, xo);
-        } else {
-          const float vr = (float)half_width(cb.w) / (float)half_width(ca.w);  // v / u = h_B / h_A
-          const float *Mb = M + (size_t)pair_src(e) * ldm;
-          T *hi = reinterpret_cast<T *>(b_hi), *lo = reinterpret_cast<T *>(b_lo);
-          if constexpr (kBF) TCStoreBF<P>::store_m(Mb, vr, valid ? 1.f : 0.f, hi, lo, xo);
-          else TCStore<P>::store_m(Mb, vr, valid ? 1.f : 0.f, hi, lo, xo);
-        }
-        asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
-        sync();
-        if (tid == 0) {
-          asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-          const uint32_t steps = (cnt + kStep - 1) / kStep;
-          for (uint32_t j = 0; j < steps; ++j) {
-            const uint32_t off = j * 32;
-            const uint64_t ah = desc_sw128(smem_u32(a_hi) + off), al = desc_sw128(smem_u32(a_lo) + off);
-            const uint64_t bh = desc_sw128(smem_u32(b_hi) + off), bl = desc_sw128(smem_u32(b_lo) + off);
-            const uint32_t acc = (!first || j != 0) ? 1u : 0u;
-            if constexpr (kBF) {
-              mma_bf16(tmem, ah, bh, IDESC, acc);
-              mma_bf16(tmem, ah, bl, IDESC, 1u);
-              mma_bf16(tmem, al, bh, IDESC, 1u);
-            } else {
-              mma_tf32(tmem, ah, bh, IDESC, acc);
-              mma_tf32(tmem, ah, bl, IDESC, 1u);
-              mma_tf32(tmem, al, bh, IDESC, 1u);
-            }
-          }
-          mma_commit(mb);
-        }
-        t0 += kChunk;
-        more = t0 < sink_end;
-        if (!more && si + 1 < ns) {
-          k = sinks[si + 1];
-          t0 = tb = beg[k];
-          te = end[k];
-          ca = cell[k];
-        }
-        fetch();
-        const bool ok = mbar_wait(mb, phase, chunk_wait);
-        phase ^= 1u;
-        if (!ok && lane == 0) {
-          atomicExch(status, 1);
-          abort_flag = 1;
-        }
-        sync();
-        if (abort_flag) break;
-        asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+    auto after = [&](Chunk c) {
+      c.t0 += kChunk;
+      if (c.t0 >= c.te && c.si < ns && ++c.si < ns) {
+        c.t0 = bounds[c.si].x;
+        c.te = bounds[c.si].y;
       }
+      return c;
+    };
+    auto entry = [&](const Chunk &c) { return c.si < ns && c.t0 + lane < c.te ? lst[c.t0 + lane] : 0ull; };
+    Chunk c0{0, bounds[0].x, bounds[0].y}, c1 = after(c0);
+    uint64_t e = entry(c0), e1 = entry(c1);
+    uint4 ca = cell[sinks[0]], cb = cell[pair_src(e)];
+    for (bool first = true; c0.si < ns;) {
+      const int si = c0.si;
+      const uint32_t cnt = c0.te - c0.t0 < (uint32_t)kChunk ? c0.te - c0.t0 : (uint32_t)kChunk;
+      const bool valid = (uint32_t)lane < cnt;
+      if (warp != 1) {  // D': a third of the coefficients each
+        float rx = 1.f, ry = 0.f, rz = 0.f, x = 1.f, u = 0.f;
+        if (valid) {
+          int dd[3];
+          half_delta32(ca, cb, pair_shift(e), dd);
+          const float Rx = -(float)dd[0], Ry = -(float)dd[1], Rz = -(float)dd[2];
+          const float r2 = Rx * Rx + Ry * Ry + Rz * Rz;
+          const float rinv = rsqrtf(r2);
+          rx = Rx * rinv;
+          ry = Ry * rinv;
+          rz = Rz * rinv;
+          x = r2 * rinv * inv_rs;
+          u = (float)(2 * half_width(ca.w)) * rinv;
+        }
+        float f[P + 1];
+        f[0] = erfcf(0.5f * x);
+        float tk = -x * kInvSqrtPi * __expf(-0.25f * x * x);
+        const float hx2 = 0.5f * x * x;
+#pragma unroll
+        for (int q = 0; q < P; ++q) {
+          f[q + 1] = -(float)(2 * q + 1) * f[q] + tk;
+          tk = -tk * hx2;
+        }
+        float U[P + 1];
+        U[0] = u;
+#pragma unroll
+        for (int q = 1; q <= P; ++q) U[q] = U[q - 1] * u;
+        T *hi = reinterpret_cast<T *>(a_hi), *lo = reinterpret_cast<T *>(a_lo);
+        using Store = typename std::conditional<kBF, TCStoreBF<P>, TCStore<P>>::type;
+        if (warp == 0) Store::template store_d<3, 0>(rx, ry, rz, f, U, hi, lo, xo);
+        else if (warp == 2) Store::template store_d<3, 1>(rx, ry, rz, f, U, hi, lo, xo);
+        else Store::template store_d<3, 2>(rx, ry, rz, f, U, hi, lo, xo);
+      } else {
+        const float vr = (float)half_width(cb.w) / (float)half_width(ca.w);  // v / u = h_B / h_A
+        const float *Mb = M + (size_t)pair_src(e) * ldm;
+        T *hi = reinterpret_cast<T *>(b_hi), *lo = reinterpret_cast<T *>(b_lo);
+        if constexpr (kBF) TCStoreBF<P>::store_m(Mb, vr, valid ? 1.f : 0.f, hi, lo, xo);
+        else TCStore<P>::store_m(Mb, vr, valid ? 1.f : 0.f, hi, lo, xo);
+      }
+      asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+      sync();
+      if (tid == 0) {
+        asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+        const uint32_t steps = (cnt + kStep - 1) / kStep;
+        for (uint32_t j = 0; j < steps; ++j) {
+          const uint32_t off = j * 32;
+          const uint64_t ah = desc_sw128(smem_u32(a_hi) + off), al = desc_sw128(smem_u32(a_lo) + off);
+          const uint64_t bh = desc_sw128(smem_u32(b_hi) + off), bl = desc_sw128(smem_u32(b_lo) + off);
+          const uint32_t acc = (!first || j != 0) ? 1u : 0u;
+          if constexpr (kBF) {
+            mma_bf16(tmem, ah, bh, IDESC, acc);
+            mma_bf16(tmem, ah, bl, IDESC, 1u);
+            mma_bf16(tmem, al, bh, IDESC, 1u);
+          } else {
+            mma_tf32(tmem, ah, bh, IDESC, acc);
+            mma_tf32(tmem, ah, bl, IDESC, 1u);
+            mma_tf32(tmem, al, bh, IDESC, 1u);
+          }
+        }
+        mma_commit(mb);
+      }
+      c0 = c1;
+      c1 = after(c1);
+      e = e1;
+      if (c0.si < ns) {
+        ca = cell[sinks[c0.si]];
+        cb = cell[pair_src(e)];
+      }
+      e1 = entry(c1);
+      const bool ok = mbar_wait(mb, phase, chunk_wait);
+      phase ^= 1u;
+      if (!ok && lane == 0) {
+        atomicExch(status, 1);
+        abort_flag = 1;
+      }
+      sync();
       if (abort_flag) break;
+      asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+      first = c0.si != si;
+      if (!first) continue;  // more chunks of this sink
       // ---- TMEM rows 32 warp + lane hold P[c][0..NCP); stage rows c < NC
       const int c = warp * 32 + lane;
       if (warp * 32 < NC) {
@@ -306,7 +326,7 @@ __global__ void __launch_bounds__(kThreads, 1)
         const unsigned quad = 0xfu << (lane & 28);
         acc += __shfl_xor_sync(quad, acc, 1);
         acc += __shfl_xor_sync(quad, acc, 2);
-        if ((o & 3) == 0) L[(size_t)sink * ldm + n] += acc;
+        if ((o & 3) == 0) atomicAdd(L + (size_t)sinks[si] * ldm + n, acc);  // no other warp does
       }
       sync();  // the operand tiles are rewritten
       asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
@@ -336,7 +356,7 @@ cudaError_t launch_tc(Ctx &c, cudaStream_t st) {
   if ((e = cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev)) != cudaSuccess) return e;
   const unsigned grid = std::min((unsigned)nsm, blocks_for((size_t)c.nnodes, kSinkBatch));  // persistent
   const float inv_rs = (float)(c.prm.box / (double)kHalfBox / c.rs);
-  k_m2l_tc<P, kBF><<<grid, kThreads, smem, st>>>(
+  k_m2l_tc<P, kBF><<<grid, 128 * workers_of(P), smem, st>>>(
       c.nnodes, hfmm::P<uint4>(c.cell), hfmm::P<uint32_t>(c.m2l_beg), hfmm::P<uint32_t>(c.m2l_end),
       hfmm::P<uint64_t>(c.m2l), hfmm::P<float>(c.M), hfmm::P<float>(c.L), c.ldm, inv_rs, ctr, status,
       c.prm.tc_wait_polls > 0 ? (uint32_t)c.prm.tc_wait_polls : c.prm.tc_wait_polls < 0 ? 0u : kWaitLimit);
