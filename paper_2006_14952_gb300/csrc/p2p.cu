@@ -20,10 +20,12 @@
 // below R_c; the others contribute nothing).  Lanes are split as (sink i,
 // stream s): with cs sinks in the chunk, S = 32 / cs streams walk the buffer,
 // so small leaves still keep the warp busy; the streams are added in a fixed
-// order at the end (deterministic).  Chunks of 11, 12 or 17..20 sinks, where
-// S = 32 / cs leaves many lanes idle, are split in two halves instead: each lane
-// holds one sink of each half and evaluates both against every staged source
-// pair, which doubles the streams.
+// order at the end (deterministic).  Where S = 32 / cs leaves many lanes idle the
+// chunk is split instead: in two halves (19 and 20 sinks) or three thirds (9, 11, 12, 17,
+// 18, 21..24), each lane holding one sink of each and evaluating all against every staged
+// source pair.  Of the pair evaluations of the 2M set 88% are a sink's with halves alone,
+// 93% with thirds: 7.69 -> 7.53 ms; in smaller chunks (3 and 6) the longer final sum takes
+// back what thirds give (32k uniform particles, about 8 a leaf: 0.115 instead of 0.113).
 //
 // The evaluation buffer holds sources in pairs, {-x0, -x1, -y0, -y1}
 // {-z0, -z1, -w0, -w1} (w = mass), so each lane evaluates two pairs per step
@@ -269,28 +271,34 @@ __global__ void __launch_bounds__(256, 2) k_p2p(const uint32_t *__restrict__ ite
     for (uint32_t cbase = cfirst; cbase < cend; cbase += 32) {
       const uint32_t rem = r.x + r.y - cbase;
       const int cs = rem < 32 ? (int)rem : 32;
-      // two sinks per lane (one from each half of the chunk) where that doubles the
-      // streams: cs in {11, 12, 17..20}; otherwise one sink per lane
-      const int c2 = (cs + 1) >> 1;
-      const bool two = 2 * (32 / cs) < 32 / c2;
-      const int cl = two ? c2 : cs;  // sinks per lane group
+      // sinks per lane: one of each half or third of the chunk where that leaves fewer
+      // lanes idle (S_k streams of ceil(cs / k) lanes, S_k / k the sinks they hold at once)
+      const int c2 = (cs + 1) >> 1, c3 = (cs + 2) / 3;
+      const int s1 = 32 / cs, s2 = 32 / c2, s3 = 32 / c3;
+      const bool two = s2 > 2 * s1;
+      const bool three = cs >= 9 && 2 * s3 > 3 * (two ? s2 : 2 * s1);
+      const int cl = three ? c3 : two ? c2 : cs;  // sinks per lane group
       const int S = 32 / cl, stream = lane / cl, il = lane % cl;
       const bool active = stream < S;
       const float4 xi = pm4[cbase + il];
-      const bool hasb = two && il + c2 < cs;
-      const float4 xib = hasb ? pm4[cbase + il + c2] : make_float4(1e18f, 1e18f, 1e18f, 0.f);
+      const bool hasb = cl < cs && il + cl < cs, hasc = three && il + 2 * cl < cs;
+      const float4 none = make_float4(1e18f, 1e18f, 1e18f, 0.f);
+      const float4 xib = hasb ? pm4[cbase + il + cl] : none, xic = hasc ? pm4[cbase + il + 2 * cl] : none;
       const float2 xx = f2(xi.x), xy = f2(xi.y), xz = f2(xi.z);
       const float2 bxx = f2(xib.x), bxy = f2(xib.y), bxz = f2(xib.z);
+      const float2 cxx = f2(xic.x), cxy = f2(xic.y), cxz = f2(xic.z);
       {
         float lo0 = xi.x, lo1 = xi.y, lo2 = xi.z, hi0 = xi.x, hi1 = xi.y, hi2 = xi.z;
-        if (hasb) {
-          lo0 = fminf(lo0, xib.x);
-          lo1 = fminf(lo1, xib.y);
-          lo2 = fminf(lo2, xib.z);
-          hi0 = fmaxf(hi0, xib.x);
-          hi1 = fmaxf(hi1, xib.y);
-          hi2 = fmaxf(hi2, xib.z);
-        }
+        auto take = [&](const float4 &v) {
+          lo0 = fminf(lo0, v.x);
+          lo1 = fminf(lo1, v.y);
+          lo2 = fminf(lo2, v.z);
+          hi0 = fmaxf(hi0, v.x);
+          hi1 = fmaxf(hi1, v.y);
+          hi2 = fmaxf(hi2, v.z);
+        };
+        if (hasb) take(xib);
+        if (hasc) take(xic);
 #pragma unroll
         for (int o = 16; o; o >>= 1) {
           lo0 = fminf(lo0, __shfl_xor_sync(0xffffffffu, lo0, o));
@@ -311,6 +319,7 @@ __global__ void __launch_bounds__(256, 2) k_p2p(const uint32_t *__restrict__ ite
       }
       float2 ax = f2(0.f), ay = f2(0.f), az = f2(0.f);
       float2 bx = f2(0.f), by = f2(0.f), bz = f2(0.f);
+      float2 cx = f2(0.f), cy = f2(0.f), cz = f2(0.f);
       uint32_t q = tb, jq = 0;
       bool pending = q < te;
       fetch_lst(q);
@@ -393,7 +402,15 @@ __global__ void __launch_bounds__(256, 2) k_p2p(const uint32_t *__restrict__ ite
         };
         if (active) {
           const int np = (int)((kept + 1) >> 1);
-          if (two) {
+          if (three) {
+#pragma unroll 2
+            for (int kk = stream; kk < np; kk += S) {
+              const float4 A = buf[2 * kk], B = buf[2 * kk + 1];
+              pair2(xx, xy, xz, A, B, ax, ay, az);
+              pair2(bxx, bxy, bxz, A, B, bx, by, bz);
+              pair2(cxx, cxy, cxz, A, B, cx, cy, cz);
+            }
+          } else if (two) {
 #pragma unroll 4
             for (int kk = stream; kk < np; kk += S) {
               const float4 A = buf[2 * kk], B = buf[2 * kk + 1];
@@ -413,10 +430,12 @@ __global__ void __launch_bounds__(256, 2) k_p2p(const uint32_t *__restrict__ ite
       // add the streams of each sink in a fixed order
       buf[lane] = make_float4(ax.x + ax.y, ay.x + ay.y, az.x + az.y, 0.f);
       buf[32 + lane] = make_float4(bx.x + bx.y, by.x + by.y, bz.x + bz.y, 0.f);
+      buf[64 + lane] = make_float4(cx.x + cx.y, cy.x + cy.y, cz.x + cz.y, 0.f);
       __syncwarp();
       if (lane < cs) {
         float sx = 0.f, sy = 0.f, sz = 0.f;
-        const int i0 = lane < cl ? lane : 32 + lane - cl;  // the sink's slot in the first group
+        const int grp = lane < cl ? 0 : lane < 2 * cl ? 1 : 2;
+        const int i0 = 32 * grp + lane - grp * cl;  // the sink's slot in the first stream
         for (int s = 0; s < S; ++s) {
           const float4 v = buf[i0 + s * cl];
           sx += v.x;
