@@ -184,7 +184,7 @@ namespace {
 template <class F>
 void for_each_buffer(Ctx &c, F f) {
   DBuf *bufs[] = {&c.key, &c.key_alt, &c.idx, &c.idx_alt, &c.xs, &c.pm4, &c.perm, &c.cell, &c.range, &c.kids,
-                  &c.leaves, &c.lev, &c.lcnt, &c.offs, &c.wnode, &c.wqueue, &c.wspill, &c.obeg, &c.ocnt, &c.open, &c.openc,
+                  &c.leaves, &c.lev, &c.lcnt, &c.offs, &c.wnode, &c.wfeat, &c.wqueue, &c.wspill, &c.obeg, &c.ocnt, &c.open, &c.openc,
                   &c.m2l, &c.m2l_alt, &c.p2p, &c.p2p_alt, &c.m2l_beg, &c.m2l_end, &c.p2p_beg, &c.p2p_end, &c.M,
                   &c.L, &c.tmp, &c.tmp2, &c.d_small, &c.hpos, &c.hmass, &c.hacc, &c.m2l_mid, &c.tab,
                   &c.mlp_w, &c.cand, &c.mlp_scratch, &c.tstate,

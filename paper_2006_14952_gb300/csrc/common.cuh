@@ -326,7 +326,7 @@ struct Ctx {
   uint64_t cap_nodes = 0;
 
   // traversal: node records, each node's parent's open list, open lists
-  DBuf wnode, wqueue, wspill, obeg, ocnt, open, openc;
+  DBuf wnode, wfeat, wqueue, wspill, obeg, ocnt, open, openc;
   DBuf offs;               // scan scratch
   int64_t frontier_items = 0;
   DBuf m2l, m2l_alt, p2p, p2p_alt;  // packed u64 entries

@@ -151,17 +151,15 @@ __device__ __forceinline__ void mlp_argmax16(const float (&l)[4], int &cls_g, in
 // 6 (level_A - level_B)/8, 7 log2(1+n_A)/16, 8 log2(1+n_B)/16,
 // 9 |dipole of B| / |monopole|, 10 |quadrupole of B| / |monopole| (scaled
 // multipoles M~ = M / h^|m|), 11 S_c/R_c.
-__device__ __forceinline__ void pair_features(uint4 ca, uint4 cb, uint32_t s, uint32_t na, uint32_t nb,
-                                              const float *__restrict__ Mb, float inv_rs_h, float inv_rc_h,
-                                              float *f) {
-  int64_t dd[3];
-  half_delta(ca, cb, s, dd);
-  const int64_t wa = half_width(ca.w), wb = half_width(cb.w), ext = wa + wb;
+// Those of the pair's geometry, from the source's centre less the sink's (half units).
+__device__ __forceinline__ void pair_shape_features(const int (&dd)[3], uint32_t la, uint32_t lb, float inv_rs_h,
+                                                    float inv_rc_h, float *f) {
+  const int wa = 1 << (kDepth - la), wb = 1 << (kDepth - lb), ext = wa + wb;
   float sc2 = 0.f, sm2 = 0.f, sx2 = 0.f;
 #pragma unroll
   for (int d = 0; d < 3; ++d) {
-    const int64_t a = dd[d] < 0 ? -dd[d] : dd[d];
-    const int64_t gp = a - ext > 0 ? a - ext : 0;
+    const int a = dd[d] < 0 ? -dd[d] : dd[d];
+    const int gp = a - ext > 0 ? a - ext : 0;
     const float fa = (float)a, fg = (float)gp, fx = (float)(a + ext);
     sc2 += fa * fa;
     sm2 += fg * fg;
@@ -176,16 +174,30 @@ __device__ __forceinline__ void pair_features(uint4 ca, uint4 cb, uint32_t s, ui
   f[3] = ha * isc;
   f[4] = hb * isc;
   f[5] = fmaxf(ha, hb) * isc;
-  f[6] = ((float)ca.w - (float)cb.w) * 0.125f;
-  f[7] = __log2f(1.f + (float)na) * 0.0625f;
-  f[8] = __log2f(1.f + (float)nb) * 0.0625f;
+  f[6] = ((float)la - (float)lb) * 0.125f;
+  f[11] = sc * inv_rc_h;
+}
+
+// Those of one cell: its particle count (feature 7 or 8) and, as a source, 9 and 10.
+__device__ __forceinline__ void node_features(const float *__restrict__ Mb, uint32_t n, float &count, float &dipole,
+                                              float &quadrupole) {
+  count = __log2f(1.f + (float)n) * 0.0625f;
   const float m0 = fabsf(Mb[0]) + 1e-30f;
-  f[9] = sqrtf(Mb[1] * Mb[1] + Mb[2] * Mb[2] + Mb[3] * Mb[3]) / m0;
+  dipole = sqrtf(Mb[1] * Mb[1] + Mb[2] * Mb[2] + Mb[3] * Mb[3]) / m0;
   float q2 = 0.f;
 #pragma unroll
   for (int c = 4; c < 10; ++c) q2 += Mb[c] * Mb[c];
-  f[10] = sqrtf(q2) / m0;
-  f[11] = sc * inv_rc_h;
+  quadrupole = sqrtf(q2) / m0;
+}
+
+__device__ __forceinline__ void pair_features(uint4 ca, uint4 cb, uint32_t s, uint32_t na, uint32_t nb,
+                                              const float *__restrict__ Mb, float inv_rs_h, float inv_rc_h,
+                                              float *f) {
+  int dd[3];
+  half_delta32(ca, cb, s, dd);
+  pair_shape_features(dd, ca.w, cb.w, inv_rs_h, inv_rc_h, f);
+  f[7] = __log2f(1.f + (float)na) * 0.0625f;
+  node_features(Mb, nb, f[8], f[9], f[10]);
 }
 
 }  // namespace hfmm

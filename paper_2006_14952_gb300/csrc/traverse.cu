@@ -184,6 +184,7 @@ struct WalkArgs {
   const uint32_t *leaves;
   const TreeState *tree;
   uint4 *wn;                             // node records
+  uint2 *wf;                             // network: per node its features as BF16 (count, dipole; quadrupole)
   uint32_t *obeg, *ocnt;                 // per node: its parent's open list
   uint32_t *open;                        // open lists: (node to visit or its first child) << 5 | shift
   uint8_t *openc;                        //   and how many nodes from there
@@ -266,12 +267,8 @@ __device__ __forceinline__ void walk_sink(const WalkArgs &A, const Mac &m, const
   const float wa = (float)(1 << (kDepth - a.lev));
   uint32_t *spill_p = spill, *spill_m = spill + kSpillP;
   uint8_t *saux_p = reinterpret_cast<uint8_t *>(spill + kSpillP + kSpillM), *saux_m = saux_p + kSpillP;
-  uint4 ca = make_uint4(0, 0, 0, 0);
-  uint32_t na = 0;
-  if (kNet) {
-    ca = A.cell[sink];
-    na = m.range[sink].y;
-  }
+  uint32_t fa = 0;  // the sink's count feature
+  if (kNet) fa = A.wf[sink].x & 0xffffu;
   unsigned long long base_m = 0, base_p = 0;
   bool fit_m = false, fit_p = false;
   uint32_t cm = 0, cp = 0;  // M2L entries; P2P entries of a leaf, open entries of a cell with children
@@ -349,11 +346,20 @@ __device__ __forceinline__ void walk_sink(const WalkArgs &A, const Mac &m, const
           if (va[0]) {
             __nv_bfloat16 *row = xs + lane * 16;
             float ft[kMlpIn];
-            pair_features(ca, A.cell[src], s, na, m.range[src].y, m.M + (size_t)src * m.ldm, m.inv_rs_h, m.inv_rc_h,
-                          ft);
-            uint32_t w[8] = {0u, 0u, 0u, 0u, 0u, 0u, 0u, 0u};
+            const Node nb = unpack_node(rec[0]);
+            const uint32_t s9 = (s * 57u) >> 9, s3 = (s * 11u) >> 5;  // s / 9, s / 3
+            const int dd[3] = {nb.x - a.x + ((int)s9 - 1) * (int)kHalfBox,
+                               nb.y - a.y + ((int)(s3 - 3u * s9) - 1) * (int)kHalfBox,
+                               nb.z - a.z + ((int)(s - 3u * s3) - 1) * (int)kHalfBox};
+            pair_shape_features(dd, a.lev, nb.lev, m.inv_rs_h, m.inv_rc_h, ft);
+            const uint2 fb = A.wf[src];
+            uint32_t w[8];
 #pragma unroll
-            for (int k = 0; k < kMlpIn / 2; ++k) w[k] = pack_bf16(ft[2 * k], ft[2 * k + 1]);
+            for (int k = 0; k < 3; ++k) w[k] = pack_bf16(ft[2 * k], ft[2 * k + 1]);
+            w[3] = (pack_bf16(ft[6], 0.f) & 0xffffu) | fa << 16;
+            w[4] = fb.x;
+            w[5] = (fb.y & 0xffffu) | pack_bf16(0.f, ft[11]);
+            w[6] = w[7] = 0u;
             reinterpret_cast<uint4 *>(row)[0] = make_uint4(w[0], w[1], w[2], w[3]);
             reinterpret_cast<uint4 *>(row)[1] = make_uint4(w[4], w[5], w[6], w[7]);
           } else {
@@ -587,7 +593,7 @@ __device__ __forceinline__ void walk_sink(const WalkArgs &A, const Mac &m, const
 // a level and 31 warp instructions a pair, and left each sink's entries in
 // pieces that were sorted and copied together.  Walk and lists, ms, before and
 // now: 0.21 -> 0.05 (1k uniform, leaf 16), 0.41 -> 0.08 (32k uniform), 0.86 ->
-// 0.21 (262k clustered, leaf 48), 3.07 -> 1.12 (2M clustered), 6.7 -> 4.5 (2M with
+// 0.21 (262k clustered, leaf 48), 3.07 -> 1.12 (2M clustered), 6.7 -> 3.6 (2M with
 // the network).  A warp a session instead of a block, with the leaves in the same
 // queue: 1.08 at 2M, but 0.14 at 32k and 0.41 at 262k.
 template <bool kNet>
@@ -612,6 +618,11 @@ __global__ void __launch_bounds__(kTT, kNet ? 3 : 4) k_walk(const __grid_constan
   for (long long k = gt; k < nn; k += nt) {
     if (A.what != kWalkLeaves) {
       A.wn[k] = pack_node(A.cell[k], A.kids[k]);
+      if (kNet) {  // once a node, not a pair (ten scattered loads, two roots, two divisions): 2M walk 4.2 -> 3.6 ms
+        float count, dipole, quadrupole;
+        node_features(m.M + (size_t)k * m.ldm, m.range[k].y, count, dipole, quadrupole);
+        A.wf[k] = make_uint2(pack_bf16(count, dipole), pack_bf16(quadrupole, 0.f));
+      }
       A.ocnt[k] = 0u;
       A.obeg[k] = 0u;
       A.queue[k] = k == 0 && nn > 1 ? 1u : 0u;  // the root is there, if it has children
@@ -830,6 +841,7 @@ cudaError_t walk_buffers(Ctx &c, const WalkPlan &w) {
   } while (0)
   const size_t nn = (size_t)(c.nnodes > 0 ? c.nnodes : 1);
   TRY(ensure(c.wnode, nn * sizeof(uint4)));
+  if (w.m.mode == 1) TRY(ensure(c.wfeat, nn * sizeof(uint2)));
   TRY(ensure(c.wqueue, nn * 4));
   TRY(ensure(c.wspill, (size_t)w.nb * kTW * kSpillBytes));
   TRY(ensure(c.obeg, nn * 4));
@@ -870,6 +882,7 @@ cudaError_t walk_launch(Ctx &c, const WalkPlan &w, cudaStream_t st, const WalkPa
   A.leaves = P<uint32_t>(c.leaves);
   A.tree = P<TreeState>(c.tstate);
   A.wn = P<uint4>(c.wnode);
+  A.wf = P<uint2>(c.wfeat);
   A.obeg = P<uint32_t>(c.obeg);
   A.ocnt = P<uint32_t>(c.ocnt);
   A.open = P<uint32_t>(c.open);
