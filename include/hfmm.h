@@ -95,8 +95,8 @@ typedef struct {
   int tile_m2l_blocks; /* cap on M2L blocks of 128 threads, per SM, 1..64 (default 64) */
   int tile_trav_blocks;/* traversal blocks of 256 threads per SM, 1..4 (default 4; capped by occupancy) */
   int use_graph;       /* 1 = hfmm_short_range_forces runs as one CUDA graph (captured on a library
-                          stream, launched on the caller's): upward pass, the walk, list grouping,
-                          M2L, L2L/L2P and P2P, with no host read-back inside; the lists take their
+                          stream, launched on the caller's): upward pass, the walk, M2L,
+                          L2L/L2P and P2P, with no host read-back inside; the lists take their
                           capacities from the last call (or the first guess), their sizes stay on
                           the device, and one read-back after the graph checks them: if a list
                           overflowed, the call runs again directly (growing the lists), so the
@@ -129,7 +129,7 @@ typedef struct {
                           Needs mac_mode 0 and size_rule 1 (the walk is then symmetric); ignores
                           use_graph.  The partials take 12 bytes per (entry, source particle). */
   int list_init;       /* initial capacity, in entries, of every traversal list (open lists, M2L, P2P;
-                          k-d tree: frontier) of a new context: 0 = a guess scaled with n and leaf_max;
+                          k-d tree too) of a new context: 0 = a guess scaled with n and leaf_max;
                           a small value makes the walk overflow and repeat with grown lists (the
                           lists come out the same either way) */
   int sink_batches;    /* hfmm_short_range_forces in batches of sinks (0 = automatic: one batch
@@ -151,9 +151,9 @@ typedef struct {
                           centre, the rules of Sec. 2.3 on the boxes in FP64 (S_c between the centres,
                           S_m and S_max from per-axis gaps and spans, side = largest extent; a pair with
                           theta S_c = 0 is never accepted), the walk opening the node of larger side.
-                          hfmm_build_tree synchronises `stream` once (the level extents); the walk is
+                          hfmm_build_tree synchronises `stream` once; the walk is
                           one cooperative launch, followed by one read-back (repeated with grown
-                          buffers when a list or the frontier outgrew its buffer).  Needs mac_mode 0,
+                          buffers when a list outgrew its buffer).  Needs mac_mode 0,
                           m2l_precision 0, m2l_tables 0, p2p_mutual 0 and order <= 6 (either split);
                           use_graph and sink_batches are ignored, and
                           HFMM_EXPORT_KEYS and HFMM_EXPORT_NODES are octree only
@@ -208,7 +208,7 @@ const char *hfmm_last_error(const hfmm_ctx *ctx);
  * (depth cap 21), per-particle FP32 offsets from the geometric leaf centre.
  * pos_soa: device FP64 [3][n], finite values (any finite position is wrapped;
  * a NaN or infinite coordinate is not checked and lands in an arbitrary cell);
- * mass: device FP32 [n]; n >= 0 (n = 0 gives an empty tree).  The levels are built in one cooperative launch; `stream` is
+ * mass: device FP32 [n]; n >= 0 (n = 0 gives an empty tree).  `stream` is
  * synchronised once to read the node and level counts back (again if the node
  * capacity had to grow).  The library keeps no reference to pos/mass after the
  * call returns.

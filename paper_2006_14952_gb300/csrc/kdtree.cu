@@ -1017,8 +1017,10 @@ cudaError_t kd_build_tree(Ctx &c, const double *pos, const float *mass, int64_t 
                                     P<uint32_t>(c.idx), P<float4>(c.pm4));
   note_launch();
   if (c.prm.profile & 1) cudaEventRecord(c.ev[2], st);
+  TRY(cudaGetLastError());
+  TRY(cudaStreamSynchronize(st));  // the caller's positions and masses have been read when the call returns
   c.have_tree = true;
-  return cudaGetLastError();
+  return cudaSuccess;
 }
 
 cudaError_t kd_interaction_counts(Ctx &c, bool conventional, int64_t *out, cudaStream_t st) {
