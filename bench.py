@@ -494,7 +494,7 @@ def main():
         flops = st["p2p_useful_pairs"] * fpp
         achieved = flops / (mean["t_p2p"] / 1e3) / 1e12
         kd_main = args.tree == "kd"
-        roof = {"kernel": "k_kd_p2p (cut-off P2P on the k-d tree)" if kd_main else "k_p2p (cut-off P2P)",
+        roof = {"kernel": "k_p2p (cut-off P2P on the k-d tree)" if kd_main else "k_p2p (cut-off P2P)",
                 "bound": "alu", "achieved": achieved, "peak": peak_fp32,
                 "unit": "TFLOP/s", "frac": achieved / peak_fp32,
                 "traffic": measured_traffic("k_p2p", "p2p.cu") if args.split == "gauss" and not kd_main else None,
@@ -558,7 +558,7 @@ def main():
                   "accuracy": None,
                   "ratio_over_octree": (whole_job_rate(ws, n, args.steps, k_tot / 1e3) / value),
                   "breakdown_ms": kmean, "launches_per_step": k_launch / args.steps,
-                  "roofline": {"kernel": "k_kd_p2p (cut-off P2P on the k-d tree)", "bound": "alu",
+                  "roofline": {"kernel": "k_p2p (cut-off P2P on the k-d tree)", "bound": "alu",
                                "achieved": k_ach, "peak": peak_fp32, "unit": "TFLOP/s",
                                "frac": k_ach / peak_fp32, "traffic": None,
                                "algorithmic": f"{kcnt['p2p_useful_pairs']} pairs inside R_c x "
