@@ -28,7 +28,16 @@ __global__ void k_keys(const double *__restrict__ pos, int64_t n, double box, do
 }
 
 constexpr int kLT = 256;        // threads of the level kernels
-constexpr int kLTile = 1024;    // particles per tile
+// Particles per tile: four rounds of the block, or one while the larger tiles would not fill
+// the GPU: a block's rounds are a chain of ballots and dependent loads.  k_levels and k_nodes
+// with 1024 and with 256, us: 7.1, 14.6 -> 4.6, 6.0 (1000 particles), 7.4, 14.7 -> 4.6, 6.3 (32k),
+// 7.5, 17.5 -> 5.1, 8.8 (100k; the scan over more tiles 4.5 -> 7.9).
+constexpr int kLTileMost = 1024, kLTileSmall = kLT;
+inline bool small_tiles(int64_t n) { return n <= 152 * (int64_t)kLTileMost; }
+inline int64_t level_tiles(int64_t n) {
+  const int64_t tile = small_tiles(n) ? kLTileSmall : kLTileMost;
+  return (n + tile - 1) / tile;
+}
 constexpr int kHalo = 64;       // leaf_max is at most 64
 constexpr int kLCnt = 2 * (kDepth + 1);  // counters per tile: nodes by level, leaves by level
 
@@ -41,6 +50,7 @@ __device__ __forceinline__ int common_level(uint64_t a, uint64_t b) {
 // lev[i]: the first level particle i starts a cell on (low byte), the level of its
 // leaf (high byte); it starts the nodes of the levels from the first to the second.
 // cnt[c][tile]: nodes (c < 22) and leaves (c - 22) by level that start in the tile.
+template <int kLTile>
 __global__ void __launch_bounds__(kLT) k_levels(const uint64_t *__restrict__ key, int64_t n, int leaf_max,
                                                 uint16_t *__restrict__ lev, uint32_t *__restrict__ cnt,
                                                 int64_t ntiles) {
@@ -163,6 +173,7 @@ __device__ __forceinline__ uint32_t pack3(uint64_t v) {
 // and FP64 offset from the leaf's geometric centre, rounded once to FP32 (the cell
 // side L 2^-level built from its bits: no FP64 division).  Cells that split get
 // their first child here, their particle and child counts from k_node_counts.
+template <int kLTile>
 __global__ void __launch_bounds__(kLT) k_nodes(const uint64_t *__restrict__ key, const uint16_t *__restrict__ lev,
                                                int64_t n, int leaf_max, const uint32_t *__restrict__ cnt,
                                                const uint32_t *__restrict__ base, int64_t ntiles,
@@ -290,7 +301,7 @@ __global__ void k_node_counts(const uint64_t *__restrict__ key, int64_t n, int l
 // Buffers of the levels for n particles and the node capacity.
 cudaError_t level_buffers(Ctx &c, int64_t n) {
   cudaError_t e;
-  const int64_t ntiles = (n + kLTile - 1) / kLTile;
+  const int64_t ntiles = level_tiles(n);
   const size_t capN = (size_t)c.cap_nodes;
   if ((e = ensure(c.lev, (size_t)n * 2)) != cudaSuccess) return e;
   if ((e = ensure(c.lcnt, (size_t)(ntiles + 1) * kLCnt * 4)) != cudaSuccess) return e;
@@ -307,18 +318,19 @@ cudaError_t level_buffers(Ctx &c, int64_t n) {
 // below 10^5 particles, four launches.  The level-synchronous build it replaced
 // (one cooperative launch, three grid barriers a level, then a thread a leaf for
 // the offsets), ms with its read-back, before and now: 0.54 -> 0.18 at 2M, 1.67 ->
-// 1.07 at 16M, 0.32 -> 0.06 at 262k, 0.17 -> 0.05 at 32k, 0.10 -> 0.05 at 1000.
+// 1.07 at 16M, 0.32 -> 0.06 at 262k, 0.17 -> 0.04 at 32k, 0.10 -> 0.03 at 1000.
 cudaError_t levels_launch(Ctx &c, const double *pos, const float *mass, int64_t n, int max_levels, cudaStream_t st) {
-  const int64_t ntiles = (n + kLTile - 1) / kLTile;
+  const int64_t ntiles = level_tiles(n);
+  const bool small = small_tiles(n);
   uint32_t *base = P<uint32_t>(c.lcnt), *cnt = base + kLCnt;
   TreeState *ts = P<TreeState>(c.tstate);
   const uint64_t *key = P<uint64_t>(c.key);
-  k_levels<<<(unsigned)ntiles, kLT, 0, st>>>(key, n, c.prm.leaf_max, P<uint16_t>(c.lev), cnt, ntiles);
+  (small ? k_levels<kLTileSmall> : k_levels<kLTileMost>)<<<(unsigned)ntiles, kLT, 0, st>>>(key, n, c.prm.leaf_max, P<uint16_t>(c.lev), cnt, ntiles);
   k_level_scan<<<1, 1024, 0, st>>>(cnt, ntiles, base, c.cap_nodes, max_levels, ts);
-  k_nodes<<<(unsigned)ntiles, kLT, 0, st>>>(key, P<uint16_t>(c.lev), n, c.prm.leaf_max, cnt, base, ntiles, ts,
-                                            P<uint4>(c.cell), P<uint2>(c.range), P<int2>(c.kids),
-                                            P<uint32_t>(c.leaves), pos, mass, P<uint32_t>(c.idx), c.prm.box,
-                                            box_inverse_if_pow2(c.prm.box), P<double>(c.xs), P<float4>(c.pm4));
+  (small ? k_nodes<kLTileSmall> : k_nodes<kLTileMost>)<<<(unsigned)ntiles, kLT, 0, st>>>(
+      key, P<uint16_t>(c.lev), n, c.prm.leaf_max, cnt, base, ntiles, ts, P<uint4>(c.cell), P<uint2>(c.range),
+      P<int2>(c.kids), P<uint32_t>(c.leaves), pos, mass, P<uint32_t>(c.idx), c.prm.box,
+      box_inverse_if_pow2(c.prm.box), P<double>(c.xs), P<float4>(c.pm4));
   k_node_counts<<<std::min(blocks_for((size_t)c.cap_nodes, 128), 152u * 16u), 128, 0, st>>>(
       key, n, c.prm.leaf_max, ts, P<uint4>(c.cell), P<uint2>(c.range), P<int2>(c.kids));
   note_launch(4);
