@@ -59,24 +59,32 @@ __global__ void __launch_bounds__(256) k_mlp_infer(const __nv_bfloat16 *__restri
 // atomics and the result does not depend on scheduling.
 //
 // Precision: weights, inputs and activations are BF16 values, so the forward
-// products are exact in FP32.  The backward operands d = dLoss/dz are FP32; each
-// is split exactly into three BF16 terms (8 + 8 + 8 significant bits), three MMAs
-// whose products are again exact in FP32.  The tensor cores do not round their
-// accumulator to nearest: chained over all of a block's tiles the gradients came
-// out 2.4e-6 from the FP64 ones (3e-7 in FP32 arithmetic), and chained over a
-// layer's 64 inputs the bias of the logits alone moved them by 1e-6.  So every
-// MMA group sums 16 terms from zero, and the groups are added in FP32.
+// products are exact in FP32; their sums are not, and the tensor cores do not
+// round a sum to nearest.  In the first layer that moved one activation in some
+// 3e5 across a BF16 rounding boundary (2^-8 of it), and through it a second-layer
+// pre-activation near zero across zero: the sample's rows of the gradient change,
+// and in a quarter of the batches of 400k samples the gradient was 7e-7 to 1.5e-6
+// from the FP64 one instead of at most 1.3e-7.  So the first layer is FP32 FMAs,
+// the bias first and the inputs in order, and a second-layer sum too close to zero
+// for its sign to be certain is formed again in the same way (gate_bound).
+// The backward operands d = dLoss/dz are FP32; each is split exactly into three
+// BF16 terms (8 + 8 + 8 significant bits), three MMAs whose products are again exact
+// in FP32.  Chained over all of a block's tiles the gradients came out 2.4e-6 from
+// the FP64 ones, so every MMA group sums 16 terms from zero, and the groups are
+// added in FP32.
 //
-// The sample tile of 64 (16 rows a warp) keeps the staged operands within 73 KB,
+// The sample tile of 64 (16 rows a warp) keeps the staged operands within 76 KB,
 // so that three blocks share an SM: 12 warps cover the latency of the staging.
-// Measured (400k samples, gradient + Adam step): 14.3 -> 0.15 ms.
+// Measured (400k samples, gradient + Adam step): 14.3 -> 0.18 ms; 0.14 with the first
+// layer on the tensor cores too.
 constexpr int kGradThreads = 128;
 constexpr int kGradTile = 64;
 constexpr int kGradBlocks = 152 * 3;
 constexpr int kLdH = 72, kLdX = 24, kLdO = 8;  // row strides (BF16): 16-byte rows, no bank conflicts
 constexpr int kFragW2T = 4 * 8 * 2 * 32, kFragW3T = 8 * 32;
-// dynamic shared memory: weight images, then the tile's operands
-constexpr int kGradWords = (kMlpSmemWords + 3) / 4 * 4 + kFragW2T + kFragW3T;
+// dynamic shared memory: weight images (W1 as FP32), then the tile's operands
+constexpr int kGradW1 = kMlpH * kMlpIn;
+constexpr int kGradWords = (kMlpSmemWords + 3) / 4 * 4 + kFragW2T + kFragW3T + kGradW1;
 constexpr size_t kGradSmem = (size_t)kGradWords * 4 + (size_t)kGradTile * (5 * kLdH + kLdX + 3 * kLdO) * 2;
 
 // x = hi + mid + lo, each BF16 (exact for finite x above the denormal range), two values per word.
@@ -112,6 +120,17 @@ __device__ __forceinline__ void mma_add(float (&c)[4], const uint32_t (&a)[4], u
   for (int q = 0; q < 4; ++q) c[q] += p[q];
 }
 
+// How far from zero the sign of a row's second-layer sums is certain.  The terms'
+// magnitudes add up to at most `terms` (the bias, and the largest activation times the
+// largest sum of |w| over a unit); an MMA group of 16 that truncates every term to 24 bits
+// below the largest is within 2^-19 of that, with the FP32 additions of the groups within
+// 2^-18.  Some 3000 of a batch's 25.6M sums are closer.  With an infinite activation the sums
+// are infinite or NaN however they are formed: they stay as they are.
+__device__ __forceinline__ float gate_bound(float terms) {
+  const float tol = 0x1p-18f * terms;
+  return tol < 3e38f ? tol : -1.f;
+}
+
 __device__ __forceinline__ void ldsm4t(uint32_t (&r)[4], const __nv_bfloat16 *p) {
   asm volatile("ldmatrix.sync.aligned.m8n8.x4.trans.shared.b16 {%0,%1,%2,%3}, [%4];"
                : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3])
@@ -133,6 +152,7 @@ __global__ void __launch_bounds__(kGradThreads, 3) k_mlp_grad(const float *__res
   extern __shared__ __align__(16) uint32_t gsm[];
   __shared__ float lsum[4];
   uint32_t *sw = gsm, *w2t = gsm + (kMlpSmemWords + 3) / 4 * 4, *w3t = w2t + kFragW2T;
+  float *w1 = reinterpret_cast<float *>(w3t + kFragW3T);
   __nv_bfloat16 *sh1 = reinterpret_cast<__nv_bfloat16 *>(gsm + kGradWords);
   __nv_bfloat16 *sh2 = sh1 + kGradTile * kLdH, *sd = sh2 + kGradTile * kLdH;  // sd: three terms of d2, then of d1
   __nv_bfloat16 *sx = sd + 3 * kGradTile * kLdH, *sd3 = sx + kGradTile * kLdX;
@@ -147,11 +167,32 @@ __global__ void __launch_bounds__(kGradThreads, 3) k_mlp_grad(const float *__res
     const int l = i & 31, nt = i >> 5, o = 2 * (l & 3), k = nt * 8 + (l >> 2);
     w3t[i] = pkw(kOffW3 + o * kMlpH + k, kOffW3 + (o + 1) * kMlpH + k);
   }
+  auto bf = [](float v) { return __bfloat162float(__float2bfloat16_rn(v)); };
+  for (int i = threadIdx.x; i < kGradW1; i += kGradThreads) w1[i] = bf(wm[kOffW1 + i]);
   __syncthreads();
   const int lane = threadIdx.x & 31, wp = threadIdx.x >> 5, g = lane >> 2, t = lane & 3;
   const float *bias = reinterpret_cast<const float *>(sw + kFragL1 + kFragL2 + kFragL3);
   const uint32_t *s2 = sw + kFragL1, *s3 = s2 + kFragL2;
   const int r0 = 16 * wp + g, r8 = r0 + 8;  // this lane's rows of the tile
+  float most_w = 0.f, most_b = 0.f;  // layer 2: the largest sum of |w| over a unit, the largest |bias|
+#pragma unroll 1
+  for (int nt = 0; nt < 8; ++nt) {  // unit 8 nt + g, its row over the quad's lanes
+    float v = 0.f;
+#pragma unroll
+    for (int j = 0; j < 8; ++j) {
+      const uint32_t wv = s2[nt * 256 + 32 * j + lane];
+      v += fabsf(__uint_as_float(wv << 16)) + fabsf(__uint_as_float(wv & 0xffff0000u));
+    }
+    v += __shfl_xor_sync(0xffffffffu, v, 1);
+    v += __shfl_xor_sync(0xffffffffu, v, 2);
+    most_w = fmaxf(most_w, v);
+    most_b = fmaxf(most_b, fabsf(bias[kMlpH + nt * 8 + g]));
+  }
+#pragma unroll
+  for (int o = 4; o < 32; o <<= 1) {
+    most_w = fmaxf(most_w, __shfl_xor_sync(0xffffffffu, most_w, o));
+    most_b = fmaxf(most_b, __shfl_xor_sync(0xffffffffu, most_b, o));
+  }
   // lane addresses of the transposed fragment loads: rows are samples
   const int m = lane >> 3, r = lane & 7;
   const int a_s = (m >> 1) * 8 + r, a_u = (m & 1) * 8;  // A: [k = sample][row = unit]
@@ -190,22 +231,65 @@ __global__ void __launch_bounds__(kGradThreads, 3) k_mlp_grad(const float *__res
     }
     // ---- forward; bits of m1, m2: z > 0 by (n-tile, fragment element)
     uint32_t f[4][4], m1 = 0, m2 = 0;
+    float tol0, tol8;  // of the rows' gates
+    {
+      float x0[kMlpIn], x8[kMlpIn];  // the whole rows, from the quad's lanes
+      __nv_bfloat162 top0 = __float2bfloat162_rn(0.f), top8 = top0;  // the rows' largest activations
 #pragma unroll
-    for (int nt = 0; nt < 8; ++nt) {
-      float c[4] = {0.f, 0.f, 0.f, 0.f};
-      mma_bf16_16816(c, a, sw[(nt * 2 + 0) * 32 + lane], sw[(nt * 2 + 1) * 32 + lane]);
+      for (int j = 0; j < kMlpIn / 2; ++j) {
+        const uint32_t v0 = __shfl_sync(0xffffffffu, j < 4 ? a[0] : a[2], (lane & 28) + (j & 3));
+        const uint32_t v8 = __shfl_sync(0xffffffffu, j < 4 ? a[1] : a[3], (lane & 28) + (j & 3));
+        x0[2 * j] = __uint_as_float(v0 << 16);
+        x0[2 * j + 1] = __uint_as_float(v0 & 0xffff0000u);
+        x8[2 * j] = __uint_as_float(v8 << 16);
+        x8[2 * j + 1] = __uint_as_float(v8 & 0xffff0000u);
+      }
 #pragma unroll
-      for (int q = 0; q < 4; ++q) c[q] += bias[nt * 8 + 2 * t + (q & 1)];
+      for (int nt = 0; nt < 8; ++nt) {
+        float c[4];
 #pragma unroll
-      for (int q = 0; q < 4; ++q) m1 |= (c[q] > 0.f ? 1u : 0u) << (4 * nt + q);
-      const uint32_t lo = pack_bf16(fmaxf(c[0], 0.f), fmaxf(c[1], 0.f));
-      const uint32_t hi = pack_bf16(fmaxf(c[2], 0.f), fmaxf(c[3], 0.f));
-      f[nt >> 1][(nt & 1) * 2 + 0] = lo;
-      f[nt >> 1][(nt & 1) * 2 + 1] = hi;
-      reinterpret_cast<uint32_t *>(sh1 + r0 * kLdH)[nt * 4 + t] = finite_or_zero(lo);
-      reinterpret_cast<uint32_t *>(sh1 + r8 * kLdH)[nt * 4 + t] = finite_or_zero(hi);
+        for (int e = 0; e < 2; ++e) {
+          const int u = nt * 8 + 2 * t + e;
+          const float4 *w4 = reinterpret_cast<const float4 *>(w1 + u * kMlpIn);
+          c[e] = c[2 + e] = bias[u];
+#pragma unroll
+          for (int j = 0; j < kMlpIn / 4; ++j) {
+            const float4 w = w4[j];
+            c[e] = fmaf(w.x, x0[4 * j], c[e]);
+            c[2 + e] = fmaf(w.x, x8[4 * j], c[2 + e]);
+            c[e] = fmaf(w.y, x0[4 * j + 1], c[e]);
+            c[2 + e] = fmaf(w.y, x8[4 * j + 1], c[2 + e]);
+            c[e] = fmaf(w.z, x0[4 * j + 2], c[e]);
+            c[2 + e] = fmaf(w.z, x8[4 * j + 2], c[2 + e]);
+            c[e] = fmaf(w.w, x0[4 * j + 3], c[e]);
+            c[2 + e] = fmaf(w.w, x8[4 * j + 3], c[2 + e]);
+          }
+        }
+#pragma unroll
+        for (int q = 0; q < 4; ++q) {
+          m1 |= (c[q] > 0.f ? 1u : 0u) << (4 * nt + q);
+          c[q] = fmaxf(c[q], 0.f);
+        }
+        const uint32_t lo = pack_bf16(c[0], c[1]), hi = pack_bf16(c[2], c[3]);
+        f[nt >> 1][(nt & 1) * 2 + 0] = lo;
+        f[nt >> 1][(nt & 1) * 2 + 1] = hi;
+        top0 = __hmax2(top0, *reinterpret_cast<const __nv_bfloat162 *>(&lo));
+        top8 = __hmax2(top8, *reinterpret_cast<const __nv_bfloat162 *>(&hi));
+        reinterpret_cast<uint32_t *>(sh1 + r0 * kLdH)[nt * 4 + t] = finite_or_zero(lo);
+        reinterpret_cast<uint32_t *>(sh1 + r8 * kLdH)[nt * 4 + t] = finite_or_zero(hi);
+      }
+      tol0 = fmaxf(__low2float(top0), __high2float(top0));
+      tol8 = fmaxf(__low2float(top8), __high2float(top8));
+#pragma unroll
+      for (int o = 1; o <= 2; o <<= 1) {
+        tol0 = fmaxf(tol0, __shfl_xor_sync(0xffffffffu, tol0, o));
+        tol8 = fmaxf(tol8, __shfl_xor_sync(0xffffffffu, tol8, o));
+      }
+      tol0 = gate_bound(fmaf(most_w, tol0, most_b));
+      tol8 = gate_bound(fmaf(most_w, tol8, most_b));
+      __syncwarp();  // a row of sh1 is its quad's
     }
-    uint32_t h2[4][4];
+    uint32_t h2[4][4], unsure = 0;
 #pragma unroll
     for (int nt = 0; nt < 8; ++nt) {
       float c[4];
@@ -215,6 +299,8 @@ __global__ void __launch_bounds__(kGradThreads, 3) k_mlp_grad(const float *__res
       for (int kt = 0; kt < 4; ++kt)
         mma_add(c, f[kt], s2[((nt * 4 + kt) * 2 + 0) * 32 + lane], s2[((nt * 4 + kt) * 2 + 1) * 32 + lane]);
 #pragma unroll
+      for (int q = 0; q < 4; ++q) unsure |= (fabsf(c[q]) < (q < 2 ? tol0 : tol8) ? 1u : 0u) << (4 * nt + q);
+#pragma unroll
       for (int q = 0; q < 4; ++q) m2 |= (c[q] > 0.f ? 1u : 0u) << (4 * nt + q);
       const uint32_t lo = pack_bf16(fmaxf(c[0], 0.f), fmaxf(c[1], 0.f));
       const uint32_t hi = pack_bf16(fmaxf(c[2], 0.f), fmaxf(c[3], 0.f));
@@ -223,6 +309,28 @@ __global__ void __launch_bounds__(kGradThreads, 3) k_mlp_grad(const float *__res
       reinterpret_cast<uint32_t *>(sh2 + r0 * kLdH)[nt * 4 + t] = lo;
       reinterpret_cast<uint32_t *>(sh2 + r8 * kLdH)[nt * 4 + t] = hi;
     }
+    while (unsure) {  // the sum again in FP32, the bias first and the inputs in order
+      const int at = __ffs(unsure) - 1, nt = at >> 2, q = at & 3, u = nt * 8 + 2 * t + (q & 1), row = q < 2 ? r0 : r8;
+      const uint32_t *h = reinterpret_cast<const uint32_t *>(sh1 + row * kLdH);
+      const uint32_t *w = s2 + nt * 256 + (u & 7) * 4;  // the unit's row: inputs 8 j + 2 i, + 1 in word 32 j + i
+      unsure &= unsure - 1u;
+      float z = bias[kMlpH + u];
+#pragma unroll 1
+      for (int j = 0; j < 8; ++j)
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+          const uint32_t wv = w[32 * j + i], hv = h[4 * j + i];
+          z = fmaf(__uint_as_float(wv << 16), __uint_as_float(hv << 16), z);
+          z = fmaf(__uint_as_float(wv & 0xffff0000u), __uint_as_float(hv & 0xffff0000u), z);
+        }
+      m2 = (m2 & ~(1u << at)) | (z > 0.f ? 1u << at : 0u);
+      uint32_t *pair = reinterpret_cast<uint32_t *>(sh2 + row * kLdH) + nt * 4 + t;
+      const uint32_t other = *pair & ((q & 1) ? 0x0000ffffu : 0xffff0000u);
+      *pair = other | ((q & 1) ? pack_bf16(0.f, fmaxf(z, 0.f)) : pack_bf16(fmaxf(z, 0.f), 0.f));
+#pragma unroll
+      for (int i = 0; i < 16; ++i) h2[i >> 2][i & 3] = i == at >> 1 ? *pair : h2[i >> 2][i & 3];
+    }
+    __syncwarp();
     const float b0 = bias[2 * kMlpH + 2 * t], b1 = bias[2 * kMlpH + 2 * t + 1];
     float z[4] = {b0, b1, b0, b1};
 #pragma unroll
