@@ -538,7 +538,7 @@ cudaError_t step_graph(Ctx &c, double *pos, float *vel, float *acc, double dt, c
   if ((e = ensure(c.M, eb)) != cudaSuccess) return e;
   if ((e = ensure(c.L, eb)) != cudaSuccess) return e;
   if ((e = traverse_graph_prepare(c)) != cudaSuccess) return e;
-  if ((e = pm_prepare(c)) != cudaSuccess) return e;
+  if ((e = pm_prepare(c, st)) != cudaSuccess) return e;
   std::vector<uint64_t> sig = step_signature(c, pos, vel, acc, dt);
   if (!c.gexec_step || sig != c.step_sig) {
     c.nm2l = (int64_t)c.cap_m2l;

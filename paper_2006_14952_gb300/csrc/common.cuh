@@ -222,6 +222,10 @@ struct DBuf {
 // (a stream capture is in progress) the old allocation is queued there instead of freed.
 cudaError_t ensure(DBuf &b, size_t bytes);
 extern thread_local std::vector<void *> *g_deferred_free;
+// A host table to b, in device memory when the call returns: a reader on any stream is
+// ordered after it (a synchronous copy from pageable memory may return before its transfer,
+// and a non-blocking stream does not wait for the stream it runs on).
+cudaError_t upload(DBuf &b, const void *src, size_t bytes, cudaStream_t st);
 // Grow b to at least `bytes`, keeping the first `keep` bytes (stream-ordered copy).
 cudaError_t ensure_keep(DBuf &b, size_t bytes, size_t keep, cudaStream_t st);
 void release(DBuf &b);
@@ -386,7 +390,7 @@ struct Ctx {
   KdTree kd;  // tree = 1
   DBuf pm_win;           // sinc window of one axis by index (PM Green function)
   DBuf pm_gtab;          // polynomial split: long-range Green function per integer |k|^2
-  size_t pm_gtab_n = 0;  // its length (0: not built)
+  size_t pm_gtab_n = 0, pm_win_n = 0;  // their lengths (0: not built)
   int pm_plan_r2c = -1, pm_plan_c2r = -1;
   const float *mass_ref = nullptr;  // the mass array of the last build_tree
 
@@ -448,7 +452,7 @@ int sink_batches_for(const Ctx &c);
 cudaError_t pm_long_range(Ctx &c, float *acc, cudaStream_t st);
 // Graph mode: the mesh buffers, FFT plans and Green-function table, made
 // outside a capture (pm_long_range calls it too).
-cudaError_t pm_prepare(Ctx &c);
+cudaError_t pm_prepare(Ctx &c, cudaStream_t st);
 void pm_release(Ctx &c);
 // A step captured as one graph: the second kick runs only when the tree and the
 // walk fitted their capacities (device flags; null pointers: always).

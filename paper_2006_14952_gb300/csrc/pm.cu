@@ -277,7 +277,7 @@ void pm_release(Ctx &c) {
   release(c.pm_a);
   release(c.pm_gtab);
   release(c.pm_win);
-  c.pm_gtab_n = 0;
+  c.pm_gtab_n = c.pm_win_n = 0;
 }
 
 namespace {
@@ -313,7 +313,7 @@ void gauss_legendre01(int n, std::vector<double> &x, std::vector<double> &w) {
 //   psi^(k) = (4 pi R_c / k) int_0^1 [1 - (15 x - 10 x^3 + 3 x^5) / 8] sin(k R_c x) dx,
 // by a 96-point Gauss-Legendre rule in FP64 (k R_c stays below 10 pi for the
 // meshes allowed, a few oscillations of a smooth integrand).
-cudaError_t green_table_poly(Ctx &c) {
+cudaError_t green_table_poly(Ctx &c, cudaStream_t st) {
   const int ng = c.prm.pm_grid, h = ng / 2;
   const size_t nt = (size_t)3 * h * h + 1;
   if (c.pm_gtab_n == nt) return cudaSuccess;
@@ -330,15 +330,14 @@ cudaError_t green_table_poly(Ctx &c) {
     }
     tab[n] = (float)(4.0 * M_PI / (k * k) - 4.0 * M_PI * rc / k * integ);
   }
-  cudaError_t e = ensure(c.pm_gtab, nt * sizeof(float));
-  if (e == cudaSuccess) e = cudaMemcpy(c.pm_gtab.p, tab.data(), nt * sizeof(float), cudaMemcpyHostToDevice);
+  const cudaError_t e = upload(c.pm_gtab, tab.data(), nt * sizeof(float), st);
   if (e == cudaSuccess) c.pm_gtab_n = nt;
   return e;
 }
 
 }  // namespace
 
-cudaError_t pm_prepare(Ctx &c) {
+cudaError_t pm_prepare(Ctx &c, cudaStream_t st) {
   const int ng = c.prm.pm_grid;
   const int64_t cells = (int64_t)ng * ng * ng, kcells = (int64_t)ng * ng * (ng / 2 + 1);
   cudaError_t e;
@@ -357,16 +356,16 @@ cudaError_t pm_prepare(Ctx &c) {
       return e;
     c.pm_plan_c2r = p;
   }
-  if (!c.pm_win.p) {  // sinc(k_i h / 2) = sinc(pi i / N_g) by axis index (i and N_g - i alike)
+  if (c.pm_win_n != (size_t)ng) {  // sinc(k_i h / 2) = sinc(pi i / N_g) by axis index (i and N_g - i alike)
     std::vector<float> win(ng);
     for (int i = 0; i < ng; ++i) {
       const double x = M_PI * (i <= ng / 2 ? i : ng - i) / ng;
       win[i] = (float)(x > 0 ? std::sin(x) / x : 1.0);
     }
-    if ((e = ensure(c.pm_win, ng * 4)) != cudaSuccess) return e;
-    if ((e = cudaMemcpy(c.pm_win.p, win.data(), ng * 4, cudaMemcpyHostToDevice)) != cudaSuccess) return e;
+    if ((e = upload(c.pm_win, win.data(), (size_t)ng * 4, st)) != cudaSuccess) return e;
+    c.pm_win_n = (size_t)ng;
   }
-  if (c.prm.split == 1 && (e = green_table_poly(c)) != cudaSuccess) return e;
+  if (c.prm.split == 1 && (e = green_table_poly(c, st)) != cudaSuccess) return e;
   return cudaSuccess;
 }
 
@@ -375,7 +374,7 @@ cudaError_t pm_long_range(Ctx &c, float *acc, cudaStream_t st) {
   const int ng = c.prm.pm_grid;
   const int64_t cells = (int64_t)ng * ng * ng, kcells = (int64_t)ng * ng * (ng / 2 + 1);
   cudaError_t e;
-  if ((e = pm_prepare(c)) != cudaSuccess) return e;
+  if ((e = pm_prepare(c, st)) != cudaSuccess) return e;
   if ((e = fft_error(cufftSetStream(c.pm_plan_r2c, st))) != cudaSuccess) return e;
   if ((e = fft_error(cufftSetStream(c.pm_plan_c2r, st))) != cudaSuccess) return e;
 

@@ -56,6 +56,12 @@ cudaError_t ensure_keep(DBuf &b, size_t bytes, size_t keep, cudaStream_t st) {
   return cudaSuccess;
 }
 
+cudaError_t upload(DBuf &b, const void *src, size_t bytes, cudaStream_t st) {
+  cudaError_t e = ensure(b, bytes);
+  if (e == cudaSuccess) e = cudaMemcpyAsync(b.p, src, bytes, cudaMemcpyHostToDevice, st);
+  return e == cudaSuccess ? cudaStreamSynchronize(st) : e;
+}
+
 void release(DBuf &b) {
   if (b.p) cudaFree(b.p);
   b.p = nullptr;
