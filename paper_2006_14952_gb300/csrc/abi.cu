@@ -928,8 +928,7 @@ int hfmm_load_mlp(hfmm_ctx *h, const void *weights_bf16, size_t bytes) {
   Ctx &c = h->c;
   const size_t need = (size_t)kMlpWeights * 2;
   if (!weights_bf16 || bytes != need) return fail(c, HFMM_ERR_ARG, "weights must be 5512 BF16 values (11024 bytes)");
-  cudaError_t e = ensure(c.mlp_w, need);
-  if (e == cudaSuccess) e = cudaMemcpy(c.mlp_w.p, weights_bf16, need, cudaMemcpyHostToDevice);
+  const cudaError_t e = upload(c.mlp_w, weights_bf16, need, cudaStreamLegacy);
   if (e != cudaSuccess) return cuda_fail(c, e, "load_mlp");
   c.have_mlp = true;
   return HFMM_OK;
