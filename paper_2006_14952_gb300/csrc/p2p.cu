@@ -2,8 +2,9 @@
 // f_(1)(r) r of Sec. 2.2, kept for 0 < r < R_c), added to the L2P accelerations
 // already in the caller's particle order (the un-permute).
 //
-// One warp per work item: a chunk of up to 32 sinks of a leaf, taken from a
-// global work counter in longest-first order (k_lpt_hist / k_lpt_place below).
+// One warp per work item: a leaf's first 32 sinks, or the others in chunks of 32 (more
+// than one such chunk only for a leaf at the depth cap, which may hold any number of
+// particles), taken from a global work counter in longest-first order (k_lpt_hist / k_lpt_place below).
 // The source particles of all leaves on the sink's list are streamed through per-warp
 // shared memory in fills of up to kCap particles.  A fill takes the next 32
 // list entries (a prefix scan of their particle counts gives each candidate
@@ -106,8 +107,8 @@ __global__ void __launch_bounds__(256, 2) k_p2p(const uint32_t *__restrict__ ite
   extern __shared__ float4 p2p_smem[];
   __shared__ float4 part[8][32];  // a shared item's sums, by warp and sink
   __shared__ unsigned next_shared, n_shared;
-  // work items: a leaf's chunk of up to 32 sinks (leaf index, chunk in bit 31); not ordered (lpt null):
-  // two for every leaf, the second possibly empty
+  // work items: a leaf's first 32 sinks, or (bit 31 beside the leaf's index) the others; not ordered
+  // (lpt null): two for every leaf, the second possibly empty
   const unsigned nl = lpt ? lpt->n_items : 2u * (unsigned)tree_leaves(tz, n_leaves);
   unsigned *taken = reinterpret_cast<unsigned *>(ctr);  // items handed out: to warps, to blocks
   if (threadIdx.x < 32) {
@@ -273,7 +274,7 @@ __global__ void __launch_bounds__(256, 2) k_p2p(const uint32_t *__restrict__ ite
       return tot;
     };
 
-    const uint32_t cfirst = r.x + 32u * (item >> 31), cend = min(cfirst + 32u, r.x + r.y);
+    const uint32_t cfirst = r.x + 32u * (item >> 31), cend = item >> 31 ? r.x + r.y : min(cfirst + 32u, r.x + r.y);
     for (uint32_t cbase = cfirst; cbase < cend; cbase += 32) {
       const uint32_t rem = r.x + r.y - cbase;
       const int cs = rem < 32 ? (int)rem : 32;
@@ -474,6 +475,7 @@ __global__ void __launch_bounds__(256, 2) k_p2p(const uint32_t *__restrict__ ite
           acc_out[n + o] += G * sy;
           acc_out[2 * n + o] += G * sz;
         }
+        if (cbase + 32u < cend) __syncthreads();  // part is rewritten by the next chunk
       }
     }
   }
@@ -491,8 +493,8 @@ __global__ void __launch_bounds__(256, 2) k_p2p(const uint32_t *__restrict__ ite
 // 1.40 -> 1.02 ms at 262k clustered particles, 0.91 -> 0.59 at 300k (polynomial
 // split), nothing at 2M, where no item is that heavy.  Shared from 2^13: 0.48
 // instead of 0.41 ms at 100k uniform; every item above half a share, whatever its
-// size: 0.15 instead of 0.115 at 32k.  An item is one chunk of up to 32 sinks of a leaf
-// (leaves of 33..64 particles give two, so the heaviest leaves' work is split
+// size: 0.15 instead of 0.115 at 32k.  An item is a leaf's first 32 sinks or its
+// others (leaves of 33..64 particles give two, so the heaviest leaves' work is split
 // between two warps; the chunks' sums are independent, so the forces do not
 // change).  An item's work is about the leaf's list entries times its sinks;
 // items are bucketed by the binary order of magnitude of that (coarse buckets
@@ -517,7 +519,7 @@ __global__ void k_lpt_hist(const uint32_t *__restrict__ leaves, int64_t nl, Node
     for (uint32_t c = 0; c < 2; ++c) {
       uint8_t b = 0xff;
       if (ent > 0 && 32u * c < cnt) {
-        const uint32_t cs = min(32u, cnt - 32u * c);
+        const uint32_t cs = c ? cnt - 32u : min(32u, cnt);
         b = (uint8_t)__clzll((unsigned long long)ent * cs);  // heavier: smaller bucket index
         atomicAdd(&h[b], 1u);
         work += (unsigned long long)ent * cs;
@@ -616,7 +618,6 @@ cudaError_t run_p2p(Ctx &c, const Nodes &nodes, float *acc, cudaStream_t st) {
                                                          P<uint32_t>(c.lpt_order), tz);
     note_launch(2);
   }
-  if (c.prm.leaf_max > 64) return cudaErrorInvalidValue;  // two chunks per leaf at most
   kern<<<g, T, dyn, st>>>(P<uint32_t>(c.lpt_order), nodes, P<uint32_t>(c.p2p_beg), P<uint32_t>(c.p2p_end),
                         P<uint64_t>(c.p2p), P<float4>(c.pm4), P<uint32_t>(c.idx), c.n, fit2, (float)c.prm.G, acc, ctr, lpt,
                         P<uint32_t>(c.leaves), c.nleaves, tz);
