@@ -447,36 +447,39 @@ __global__ void __launch_bounds__(256) k_p2p_reactions(const uint32_t *__restric
     const uint32_t b = leaves[t];
     const uint2 rb = range[b];
     const uint32_t lo = rbeg[b], hi = rend[b];
-    float sx0 = 0.f, sy0 = 0.f, sz0 = 0.f, sx1 = 0.f, sy1 = 0.f, sz1 = 0.f;
-    for (uint32_t i0 = lo; i0 < hi; i0 += 32) {
-      // the partial offsets of the next 32 entries, one per lane, then broadcast
-      uint32_t po = 0;
-      if (i0 + lane < hi) po = poff[ents[i0 + lane]];
-      const int m = hi - i0 < 32u ? (int)(hi - i0) : 32;
+    if (hi <= lo) continue;
+    // 64 particles at a time (more only in a leaf at the depth cap)
+    for (uint32_t p0 = lane; p0 < (rb.y + 31u) / 32u * 32u; p0 += 64) {
+      const bool v0 = p0 < rb.y, v1 = p0 + 32u < rb.y;
+      float sx0 = 0.f, sy0 = 0.f, sz0 = 0.f, sx1 = 0.f, sy1 = 0.f, sz1 = 0.f;
+      for (uint32_t i0 = lo; i0 < hi; i0 += 32) {
+        // the partial offsets of the next 32 entries, one per lane, then broadcast
+        uint32_t po = 0;
+        if (i0 + lane < hi) po = poff[ents[i0 + lane]];
+        const int m = hi - i0 < 32u ? (int)(hi - i0) : 32;
 #pragma unroll 4
-      for (int j = 0; j < m; ++j) {
-        const uint64_t base = __shfl_sync(0xffffffffu, po, j);
-        if ((uint32_t)lane < rb.y) {
-          sx0 += part[base + lane];
-          sy0 += part[npart + base + lane];
-          sz0 += part[2 * npart + base + lane];
-        }
-        if ((uint32_t)lane + 32u < rb.y) {
-          sx1 += part[base + lane + 32];
-          sy1 += part[npart + base + lane + 32];
-          sz1 += part[2 * npart + base + lane + 32];
+        for (int j = 0; j < m; ++j) {
+          const uint64_t base = (uint64_t)__shfl_sync(0xffffffffu, po, j) + p0;
+          if (v0) {
+            sx0 += part[base];
+            sy0 += part[npart + base];
+            sz0 += part[2 * npart + base];
+          }
+          if (v1) {
+            sx1 += part[base + 32];
+            sy1 += part[npart + base + 32];
+            sz1 += part[2 * npart + base + 32];
+          }
         }
       }
-    }
-    if (hi > lo) {
-      if ((uint32_t)lane < rb.y) {
-        const uint32_t o = perm[rb.x + lane];
+      if (v0) {
+        const uint32_t o = perm[rb.x + p0];
         acc_out[o] += G * sx0;
         acc_out[n + o] += G * sy0;
         acc_out[2 * n + o] += G * sz0;
       }
-      if ((uint32_t)lane + 32u < rb.y) {
-        const uint32_t o = perm[rb.x + lane + 32];
+      if (v1) {
+        const uint32_t o = perm[rb.x + p0 + 32];
         acc_out[o] += G * sx1;
         acc_out[n + o] += G * sy1;
         acc_out[2 * n + o] += G * sz1;

@@ -14,22 +14,26 @@ pytestmark = pytest.mark.gpu
 
 
 def crowded(n, crowd, seed):
-    """n uniform particles, the first `crowd` of them moved to one point, in input order at random."""
+    """n uniform particles, 2 `crowd` of them moved to two points, in input order at random.
+    (Mutual P2P: of two leaves the deeper one owns a pair, so only two such leaves react.)"""
     rng = np.random.default_rng(seed)
     pos, mass = W.uniform(n, seed)
     pos[:, :crowd] = np.array([0.3137, 0.7071, 0.5772])[:, None]
+    pos[:, crowd:2 * crowd] = np.array([0.4142, 0.6931, 0.6180])[:, None]
     order = rng.permutation(n)
-    return np.ascontiguousarray(pos[:, order]), mass, order < crowd
+    return np.ascontiguousarray(pos[:, order]), mass, order < 2 * crowd
 
 
-@pytest.mark.parametrize("opts", [{}, {"sink_batches": 3}, {"split": 1}], ids=["plain", "batches", "poly"])
+@pytest.mark.parametrize("opts", [{}, {"sink_batches": 3}, {"split": 1}, {"p2p_mutual": 1}],
+                         ids=["plain", "batches", "poly", "mutual"])
 @pytest.mark.parametrize("n", [700, 12000])
 @pytest.mark.parametrize("crowd", [65, 96, 100, 300])
 def test_theta_zero_equals_direct_sum(crowd, n, opts):
-    pos, mass, is_crowd = crowded(n + crowd, crowd, 31 + crowd)
+    pos, mass, is_crowd = crowded(n + 2 * crowd, crowd, 31 + crowd)
     s, acc = run_gpu(pos, mass, pm_grid=24, theta=0.0, leaf_max=16, **opts)
     assert (s.get_stats()["nleaves"] < 512) == (n == 700)
-    assert s.export("nodes")[:, 5].max() >= crowd
+    nodes = s.export("nodes")
+    assert (nodes[nodes[:, 6] < 0, 5] == crowd).sum() == 2
     ref = oracle.direct_sr(pos, mass, 1.0, s.rs, s.rc, **({"split": "poly"} if opts.get("split") else {}))
     for which in (slice(None), is_crowd):
         a, r = acc[:, which], ref[:, which]
