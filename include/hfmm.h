@@ -159,6 +159,9 @@ typedef struct {
                           HFMM_EXPORT_KEYS and HFMM_EXPORT_NODES are octree only
                           (HFMM_EXPORT_KD_NODES and _KD_BOXES describe this tree).  The conventional
                           walk of hfmm_interaction_counts uses the same boxes and opening order. */
+  int wait_polls;      /* polls of the octree walk's bounded waits (for a cell whose parent is being
+                          visited) before the call gives up with HFMM_ERR_TIMEOUT (0 = 2^22; -1 = none
+                          at all: a test of the error path) */
 } hfmm_params;
 
 /* Counters and timings of the last build_tree / short_range_forces call. */

@@ -22,7 +22,8 @@ int fail(Ctx &c, int code, const std::string &msg) {
 }
 
 int cuda_fail(Ctx &c, cudaError_t e, const char *where) {
-  int code = e == cudaErrorMemoryAllocation ? HFMM_ERR_OOM : HFMM_ERR_CUDA;
+  // (cudaErrorTimeout: the walk's own, for a wait that gave up)
+  int code = e == cudaErrorMemoryAllocation ? HFMM_ERR_OOM : e == cudaErrorTimeout ? HFMM_ERR_TIMEOUT : HFMM_ERR_CUDA;
   c.err = std::string(where) + ": " + cudaGetErrorString(e);
   return code;
 }
@@ -54,6 +55,7 @@ bool valid_params(const hfmm_params &p, std::string &why) {
   if (p.list_init < 0) return why = "list_init must be >= 0", false;
   if (p.sink_batches < 0 || p.sink_batches > 4096) return why = "sink_batches must be in 0..4096", false;
   if (p.tc_wait_polls < -1) return why = "tc_wait_polls must be >= -1", false;
+  if (p.wait_polls < -1) return why = "wait_polls must be >= -1", false;
   if (p.split != 0 && p.split != 1) return why = "split must be 0 (Gaussian) or 1 (polynomial)", false;
   if (p.split == 1 && (p.mac_mode != 0 || p.m2l_precision != 0 || p.m2l_tables != 0))
     return why = "split 1 needs mac_mode 0, m2l_precision 0 and m2l_tables 0", false;

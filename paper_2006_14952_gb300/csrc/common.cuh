@@ -460,6 +460,10 @@ struct StepGuard {
   const int *tree_overflow = nullptr, *walk_overflow = nullptr;
 };
 StepGuard step_guard(Ctx &c);
+// The polls a bounded wait of the walk takes before it gives up (hfmm_params.wait_polls).
+inline unsigned wait_polls(const Ctx &c, unsigned usual) {
+  return c.prm.wait_polls > 0 ? (unsigned)c.prm.wait_polls : c.prm.wait_polls < 0 ? 0u : usual;
+}
 cudaError_t kick_guarded(float *vel, const float *acc, int64_t n, double h, StepGuard g, cudaStream_t st);
 // vel += h acc and pos += dt vel (wrapped), [3][n] arrays.
 cudaError_t kick(float *vel, const float *acc, int64_t n, double h, cudaStream_t st);

@@ -173,7 +173,7 @@ struct TravState {
   unsigned next, tail;                   // queue of cells with children: tickets handed out, cells put in
   int cells_left;                        // cells put in and not finished
   unsigned leaf_next;                    // leaves handed out
-  int overflow;                          // 1: a list did not fit, 3: the tree did not fit, 4: a wait gave up
+  int overflow;                          // the largest of 1: a list did not fit, 3: the tree did not, 4: a wait gave up
   int ovf_lists;                         // bit 0 M2L, 1 P2P, 2 open lists
   int levels;                            // levels of the deepest pair, less one
 };
@@ -196,6 +196,7 @@ struct WalkArgs {
   uint32_t *spill;                       // per warp: staged entries beyond the stage
   long long leaf_lo, leaf_hi;            // a batch of leaves, by position in `leaves`
   int what;                              // kWalkAll, kWalkCells, kWalkLeaves
+  unsigned polls;                        // of a node's slot before the wait gives up
 };
 
 enum : int { kWalkAll = 0, kWalkCells = 1, kWalkLeaves = 2 };
@@ -207,7 +208,8 @@ constexpr int kStack = 512;  // nodes a leaf's walk has still to visit
 constexpr int kStage = 480;  // entries staged in shared memory
 constexpr int kSpillP = 4096, kSpillM = 2048;  // entries a warp can put aside in memory
 constexpr size_t kSpillBytes = (size_t)(kSpillP + kSpillM) * 5;
-constexpr unsigned kWaitPolls = 1u << 22;  // of a node's slot, about a microsecond each
+constexpr unsigned kWaitPolls = 1u << 22;  // about a microsecond each
+constexpr uint32_t kGaveUp = ~0u;          // in place of a cell
 template <bool kNet>
 struct WalkSize {
   static constexpr int kNetWait = kNet ? 64 : 0;  // candidates waiting for the network
@@ -495,7 +497,7 @@ __device__ __forceinline__ void walk_sink(const WalkArgs &A, const Mac &m, const
         }
         if ((cm && !fit_m) || (cp && !fit_p)) {
           atomicOr(&A.st->ovf_lists, (cm && !fit_m ? 1 : 0) | (cp && !fit_p ? 2 : 0));
-          atomicExch(&A.st->overflow, 1);
+          atomicMax(&A.st->overflow, 1);
         }
       }
     } else {
@@ -525,7 +527,7 @@ __device__ __forceinline__ void walk_sink(const WalkArgs &A, const Mac &m, const
           const bool fm = bm + all_m <= A.cap_m2l, fp = bp + all_p <= A.cap_open;
           if (!fm || !fp) {
             atomicOr(&A.st->ovf_lists, (fm ? 0 : 1) | (fp ? 0 : 4));
-            atomicExch(&A.st->overflow, 1);
+            atomicMax(&A.st->overflow, 1);
           }
           if (fm && all_m) {
             A.mb[sink] = A.mm[sink] = (uint32_t)bm;
@@ -583,7 +585,8 @@ __device__ __forceinline__ void walk_sink(const WalkArgs &A, const Mac &m, const
 // once its parent is done.  Done cells put theirs into a queue; each block takes
 // the next ticket and waits for its cell.  A cell is put in at most once; when
 // none is left unfinished the queue is complete, and the tickets beyond its end
-// go on to the leaves: handed out to warps from a counter.  (Sink batches: a
+// go on to the leaves: handed out to warps from a counter.  A block whose wait for
+// a cell gives up leaves there: the open lists are not complete.  (Sink batches: a
 // launch for the first phase, then one for each range of the leaves.)
 //
 // What bounds it: the first phase by latency, one session a level along the
@@ -647,13 +650,14 @@ __global__ void __launch_bounds__(kTT, kNet ? 3 : 4) k_walk(const __grid_constan
   uint32_t maxlev = 0;
   grid.sync();
   volatile TravState *vst = A.st;
+  bool lost = false;
   if (A.what != kWalkLeaves) {
     for (;;) {
       if (tid == 0) {
         const unsigned t = atomicAdd(&A.st->next, 1u);
         uint32_t k = 0;
         unsigned poll = 0;
-        for (; poll < kWaitPolls; ++poll) {
+        for (; poll < A.polls; ++poll) {
           if ((long long)t < nn) k = *(volatile uint32_t *)(A.queue + t);
           if (k) break;
           if (vst->cells_left == 0) {  // complete (read before the tail): nothing more will come
@@ -662,13 +666,17 @@ __global__ void __launch_bounds__(kTT, kNet ? 3 : 4) k_walk(const __grid_constan
           }
           __nanosleep(poll < 64 ? 20 : 200);
         }
-        if (poll == kWaitPolls) atomicExch(&A.st->overflow, 4);
+        if (poll == A.polls) {
+          atomicMax(&A.st->overflow, 4);
+          k = kGaveUp;
+        }
         __threadfence();  // the parent's open list was written before the slot
         B.cell = k;
       }
       __syncthreads();
       const uint32_t k = B.cell;
-      if (k == 0) break;
+      lost = k == kGaveUp;
+      if (k == 0 || lost) break;
       const Node a = unpack_node(A.wn[k - 1]);
       walk_sink<kNet, false>(A, m, mf, k - 1, a, W, B, spill, sw, xs[wp], dec[wp], items, maxlev);
       // the open list, then the children's slots, then this cell is finished
@@ -686,7 +694,7 @@ __global__ void __launch_bounds__(kTT, kNet ? 3 : 4) k_walk(const __grid_constan
   }
   const long long leaf_lo = A.what == kWalkLeaves ? A.leaf_lo : 0,
                   leaf_hi = A.what == kWalkAll ? (long long)ts->nleaves : A.leaf_hi;
-  for (;;) {
+  while (!lost) {
     unsigned t = 0;
     if (lane == 0) t = atomicAdd(&A.st->leaf_next, 1u);
     t = __shfl_sync(0xffffffffu, t, 0);
@@ -902,6 +910,7 @@ cudaError_t walk_launch(Ctx &c, const WalkPlan &w, cudaStream_t st, const WalkPa
   A.what = part.what;
   A.leaf_lo = part.leaf_lo;
   A.leaf_hi = part.leaf_hi;
+  A.polls = wait_polls(c, kWaitPolls);
   Mac m = w.m;
   const bool net = m.mode == 1;
   const void *kern = net ? (const void *)k_walk<true> : (const void *)k_walk<false>;
@@ -950,7 +959,7 @@ cudaError_t walk_part(Ctx &c, const WalkPlan &w, const WalkPart &part, cudaStrea
     if ((e = walk_launch(c, w, st, part)) != cudaSuccess) return e;
     if ((e = walk_read(c, st, hs)) != cudaSuccess) return e;
     if (!hs.overflow) return cudaSuccess;
-    if (hs.overflow == 4) return cudaErrorLaunchTimeout;
+    if (hs.overflow == 4) return cudaErrorTimeout;  // HFMM_ERR_TIMEOUT
     walk_grow(c, hs);
   }
   return cudaErrorInvalidValue;
