@@ -184,7 +184,6 @@ cudaError_t collect_pairs(Ctx &c, int64_t max_pairs, uint32_t sample_mod, float 
   if ((e = ensure(c.cand, (size_t)(max_pairs > 0 ? max_pairs : 1) * 8)) != cudaSuccess) return e;
   c.cand_cap = (uint64_t)max_pairs;
   c.sample_mod = sample_mod ? sample_mod : 1u;
-  if ((e = cudaMemsetAsync(P<uint64_t>(c.d_small) + 7, 0, 8, st)) != cudaSuccess) return e;
   size_t eb = (size_t)c.nnodes * c.ldm * sizeof(float);
   if ((e = ensure(c.M, eb)) != cudaSuccess) return e;
   if ((e = upward(c, st)) != cudaSuccess) return e;

@@ -912,6 +912,8 @@ cudaError_t walk_launch(Ctx &c, const WalkPlan &w, cudaStream_t st, const WalkPa
   A.leaf_hi = part.leaf_hi;
   A.polls = wait_polls(c, kWaitPolls);
   Mac m = w.m;
+  // collected candidates: those of this walk alone (a walk whose lists overflowed is repeated)
+  if (m.mode == 2 && (e = cudaMemsetAsync(m.ncand, 0, 8, st)) != cudaSuccess) return e;
   const bool net = m.mode == 1;
   const void *kern = net ? (const void *)k_walk<true> : (const void *)k_walk<false>;
   void *args[] = {(void *)&A, (void *)&m};
