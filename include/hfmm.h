@@ -159,9 +159,11 @@ typedef struct {
                           HFMM_EXPORT_KEYS and HFMM_EXPORT_NODES are octree only
                           (HFMM_EXPORT_KD_NODES and _KD_BOXES describe this tree).  The conventional
                           walk of hfmm_interaction_counts uses the same boxes and opening order. */
-  int wait_polls;      /* polls of the octree walk's bounded waits (for a cell whose parent is being
-                          visited) before the call gives up with HFMM_ERR_TIMEOUT (0 = 2^22; -1 = none
-                          at all: a test of the error path) */
+  int wait_polls;      /* polls of the bounded waits inside a kernel (0 = the defaults below; -1 = none at
+                          all: a test of what comes after).  The octree walk's, for a cell whose parent
+                          is being visited (2^22): the call gives up with HFMM_ERR_TIMEOUT.  Those of
+                          the key sorts and of the k-d build's partition, for the counts of the tiles
+                          before (2^20): the tile counts by itself, with the same result. */
 } hfmm_params;
 
 /* Counters and timings of the last build_tree / short_range_forces call. */

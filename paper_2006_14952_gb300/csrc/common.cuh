@@ -242,16 +242,20 @@ cudaError_t scan_u32(const uint32_t *in, uint32_t *out, uint64_t *total, size_t 
 
 // Stable LSD radix sort of uint64 keys on bits [bit_lo, bit_hi), optionally
 // carrying uint32 values.  Ping-pongs between (keys, vals) and (keys_alt,
-// vals_alt); returns in *in_alt whether the result ended in the alt buffers.
+// vals_alt); returns in *in_alt whether the result ended in the alt buffers.  A tile's
+// wait for its predecessors' counts takes look_polls polls at most (0: no look at all)
+// and then counts by itself, with the same result.
+constexpr unsigned kLookPolls = 1u << 20;
 cudaError_t radix_sort_u64(uint64_t *keys, uint32_t *vals, uint64_t *keys_alt, uint32_t *vals_alt, size_t n,
-                           int bit_lo, int bit_hi, bool *in_alt, DBuf &tmp, cudaStream_t st);
+                           int bit_lo, int bit_hi, bool *in_alt, DBuf &tmp, cudaStream_t st,
+                           unsigned look_polls = kLookPolls);
 
 // The same sort with all scratch in a caller-provided region (no allocation);
 // radix_sort_scratch_bytes(n) is the size that region needs.
 size_t radix_sort_scratch_bytes(size_t n);
 cudaError_t radix_sort_u64_into(uint64_t *keys, uint32_t *vals, uint64_t *keys_alt, uint32_t *vals_alt, size_t n,
                                 int bit_lo, int bit_hi, bool *in_alt, void *scratch, size_t scratch_bytes,
-                                cudaStream_t st);
+                                cudaStream_t st, unsigned look_polls = kLookPolls);
 
 // ---------------------------------------------------------------- pair force
 // 1/L when the box side L is a power of two (then exact), else 0
@@ -460,7 +464,7 @@ struct StepGuard {
   const int *tree_overflow = nullptr, *walk_overflow = nullptr;
 };
 StepGuard step_guard(Ctx &c);
-// The polls a bounded wait of the walk takes before it gives up (hfmm_params.wait_polls).
+// The polls a bounded wait of the tree build or the walk takes before it gives up (hfmm_params.wait_polls).
 inline unsigned wait_polls(const Ctx &c, unsigned usual) {
   return c.prm.wait_polls > 0 ? (unsigned)c.prm.wait_polls : c.prm.wait_polls < 0 ? 0u : usual;
 }

@@ -202,11 +202,11 @@ __global__ void k_kd_side(int64_t n, int level, const int *__restrict__ axis, Kd
 // side flags, the flags of all tiles before (published counts, looked back over), less
 // those of the nodes before, whose second children are known from the counts alone.
 constexpr int kPartItems = 8, kPartTile = kT * kPartItems;
-constexpr unsigned kPartPolls = 1u << 20;
 __global__ void __launch_bounds__(kT) k_kd_part(int64_t n, int level, KdOrders O, uint32_t *__restrict__ r0,
                                                 uint32_t *__restrict__ r1, uint32_t *__restrict__ r2,
                                                 const uint8_t *__restrict__ side, unsigned *__restrict__ ticket,
-                                                volatile unsigned long long *look, unsigned ntiles) {
+                                                volatile unsigned long long *look, unsigned ntiles,
+                                                unsigned look_polls) {
   __shared__ uint32_t wsum[kT / 32];
   __shared__ unsigned tile_s;
   __shared__ unsigned long long before_s;
@@ -242,13 +242,13 @@ __global__ void __launch_bounds__(kT) k_kd_part(int64_t n, int level, KdOrders O
     if (lane == 0) look[tile] = (t == 0 ? kInc : kAgg) | all;
     // look back, 32 tiles at a time: up to the nearest published inclusive count
     unsigned long long before = 0;
-    bool lost = false;
-    for (long long at = (long long)t - 1; at >= 0;) {
+    bool lost = look_polls == 0;
+    for (long long at = (long long)t - 1; at >= 0 && !lost;) {
       unsigned long long x = kInc;  // before the order's first tile: nothing
       for (unsigned poll = 0;; ++poll) {
         if (at - lane >= 0) x = look[d * ntiles + (unsigned)(at - lane)];
         if (__all_sync(0xffffffffu, (x >> 62) != 0)) break;
-        if (poll == kPartPolls) {
+        if (poll == look_polls) {
           lost = true;
           break;
         }
@@ -972,7 +972,7 @@ cudaError_t kd_build_tree(Ctx &c, const double *pos, const float *mass, int64_t 
     note_launch();
     bool alt = false;
     TRY(radix_sort_u64(P<uint64_t>(c.key), P<uint32_t>(kd.ord[d]), P<uint64_t>(c.key_alt), P<uint32_t>(kd.ord2[d]),
-                       (size_t)n, 0, 64, &alt, c.tmp, st));
+                       (size_t)n, 0, 64, &alt, c.tmp, st, wait_polls(c, kLookPolls)));
     if (alt) std::swap(kd.ord[d], kd.ord2[d]);
   }
   if (c.prm.profile & 1) cudaEventRecord(c.ev[1], st);
@@ -996,7 +996,8 @@ cudaError_t kd_build_tree(Ctx &c, const double *pos, const float *mass, int64_t 
       unsigned long long *lw = P<unsigned long long>(c.tmp2) + (size_t)l * words;
       k_kd_part<<<3 * ntiles, kT, 0, st>>>(n, l, orders(), P<uint32_t>(kd.ord2[0]), P<uint32_t>(kd.ord2[1]),
                                            P<uint32_t>(kd.ord2[2]), P<uint8_t>(kd.side),
-                                           reinterpret_cast<unsigned *>(lw), lw + 1, ntiles);
+                                           reinterpret_cast<unsigned *>(lw), lw + 1, ntiles,
+                                           wait_polls(c, kLookPolls));
       note_launch(3);
       for (int d = 0; d < 3; ++d) std::swap(kd.ord[d], kd.ord2[d]);
     }

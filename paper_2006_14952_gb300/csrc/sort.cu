@@ -196,7 +196,7 @@ cudaError_t scan_u32(const uint32_t *in, uint32_t *out, uint64_t *total, size_t 
 // values): 2M 0.44 -> 0.29 ms, 16M 2.95 -> 1.6, 32k 0.23 -> 0.08, 1000 0.19 -> 0.02.
 //
 // Tiles are numbered in the order their blocks start, so every predecessor is
-// already running.  A look-back that has polled kLookPolls times gives up waiting
+// already running.  A look-back that has polled look_polls times gives up waiting
 // and counts the digits before its tile from the keys themselves: slow, but it
 // ends, with the same result.
 namespace {
@@ -204,7 +204,6 @@ namespace {
 constexpr int kSortThreads = 256;
 constexpr int kSortWarps = kSortThreads / 32;
 constexpr int kMaxPasses = 8;
-constexpr unsigned kLookPolls = 1u << 20;
 constexpr int kLookAhead = 4;
 // scratch: digit totals of all passes, tickets, then two look-back tables used in turn
 // (a pass clears the table of the next one)
@@ -261,7 +260,7 @@ __global__ void __launch_bounds__(kSortThreads, 3) k_radix_pass(const uint64_t *
                                                              size_t n, int shift, uint32_t mask,
                                                              const uint32_t *__restrict__ hist,
                                                              unsigned *__restrict__ ticket, volatile Word *look,
-                                                             Word *__restrict__ clear) {
+                                                             Word *__restrict__ clear, unsigned look_polls) {
   constexpr int kTile = kSortThreads * kItems;
   constexpr int kFlag = 8 * (int)sizeof(Word) - 2;
   constexpr Word kCount = ((Word)1 << kFlag) - 1;
@@ -314,7 +313,7 @@ __global__ void __launch_bounds__(kSortThreads, 3) k_radix_pass(const uint64_t *
   const uint32_t local = block_exclusive_scan<uint32_t>(c, nullptr);
   const unsigned long long base = block_exclusive_scan<unsigned long long>(hist[tid], nullptr);
   unsigned long long before = 0;
-  bool lost = false;
+  bool lost = tile > 0 && look_polls == 0;
   if (tile > 0) {
     // kLookAhead predecessors' words in flight at a time: the first wave's tiles all look back
     // over each other's aggregates, and one load a step made that the longest part of a pass
@@ -338,7 +337,7 @@ __global__ void __launch_bounds__(kSortThreads, 3) k_radix_pass(const uint64_t *
         found = flag == 2;  // the first tile publishes nothing else
         --t;
       }
-      if (wait && ++polls > kLookPolls) lost = true;
+      if (wait && ++polls > look_polls) lost = true;
     }
   }
   if (__syncthreads_or(lost)) {  // count the digits before this tile from the keys
@@ -464,7 +463,7 @@ cudaError_t radix_block(uint64_t *keys, uint32_t *vals, size_t n, int bit_lo, in
 
 template <bool kVals, int kItems, class Word>
 cudaError_t radix_passes(uint64_t *ka, uint32_t *va, uint64_t *kb, uint32_t *vb, size_t n, int bit_lo, int bit_hi,
-                         bool *in_alt, void *scratch, cudaStream_t st) {
+                         bool *in_alt, void *scratch, unsigned look_polls, cudaStream_t st) {
   const unsigned ntiles = (unsigned)sort_tiles(n);
   uint32_t *hist = static_cast<uint32_t *>(scratch);
   unsigned *ticket = hist + kMaxPasses * 256;
@@ -485,7 +484,8 @@ cudaError_t radix_passes(uint64_t *ka, uint32_t *va, uint64_t *kb, uint32_t *vb,
   for (int sh = bit_lo; sh < bit_hi; sh += 8, ++pass) {
     const uint32_t mask = bit_hi - sh < 8 ? (1u << (bit_hi - sh)) - 1u : 255u;
     kern<<<ntiles, kSortThreads, smem, st>>>(alt ? kb : ka, alt ? vb : va, alt ? ka : kb, alt ? va : vb, n, sh, mask,
-                                             hist + 256 * pass, ticket + pass, look[pass & 1], look[(pass + 1) & 1]);
+                                             hist + 256 * pass, ticket + pass, look[pass & 1], look[(pass + 1) & 1],
+                                             look_polls);
     note_launch();
     alt = !alt;
   }
@@ -499,7 +499,7 @@ size_t radix_sort_scratch_bytes(size_t n) { return kSortHead + 2 * sort_tiles(n)
 
 cudaError_t radix_sort_u64_into(uint64_t *keys, uint32_t *vals, uint64_t *keys_alt, uint32_t *vals_alt, size_t n,
                                 int bit_lo, int bit_hi, bool *in_alt, void *scratch, size_t scratch_bytes,
-                                cudaStream_t st) {
+                                cudaStream_t st, unsigned look_polls) {
   *in_alt = false;
   if (n <= 1 || bit_hi <= bit_lo) return cudaSuccess;
   if (radix_sort_scratch_bytes(n) > scratch_bytes || bit_hi - bit_lo > 8 * kMaxPasses) return cudaErrorInvalidValue;
@@ -512,7 +512,9 @@ cudaError_t radix_sort_u64_into(uint64_t *keys, uint32_t *vals, uint64_t *keys_a
                      : n <= 4096 ? block(radix_block<false, 4>) : block(radix_block<false, 8>);
   }
   const bool small = sort_items(n) == 8, wide = sort_word(n) == 8;
-  auto run = [&](auto f) { return f(keys, vals, keys_alt, vals_alt, n, bit_lo, bit_hi, in_alt, scratch, st); };
+  auto run = [&](auto f) {
+    return f(keys, vals, keys_alt, vals_alt, n, bit_lo, bit_hi, in_alt, scratch, look_polls, st);
+  };
   if (vals)
     return small ? run(radix_passes<true, 8, uint32_t>)
                  : wide ? run(radix_passes<true, 16, uint64_t>) : run(radix_passes<true, 16, uint32_t>);
@@ -521,12 +523,13 @@ cudaError_t radix_sort_u64_into(uint64_t *keys, uint32_t *vals, uint64_t *keys_a
 }
 
 cudaError_t radix_sort_u64(uint64_t *keys, uint32_t *vals, uint64_t *keys_alt, uint32_t *vals_alt, size_t n,
-                           int bit_lo, int bit_hi, bool *in_alt, DBuf &tmp, cudaStream_t st) {
+                           int bit_lo, int bit_hi, bool *in_alt, DBuf &tmp, cudaStream_t st, unsigned look_polls) {
   *in_alt = false;
   if (n <= 1 || bit_hi <= bit_lo) return cudaSuccess;
   const cudaError_t e = ensure(tmp, radix_sort_scratch_bytes(n));
   if (e != cudaSuccess) return e;
-  return radix_sort_u64_into(keys, vals, keys_alt, vals_alt, n, bit_lo, bit_hi, in_alt, tmp.p, tmp.cap, st);
+  return radix_sort_u64_into(keys, vals, keys_alt, vals_alt, n, bit_lo, bit_hi, in_alt, tmp.p, tmp.cap, st,
+                             look_polls);
 }
 
 }  // namespace hfmm

@@ -368,7 +368,7 @@ cudaError_t build_tree(Ctx &c, const double *pos, const float *mass, int64_t n, 
   note_launch();
   bool alt = false;
   TRY(radix_sort_u64(P<uint64_t>(c.key), P<uint32_t>(c.idx), P<uint64_t>(c.key_alt), P<uint32_t>(c.idx_alt), n, 0,
-                     63, &alt, c.tmp, st));
+                     63, &alt, c.tmp, st, wait_polls(c, kLookPolls)));
   if (alt) {
     std::swap(c.key, c.key_alt);
     std::swap(c.idx, c.idx_alt);
@@ -437,7 +437,7 @@ cudaError_t build_tree_launch(Ctx &c, const double *pos, const float *mass, int6
   note_launch();
   bool alt = false;
   if ((e = radix_sort_u64(P<uint64_t>(c.key), P<uint32_t>(c.idx), P<uint64_t>(c.key_alt), P<uint32_t>(c.idx_alt), n,
-                          0, 63, &alt, c.tmp, st)) != cudaSuccess)
+                          0, 63, &alt, c.tmp, st, wait_polls(c, kLookPolls))) != cudaSuccess)
     return e;
   if (alt) {
     std::swap(c.key, c.key_alt);
