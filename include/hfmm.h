@@ -385,7 +385,8 @@ int hfmm_mlp_infer(const void *weights_bf16, const float *features, int64_t n, f
  * Mean softmax cross-entropy over n samples and its gradient (device
  * pointers): weights = FP32 master copy [5512] (rounded to BF16 in the
  * forward pass, as the inference does), labels [n] in 0..7, class_weights
- * [8] or NULL; grad [5512] and loss [1] are written.  Uses ctx's scratch.
+ * [8] or NULL (with them, a sample of another label weighs nothing); grad [5512] and
+ * loss [1] are written.  Uses ctx's scratch.
  */
 int hfmm_mlp_grad(hfmm_ctx *ctx, const float *weights, const float *features, const int32_t *labels,
                   const float *class_weights, int64_t n, float *grad, float *loss, void *stream);

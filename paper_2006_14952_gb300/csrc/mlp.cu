@@ -220,7 +220,11 @@ __global__ void __launch_bounds__(kGradThreads, 3) k_mlp_grad(const float *__res
       if (t < 2) a[3] = pack_bf16(x[i8 * kMlpIn + 8 + 2 * t], x[i8 * kMlpIn + 9 + 2 * t]);
     }
     const int lab0 = v0 ? labels[i0] : -1, lab8 = v8 ? labels[i8] : -1;
-    const float wg0 = v0 ? (cw ? cw[lab0] : 1.f) : 0.f, wg8 = v8 ? (cw ? cw[lab8] : 1.f) : 0.f;
+    // (class weights cover the labels 0..7: another label has none)
+    auto weight = [&](bool valid, int lab) {
+      return !valid ? 0.f : !cw ? 1.f : (unsigned)lab < (unsigned)kMlpOut ? cw[lab] : 0.f;
+    };
+    const float wg0 = weight(v0, lab0), wg8 = weight(v8, lab8);
     {
       // the gradient's copy: column 12 is one, so that column of d1^T x is the bias gradient
       uint32_t *q0 = reinterpret_cast<uint32_t *>(sx + r0 * kLdX), *q8 = reinterpret_cast<uint32_t *>(sx + r8 * kLdX);
