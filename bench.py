@@ -4,7 +4,7 @@ r_s = 1.25 cells, R_c = 4.5 r_s; solved with leaves <= 48, theta 0.35, p 6, the
 setting that meets the 1e-4 RMS accuracy bar), one GB300.
 
 One step = one pass of the whole short-range path over the resident particle
-set: wrap + Morton keys, sort, octree, P2M/M2M, traversal, list grouping, M2L,
+set: wrap + Morton keys, sort, octree, P2M/M2M, traversal, M2L,
 L2L, L2P + P2P, accelerations in input order.  L2 is flushed (a 512 MB write)
 before every timed step.  `value` counts particles with forces per second of
 device time (CUDA events on the launching stream); `e2e` repeats the step

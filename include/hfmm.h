@@ -169,7 +169,8 @@ typedef struct {
 /* Counters and timings of the last build_tree / short_range_forces call. */
 typedef struct {
   int64_t n, nnodes, nleaves;
-  int32_t nlevels, traverse_iters;
+  int32_t nlevels;
+  int32_t traverse_iters; /* tree levels the last walk met (octree: the deepest cell's; tree 1: levels walked) */
   int64_t np2p;           /* P2P leaf pairs */
   int64_t nm2l;           /* M2L cell pairs */
   int64_t p2p_particle_pairs; /* particle pairs evaluated by P2P incl. masked (profile bit 1, else -1) */

@@ -316,7 +316,7 @@ bool graph_eligible(const Ctx &c) {
 // The whole short-range call captured as one CUDA graph on the context's own
 // stream and replayed on `st`: upward pass, the walk (its list sizes stay on
 // the device: the lists have their capacities from the last call or the first
-// guess), list grouping (run counts read on the device), M2L, L2L/L2P and P2P.
+// guess), M2L, L2L/L2P and P2P.
 // Every buffer is sized before the capture.  After the graph, one read-back
 // of the walk's state: *ok is false when a list overflowed (the caller then
 // runs the direct path, which grows the lists).  With profiling the graph is
@@ -518,7 +518,7 @@ std::vector<uint64_t> step_signature(Ctx &c, const double *pos, const float *vel
 
 // The kick-drift-kick step as one CUDA graph (Sec. 4's synchronised step):
 // first kick, drift, the octree build (its sizes stay on the device), the
-// short-range call (upward pass, walk, list grouping, M2L, L2L/L2P, P2P), the
+// short-range call (upward pass, walk, M2L, L2L/L2P, P2P), the
 // PM long range and the second kick.  Kernels after the build read the tree's
 // extent from the device state and treat an overflowed tree as empty; the
 // second kick runs only when the tree and the walk fitted.  Buffers are sized

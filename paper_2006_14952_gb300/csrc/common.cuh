@@ -44,7 +44,7 @@ __host__ __device__ inline void mdecode(int c, int &nx, int &ny, int &nz) {
 
 // ---------------------------------------------------------------- lists
 // Packed (sink node, source node, shift, order) entry:
-//   bits 61..63  expansion order - 1 of an M2L entry (0 for P2P and frontier entries)
+//   bits 61..63  expansion order - 1 of an M2L entry (0 for P2P entries)
 //   bits 34..60  sink node (27 bits)
 //   bit  33      M2L entries: 1 = the operator is evaluated per pair, 0 = it is read
 //                from the (level, offset) table (sorting on bits 33.. puts a sink's
@@ -226,8 +226,6 @@ extern thread_local std::vector<void *> *g_deferred_free;
 // ordered after it (a synchronous copy from pageable memory may return before its transfer,
 // and a non-blocking stream does not wait for the stream it runs on).
 cudaError_t upload(DBuf &b, const void *src, size_t bytes, cudaStream_t st);
-// Grow b to at least `bytes`, keeping the first `keep` bytes (stream-ordered copy).
-cudaError_t ensure_keep(DBuf &b, size_t bytes, size_t keep, cudaStream_t st);
 void release(DBuf &b);
 
 template <class T>
@@ -267,9 +265,10 @@ inline double box_inverse_if_pow2(double box) {
 // S(x) = erfc(x/2) + x e^(-x^2/4) / sqrt(pi) = exp2(r^2 kexp) Q(x), x = r / r_s,
 // Q(x) = e^(x^2/4) erfc(x/2) + x / sqrt(pi), kexp = -log2(e) / (4 r_s^2).  Q is
 // evaluated as sum_k c[k] v^k + a r, v = r / (1 + p r): the first part decays like
-// 1/x, which a degree-4 polynomial in v follows to 5.5e-7 at R_c = 4.5 r_s (a
-// polynomial in r needs degree 9 for 1.2e-6), and v = 1 / (1/r + p) is one
-// reciprocal.
+// 1/x, which a degree-4 polynomial in v follows, and v = 1 / (1/r + p) is one
+// reciprocal.  Largest relative error of the fit, and of a polynomial of degree 9 in r:
+// at R_c = 2 r_s 3.4e-8 and 2.4e-9 (FP32 rounds at 6e-8), 3 r_s 8e-8 and 6e-8, 4.5 r_s
+// 5.5e-7 and 1.2e-6, 6 r_s 9.8e-7 and 7.8e-6, 10 r_s 4.5e-6 and 1.4e-4.
 struct PairFit {
   float c[5], a, p, rc2, kexp;
 };
@@ -297,7 +296,7 @@ struct KdTree {
   DBuf ctr;                      // u64 [16]: the walk's counters
   std::vector<int64_t> level_start;
   int64_t cap = 0;
-  uint64_t caps[3] = {0, 0, 0};  // frontier, M2L and P2P capacities of the last walk
+  uint64_t caps[3] = {0, 0, 0};  // open-list, M2L and P2P capacities of the last walk
 };
 
 struct Ctx {

@@ -820,8 +820,6 @@ cudaError_t read_u64(Ctx &c, const void *src, uint64_t *out, int count, cudaStre
   return cudaSuccess;
 }
 
-KdGeo kd_geo(Ctx &c) { return KdGeo{P<double>(c.kd.geo), P<float>(c.kd.geof), c.kd.cap}; }
-
 // The walk (one cooperative launch, repeated with grown buffers while one is outgrown).
 cudaError_t kd_walk(Ctx &c, cudaStream_t st, bool conventional = false) {
   KdTree &kd = c.kd;

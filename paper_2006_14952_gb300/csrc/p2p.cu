@@ -602,8 +602,9 @@ cudaError_t run_p2p(Ctx &c, const Nodes &nodes, float *acc, cudaStream_t st) {
   if (e == cudaSuccess) e = cudaMemsetAsync(ctr, 0, 8, st);
   if (e != cudaSuccess) return e;
   // The leaves longest first; below kLptMin each has a warp to itself at once whatever the
-  // order, and no list is long enough to be shared (a work of 2^14 takes 512 entries): two
-  // launches less, 1000 uniform particles 162 -> 150 us a call.
+  // order: two launches less, 1000 uniform particles 162 -> 150 us a call.  No item is shared
+  // by a block there: its work of 2^14 takes 512 entries, more than the leaves unless some
+  // occur under several shifts (a cut-off near half the box).
   const TreeState *tz = c.graph_tree ? P<TreeState>(c.tstate) : nullptr;
   LptState *lpt = nullptr;
   if (c.nleaves >= kLptMin) {

@@ -1,5 +1,6 @@
 // Device primitives: buffer growth, exclusive scan and a stable LSD radix sort.
-// Used by the tree build (Morton-key sort) and the list grouping by sink.
+// Used by the tree builds (key sorts), the M2L lists of the learned acceptance and the
+// operator tables, and the mutual P2P.
 #include <vector>
 
 #include "common.cuh"
@@ -28,30 +29,6 @@ cudaError_t ensure(DBuf &b, size_t bytes) {
     b.p = nullptr;
     return e;
   }
-  b.cap = want;
-  return cudaSuccess;
-}
-
-cudaError_t ensure_keep(DBuf &b, size_t bytes, size_t keep, cudaStream_t st) {
-  if (bytes <= b.cap) return cudaSuccess;
-  size_t want = bytes + bytes / 2 + 256;
-  void *np = nullptr;
-  cudaError_t e = cudaMalloc(&np, want);
-  if (e != cudaSuccess) return e;
-  if (b.p && keep) {
-    e = cudaMemcpyAsync(np, b.p, keep, cudaMemcpyDeviceToDevice, st);
-    if (e != cudaSuccess) {
-      cudaFree(np);
-      return e;
-    }
-    e = cudaStreamSynchronize(st);
-    if (e != cudaSuccess) {
-      cudaFree(np);
-      return e;
-    }
-  }
-  if (b.p) cudaFree(b.p);
-  b.p = np;
   b.cap = want;
   return cudaSuccess;
 }
@@ -183,7 +160,8 @@ cudaError_t scan_u32(const uint32_t *in, uint32_t *out, uint64_t *total, size_t 
 }
 
 // ------------------------------------------------------------------ radix sort
-// Stable LSD radix sort, 8 bits a pass, one kernel a pass: a tile's keys are
+// Stable LSD radix sort, 8 bits a pass, one kernel a pass (decoupled look-back: Merrill
+// and Garland 2016, "Single-pass parallel prefix scan with decoupled look-back"): a tile's keys are
 // ranked in registers and shared memory, the tile finds the number of equal
 // digits before it by looking back over its predecessors' published counts, and
 // writes its keys out in digit order (runs of a digit are contiguous).  The digit
