@@ -601,18 +601,32 @@ constexpr int kStack = 512, kSoft = 448;  // sources a sink has still to visit
 constexpr int kStage = 1024;              // entries staged in shared memory
 constexpr int kWalkWarpWords = kStack + kStage;
 
-// One sink's session, a warp: every pair (sink, b, s) the walk meets is classified.  The
+constexpr int kKdWarps = kT / 32;
+// A group of warps that share a session: its part of the block's shared memory, and its barrier.
+struct KdGroup {
+  unsigned long long bm, bp;
+  uint32_t nm[kKdWarps], np[kKdWarps];
+};
+__device__ __forceinline__ void kd_sync(int group, int warps) {
+  asm volatile("bar.sync %0, %1;" ::"r"(group + 1), "r"(32 * warps) : "memory");
+}
+
+// One sink's session, a warp's or (kShared) that of a group of `warps` warps, each its part
+// of the parent's list: every pair (sink, b, s) the walk meets is classified.  The
 // pairs start from those its parent left open (the root: its 27 images, or itself alone in
 // the conventional walk).  The larger of the two opens, at equal sizes both, and only a node
 // with children: a source that opens alone stays with this sink (its children go on a
 // stack), and where the sink opens, alone or with the source, the source or its children go
 // to the open list both its children start from.  The M2L entries and the P2P or open
-// entries are staged, their ranges taken with one atomic per list at the end; a session with
+// entries are staged, their ranges taken with one atomic per list at the end (a group's
+// entries in warp order); a session with
 // more entries than the stage holds counts them and walks again, writing in place.
 // Above kSoft waiting the stack is taken one source at a time: each adds one at most per
 // level of the tree (27 levels: node numbers are below 2^27), so it holds.
+template <bool kShared>
 __device__ __forceinline__ void kd_session(const KdWalk &W, uint32_t k, int level, uint32_t *stack, uint32_t *stage,
-                                           unsigned long long *nopen, unsigned long long &items) {
+                                           KdGroup *groups, int warps, unsigned long long *nopen,
+                                           unsigned long long &items) {
   const int lane = threadIdx.x & 31;
   const unsigned lt = (1u << lane) - 1u;
   float4 A0, A1;
@@ -627,13 +641,21 @@ __device__ __forceinline__ void kd_session(const KdWalk &W, uint32_t k, int leve
     ibeg = W.obeg[p];
     icnt = W.ocnt[p];
   }
+  const int group = (threadIdx.x >> 5) / warps, wp = (threadIdx.x >> 5) % warps;
+  KdGroup &B = groups[kShared ? group : 0];
+  uint32_t ifirst = 0;
+  if (kShared) {
+    const uint32_t share = (icnt + warps - 1) / warps;
+    ifirst = min(share * wp, icnt);
+    icnt = min(ifirst + share, icnt);
+  }
   uint64_t *const m2l = W.m2l, *const p2p = W.p2p;
   uint32_t *const out = W.open[level & 1];
   unsigned long long bm = 0, bp = 0;
   bool fit_m = false, fit_p = false;
   uint32_t nm = 0, np = 0;  // M2L entries; P2P (a leaf's) or open entries
   for (int pass = 0; pass < 2; ++pass) {
-    uint32_t pi = 0;
+    uint32_t pi = ifirst;
     int sp = 0;
     bool over = false;
     nm = np = 0;
@@ -715,25 +737,54 @@ __device__ __forceinline__ void kd_session(const KdWalk &W, uint32_t k, int leve
       __syncwarp();
     }
     if (pass == 1) break;
-    // ---- the entries' ranges
-    if (lane == 0) {
-      if (nm) bm = atomicAdd(W.ctr + 0, (unsigned long long)nm);
-      if (np) bp = atomicAdd(leaf ? W.ctr + 1 : nopen, (unsigned long long)np);
-    }
-    bm = __shfl_sync(0xffffffffu, bm, 0);
-    bp = __shfl_sync(0xffffffffu, bp, 0);
-    fit_m = nm > 0 && bm + nm <= W.cap_m2l;
-    fit_p = np > 0 && bp + np <= (leaf ? W.cap_p2p : W.cap_open);
-    if (lane == 0) {
-      W.mb[k] = (uint32_t)bm;
-      W.me[k] = (uint32_t)bm + (fit_m ? nm : 0u);
-      W.pb[k] = leaf ? (uint32_t)bp : 0u;
-      W.pe[k] = leaf ? (uint32_t)bp + (fit_p ? np : 0u) : 0u;
-      if (!leaf) {
-        W.obeg[k] = bp;
-        W.ocnt[k] = fit_p ? np : 0u;
+    // ---- the entries' ranges: the sink's, and in them this warp's
+    uint32_t all_m = nm, all_p = np, before_m = 0, before_p = 0;
+    if (kShared) {
+      if (lane == 0) {
+        B.nm[wp] = nm;
+        B.np[wp] = np;
+      }
+      kd_sync(group, warps);
+      all_m = all_p = 0;
+      for (int q = 0; q < warps; ++q) {
+        if (q == wp) {
+          before_m = all_m;
+          before_p = all_p;
+        }
+        all_m += B.nm[q];
+        all_p += B.np[q];
       }
     }
+    if (lane == 0 && (!kShared || wp == 0)) {
+      if (all_m) bm = atomicAdd(W.ctr + 0, (unsigned long long)all_m);
+      if (all_p) bp = atomicAdd(leaf ? W.ctr + 1 : nopen, (unsigned long long)all_p);
+      if (kShared) {
+        B.bm = bm;
+        B.bp = bp;
+      }
+    }
+    if (kShared) {
+      kd_sync(group, warps);
+      bm = B.bm;
+      bp = B.bp;
+    } else {
+      bm = __shfl_sync(0xffffffffu, bm, 0);
+      bp = __shfl_sync(0xffffffffu, bp, 0);
+    }
+    fit_m = all_m > 0 && bm + all_m <= W.cap_m2l;
+    fit_p = all_p > 0 && bp + all_p <= (leaf ? W.cap_p2p : W.cap_open);
+    if (lane == 0 && (!kShared || wp == 0)) {
+      W.mb[k] = (uint32_t)bm;
+      W.me[k] = (uint32_t)bm + (fit_m ? all_m : 0u);
+      W.pb[k] = leaf ? (uint32_t)bp : 0u;
+      W.pe[k] = leaf ? (uint32_t)bp + (fit_p ? all_p : 0u) : 0u;
+      if (!leaf) {
+        W.obeg[k] = bp;
+        W.ocnt[k] = fit_p ? all_p : 0u;
+      }
+    }
+    bm += before_m;
+    bp += before_p;
     if (!over) {
       if (fit_m)
         for (uint32_t i = lane; i < nm; i += 32) m2l[bm + i] = pack_pair(k, 0, 0) | stage[kStage - 1 - i];
@@ -765,6 +816,7 @@ __global__ void __launch_bounds__(kT, 4) k_kd_walk(const __grid_constant__ KdWal
   extern __shared__ uint32_t walk_smem[];
   const int lane = threadIdx.x & 31;
   uint32_t *stack = walk_smem + (threadIdx.x >> 5) * kWalkWarpWords, *stage = stack + kStack;
+  __shared__ KdGroup groups[kKdWarps / 2];
   const bool first = blockIdx.x == 0 && threadIdx.x == 0;
   const int levels = W.S.depth + 1 + (W.S.nsplit ? 1 : 0);
   unsigned long long items = 0, most = 0;
@@ -774,12 +826,19 @@ __global__ void __launch_bounds__(kT, 4) k_kd_walk(const __grid_constant__ KdWal
     const uint32_t hi = level <= W.S.depth ? (uint32_t)(((int64_t)2 << level) - 1) : (uint32_t)W.S.nodes();
     unsigned long long *nopen = W.ctr + 5 + level % 3, *ticket = W.ctr + 8 + level % 3;
     if (first) W.ctr[5 + (level + 1) % 3] = W.ctr[8 + (level + 1) % 3] = 0;
-    for (;;) {
-      unsigned long long t = 0;
-      if (lane == 0) t = atomicAdd(ticket, 1ull);
-      t = __shfl_sync(0xffffffffu, t, 0);
-      if (t >= hi - lo) break;
-      kd_session(W, lo + (uint32_t)t, level, stack, stage, nopen, items);
+    int warps = kKdWarps;  // a session's: as many as leave every node of the level a group
+    while (warps > 1 && hi - lo > gridDim.x * (uint32_t)(kKdWarps / warps)) warps >>= 1;
+    if (warps > 1) {
+      const uint32_t t = blockIdx.x * (uint32_t)(kKdWarps / warps) + (threadIdx.x >> 5) / warps;
+      if (t < hi - lo) kd_session<true>(W, lo + t, level, stack, stage, groups, warps, nopen, items);
+    } else {
+      for (;;) {
+        unsigned long long t = 0;
+        if (lane == 0) t = atomicAdd(ticket, 1ull);
+        t = __shfl_sync(0xffffffffu, t, 0);
+        if (t >= hi - lo) break;
+        kd_session<false>(W, lo + (uint32_t)t, level, stack, stage, groups, 1, nopen, items);
+      }
     }
     grid.sync();
     // every block reads the same count, and so takes the same decision; the M2L and P2P
@@ -844,7 +903,8 @@ cudaError_t kd_walk(Ctx &c, cudaStream_t st, bool conventional = false) {
   TRY(cudaFuncSetAttribute(k_kd_walk, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
   TRY(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_kd_walk, kT, smem));
   if (per_sm < 1) return cudaErrorInvalidConfiguration;
-  const unsigned nb = (unsigned)(nsm * std::min(per_sm, 4));
+  // two warps a leaf at most: a level's barrier costs more the more blocks it spans
+  const unsigned nb = std::min((unsigned)(nsm * std::min(per_sm, 4)), blocks_for((size_t)nl, 4));
   KdWalk W;
   W.S = kd_shape(c.n, c.prm.leaf_max);
   W.G = KdGeo{P<double>(kd.geo), P<float>(kd.geof), kd.cap};
