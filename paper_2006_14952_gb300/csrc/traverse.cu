@@ -209,7 +209,6 @@ constexpr int kStage = 480;  // entries staged in shared memory
 constexpr int kSpillP = 4096, kSpillM = 2048;  // entries a warp can put aside in memory
 constexpr size_t kSpillBytes = (size_t)(kSpillP + kSpillM) * 5;
 constexpr unsigned kWaitPolls = 1u << 22;  // about a microsecond each
-constexpr uint32_t kGaveUp = ~0u;          // in place of a cell
 template <bool kNet>
 struct WalkSize {
   static constexpr int kNetWait = kNet ? 64 : 0;  // candidates waiting for the network
@@ -220,6 +219,7 @@ struct WalkSize {
 struct BlockMem {
   unsigned long long base_m, base_p;
   uint32_t cnt_m[kTW], cnt_p[kTW], fit, put, at, cell;
+  uint32_t lost;  // a wait gave up
 };
 
 // A warp's shared memory.
@@ -599,7 +599,10 @@ __device__ __forceinline__ void walk_sink(const WalkArgs &A, const Mac &m, const
 // 0.21 (262k clustered, leaf 48), 3.07 -> 1.12 (2M clustered), 6.7 -> 3.6 (2M with
 // the network).  A warp a session instead of a block, with the leaves in the same
 // queue: 1.08 at 2M, but 0.14 at 32k and 0.41 at 262k.
-template <bool kNet>
+//
+// kPolls: the wait's limit from the arguments (hfmm_params.wait_polls).  As a variable in
+// every launch it cost the network's walk a third (3.6 -> 4.8 ms at 2M particles).
+template <bool kNet, bool kPolls>
 __global__ void __launch_bounds__(kTT, kNet ? 3 : 4) k_walk(const __grid_constant__ WalkArgs A,
                                                            const __grid_constant__ Mac m) {
   cg::grid_group grid = cg::this_grid();
@@ -637,6 +640,7 @@ __global__ void __launch_bounds__(kTT, kNet ? 3 : 4) k_walk(const __grid_constan
   }
   if (kNet) mlp_stage(m.w, sw);
   mac_f(m, mf);
+  if (tid == 0) B.lost = 0u;
   WarpMem W;
   W.cand = reinterpret_cast<uint32_t *>(wsm + (size_t)wp * WalkSize<kNet>::kWarpBytes);
   W.net = W.cand + kCand;
@@ -650,14 +654,14 @@ __global__ void __launch_bounds__(kTT, kNet ? 3 : 4) k_walk(const __grid_constan
   uint32_t maxlev = 0;
   grid.sync();
   volatile TravState *vst = A.st;
-  bool lost = false;
+  const unsigned polls = kPolls ? A.polls : kWaitPolls;
   if (A.what != kWalkLeaves) {
     for (;;) {
       if (tid == 0) {
         const unsigned t = atomicAdd(&A.st->next, 1u);
         uint32_t k = 0;
         unsigned poll = 0;
-        for (; poll < A.polls; ++poll) {
+        for (; poll < polls; ++poll) {
           if ((long long)t < nn) k = *(volatile uint32_t *)(A.queue + t);
           if (k) break;
           if (vst->cells_left == 0) {  // complete (read before the tail): nothing more will come
@@ -666,17 +670,16 @@ __global__ void __launch_bounds__(kTT, kNet ? 3 : 4) k_walk(const __grid_constan
           }
           __nanosleep(poll < 64 ? 20 : 200);
         }
-        if (poll == A.polls) {
+        if (poll == polls) {
           atomicMax(&A.st->overflow, 4);
-          k = kGaveUp;
+          B.lost = 1u;
         }
         __threadfence();  // the parent's open list was written before the slot
         B.cell = k;
       }
       __syncthreads();
       const uint32_t k = B.cell;
-      lost = k == kGaveUp;
-      if (k == 0 || lost) break;
+      if (k == 0) break;
       const Node a = unpack_node(A.wn[k - 1]);
       walk_sink<kNet, false>(A, m, mf, k - 1, a, W, B, spill, sw, xs[wp], dec[wp], items, maxlev);
       // the open list, then the children's slots, then this cell is finished
@@ -693,8 +696,8 @@ __global__ void __launch_bounds__(kTT, kNet ? 3 : 4) k_walk(const __grid_constan
     }
   }
   const long long leaf_lo = A.what == kWalkLeaves ? A.leaf_lo : 0,
-                  leaf_hi = A.what == kWalkAll ? (long long)ts->nleaves : A.leaf_hi;
-  while (!lost) {
+                  leaf_hi = B.lost ? 0 : A.what == kWalkAll ? (long long)ts->nleaves : A.leaf_hi;
+  for (;;) {
     unsigned t = 0;
     if (lane == 0) t = atomicAdd(&A.st->leaf_next, 1u);
     t = __shfl_sync(0xffffffffu, t, 0);
@@ -777,6 +780,11 @@ struct WalkPlan {
   unsigned nb;
 };
 
+const void *walk_kernel(const Ctx &c, bool net) {
+  if (c.prm.wait_polls) return net ? (const void *)k_walk<true, true> : (const void *)k_walk<false, true>;
+  return net ? (const void *)k_walk<true, false> : (const void *)k_walk<false, false>;
+}
+
 size_t walk_smem(bool net) {
   return (size_t)kTW * (net ? WalkSize<true>::kWarpBytes : WalkSize<false>::kWarpBytes);
 }
@@ -809,7 +817,7 @@ cudaError_t walk_plan(Ctx &c, WalkPlan &w) {
   if ((e = cudaGetDevice(&dev)) != cudaSuccess) return e;
   if ((e = cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev)) != cudaSuccess) return e;
   const bool net = m.mode == 1;
-  const void *kern = net ? (const void *)k_walk<true> : (const void *)k_walk<false>;
+  const void *kern = walk_kernel(c, net);
   const size_t smem = walk_smem(net);
   if ((e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem)) != cudaSuccess) return e;
   e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, kTT, smem);
@@ -915,7 +923,7 @@ cudaError_t walk_launch(Ctx &c, const WalkPlan &w, cudaStream_t st, const WalkPa
   // collected candidates: those of this walk alone (a walk whose lists overflowed is repeated)
   if (m.mode == 2 && (e = cudaMemsetAsync(m.ncand, 0, 8, st)) != cudaSuccess) return e;
   const bool net = m.mode == 1;
-  const void *kern = net ? (const void *)k_walk<true> : (const void *)k_walk<false>;
+  const void *kern = walk_kernel(c, net);
   void *args[] = {(void *)&A, (void *)&m};
   e = cudaLaunchCooperativeKernel(kern, dim3(w.nb), dim3(kTT), args, walk_smem(net), st);
   note_launch();
