@@ -802,15 +802,18 @@ __device__ __forceinline__ void kd_session(const KdWalk &W, uint32_t k, int leve
 
 // The whole walk in one cooperative launch, the tree's levels in turn with a grid-wide
 // barrier between them (an open list is complete before the children start from it), a
-// level's nodes to warps from a counter, until the last level or open lists that outgrow
+// level's nodes to warps (a large level's from a counter), until the last level or open lists that outgrow
 // their buffer (the caller grows the buffers that were outgrown and walks again).  Each
 // sink's entries lie together, in an order that does not depend on the schedule.
 //
 // What bounds it: instructions, in the last two levels (two thirds of the pairs); the levels
-// above by latency, one session and one barrier each.  A walk over a frontier of (sink,
+// above by latency, one session and one barrier each: there a group of as many warps shares
+// a session as leaves every node of the level a group (one warp a session everywhere, the
+// walk alone: 121 -> 94 us at 2000 clustered particles, 271 -> 191 at 30k, 436 -> 345 at 100k,
+// 1.46 -> 1.24 ms at 2M).  A walk over a frontier of (sink,
 // source) pairs, two entries of 8 bytes written and read a pair, left lists to be sorted
 // by (sink, source, shift): 2.0 + 1.5 ms for 46M pairs and 21M entries (2M clustered
-// particles) instead of 1.46.
+// particles) instead of 1.24.
 __global__ void __launch_bounds__(kT, 4) k_kd_walk(const __grid_constant__ KdWalk W) {
   cg::grid_group grid = cg::this_grid();
   extern __shared__ uint32_t walk_smem[];
